@@ -22,133 +22,190 @@ namespace sb {
 
 namespace {
 
-constexpr int PRE_RC = 64;  // rows of L_k per partial of z_k(c)
+// An SM's FP64 pipe takes one warp instruction per 19 cycles (64 per scheduler) whatever
+// its active lanes: the two passes over the L_k are bound by their 1.5 K d^2 FMAs (24 us at
+// d = 1024, K = 8; the bytes 5 us), the small kernels by their chains of dependent FP64
+// instructions, which are spread over lanes (an exponential per lane). Device time of the
+// five launches at d = 1024, K = 8 (cold caches): 297 us -> 85 us, the two passes 114 -> 49.
+constexpr int PRE_RC = 32;    // rows of L_k per partial of z_k(c)
+constexpr int PRE_COLS = 128; // columns per CTA of z_k(c)
 
-// part[k][chunk][j] = sum over rows i of the chunk (i >= j) of L_k[i][j] (c_i - mu_k,i)
-__global__ void __launch_bounds__(256) k_pre_z0_part(int d, const double *L, const double *mu, const double *c,
-                                                     double *part) {
-    const int chunk = blockIdx.x, k = blockIdx.y, nch = gridDim.x;
+// part[k][chunk][j] = sum over rows i of the chunk (i >= j) of L_k[i][j] (c_i - mu_k,i): one
+// CTA per 32 x 128 tile of the triangle, so that every SM gets a share of the FMAs (whole
+// 64-row chunks: 84 us at d = 1024, K = 8)
+__global__ void __launch_bounds__(PRE_COLS) k_pre_z0_part(int d, const double *L, const double *mu, const double *c,
+                                                          double *part) {
+    __shared__ double dl[PRE_RC];
+    const int chunk = blockIdx.y, k = blockIdx.z, nch = gridDim.y;
     const int i0 = chunk * PRE_RC, i1 = min(d, i0 + PRE_RC);
+    if ((int)blockIdx.x * PRE_COLS >= i1) return;
     const double *Lk = L + (size_t)k * d * d;
     const double *mk = mu + (size_t)k * d;
-    for (int j = threadIdx.x; j < d; j += blockDim.x) {
-        double acc = 0.0;
-        for (int i = max(i0, j); i < i1; ++i) acc += Lk[(size_t)i * d + j] * (c[i] - mk[i]);
-        part[((size_t)k * nch + chunk) * d + j] = acc;
+    if (threadIdx.x < PRE_RC && i0 + (int)threadIdx.x < d) dl[threadIdx.x] = c[i0 + threadIdx.x] - mk[i0 + threadIdx.x];
+    __syncthreads();
+    const int j = blockIdx.x * PRE_COLS + threadIdx.x;
+    if (j >= i1) return;
+    double acc = 0.0;
+    if (j <= i0 && i1 - i0 == PRE_RC) {
+#pragma unroll 16
+        for (int r = 0; r < PRE_RC; ++r) acc = fma(Lk[(size_t)(i0 + r) * d + j], dl[r], acc);
+    } else {
+        for (int i = max(i0, j); i < i1; ++i) acc = fma(Lk[(size_t)i * d + j], dl[i - i0], acc);
     }
+    part[((size_t)k * nch + chunk) * d + j] = acc;
 }
 
-// z0[k][j] = sum of the partials (chunk order); e0[k] = a_k - |z0_k|^2 / 2
-__global__ void __launch_bounds__(256) k_pre_z0_fin(int d, int nch, const double *part, const double *a, double *z0,
-                                                    double *e0) {
-    __shared__ double sh[256 / 32];
-    const int k = blockIdx.x;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double ss = 0.0;
-    for (int j = threadIdx.x; j < d; j += blockDim.x) {
-        double z = 0.0;
-        for (int q = 0; q < nch; ++q) z += part[((size_t)k * nch + q) * d + j];
+// z0[k][j] = sum of the partials of the chunks that reach column j (chunk order), and the
+// block's share of |z0_k|^2 (one CTA per component took 31 us at d = 1024, K = 8)
+__global__ void __launch_bounds__(PRE_COLS) k_pre_z0_fin(int d, int nch, const double *part, double *z0, double *ssp) {
+    __shared__ double sh[PRE_COLS / 32];
+    const int k = blockIdx.y, j = blockIdx.x * PRE_COLS + threadIdx.x;
+    double z = 0.0;
+    if (j < d) {
+#pragma unroll 8
+        for (int q = j / PRE_RC; q < nch; ++q) z += part[((size_t)k * nch + q) * d + j];
         z0[(size_t)k * d + j] = z;
-        ss += z * z;
     }
-    ss = warp_sum(ss);
-    if (lane == 0) sh[wid] = ss;
+    const double ss = warp_sum(z * z);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ss;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < 256 / 32; ++w) t += sh[w];
-        e0[k] = a[k] - 0.5 * t;
+        for (int w = 0; w < PRE_COLS / 32; ++w) t += sh[w];
+        ssp[(size_t)k * gridDim.x + blockIdx.x] = t;
     }
 }
 
-// warp per (k, i): dot[k][i] = z0_k . L_k[i, :], nrm[k][i] = |L_k[i, :]|^2 (j <= i)
+// warp per two rows i, i + 1 of L_k: dot[k][i] = z0_k . L_k[i, :], nrm[k][i] = |L_k[i, :]|^2
+// (j <= i). The four sums are reduced together (each exchange halves the values a lane
+// holds): 6 FP64 adds for two rows instead of 20.
 __global__ void __launch_bounds__(256) k_pre_rows(int d, const double *L, const double *z0, double *dot, double *nrm) {
     const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), k = blockIdx.y;
+    const int i = 2 * (blockIdx.x * 8 + (threadIdx.x >> 5)), k = blockIdx.y;
     if (i >= d) return;
-    const double *row = L + ((size_t)k * d + i) * d;
+    const bool two = i + 1 < d;
+    const double *row0 = L + ((size_t)k * d + i) * d;
+    const double *row1 = two ? row0 + d : row0;
     const double *zk = z0 + (size_t)k * d;
-    double sd = 0.0, sn = 0.0;
-    for (int j = lane; j <= i; j += 32) {
-        const double v = row[j];
-        sd += v * zk[j];
-        sn += v * v;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};  // dot and norm of row i, of row i + 1
+    for (int j0 = 0; j0 <= i + 1; j0 += 128) {
+        double a[4], b[4], z[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 32 * u + lane;
+            a[u] = j <= i ? row0[j] : 0.0;
+            b[u] = two && j <= i + 1 ? row1[j] : 0.0;
+            z[u] = j <= i + 1 && j < d ? zk[j] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (j0 + 32 * u > i + 1) break;
+            v[0] = fma(a[u], z[u], v[0]);
+            v[1] = fma(a[u], a[u], v[1]);
+            v[2] = fma(b[u], z[u], v[2]);
+            v[3] = fma(b[u], b[u], v[3]);
+        }
     }
-    sd = warp_sum(sd);
-    sn = warp_sum(sn);
-    if (lane == 0) {
-        dot[(size_t)k * d + i] = sd;
-        nrm[(size_t)k * d + i] = sn;
-    }
+    // lanes with bit 16 keep row i + 1, lanes with bit 8 the norm
+    const bool h1 = lane & 16, h0 = lane & 8;
+    double p0 = (h1 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h1 ? v[0] : v[2], 16);
+    double p1 = (h1 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h1 ? v[1] : v[3], 16);
+    double q = (h0 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h0 ? p0 : p1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if ((lane & 7) == 0 && (!h1 || two)) (h0 ? nrm : dot)[(size_t)k * d + i + (h1 ? 1 : 0)] = q;
 }
 
-// l(c + t e_i) - l(c) for t = +-Delta_i, and s_i = |up| + |down|
-__global__ void __launch_bounds__(256) k_pre_sens(int d, int K, const double *e0, const double *dot,
-                                                  const double *nrm, const double *half, double *s) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d) return;
-    double m0 = -INFINITY;
-    for (int k = 0; k < K; ++k) m0 = fmax(m0, e0[k]);
-    double s0 = 0.0;
-    for (int k = 0; k < K; ++k) s0 += exp(e0[k] - m0);
-    const double l0 = m0 + log(s0);
-    const double t = half[i];
-    double out = 0.0;
-    for (int sgn = 0; sgn < 2; ++sgn) {
-        const double tt = sgn ? -t : t;
-        double m = -INFINITY;
-        for (int k = 0; k < K; ++k) {
-            const double v = (e0[k] - l0) - tt * dot[(size_t)k * d + i] - 0.5 * tt * tt * nrm[(size_t)k * d + i];
-            m = fmax(m, v);
-        }
-        double acc = 0.0;
-        for (int k = 0; k < K; ++k) {
-            const double v = (e0[k] - l0) - tt * dot[(size_t)k * d + i] - 0.5 * tt * tt * nrm[(size_t)k * d + i];
-            acc += exp(v - m);
-        }
-        out += fabs(m + log(acc));
+__device__ __forceinline__ double group8_sum(double v) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// up / down changes l(c +- Delta_i e_i) - l(c), s_i = |up| + |down|: eight lanes per
+// (coordinate, sign), lane q over the components q, q + 8, ... (an exponential is about 40
+// FP64 instructions; K of them in turn in each of d threads on d / 256 CTAs took 55 us)
+__global__ void __launch_bounds__(128) k_pre_sens(int d, int K, int nblk, const double *a, const double *ssp,
+                                                  const double *dot, const double *nrm, const double *half,
+                                                  double *s) {
+    __shared__ double s_e[kMaxK];
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        double t = 0.0;
+        for (int q = 0; q < nblk; ++q) t += ssp[(size_t)k * nblk + q];
+        s_e[k] = a[k] - 0.5 * t;
     }
-    s[i] = out;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, q = lane & 7;
+    double m0 = -INFINITY;
+    for (int k = 0; k < K; ++k) m0 = s_e[k] > m0 ? s_e[k] : m0;
+    double s0 = 0.0;
+    for (int k = q; k < K; k += 8) s0 += exp(s_e[k] - m0);
+    const double l0 = m0 + log(group8_sum(s0));
+    const int pair = blockIdx.x * 16 + (threadIdx.x >> 3);  // 2 i + sign
+    const int i = pair >> 1;
+    const bool live = i < d;
+    const double t = live ? ((pair & 1) ? -half[i] : half[i]) : 0.0;
+    auto term = [&](int k) {
+        return (s_e[k] - l0) - t * dot[(size_t)k * d + i] - 0.5 * t * t * nrm[(size_t)k * d + i];
+    };
+    double m = -INFINITY;
+    if (live)
+        for (int k = q; k < K; k += 8) m = fmax(m, term(k));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    double acc = 0.0;
+    if (live)
+        for (int k = q; k < K; k += 8) acc += exp(term(k) - m);
+    acc = group8_sum(acc);
+    const double out = live ? fabs(m + log(acc)) : 0.0;
+    const double other = __shfl_xor_sync(0xffffffffu, out, 8);  // the other sign of the coordinate
+    if (live && (lane & 15) == 0) s[i] = out + other;
 }
 
 constexpr int PRE_SORT = 1024;  // >= kMaxD
 
+// One CTA: the sort runs on order-preserving integer keys (FP64 compares share the SM's
+// two FP64 lanes) and the marginal terms are summed by a fixed tree; thread 0 walking the
+// d terms took most of this kernel's former 98 us at d = 1024.
 __global__ void __launch_bounds__(PRE_SORT) k_pre_classify(int d, const double *s, const double *half,
                                                           double eps_flat, double eps_soft, int8_t *cls,
                                                           double *log_int, double *log_vol, int32_t *n_active) {
-    __shared__ double v[PRE_SORT];
-    __shared__ double term_i[PRE_SORT], term_v[PRE_SORT];
-    __shared__ int s_nf;
-    const int t = threadIdx.x;
+    __shared__ uint64_t v[PRE_SORT];
+    __shared__ double sh_i[PRE_SORT / 32], sh_v[PRE_SORT / 32];
+    __shared__ int sh_n[PRE_SORT / 32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const double st = t < d ? s[t] : INFINITY;
-    v[t] = isfinite(st) ? st : INFINITY;
-    if (t == 0) s_nf = 0;
-    __syncthreads();
-    if (t < d && isfinite(st)) atomicAdd(&s_nf, 1);
+    v[t] = ordered_bits(isfinite(st) ? st : INFINITY);
+    const int nf = __syncthreads_count(t < d && isfinite(st));
+    int n2 = 2;  // the sort covers the power of two that holds d
+    while (n2 < d) n2 <<= 1;
     // bitonic sort, ascending (non-finite and padding as +inf at the end)
-    for (int size = 2; size <= PRE_SORT; size <<= 1) {
+    for (int size = 2; size <= n2; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            __syncthreads();
             const int p = t ^ stride;
-            if (p > t) {
+            if (t < n2 && p > t) {
                 const bool up = (t & size) == 0;
-                const double a = v[t], b = v[p];
+                const uint64_t a = v[t], b = v[p];
                 if ((a > b) == up) {
                     v[t] = b;
                     v[p] = a;
                 }
             }
+            __syncthreads();
         }
     }
-    __syncthreads();
-    const int nf = s_nf;
+    // the inverse of ordered_bits (the sensitivities are >= 0: the sign bit is set)
+    auto value = [&](int i) {
+        const uint64_t b = v[i];
+        return __longlong_as_double((long long)((b >> 63) ? b & 0x7fffffffffffffffull : ~b));
+    };
     double med = 0.0, smax = 0.0;
     if (nf > 0) {
-        med = (nf & 1) ? v[nf / 2] : 0.5 * (v[nf / 2 - 1] + v[nf / 2]);
-        smax = v[nf - 1];
+        med = (nf & 1) ? value(nf / 2) : 0.5 * (value(nf / 2 - 1) + value(nf / 2));
+        smax = value(nf - 1);
     }
-    term_i[t] = 0.0;
-    term_v[t] = 0.0;
+    double ti = 0.0, tv = 0.0;
+    int act = 0;
     if (t < d) {
         int8_t cl = 0;
         if (isfinite(st)) {
@@ -158,51 +215,62 @@ __global__ void __launch_bounds__(PRE_SORT) k_pre_classify(int d, const double *
                 cl = 2;
         }
         cls[t] = cl;
+        act = cl == 0;
         if (cl != 0) {
             const double w = log(2.0 * half[t]);
-            term_v[t] = w;
-            term_i[t] = cl == 1 ? w : 0.5 * SB_LOG_2PI + log(half[t] / sqrt(st));
+            tv = w;
+            ti = cl == 1 ? w : 0.5 * SB_LOG_2PI + log(half[t] / sqrt(st));
         }
     }
+    const int na = __popc(__ballot_sync(0xffffffffu, act));
+    if (__any_sync(0xffffffffu, t < d && !act)) {  // some coordinate of the warp is flagged
+        ti = warp_sum(ti);
+        tv = warp_sum(tv);
+    }
+    if (lane == 0) {
+        sh_i[wid] = ti;
+        sh_v[wid] = tv;
+        sh_n[wid] = na;
+    }
     __syncthreads();
-    if (t == 0) {
-        double li = 0.0, lv = 0.0;
-        int na = 0;
-        for (int i = 0; i < d; ++i) {
-            li += term_i[i];
-            lv += term_v[i];
-            na += cls[i] == 0;
+    if (t < 32) {
+        ti = warp_sum(sh_i[lane]);
+        tv = warp_sum(sh_v[lane]);
+        int n = sh_n[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+        if (lane == 0) {
+            *log_int = ti;
+            *log_vol = tv;
+            *n_active = n;
         }
-        *log_int = li;
-        *log_vol = lv;
-        *n_active = na;
     }
 }
 
 }  // namespace
 
 size_t precheck_scratch_elems(int d, int K) {
-    const int nch = (d + PRE_RC - 1) / PRE_RC;
-    return (size_t)K * nch * d + 3 * (size_t)K * d + (size_t)K;
+    const int nch = (d + PRE_RC - 1) / PRE_RC, nblk = (d + PRE_COLS - 1) / PRE_COLS;
+    return (size_t)K * nch * d + 3 * (size_t)K * d + (size_t)K * nblk;
 }
 
 void launch_precheck(const ProbView &pv, double eps_flat, double eps_soft, double *scratch, double *s, int8_t *cls,
                      double *log_int, double *log_vol, int32_t *n_active, cudaStream_t st) {
     const int d = pv.d, K = pv.K;
-    const int nch = (d + PRE_RC - 1) / PRE_RC;
+    const int nch = (d + PRE_RC - 1) / PRE_RC, nblk = (d + PRE_COLS - 1) / PRE_COLS;
     double *part = scratch;
     double *z0 = part + (size_t)K * nch * d;
     double *dot = z0 + (size_t)K * d;
     double *nrm = dot + (size_t)K * d;
-    double *e0 = nrm + (size_t)K * d;
+    double *ssp = nrm + (size_t)K * d;
     note_launch();
-    k_pre_z0_part<<<dim3(nch, K), 256, 0, st>>>(d, pv.L, pv.mu, pv.c, part);
+    k_pre_z0_part<<<dim3(nblk, nch, K), PRE_COLS, 0, st>>>(d, pv.L, pv.mu, pv.c, part);
     note_launch();
-    k_pre_z0_fin<<<K, 256, 0, st>>>(d, nch, part, pv.a, z0, e0);
+    k_pre_z0_fin<<<dim3(nblk, K), PRE_COLS, 0, st>>>(d, nch, part, z0, ssp);
     note_launch();
-    k_pre_rows<<<dim3((d + 7) / 8, K), 256, 0, st>>>(d, pv.L, z0, dot, nrm);
+    k_pre_rows<<<dim3((d + 15) / 16, K), 256, 0, st>>>(d, pv.L, z0, dot, nrm);
     note_launch();
-    k_pre_sens<<<(d + 255) / 256, 256, 0, st>>>(d, K, e0, dot, nrm, pv.half, s);
+    k_pre_sens<<<(2 * d + 15) / 16, 128, 0, st>>>(d, K, nblk, pv.a, ssp, dot, nrm, pv.half, s);
     note_launch();
     k_pre_classify<<<1, PRE_SORT, 0, st>>>(d, s, pv.half, eps_flat, eps_soft, cls, log_int, log_vol, n_active);
 }
