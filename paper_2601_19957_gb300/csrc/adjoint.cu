@@ -25,207 +25,317 @@
 //   gam'_k  = 2 r_k W (gbar - g_k),  t = sum_k (eps'_k g_k - P_k gam'_k).
 // tr(W P_k) = <W L_k, L_k>_F. Components with r_k == 0 contribute exactly zero
 // and are skipped. H is recomputed at every mode (not stored by the forward),
-// factored H = C C^T, and W is applied through triangular solves: W B =
-// C^-T (C^-1 B) for the d right-hand sides of L_k and for vectors. At a one-hot
-// mode (r_k = 1, the other r exactly 0) H = P_k and C = L_k, so W L_k = L_k^-T:
-// tr(W P_k) = d and lower[W L_k] = diag(1 / L_ii), with no d x d solve. Products
-// with P_k are formed as L_k (L_k^T v); P_k itself is built only for the Hessian
-// of a mode that is not one-hot.
+// factored H = C C^T, and C^-1 is formed once (its 32 x 32 diagonal blocks by
+// substitution, then pairs of blocks merged level by level), so that everything with W =
+// C^-T C^-1 is a product over all components at once: X_k = C^-1 L_k (lower triangular),
+// tr(W P_k) = |X_k|_F^2, the lower triangle of W L_k = C^-T X_k (added to dL_k as it
+// leaves the GEMM), and W v = C^-T (C^-1 v). At a one-hot mode (r_k = 1, the other r
+// exactly 0) H = P_k and C = L_k, so W L_k = L_k^-T: tr(W P_k) = d and lower[W L_k] =
+// diag(1 / L_ii), with no GEMM. Products with P_k are formed as L_k (L_k^T v); P_k itself
+// is built only for the Hessian of a mode that is not one-hot. Nothing is read back to
+// the host: every skip is decided from R and the one-hot flag on the device.
+//
+// The bound is the FP64 pipe (one warp instruction per 19 cycles and SM): per mode K d^3 /
+// 3 fused multiply-adds in the two GEMMs, d^3 / 6 each in the factor and its inverse.
 #include "sb_adjoint.cuh"
 
 namespace sb {
 
 namespace {
 
-constexpr int TB = 32;  // triangular-solve row block
+constexpr int TB = 32;  // output tile and K chunk of the GEMMs, block of the inverse's first level
 
-// ------------------------------------------------------------------ blocked TRSM, row-major B [d][n]
-// Right-looking: once row block I of X is solved, every later row block J takes
-// its update B_J -= A_JI X_I in one launch over (J, 64-column tile), so a launch
-// has up to (row blocks left) x n / 64 CTAs. Lower (X = C^-1 B): A_JI = C_JI for
-// J > I. Upper (X = C^-T B, row blocks in reverse): A_JI = (C_IJ)^T for J < I.
-__global__ void __launch_bounds__(256) k_trsm_right(int d, int n, int I, bool upper, const double *C, double *B) {
-    const int c0 = blockIdx.x * 64;
-    const int J = upper ? (int)blockIdx.y : I + 1 + (int)blockIdx.y;
-    const int rJ = J * TB, rI = I * TB;
-    __shared__ double As[TB][TB + 1];
-    __shared__ double Xs[TB][64 + 1];
-    const int tid = threadIdx.x, tc = tid & 63, tr = tid >> 6;  // 4 row groups x 64 columns
-    for (int e = tid; e < TB * TB; e += 256) {
-        const int i = e / TB, k = e % TB;
-        const int gi = rJ + i, gk = rI + k;
-        double v = 0.0;
-        if (gi < d && gk < d) v = upper ? C[(size_t)gk * d + gi] : C[(size_t)gi * d + gk];
-        As[i][k] = v;
-    }
-    for (int e = tid; e < TB * 64; e += 256) {
-        const int k = e / 64, c = e % 64;
-        const int gk = rI + k, gc = c0 + c;
-        Xs[k][c] = (gk < d && gc < n) ? B[(size_t)gk * n + gc] : 0.0;
-    }
-    __syncthreads();
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+// ------------------------------------------------------------------ C^-1 and the GEMMs
+// 32 x 32 output tiles, 256 threads with 2 x 2 outputs each, K chunks of 32: the longest
+// tile (a whole row of the triangle) is then d warp instructions per warp and output pair,
+// a sixth of the GEMM's time at d = 512; 64 x 64 tiles would put half of it on one SM.
+struct TileBuf {
+    double A[TB][TB + 1], B[TB][TB + 1];
+};
+
+// acc += sum over l in [l0, l1) of a(i, l) b(l, j) for the tile's rows i0 + ty (+16) and columns j0 + tx (+16);
+// a and b return zero outside their triangles.
+template <typename FA, typename FB>
+__device__ __forceinline__ void tile_gemm(TileBuf &sm, int l0, int l1, double (&acc)[2][2], FA a, FB b) {
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    for (int l = l0; l < l1; l += TB) {
 #pragma unroll
-    for (int k = 0; k < TB; ++k) {
-        const double x = Xs[k][tc];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[q] = fma(As[tr + 4 * q][k], x, acc[q]);
-    }
-    const int gc = c0 + tc;
-    if (gc < n)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int gi = rJ + tr + 4 * q;
-            if (gi < d) B[(size_t)gi * n + gc] -= acc[q];
+        for (int e = tid; e < TB * TB; e += 256) {
+            const int r = e >> 5, c = e & 31;
+            sm.A[r][c] = a(r, l + c);  // A[row][l]
+            sm.B[r][c] = b(l + r, c);  // B[l][column]
         }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < TB; ++q) {
+            const double a0 = sm.A[ty][q], a1 = sm.A[ty + 16][q];
+            const double b0 = sm.B[q][tx], b1 = sm.B[q][tx + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
+        }
+        __syncthreads();
+    }
 }
 
-// Diagonal block solve for 32 columns per CTA: the 32 x 32 block of B is staged
-// in shared memory, each warp solves four columns with lanes over rows (one
-// shuffle per unknown, multiplication by the diagonal's reciprocals).
-__global__ void __launch_bounds__(256) k_trsm_diag(int d, int n, int I, bool upper, const double *C, double *B) {
+// The inverses of the 32 x 32 diagonal blocks of C (identity past d): a warp per four
+// columns, lanes over rows, multiplication by the diagonal's reciprocals. Also zeroes the
+// rest of the block row, which the merges fill below the diagonal.
+__global__ void __launch_bounds__(256) k_inv_diag(int d, const double *C, double *Ci) {
     __shared__ double Cs[TB][TB + 1];
-    __shared__ double Bs[TB][TB + 1];
     __shared__ double inv[TB];
-    const int r0 = I * TB, c0 = blockIdx.x * TB;
-    const int rows = min(TB, d - r0);
-    for (int e = threadIdx.x; e < TB * TB; e += blockDim.x) {
-        const int i = e / TB, k = e % TB;
-        const int gi = r0 + i, gk = r0 + k;
-        double v = (i == k) ? 1.0 : 0.0;
-        if (gi < d && gk < d) v = upper ? C[(size_t)gk * d + gi] : C[(size_t)gi * d + gk];
-        Cs[i][k] = v;
-        Bs[i][k] = (i < rows && c0 + k < n) ? B[(size_t)(r0 + i) * n + c0 + k] : 0.0;
+    const int r0 = blockIdx.x * TB;
+    for (int e = threadIdx.x; e < TB * TB; e += 256) {
+        const int i = r0 + e / TB, j = r0 + e % TB;
+        Cs[e / TB][e % TB] = i < d && j <= i ? C[(size_t)i * d + j] : (i == j ? 1.0 : 0.0);
     }
     __syncthreads();
     if (threadIdx.x < TB) inv[threadIdx.x] = 1.0 / Cs[threadIdx.x][threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int col = wid; col < TB; col += (int)(blockDim.x >> 5)) {
-        double b = Bs[lane][col];
-        if (!upper) {
-            for (int i = 0; i < TB; ++i) {
-                const double xi = __shfl_sync(0xffffffffu, b, i) * inv[i];
-                if (lane == i) b = xi;
-                else if (lane > i) b -= Cs[lane][i] * xi;
-            }
-        } else {
-            for (int i = TB - 1; i >= 0; --i) {
-                const double xi = __shfl_sync(0xffffffffu, b, i) * inv[i];
-                if (lane == i) b = xi;
-                else if (lane < i) b -= Cs[lane][i] * xi;
-            }
+    double b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = lane == wid * 4 + q ? 1.0 : 0.0;
+    for (int i = wid * 4; i < TB; ++i) {  // rows above the warp's columns stay zero
+        const double c = lane > i ? Cs[lane][i] : 0.0, iv = inv[i];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double xi = __shfl_sync(0xffffffffu, b[q], i) * iv;
+            b[q] = lane == i ? xi : fma(-c, xi, b[q]);
         }
-        Bs[lane][col] = b;
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < TB * TB; e += blockDim.x) {
-        const int i = e / TB, k = e % TB;
-        if (i < rows && c0 + k < n) B[(size_t)(r0 + i) * n + c0 + k] = Bs[i][k];
+    const int i = r0 + lane;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int j = r0 + wid * 4 + q;
+        if (i < d && j < d) Ci[(size_t)i * d + j] = b[q];
     }
 }
 
-// W B = C^-T C^-1 B in place (B row-major [d][n]).
-void apply_W(int d, int n, const double *C, double *B, cudaStream_t s) {
-    const int nb = (d + TB - 1) / TB;
-    const int gc = (n + 63) / 64, gd = (n + TB - 1) / TB;
-    for (int I = 0; I < nb; ++I) {
-        note_launch();
-        k_trsm_diag<<<gd, 256, 0, s>>>(d, n, I, false, C, B);
-        if (I < nb - 1) {
-            note_launch();
-            k_trsm_right<<<dim3(gc, nb - 1 - I), 256, 0, s>>>(d, n, I, false, C, B);
-        }
+// One level of the merge [A 0; B D]^-1 = [A^-1 0; -D^-1 B A^-1, D^-1] for every pair of
+// blocks of s rows (blockIdx.z): pass 0 T = B A^-1, pass 1 Ci = -D^-1 T.
+template <int PASS>
+__global__ void __launch_bounds__(256) k_inv_merge(int d, int s, const double *C, double *Ci, double *T) {
+    __shared__ TileBuf sm;
+    const int p0 = blockIdx.z * 2 * s, q0 = p0 + s;  // first rows of the A and the D block
+    const int i0 = q0 + blockIdx.y * TB, j0 = p0 + blockIdx.x * TB;
+    if (i0 >= d) return;
+    double acc[2][2] = {};
+    if (PASS == 0) {
+        tile_gemm(
+            sm, j0, q0, acc, [&](int r, int l) { return i0 + r < d ? C[(size_t)(i0 + r) * d + l] : 0.0; },
+            [&](int l, int c) { return j0 + c <= l ? Ci[(size_t)l * d + j0 + c] : 0.0; });
+    } else {
+        tile_gemm(
+            sm, q0, min(d, i0 + TB), acc,
+            [&](int r, int l) { return i0 + r < d && l <= i0 + r ? Ci[(size_t)(i0 + r) * d + l] : 0.0; },
+            [&](int l, int c) { return l < d ? T[(size_t)l * d + j0 + c] : 0.0; });
     }
-    for (int I = nb - 1; I >= 0; --I) {
-        note_launch();
-        k_trsm_diag<<<gd, 256, 0, s>>>(d, n, I, true, C, B);
-        if (I > 0) {
-            note_launch();
-            k_trsm_right<<<dim3(gc, I), 256, 0, s>>>(d, n, I, true, C, B);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+            if (i < d) (PASS == 0 ? T : Ci)[(size_t)i * d + j] = PASS == 0 ? acc[r][c] : -acc[r][c];
         }
+}
+
+void launch_tri_inverse(int d, const double *C, double *Ci, double *T, cudaStream_t st) {
+    note_launch();
+    k_inv_diag<<<(d + TB - 1) / TB, 256, 0, st>>>(d, C, Ci);
+    for (int s = TB; s < d; s *= 2) {
+        const int pairs = (d + 2 * s - 1) / (2 * s);
+        const dim3 g(s / TB, s / TB, pairs);
+        note_launch();
+        k_inv_merge<0><<<g, 256, 0, st>>>(d, s, C, Ci, T);
+        note_launch();
+        k_inv_merge<1><<<g, 256, 0, st>>>(d, s, C, Ci, T);
     }
+}
+
+// Whether W L_k is formed for component k: r_k > 0 and the mode is not one-hot.
+__device__ __forceinline__ bool needs_product(const double *R, const int32_t *onehot, int k) {
+    return R[k] != 0.0 && onehot[0] < 0;
+}
+
+// Tile (I, J <= I) of the lower triangle from a flat index, the longest (J far left of a
+// low row) first.
+__device__ __forceinline__ void tile_from(int t, int nt, int &I, int &J) {
+    const int e = nt * (nt + 1) / 2 - 1 - t;
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while (i * (i + 1) / 2 > e) --i;
+    while ((i + 1) * (i + 2) / 2 <= e) ++i;
+    I = i;
+    J = i - (e - i * (i + 1) / 2);
+}
+
+// X_k = C^-1 L_k (lower triangular) and the tile's share of |X_k|_F^2 = tr(W P_k).
+__global__ void __launch_bounds__(256) k_adj_X(int d, const double *Ci, const double *L, const double *R,
+                                               const int32_t *onehot, double *X, double *trp) {
+    __shared__ TileBuf sm;
+    __shared__ double sh[8];
+    const int k = blockIdx.y;
+    if (!needs_product(R, onehot, k)) return;
+    int I, J;
+    tile_from(blockIdx.x, (d + TB - 1) / TB, I, J);
+    const int i0 = I * TB, j0 = J * TB;
+    const double *Lk = L + (size_t)k * d * d;
+    double acc[2][2] = {};
+    tile_gemm(
+        sm, j0, min(d, i0 + TB), acc,
+        [&](int r, int l) { return i0 + r < d && l <= i0 + r ? Ci[(size_t)(i0 + r) * d + l] : 0.0; },
+        [&](int l, int c) { return l < d && j0 + c <= l ? Lk[(size_t)l * d + j0 + c] : 0.0; });
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    double ss = 0.0;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+            if (i < d && j < d) {
+                const double v = j <= i ? acc[r][c] : 0.0;
+                X[((size_t)k * d + i) * d + j] = v;
+                ss = fma(v, v, ss);
+            }
+        }
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += sh[w];
+        trp[(size_t)k * gridDim.x + blockIdx.x] = t;
+    }
+}
+
+// dL_k += pi lower[ eps (diag(1/L) - delta z^T) - gam z^T - delta u^T - r W L_k ] with u =
+// L^T gam and the tile of W L_k = C^-T X_k formed here (at a one-hot mode lower[W L_k] =
+// diag(1 / L_ii)).
+__global__ void __launch_bounds__(256) k_adj_dL(int d, const double *pi, const double *R, const double *eps,
+                                                const int32_t *onehot, const double *L, const double *x,
+                                                const double *mu, const double *Z, const double *gam,
+                                                const double *U, const double *Ci, const double *X, double *dL) {
+    __shared__ TileBuf sm;
+    const int k = blockIdx.y;
+    const double rk = R[k];
+    if (rk == 0.0) return;
+    int I, J;
+    tile_from(blockIdx.x, (d + TB - 1) / TB, I, J);
+    const int i0 = I * TB, j0 = J * TB;
+    const double *Lk = L + (size_t)k * d * d, *Xk = X + (size_t)k * d * d;
+    const bool oh = onehot[0] >= 0;
+    double acc[2][2] = {};
+    if (!oh)
+        tile_gemm(
+            sm, i0, d, acc,
+            [&](int r, int l) { return l < d && i0 + r <= l ? Ci[(size_t)l * d + i0 + r] : 0.0; },
+            [&](int l, int c) { return l < d && j0 + c < d ? Xk[(size_t)l * d + j0 + c] : 0.0; });
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const double p = pi[0], ek = eps[k];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+            if (i >= d || j > i) continue;
+            const size_t e = (size_t)i * d + j, kd = (size_t)k * d;
+            const double di = x[i] - mu[kd + i], zj = Z[kd + j];
+            const double wl = oh ? (i == j ? 1.0 / Lk[e] : 0.0) : acc[r][c];
+            double v = -ek * di * zj - gam[kd + i] * zj - di * U[kd + j] - rk * wl;
+            if (i == j) v += ek / Lk[e];
+            dL[(size_t)k * d * d + e] += p * v;
+        }
 }
 
 // ------------------------------------------------------------------ per-mode vector algebra
-// Column vectors for the right-hand-side block V [d][nv] (row-major, so W acts on columns):
-// columns 0..K-1 = g_k (active only, else 0), K = gbar.
+// Vectors are rows of [nv][d]. Rows of V: 0 .. K-1 = g_k (active only, else 0), K = gbar.
 __global__ void k_pack_rhs(int d, int K, const double *GK, const double *gbar, const double *R, double *V) {
-    const int nv = K + 1;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * nv; e += gridDim.x * blockDim.x) {
-        const int i = e / nv, c = e % nv;
-        double v;
-        if (c < K)
-            v = R[c] != 0.0 ? GK[(size_t)c * d + i] : 0.0;
-        else
-            v = gbar[i];
-        V[e] = v;
-    }
+    const int c = blockIdx.y;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < d) V[(size_t)c * d + i] = c < K ? (R[c] != 0.0 ? GK[(size_t)c * d + i] : 0.0) : gbar[i];
 }
 
-// copy L_k (lower, zero above) into M [d][d]
-__global__ void k_copy_lower(int d, const double *Lk, double *M) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < (size_t)d * d;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / d), j = (int)(e % d);
-        M[e] = j <= i ? Lk[e] : 0.0;
-    }
-}
-
-template <typename T>
-__device__ T block_sum256(T v, T *sh) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    T t = 0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += sh[q];
-    __syncthreads();
-    return t;
-}
-
-// tr(W P_k) = <W L_k, L_k>_F over the lower triangle (W L_k in M).
-__global__ void __launch_bounds__(256) k_trace_WP(int d, const double *M, const double *Lk, double *out) {
-    __shared__ double sh[8];
+// y_c = T_c v_c for a lower triangular matrix T (T_c = T + c tstride), a warp per row.
+// R given: vectors c < K with R[c] == 0 are skipped.
+// dmu given: dmu_c += pi (-eps_c g_c + y_c) instead of storing y_c.
+__global__ void __launch_bounds__(256) k_adj_lower(int d, const double *T, size_t tstride, const double *V,
+                                                   const double *R, int K, double *Y, const double *pi,
+                                                   const double *eps, const double *GK, double *dmu) {
+    const int c = blockIdx.y;
+    if (R && c < K && R[c] == 0.0) return;
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= d) return;
+    const double *row = T + c * tstride + (size_t)i * d, *v = V + (size_t)c * d;
     double s = 0.0;
-    for (size_t e = threadIdx.x; e < (size_t)d * d; e += blockDim.x) {
-        const int i = (int)(e / d), j = (int)(e % d);
-        if (j <= i) s += M[e] * Lk[e];
-    }
-    s = block_sum256(s, sh);
-    if (threadIdx.x == 0) *out = s;
+#pragma unroll 4
+    for (int j = lane; j <= i; j += 32) s = fma(row[j], v[j], s);
+    s = warp_sum(s);
+    if (lane != 0) return;
+    const size_t o = (size_t)c * d + i;
+    if (dmu)
+        dmu[o] += pi[0] * (-eps[c] * GK[o] + s);
+    else
+        Y[o] = s;
 }
 
-// One CTA: given WV (W applied to [g_0..g_{K-1}, gbar]) and tr(W P_k), form t (stage 0),
-// or with Wt known form c, eps, gam (stage 1). Vectors of length d in global scratch.
-__global__ void __launch_bounds__(256) k_adj_stage(int stage, int d, int K, const double *R, const double *GK,
-                                                   const double *gbar, const double *WV, const double *trWP,
-                                                   const double *PY, const double *Wt, double *t_out, double *eps,
-                                                   double *gam, double *cvec) {
-    __shared__ double sh[8];
+// y_c = T_c^T v_c (v_c = diff - v_c when diff is given): a CTA per 32 columns, a lane per column, the eight warps
+// over interleaved rows, partials summed in a fixed order.
+__global__ void __launch_bounds__(256) k_adj_upper(int d, const double *T, size_t tstride, const double *V,
+                                                   const double *diff, const double *R, int K, double *Y) {
+    __shared__ double part[8][32];
+    const int c = blockIdx.y;
+    if (R && c < K && R[c] == 0.0) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, j0 = blockIdx.x * 32, j = j0 + lane;
+    const double *Tc = T + c * tstride, *v = V + (size_t)c * d;
+    double s = 0.0;
+    if (j < d) {
+#pragma unroll 4
+        for (int i = j0 + wid; i < d; i += 8) {
+            const double t = i >= j ? Tc[(size_t)i * d + j] : 0.0;
+            s = fma(t, diff ? diff[i] - v[i] : v[i], s);
+        }
+    }
+    part[wid][lane] = s;
+    __syncthreads();
+    if (wid == 0 && j < d) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += part[w][lane];
+        Y[(size_t)c * d + j] = t;
+    }
+}
+
+// One CTA of 1024 threads: given WV (rows W g_0 .. W g_{K-1}, W gbar) and the partials of
+// tr(W P_k), form t (stage 0), or with Wt known form eps and gam (stage 1). A warp per
+// component for the inner products.
+__global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, int n_part, const double *R,
+                                                    const int32_t *onehot, const double *GK, const double *gbar,
+                                                    const double *WV, const double *trp, const double *PY,
+                                                    const double *Wt, double *t_out, double *eps, double *gam) {
     __shared__ double s_beta[kMaxK];
-    const int nv = K + 1;
-    // per active component: dot products g_k^T W g_k, gbar^T W g_k, c^T g_k
-    for (int k = 0; k < K; ++k) {
-        const double r = R[k];
-        if (r == 0.0) {
-            if (threadIdx.x == 0) s_beta[k] = 0.0;
-            continue;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const double *Wg = WV + (size_t)K * d;  // W gbar
+    const bool oh = onehot[0] >= 0;
+    for (int k = wid; k < K; k += 32) {
+        double beta = 0.0;
+        if (R[k] != 0.0) {
+            const double *gk = GK + (size_t)k * d, *wgk = WV + (size_t)k * d;
+            double a1 = 0.0, a2 = 0.0, tr = 0.0;
+            for (int i = lane; i < d; i += 32) {
+                a1 = fma(gk[i], wgk[i], a1);  // g_k^T W g_k
+                // gbar^T W g_k, or c^T g_k with c = -W gbar - W t / 2
+                a2 = stage == 0 ? fma(gbar[i], wgk[i], a2) : fma(fma(-0.5, Wt[i], -Wg[i]), gk[i], a2);
+            }
+            if (!oh)
+                for (int q = lane; q < n_part; q += 32) tr += trp[(size_t)k * n_part + q];
+            a1 = warp_sum(a1);
+            a2 = warp_sum(a2);
+            tr = oh ? (double)d : warp_sum(tr);
+            beta = stage == 0 ? (tr - a1 + 2.0 * a2) : (-0.5 * (tr - a1) + a2);
         }
-        double a1 = 0.0, a2 = 0.0;
-        for (int i = threadIdx.x; i < d; i += blockDim.x) {
-            const double gk = GK[(size_t)k * d + i];
-            const double wgk = WV[(size_t)i * nv + k];
-            a1 += gk * wgk;                     // g_k^T W g_k
-            if (stage == 0)
-                a2 += gbar[i] * wgk;            // gbar^T W g_k
-            else
-                a2 += (-WV[(size_t)i * nv + K] - 0.5 * Wt[i]) * gk;  // c^T g_k
-        }
-        a1 = block_sum256(a1, sh);
-        a2 = block_sum256(a2, sh);
-        if (threadIdx.x == 0)
-            s_beta[k] = stage == 0 ? (trWP[k] - a1 + 2.0 * a2) : (-0.5 * (trWP[k] - a1) + a2);
+        if (lane == 0) s_beta[k] = beta;
     }
     __syncthreads();
     double sb = 0.0;
@@ -245,72 +355,15 @@ __global__ void __launch_bounds__(256) k_adj_stage(int stage, int d, int K, cons
             t_out[i] = ti;
         }
     } else {
-        if (threadIdx.x < K) {
+        if ((int)threadIdx.x < K) {
             const int k = threadIdx.x;
             eps[k] = R[k] == 0.0 ? 0.0 : R[k] + R[k] * (s_beta[k] - sb);
         }
         for (int i = threadIdx.x; i < d; i += blockDim.x) {
-            const double c = -WV[(size_t)i * nv + K] - 0.5 * Wt[i];
-            cvec[i] = c;
-            for (int k = 0; k < K; ++k) gam[(size_t)k * d + i] = R[k] == 0.0 ? 0.0 : R[k] * (WV[(size_t)i * nv + k] + c);
+            const double c = -Wg[i] - 0.5 * Wt[i];
+            for (int k = 0; k < K; ++k) gam[(size_t)k * d + i] = R[k] == 0.0 ? 0.0 : R[k] * (WV[(size_t)k * d + i] + c);
         }
     }
-}
-
-// dmu_k += pi (-eps_k g_k + P_k gam_k) for one component, P_k gam_k given (y).
-__global__ void __launch_bounds__(256) k_adj_dmu(int d, int k, double pi, const double *eps, const double *GK,
-                                                 const double *y, double *dmu) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d) return;
-    dmu[(size_t)k * d + i] += pi * (-eps[k] * GK[(size_t)k * d + i] + y[i]);
-}
-
-// v = W gbar - W g_k (columns K and k of WV [d][K + 1]).
-__global__ void __launch_bounds__(256) k_adj_wdiff(int d, int K, int k, const double *WV, double *v) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < d) v[i] = WV[(size_t)i * (K + 1) + K] - WV[(size_t)i * (K + 1) + k];
-}
-
-// y = L_k u (lower triangular), a warp per row: y_i = sum_{j <= i} L[i][j] u_j.
-__global__ void __launch_bounds__(256) k_adj_Lu(int d, const double *Lk, const double *u, double *y) {
-    const int lane = threadIdx.x & 31;
-    const int i = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-    if (i >= d) return;
-    double s = 0.0;
-    for (int j = lane; j <= i; j += 32) s += Lk[(size_t)i * d + j] * u[j];
-    s = warp_sum(s);
-    if (lane == 0) y[i] = s;
-}
-
-// L^T gam for component k (u[j] = sum_i L[i][j] gam[i]).
-__global__ void __launch_bounds__(256) k_adj_Ltg(int d, const double *Lk, const double *g, double *u) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d) return;
-    double s = 0.0;
-    for (int i = j; i < d; ++i) s += Lk[(size_t)i * d + j] * g[i];
-    u[j] = s;
-}
-
-// dL_k += pi lower[ eps (diag(1/L) - delta z^T) - gam z^T - delta u^T - r M ],  M = W L_k, u = L^T gam.
-// M null: the one-hot case W = (L_k L_k^T)^-1, where W L_k = L_k^-T, whose lower
-// triangle is diag(1 / L_ii).
-__global__ void __launch_bounds__(256) k_adj_dL(int d, double pi, double r, double eps, const double *Lk,
-                                                const double *x, const double *mu, const double *z, const double *gam,
-                                                const double *u, const double *M, double *dL) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < (size_t)d * d;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / d), j = (int)(e % d);
-        if (j > i) continue;
-        const double di = x[i] - mu[i];
-        const double wl = M ? M[e] : (i == j ? 1.0 / Lk[e] : 0.0);
-        double v = -eps * di * z[j] - gam[i] * z[j] - di * u[j] - r * wl;
-        if (i == j) v += eps / Lk[e];
-        dL[e] += pi * v;
-    }
-}
-
-__global__ void k_set_f64(double *p, double v) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *p = v;
 }
 
 __global__ void k_softmax_pi(int n, const double *logZk, double g, double *pi) {
@@ -325,10 +378,13 @@ __global__ void k_softmax_pi(int n, const double *logZk, double g, double *pi) {
 }  // namespace
 
 void adjoint_carve(Carver &cv, AdjWs &w, int d, int K) {
-    const int nJT = (d + 63) / 64;
+    const int nJT = (d + 63) / 64, nt = (d + TB - 1) / TB;
     w.P = cv.take<double>((size_t)K * d * d);
     w.H = cv.take<double>((size_t)d * d);
-    w.M = cv.take<double>((size_t)K * d * d);
+    w.Ci = cv.take<double>((size_t)d * d);
+    w.T2 = cv.take<double>((size_t)d * d);
+    w.X = cv.take<double>((size_t)K * d * d);
+    w.trp = cv.take<double>((size_t)K * nt * (nt + 1) / 2);
     w.Z = cv.take<double>((size_t)K * d);
     w.R = cv.take<double>((size_t)K);
     w.qpart = cv.take<double>((size_t)K * nJT);
@@ -336,19 +392,24 @@ void adjoint_carve(Carver &cv, AdjWs &w, int d, int K) {
     w.ell = cv.take<double>(1);
     w.GK = cv.take<double>((size_t)K * d);
     w.V = cv.take<double>((size_t)d * (K + 1));
+    w.Y = cv.take<double>((size_t)d * (K + 1));
+    w.WV = cv.take<double>((size_t)d * (K + 1));
     w.T = cv.take<double>(d);
-    w.cvec = cv.take<double>(d);
     w.eps = cv.take<double>(K);
     w.gam = cv.take<double>((size_t)K * d);
-    w.u = cv.take<double>(d);
-    w.trWP = cv.take<double>(K);
+    w.U = cv.take<double>((size_t)K * d);
     w.PY = cv.take<double>((size_t)K * d);
-    w.y = cv.take<double>(d);
     w.pi = cv.take<double>(kMaxAdjModes);
     w.info = cv.take<int32_t>(1);
     w.one = cv.take<int32_t>(1);
     w.onehot = cv.take<int32_t>(1);
+    w.p_done = cv.take<int32_t>(kMaxK);
+    w.p_need = cv.take<int32_t>(kMaxK);
     w.bar = cv.take<uint32_t>(2);
+}
+
+__global__ void k_set_one(int32_t *p) {
+    if (threadIdx.x == 0) *p = 1;
 }
 
 sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, const double *logZk, int n_modes,
@@ -357,19 +418,25 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
     if (n_modes < 1 || n_modes > kMaxAdjModes) return SB_ERR_INVALID_ARG;
     SB_CUDA_TRY(cudaMemsetAsync(dmu, 0, sizeof(double) * K * d, s));
     SB_CUDA_TRY(cudaMemsetAsync(dL, 0, sizeof(double) * (size_t)K * d * d, s));
-    const int32_t one = 1;
-    SB_CUDA_TRY(cudaMemcpyAsync(w.one, &one, sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    SB_CUDA_TRY(cudaMemsetAsync(w.p_done, 0, sizeof(int32_t) * kMaxK, s));
+    note_launch();
+    k_set_one<<<1, 32, 0, s>>>(w.one);
     note_launch();
     k_softmax_pi<<<1, 32, 0, s>>>(n_modes, logZk, grad_logZ, w.pi);
-    // P_k = L_k L_k^T is formed only for the Hessian at a mode that is not one-hot;
-    // every product with P_k below is L_k (L_k^T v)
-    bool p_ready = false;
-    std::vector<double> pis(n_modes), Rh(K), epsh(K);
-    SB_CUDA_TRY(cudaMemcpyAsync(pis.data(), w.pi, sizeof(double) * n_modes, cudaMemcpyDeviceToHost, s));
-    SB_CUDA_TRY(cudaStreamSynchronize(s));
+    const int nt = (d + TB - 1) / TB, tiles = nt * (nt + 1) / 2;
+    const unsigned rows8 = (unsigned)((d + 7) / 8), cols32 = (unsigned)((d + 31) / 32);
+    const size_t dd = (size_t)d * d;
+    // W v for the rows of V [nv][d] (rows c < nk with R[c] == 0 skipped: their V is zero and unread)
+    auto apply_W = [&](int nv, const double *V, double *out, const double *R, int nk) {
+        note_launch(2);
+        k_adj_lower<<<dim3(rows8, nv), 256, 0, s>>>(d, w.Ci, 0, V, R, nk, w.Y, nullptr, nullptr, nullptr, nullptr);
+        k_adj_upper<<<dim3(cols32, nv), 256, 0, s>>>(d, w.Ci, 0, w.Y, nullptr, R, nk, out);
+    };
     for (int mo = 0; mo < n_modes; ++mo) {
         const double *x = modes + (size_t)mo * d;
+        const double *pi = w.pi + mo;
         // l, grad l, z_k, r_k at x (FP64 likelihood kernels), then g_k, H and H = C C^T
+        // (at a one-hot mode C = L_k is copied, as in the Laplace stage), C^-1
         LikF64Args la{};
         la.d = d;
         la.K = K;
@@ -387,82 +454,36 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
         la.grad_sign = -1.0;
         la.out_by_walker = 0;
         launch_lik_f64_few(la, true, s);
-        SB_CUDA_TRY(cudaMemcpyAsync(Rh.data(), w.R, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
-        SB_CUDA_TRY(cudaStreamSynchronize(s));
-        // at a one-hot mode (r_k = 1, every other r exactly 0) H = P_k, whose factor is
-        // L_k: copied, not assembled and factored (as in the Laplace stage)
-        int oh = -1, nz = 0;
-        for (int k = 0; k < K; ++k)
-            if (Rh[k] != 0.0) {
-                ++nz;
-                oh = Rh[k] == 1.0 ? k : -2;
-            }
-        if (nz != 1 || oh < 0) oh = -1;
-        if (oh < 0 && !p_ready) {
-            launch_precision(d, K, pv.L, w.P, s);
-            p_ready = true;
-        }
         launch_onehot(K, w.R, w.one, 1, w.onehot, s);
+        launch_precision_needed(d, K, pv.L, w.R, w.one, w.p_done, w.p_need, w.P, s, w.onehot);
         launch_hessian_chol(d, K, 1, pv.L, w.P, w.Z, w.R, w.gbar, w.one, w.GK, w.H, w.info, w.bar, pv.status, s,
                             w.onehot);
-        // W [g_0 .. g_{K-1}, gbar]
+        launch_tri_inverse(d, w.H, w.Ci, w.T2, s);
+        // W [g_0 .. g_{K-1}, gbar]; X_k = C^-1 L_k and tr(W P_k)
         note_launch();
-        k_pack_rhs<<<(d * (K + 1) + 255) / 256, 256, 0, s>>>(d, K, w.GK, w.gbar, w.R, w.V);
-        apply_W(d, K + 1, w.H, w.V, s);
-        // W L_k and tr(W P_k) = <W L_k, L_k>_F for the components with r_k > 0. At a
-        // one-hot mode the factor is L_k, so W L_k = L_k^-T and tr(W P_k) = d exactly:
-        // no d x d solve
-        for (int k = 0; k < K; ++k) {
-            if (Rh[k] == 0.0) continue;
-            if (k == oh) {
-                note_launch();
-                k_set_f64<<<1, 32, 0, s>>>(w.trWP + k, (double)d);
-                continue;
-            }
-            double *Mk = w.M + (size_t)k * d * d;
-            note_launch();
-            k_copy_lower<<<1184, 256, 0, s>>>(d, pv.L + (size_t)k * d * d, Mk);
-            apply_W(d, d, w.H, Mk, s);
-            note_launch();
-            k_trace_WP<<<1, 256, 0, s>>>(d, Mk, pv.L + (size_t)k * d * d, w.trWP + k);
-        }
-        // P_k (W gbar - W g_k) for the components with r_k > 0
-        for (int k = 0; k < K; ++k) {
-            if (Rh[k] == 0.0) continue;
-            const double *Lk = pv.L + (size_t)k * d * d;
-            note_launch();
-            k_adj_wdiff<<<(d + 255) / 256, 256, 0, s>>>(d, K, k, w.V, w.y);
-            note_launch();
-            k_adj_Ltg<<<(d + 255) / 256, 256, 0, s>>>(d, Lk, w.y, w.u);
-            note_launch();
-            k_adj_Lu<<<(d * 32 + 255) / 256, 256, 0, s>>>(d, Lk, w.u, w.PY + (size_t)k * d);
-        }
-        // t = grad_x log det H, then v = W t (in place)
+        k_pack_rhs<<<dim3((d + 255) / 256, K + 1), 256, 0, s>>>(d, K, w.GK, w.gbar, w.R, w.V);
+        apply_W(K + 1, w.V, w.WV, w.R, K);
         note_launch();
-        k_adj_stage<<<1, 256, 0, s>>>(0, d, K, w.R, w.GK, w.gbar, w.V, w.trWP, w.PY, nullptr, w.T, nullptr, nullptr,
-                                      nullptr);
-        apply_W(d, 1, w.H, w.T, s);
-        // c, eps_k, gam_k
+        k_adj_X<<<dim3(tiles, K), 256, 0, s>>>(d, w.Ci, pv.L, w.R, w.onehot, w.X, w.trp);
+        // P_k (W gbar - W g_k) = L_k (L_k^T (W gbar - W g_k))
+        note_launch(2);
+        k_adj_upper<<<dim3(cols32, K), 256, 0, s>>>(d, pv.L, dd, w.WV, w.WV + (size_t)K * d, w.R, K, w.U);
+        k_adj_lower<<<dim3(rows8, K), 256, 0, s>>>(d, pv.L, dd, w.U, w.R, K, w.PY, nullptr, nullptr, nullptr,
+                                                   nullptr);
+        // t = grad_x log det H, then v = W t (into V's first row), then c, eps_k, gam_k
         note_launch();
-        k_adj_stage<<<1, 256, 0, s>>>(1, d, K, w.R, w.GK, w.gbar, w.V, w.trWP, w.PY, w.T, nullptr, w.eps, w.gam,
-                                      w.cvec);
-        SB_CUDA_TRY(cudaMemcpyAsync(epsh.data(), w.eps, sizeof(double) * K, cudaMemcpyDeviceToHost, s));
-        SB_CUDA_TRY(cudaStreamSynchronize(s));
-        for (int k = 0; k < K; ++k) {
-            if (Rh[k] == 0.0) continue;
-            const double *Lk = pv.L + (size_t)k * d * d;
-            // u = L_k^T gam_k, then P_k gam_k = L_k u for dmu_k
-            note_launch();
-            k_adj_Ltg<<<(d + 255) / 256, 256, 0, s>>>(d, Lk, w.gam + (size_t)k * d, w.u);
-            note_launch();
-            k_adj_Lu<<<(d * 32 + 255) / 256, 256, 0, s>>>(d, Lk, w.u, w.y);
-            note_launch();
-            k_adj_dmu<<<(d + 255) / 256, 256, 0, s>>>(d, k, pis[mo], w.eps, w.GK, w.y, dmu);
-            note_launch();
-            k_adj_dL<<<1184, 256, 0, s>>>(d, pis[mo], Rh[k], epsh[k], Lk, x, pv.mu + (size_t)k * d,
-                                          w.Z + (size_t)k * d, w.gam + (size_t)k * d, w.u,
-                                          k == oh ? nullptr : w.M + (size_t)k * d * d, dL + (size_t)k * d * d);
-        }
+        k_adj_stage<<<1, 1024, 0, s>>>(0, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, nullptr, w.T,
+                                       nullptr, nullptr);
+        apply_W(1, w.T, w.V, nullptr, 0);
+        note_launch();
+        k_adj_stage<<<1, 1024, 0, s>>>(1, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, w.V, nullptr,
+                                       w.eps, w.gam);
+        // u_k = L_k^T gam_k, dmu_k += pi (-eps_k g_k + L_k u_k), dL_k
+        note_launch(3);
+        k_adj_upper<<<dim3(cols32, K), 256, 0, s>>>(d, pv.L, dd, w.gam, nullptr, w.R, K, w.U);
+        k_adj_lower<<<dim3(rows8, K), 256, 0, s>>>(d, pv.L, dd, w.U, w.R, K, nullptr, pi, w.eps, w.GK, dmu);
+        k_adj_dL<<<dim3(tiles, K), 256, 0, s>>>(d, pi, w.R, w.eps, w.onehot, pv.L, x, pv.mu, w.Z, w.gam, w.U, w.Ci,
+                                                w.X, dL);
     }
     SB_CUDA_TRY(cudaGetLastError());
     return SB_OK;
