@@ -15,6 +15,7 @@
 // columns j < i0 + 64. FP64 throughput bounds this path; it exists as the
 // exact reference path and the plain-FP64 comparator of the tensor-core path.
 #include "sb_internal.cuh"
+#include "sb_small_f64.cuh"
 
 namespace sb {
 
@@ -396,6 +397,7 @@ void launch_lik_f64_z(const LikF64Args &a, cudaStream_t s) {
 
 void launch_lik_f64_rays(const LikF64Args &a, cudaStream_t s) {
     if (a.n_rows <= 0) return;
+    if (small_f64_fits(a.d, a.K, 0)) return launch_small_points_f64(a, true, s);
     dim3 g((a.n_rows + BM - 1) / BM, (a.d + BN - 1) / BN, a.K);
     {
         ProfScope prof(PROF_F64_Z, s);
@@ -408,6 +410,11 @@ void launch_lik_f64_rays(const LikF64Args &a, cudaStream_t s) {
 
 void launch_lik_f64_points(const LikF64Args &a, bool want_grad, cudaStream_t s) {
     if (a.n_rows <= 0) return;
+    if (small_f64_fits(a.d, a.K, 0)) {
+        LikF64Args b = a;
+        if (!want_grad) b.G = nullptr;
+        return launch_small_points_f64(b, false, s);
+    }
     dim3 g((a.n_rows + BM - 1) / BM, (a.d + BN - 1) / BN, a.K);
     if (want_grad) {
         {

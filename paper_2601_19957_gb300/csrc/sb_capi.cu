@@ -19,6 +19,7 @@
 #include "sb_internal.cuh"
 #include "sb_laplace.cuh"
 #include "sb_lbfgs.cuh"
+#include "sb_small_f64.cuh"
 #include "sb_tc.cuh"
 #include "sb_graph.cuh"
 
@@ -464,6 +465,12 @@ sb_status run_refine(const ProbView &pv, const sb_config *c, const RefineWs<T> &
     RefineWs<T> rr = r;
     rr.lb = a;
     int64_t *ev = n_evals ? n_evals : r.n_evals;
+    if constexpr (std::is_same<T, double>::value)
+        if (small_f64_fits(pv.d, pv.K, c->m)) {  // every walker to its end in one launch
+            launch_small_refine_f64(pv, a, starts, n, r.Z, x_out, ell_out, status_out, iters_out, ev, s);
+            SB_CUDA_TRY(cudaGetLastError());
+            return SB_OK;
+        }
     launch_lbfgs_init<T>(n, pv.d, starts, a, ev, s);
     if constexpr (std::is_same<T, float>::value) tc_walkers_reset(r.tc, n, s);
     // every accepted step takes at most 2 (max_backtracks + 2) rounds
