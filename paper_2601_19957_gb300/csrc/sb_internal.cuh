@@ -133,6 +133,34 @@ __device__ __forceinline__ double warp_exit_min(int lane, int d, const double *u
 __device__ __forceinline__ bool is_finite(double v) { return isfinite(v); }
 __device__ __forceinline__ bool is_finite(float v) { return isfinite(v); }
 
+// FP64 <-> FP32 conversions on the integer units. The FP64 pipe, which also does the
+// hardware conversions, takes one warp instruction per 19 cycles and SM: a pass that
+// converts every element it moves is bound by it (8 bytes a lane and 19 cycles are 13
+// bytes a cycle and SM, well below HBM). Same results as the hardware conversions
+// (round to nearest even), which serve the rare exponents.
+__device__ __forceinline__ float f64_to_f32(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    const uint32_t sign = hi & 0x80000000u;
+    if (e - 897u > 253u) {  // not a normal float (zero, below 2^-126, above 2^127)
+        if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(sign);
+        return (float)v;
+    }
+    const uint32_t m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const uint32_t rest = lo & 0x1fffffffu;
+    // up when more than half a unit is dropped, or half and the kept part is odd (the
+    // carry runs into the exponent as it should)
+    return __uint_as_float(sign | (m + ((rest + (m & 1u)) > 0x10000000u ? 1u : 0u)));
+}
+__device__ __forceinline__ double f32_to_f64(float v) {
+    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xffu;
+    const uint32_t sign = u & 0x80000000u;
+    if (e - 1u > 253u) {  // zero, subnormal, infinity or NaN
+        if ((u & 0x7fffffffu) == 0u) return __hiloint2double((int)sign, 0);
+        return (double)v;
+    }
+    return __hiloint2double((int)(sign | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
 __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): 10 rounds, Weyl key bumps.

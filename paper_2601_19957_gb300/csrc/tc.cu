@@ -601,60 +601,76 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
 // LSE over components from the FP32 |z|^2 partials: e_k and the maximum in
 // FP64, exp/log of the shifted values (in [0, 1] and [1, K]) in FP32, whose
 // absolute error stays below the FP32 resolution of the outputs.
-// mode 0: walkers (FT[act[n]] = -l, R); mode 1: ray samples (ell[flat0 + n] = l);
-// mode 2: points (ell[n] = l, R). Modes 0 and 2 also raise rflag[block][k] when
-// some row of the 128-row block has r_nk > 0 (GEMM2 and the scaling pass skip
-// the other (block, component) pairs, whose terms are exactly zero).
-__global__ void __launch_bounds__(128) k_tc_lse(int mode, int K, int n_ntile, const int32_t *n_rows_dev,
-                                                int n_rows_max, const int32_t *act, const float *qpart,
-                                                const double *a_k, float *R, float *FT, double *ell,
-                                                uint32_t *rflag, const uint32_t *zmask, float *zb, int32_t *jst,
-                                                float *zst) {
+// mode 0: walkers (FT[act[n]] = -l, R); mode 2: points (ell[n] = l, R). Both raise
+// rflag[block][k] when some row of the 128-row block has r_nk > 0 (GEMM2 and the scaling
+// pass skip the other (block, component) pairs, whose terms are exactly zero).
+// Bound by the FP64 pipe (one warp instruction per 19 cycles and SM): each e_k is formed
+// once and kept in shared memory (n_ntile + 1 FP64 instructions per row and evaluated
+// component; it was three times that, an FP64 square root and the conversions), the
+// conversions run on the integer units and the bounds in FP32 with directed rounding. At
+// 16384 walkers, d = 1024, K = 8 a launch takes 9.6 us (16.5 before), cold caches.
+constexpr int LSE_ROWS = 128;
+__global__ void __launch_bounds__(LSE_ROWS) k_tc_lse(int mode, int K, int n_ntile, const int32_t *n_rows_dev,
+                                                     int n_rows_max, const int32_t *act, const float *qpart,
+                                                     const double *a_k, float *R, float *FT, double *ell,
+                                                     uint32_t *rflag, const uint32_t *zmask, float *zb, int32_t *jst,
+                                                     float *zst) {
+    extern __shared__ double s_e[];  // [K][LSE_ROWS]: e_k, then (as float) exp(e_k - max)
     const int n_rows = n_rows_dev ? *n_rows_dev : n_rows_max;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if ((int)blockIdx.x * LSE_ROWS >= n_rows) return;
+    const int n = blockIdx.x * LSE_ROWS + threadIdx.x;
     const bool valid = n < n_rows;
-    // components the |z|^2 pass skipped for this row block (zmask): e_k = -inf. Each
-    // pass below recomputes e_k from the partials (the same sum in the same order, so
-    // the same value), which keeps the terms out of a local-memory array.
+    // components the |z|^2 pass skipped for this row block (zmask): e_k = -inf
     const uint64_t km = zmask ? block_kmask(zmask, n / BM, K) : ~0ull;
-    auto term = [&](int k) -> double {
-        if (!((km >> k) & 1ull)) return -INFINITY;
-        const float *qp = qpart + ((size_t)n * K + k) * n_ntile;
-        double q = 0.0;
-        for (int t = 0; t < n_ntile; ++t) q += (double)qp[t];
-        return a_k[k] - 0.5 * q;
-    };
     double emax = -INFINITY;
     float s = 0.f;
+    auto slot = [&](int k) -> double & { return s_e[k * LSE_ROWS + threadIdx.x]; };
     if (valid) {
-        for (int k = 0; k < K; ++k) emax = fmax(emax, term(k));
+        // the largest term, compared as order-preserving integers (a NaN is never the largest)
+        auto order = [](double e) -> long long {
+            const long long b = __double_as_longlong(e);
+            if ((b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) return (long long)0x8000000000000000ull;
+            return b >= 0 ? b : b ^ 0x7fffffffffffffffll;
+        };
         // bounds for the next round's skip (k_tc_need): |z_k| of the evaluated
         // components, lowered by a 1/32 margin for the GEMM's rounding, and the
         // largest term's |z|, raised by the same margin
         const int w = zb ? (act ? act[n] : n) : 0;
         int jm = -1;
-        double ejm = 0.0;
+        long long top = order(-INFINITY);
+        float qtop = 0.f;
         for (int k = 0; k < K; ++k) {
-            const double e = term(k);
-            s += __expf((float)(e - emax));
-            if (zb && isfinite(e)) {
-                zb[(size_t)w * K + k] = __double2float_rd(sqrt(fmax((a_k[k] - e) * 2.0, 0.0)) * (1.0 - 1.0 / 32));
-                if (e == emax && jm < 0) {
-                    jm = k;
-                    ejm = e;
-                }
+            if (!((km >> k) & 1ull)) continue;
+            const float *qp = qpart + ((size_t)n * K + k) * n_ntile;
+            double q = f32_to_f64(qp[0]);
+            for (int t = 1; t < n_ntile; ++t) q += f32_to_f64(qp[t]);
+            const double e = a_k[k] - 0.5 * q;
+            slot(k) = e;
+            const long long o = order(e);
+            const bool fin = finite_bits(e);
+            if (o > top) {
+                top = o;
+                emax = e;
+                jm = fin ? k : -1;
             }
+            if (zb && fin) {
+                const float qf = f64_to_f32(q);  // within 2^-24
+                if (jm == k) qtop = qf;
+                zb[(size_t)w * K + k] = __fmul_rd(__fsqrt_rd(qf), 1.0f - 1.0f / 32 - 0x1p-22f);
+            }
+        }
+        for (int k = 0; k < K; ++k) {
+            float x = 0.f;
+            if ((km >> k) & 1ull) x = __expf(f64_to_f32(slot(k) - emax));
+            s += x;
+            reinterpret_cast<float &>(slot(k)) = x;
         }
         if (zb) {
             jst[w] = jm;
-            if (jm >= 0) zst[w] = __double2float_ru(sqrt(fmax((a_k[jm] - ejm) * 2.0, 0.0)) * (1.0 + 1.0 / 32));
+            if (jm >= 0) zst[w] = __fmul_ru(__fsqrt_ru(qtop), 1.0f + 1.0f / 32 + 0x1p-22f);
         }
     }
-    const double l = emax + (double)__logf(s);
-    if (mode == 1) {
-        if (valid) ell[n] = l;
-        return;
-    }
+    const double l = emax + f32_to_f64(__logf(s));
     const float inv = 1.f / s;
     // One CTA is one 128-row block. Flag of (block, component k): bit 0 when some row
     // has r_nk > 0; bit 1 as well when every live row has r_nk == 1 exactly (all other
@@ -667,7 +683,7 @@ __global__ void __launch_bounds__(128) k_tc_lse(int mode, int K, int n_ntile, co
     __syncthreads();
     uint64_t any_m = 0, one_m = 0;
     for (int k = 0; k < K; ++k) {
-        const float r = valid ? __expf((float)(term(k) - emax)) * inv : 0.f;
+        const float r = valid ? reinterpret_cast<float &>(slot(k)) * inv : 0.f;
         if (valid) R[(size_t)n * K + k] = r;
         if (__any_sync(0xffffffffu, r > 0.f)) any_m |= 1ull << k;
         if (__all_sync(0xffffffffu, !valid || r == 1.f)) one_m |= 1ull << k;
@@ -684,7 +700,7 @@ __global__ void __launch_bounds__(128) k_tc_lse(int mode, int K, int n_ntile, co
     }
     if (!valid) return;
     if (mode == 0)
-        FT[act ? act[n] : n] = (float)(-l);
+        FT[act ? act[n] : n] = f64_to_f32(-l);
     else
         ell[n] = l;
 }
@@ -761,7 +777,7 @@ __global__ void __launch_bounds__(256) k_tc_scale_z(int K, int ldz, int z_rows, 
 // and the (row block, component) pair is visited unless every row of the block has
 // a_k - zb_k(new)^2 / 2 < e_lb - kSkipNats. The largest term's component is always
 // visited, so the LSE's maximum is at least e_lb.
-constexpr double kSkipNats = 110.0;
+constexpr float kSkipNats = 110.0f;
 __global__ void __launch_bounds__(128) k_tc_need(int K, const int32_t *n_rows_dev, int n_rows_max,
                                                  const int32_t *act, const double *a_k, const float *lnorm, float *zb,
                                                  const int32_t *jst, const float *zst, const float *dist,
@@ -773,10 +789,17 @@ __global__ void __launch_bounds__(128) k_tc_need(int K, const int32_t *n_rows_de
     const int j = valid ? jst[w] : -1;
     const float D = valid ? dist[w] : 0.f;
     const bool bounded = j >= 0 && D >= 0.f && isfinite(D);
-    double elb = 0.0;
+    // the test in FP32 with directed rounding (a_k widened by 2^-22 of itself): it only
+    // ever visits more than the FP64 test would, by about 0.1 nats at |e| ~ 1e6
+    auto a_up = [&](int k) {
+        const float f = f64_to_f32(a_k[k]);
+        return __fmaf_ru(fabsf(f), 0x1p-22f, f);
+    };
+    float elb = 0.f;
     if (bounded) {
-        const double ub = (double)__fmaf_ru(lnorm[j], D, zst[w]);
-        elb = a_k[j] - 0.5 * ub * ub;
+        const float f = f64_to_f32(a_k[j]);
+        const float ub = __fmaf_ru(lnorm[j], D, zst[w]);
+        elb = __fadd_rd(__fmaf_rd(-0.5f, __fmul_ru(ub, ub), __fmaf_rd(-fabsf(f), 0x1p-22f, f)), -kSkipNats);
     }
     // one CTA is one 128-row block: it writes every component's word of its block
     __shared__ unsigned long long s_need;
@@ -788,7 +811,7 @@ __global__ void __launch_bounds__(128) k_tc_need(int K, const int32_t *n_rows_de
         if (bounded) {
             const float b = fmaxf(__fmaf_rd(-lnorm[k], D, zb[(size_t)w * K + k]), 0.f);
             zb[(size_t)w * K + k] = b;
-            need = !(a_k[k] - 0.5 * (double)b * (double)b < elb - kSkipNats);
+            need = !(__fmaf_ru(-0.5f, __fmul_rd(b, b), a_up(k)) < elb);
         }
         if (__any_sync(0xffffffffu, need)) mk |= 1ull << k;
     }
@@ -1103,6 +1126,15 @@ void launch_center(const TcWs &t, int d, int K, const int32_t *n_rows_dev, int n
     else
         k_tc_center<SB_PREC_TF32><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, n_rows_dev, n_rows_max, act, X, d,
                                                       (const float *)t.p[2], t.p[9], zmask);
+}
+
+size_t lse_smem(int K) {
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_tc_lse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(double) * kMaxK * LSE_ROWS);
+    });
+    return sizeof(double) * (size_t)K * LSE_ROWS;
 }
 
 TcArgs base_args(const ProbView &pv, const TcWs &t) {
@@ -1648,7 +1680,7 @@ void tc_eval_walkers(const ProbView &pv, const sb_config *c, const TcWs &t, cons
     a.zmask = nullptr;
     a.rflag = (const uint32_t *)t.p[10];  // written for every block by k_tc_lse
     note_launch();
-    k_tc_lse<<<(n + 127) / 128, 128, 0, s>>>(0, pv.K, a.n_ntile, n_act, n, act, a.qpart, pv.a, (float *)t.p[6], FT,
+    k_tc_lse<<<(n + LSE_ROWS - 1) / LSE_ROWS, LSE_ROWS, lse_smem(pv.K), s>>>(0, pv.K, a.n_ntile, n_act, n, act, a.qpart, pv.a, (float *)t.p[6], FT,
                                              nullptr, (uint32_t *)t.p[10], zmask, (float *)t.p[11],
                                              (int32_t *)t.p[12], (float *)t.p[13]);
     launch_scale_z(pv, t, n_act, n, s);
@@ -1675,7 +1707,7 @@ sb_status tc_loglik_points(const ProbView &pv, const sb_config *c, const TcWs &t
     launch_gemm_any(t.prec, grad ? MODE_ZW : MODE_ZR, t.bn, t.mapA1, t.mapT, a, s);
     a.rflag = (const uint32_t *)t.p[10];  // written for every block by k_tc_lse
     note_launch();
-    k_tc_lse<<<(n + 127) / 128, 128, 0, s>>>(2, pv.K, a.n_ntile, nullptr, n, nullptr, a.qpart, pv.a,
+    k_tc_lse<<<(n + LSE_ROWS - 1) / LSE_ROWS, LSE_ROWS, lse_smem(pv.K), s>>>(2, pv.K, a.n_ntile, nullptr, n, nullptr, a.qpart, pv.a,
                                              (float *)t.p[6], nullptr, ell, (uint32_t *)t.p[10], nullptr, nullptr,
                                              nullptr, nullptr);
     if (grad) {
