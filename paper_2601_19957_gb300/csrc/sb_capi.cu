@@ -387,7 +387,7 @@ sb_status run_discover(const ProbView &pv, const sb_config *c, const Layout &L, 
     } else {
         // one GEMM of the directions, l at the samples from three scalars per (ray, component)
         const sb_status st = tc_ray_loglik_quad(pv, c->n_rays, c->n_steps, c->prec, L.di.tc.bn, L.di.quad, L.di.u,
-                                                L.di.texit, L.di.ell_all, s);
+                                                L.di.texit, false, L.di.ell_all, s);
         if (st != SB_OK) return st;
     }
     launch_select_starts(L.di.ell_all, c->n_rays, c->n_steps, c->n_starts, L.di.sel, s);
@@ -1773,8 +1773,7 @@ extern "C" sb_status sb_ray_loglik_quad(const sb_problem *p, int32_t form, const
     else {
         const int prec = form == 2 ? SB_PREC_BF16 : SB_PREC_TF32;
         if (!tc_available(prec)) return SB_ERR_UNSUPPORTED;
-        launch_ray_texit(pv, u, n_rays, w.scratch, cs);
-        st = tc_ray_loglik_quad(pv, n_rays, n_steps, prec, 0, w.quad, u, w.scratch, ell, cs);
+        st = tc_ray_loglik_quad(pv, n_rays, n_steps, prec, 0, w.quad, u, w.scratch, true, ell, cs);
         if (st != SB_OK) return st;
     }
     SB_CUDA_TRY(cudaGetLastError());

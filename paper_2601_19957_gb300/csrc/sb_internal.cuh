@@ -137,14 +137,17 @@ __device__ __forceinline__ bool is_finite(float v) { return isfinite(v); }
 // hardware conversions, takes one warp instruction per 19 cycles and SM: a pass that
 // converts every element it moves is bound by it (8 bytes a lane and 19 cycles are 13
 // bytes a cycle and SM, well below HBM). Same results as the hardware conversions
-// (round to nearest even), which serve the rare exponents.
+// (round to nearest even), which serve the rare exponents, by a call: inlined they would
+// be predicated and take their turns on the pipe all the same.
+static __device__ __noinline__ float cvt_f32_slow(double v) { return (float)v; }
+static __device__ __noinline__ double cvt_f64_slow(float v) { return (double)v; }
 __device__ __forceinline__ float f64_to_f32(double v) {
     const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
     const uint32_t e = (hi >> 20) & 0x7ffu;
     const uint32_t sign = hi & 0x80000000u;
     if (e - 897u > 253u) {  // not a normal float (zero, below 2^-126, above 2^127)
         if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(sign);
-        return (float)v;
+        return cvt_f32_slow(v);
     }
     const uint32_t m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
     const uint32_t rest = lo & 0x1fffffffu;
@@ -157,7 +160,7 @@ __device__ __forceinline__ double f32_to_f64(float v) {
     const uint32_t sign = u & 0x80000000u;
     if (e - 1u > 253u) {  // zero, subnormal, infinity or NaN
         if ((u & 0x7fffffffu) == 0u) return __hiloint2double((int)sign, 0);
-        return (double)v;
+        return cvt_f64_slow(v);
     }
     return __hiloint2double((int)(sign | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
 }

@@ -46,17 +46,19 @@ void tc_to_f32(const double *x, float *y, size_t n, cudaStream_t s);
 struct TcQuadWs {
     void *A2, *B2;                   // [rows][2 dK] direction splits, [K][d][2 dK] L_k^T splits
     float *alpha, *qpart1, *qpart2;  // [K][ald] z_k(c) in FP32 (zero past d); partials [rows][K][nct]
-    double *zc, *q0;                 // [K][d] z_k(c), [K] |z_k(c)|^2
-    double2 *q12;                    // [n_rays][K] (z_k(c) . w_rk, |w_rk|^2) in FP64
+    double *zc, *q0;                 // parts of z_k(c) [.][K][d], [K] |z_k(c)|^2
+    double *co;                      // [n_rays][K][3] coefficients of e_k in tau (FP64)
+    float4 *cf;                      // [n_rays][K] the same in FP32
     int rows, dK, ald;
     CUtensorMap mapU, mapL;
 };
 void carve_tc_quad(Carver &cv, TcQuadWs &q, int n_rays, int d, int K, int prec);
-// l at every ray sample from the FP64 directions u [n_rays][d] and t_exit; ell_all[r n_steps + j].
+// l at every ray sample from the FP64 directions u [n_rays][d] and t_exit (exits: computed
+// here, from pv.half, in the pass that splits u); ell_all[r n_steps + j].
 // bn: the GEMM's column tile (64, 128 or 256; 0: the width tuned for (d, K, prec) in
 // this process, else the heuristic one). pv needs a_k, mu, L and c.
 sb_status tc_ray_loglik_quad(const ProbView &pv, int n_rays, int n_steps, int prec, int bn, TcQuadWs q,
-                             const double *u, const double *texit, double *ell_all, cudaStream_t s);
+                             const double *u, double *texit, bool exits, double *ell_all, cudaStream_t s);
 // Rays from per-ray origins, x = o_r + tau u_r, in the same quadratic form:
 // z_k(o_r + tau u_r) = z_k(o_r) + tau w_rk, z_k(o_r) = o_r L_k - mu_k L_k from a split
 // GEMM of the origins (FP32 result, stored, with the FP32 -mu_k L_k added in the
@@ -64,8 +66,7 @@ sb_status tc_ray_loglik_quad(const ProbView &pv, int n_rays, int n_steps, int pr
 // dot products with the stored z_k(o_r).
 struct TcOriginWs {
     float *zo, *off, *qp0;  // [rows][K][ald] z_k(o_r); [K][ald] -mu_k L_k (FP32); [rows][K][nct] |z|^2 partials
-    double *negm, *q0k;     // [K][d] -mu_k L_k (FP64); [K] scratch
-    double *q0r;            // [rows][K] |z_k(o_r)|^2
+    double *negm, *q0k;     // parts of -mu_k L_k [.][K][d] (FP64); [K] scratch
 };
 void carve_tc_origins(Carver &cv, TcOriginWs &o, int n_rays, int d, int K, int prec);
 // Split L_k^T into q.B2 and -mu_k L_k into o.off (once per problem and call).

@@ -967,26 +967,98 @@ __global__ void __launch_bounds__(256) k_tc_center(int d, int K, int rows_cap, i
     }
 }
 
-template <typename E>
-__global__ void k_tc_convert_L(int d, int K, int ldp, const double *L, E *LT, E *LB) {
-    const size_t tot = (size_t)K * d * ldp;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(e / ((size_t)d * ldp));
-        const size_t rem = e % ((size_t)d * ldp);
-        const int row = (int)(rem / ldp), col = (int)(rem % ldp);
-        double lt = 0.0, lb = 0.0;
-        if (col < d) {
-            const double *Lk = L + (size_t)k * d * d;
-            if (col >= row) lt = Lk[(size_t)col * d + row];  // LT[k][j=row][i=col] = L[i][j], i >= j
-            if (col <= row) lb = Lk[(size_t)row * d + col];  // LB[k][i=row][j=col] = L[i][j], j <= i
-        }
-        if (sizeof(E) == 2) {
-            reinterpret_cast<__nv_bfloat16 *>(LT)[e] = __double2bfloat16(lt);
-            reinterpret_cast<__nv_bfloat16 *>(LB)[e] = __double2bfloat16(lb);
-        } else {
-            reinterpret_cast<float *>(LT)[e] = to_tf32((float)lt);
-            reinterpret_cast<float *>(LB)[e] = to_tf32((float)lb);
-        }
+// ------------------------------------------------------------------ operands from FP64
+// A double as its 24-bit truncation t plus the rest (x = t + rest exactly for the
+// exponents it accepts; zero gives zeros). On the integer units: the FP64 pipe, which also
+// does the hardware conversions, was the bound of every pass that converted (see
+// f64_to_f32).
+__device__ __forceinline__ bool split24(double x, float &t, float &rest) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+    t = rest = 0.f;
+    if (e - 960u > 126u) return ((hi & 0x7fffffffu) | lo) == 0u;  // outside [2^-63, 2^64)
+    t = __uint_as_float(sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    // 29 bits of weight 2^(e - 1023 - 52)
+    rest = __uint2float_rn(lo & 0x1fffffffu) * __uint_as_float(sign | ((e - 948u) << 23));
+    return true;
+}
+// The same through FP64 arithmetic, for what the integer route does not cover (calls, so
+// that they are not predicated into it).
+template <int PREC>
+__device__ __noinline__ float round_op_slow(double x) {
+    return PREC == SB_PREC_BF16 ? __bfloat162float(__double2bfloat16(x)) : to_tf32((float)x);
+}
+// x rounded to nearest bf16 / tf32 (the tf32 rounding as of (float) x)
+template <int PREC>
+__device__ __forceinline__ float round_op(double x) {
+    if (PREC == SB_PREC_BF16) {
+        float t, rest;
+        if (!split24(x, t, rest)) return round_op_slow<PREC>(x);
+        // the dropped bits as a sticky last bit: rounding t to 8 bits is then rounding x
+        if (rest != 0.f) t = __uint_as_float(__float_as_uint(t) | 1u);
+        return __bfloat162float(__float2bfloat16_rn(t));
+    }
+    return to_tf32(f64_to_f32(x));
+}
+// x split into hi + lo of the operand precision: hi = round(x), lo = round(x - hi). x - hi =
+// (t - hi) + rest with t - hi exact; its FP32 rounding decides lo unless it falls on (bf16),
+// or next to (tf32), the midpoint of two operand values, where FP64 does.
+template <int PREC>
+__device__ __noinline__ float split_lo_slow(double x, float hi) {
+    return round_op_slow<PREC>(x - (double)hi);
+}
+template <int PREC>
+__device__ __forceinline__ void split_op(double x, float &hi, float &lo) {
+    float t, rest;
+    const bool ok = split24(x, t, rest);
+    hi = round_op<PREC>(x);
+    float r = (t - hi) + rest;
+    const uint32_t low = __float_as_uint(r);
+    const bool mid = PREC == SB_PREC_BF16 ? (low & 0xffffu) == 0x8000u : ((low + 1u) & 0x1fffu) - 0x1000u <= 2u;
+    if (!ok || mid) {
+        lo = split_lo_slow<PREC>(x, hi);
+        return;
+    }
+    lo = PREC == SB_PREC_BF16 ? __bfloat162float(__float2bfloat16_rn(r)) : to_tf32(r);
+}
+// Two neighbouring elements (values of the operand precision) at an even index.
+template <int PREC>
+__device__ __forceinline__ void put_pair(void *base, size_t e, float a, float b) {
+    if (PREC == SB_PREC_BF16)
+        reinterpret_cast<uint32_t *>(base)[e / 2] = pack_bf16x2(a, b);
+    else
+        reinterpret_cast<float2 *>(base)[e / 2] = make_float2(a, b);
+}
+
+// The tensor-core copies LT[k][j][i] = LB[k][i][j] = round(L_k[i][j]) for i >= j, zeros
+// elsewhere (rows of ldp elements), by 64 x 32 tiles of L_k through shared memory: L is
+// read once, along its rows, and both copies are written in whole rows of a tile (an
+// element per thread read L_k down its columns: 38 us at d = 1024, K = 8, 19 us now; 100
+// MB of traffic are 15 us).
+constexpr int CV_I = 64, CV_J = 32;
+template <int PREC>
+__global__ void __launch_bounds__(256) k_tc_convert_L(int d, int ldp, const double *L, void *LT, void *LB) {
+    __shared__ float t[CV_J][CV_I + 2];
+    const int i0 = blockIdx.x * CV_I, j0 = blockIdx.y * CV_J, k = blockIdx.z;
+    const double *Lk = L + (size_t)k * d * d;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < CV_I / 8; ++q) {
+        const int i = i0 + wid + 8 * q, j = j0 + lane;
+        t[lane][wid + 8 * q] = i < d && j <= i ? round_op<PREC>(Lk[(size_t)i * d + j]) : 0.f;
+    }
+    __syncthreads();
+    // LT: rows j, pairs along i
+#pragma unroll
+    for (int q = 0; q < CV_J / 8; ++q) {
+        const int jj = wid + 8 * q, j = j0 + jj, i = i0 + 2 * lane;
+        if (j < d && i < ldp) put_pair<PREC>(LT, ((size_t)k * d + j) * ldp + i, t[jj][2 * lane], t[jj][2 * lane + 1]);
+    }
+    // LB: rows i, pairs along j (16 lanes a row)
+#pragma unroll
+    for (int q = 0; q < CV_I / 16; ++q) {
+        const int ii = 16 * q + 2 * wid + (lane >> 4), i = i0 + ii, jj = 2 * (lane & 15), j = j0 + jj;
+        if (i < d && j < ldp) put_pair<PREC>(LB, ((size_t)k * d + i) * ldp + j, t[jj][ii], t[jj + 1][ii]);
     }
 }
 
@@ -1316,11 +1388,12 @@ int tc_tuned_tile(int d, int K, int prec) {
 sb_status tc_prepare(const ProbView &pv, TcWs &t, cudaStream_t s, bool skip_bounds) {
     const int d = pv.d, K = pv.K;
     const int ldp = ldp_of(d, t.prec);
+    const dim3 gc((unsigned)((ldp + CV_I - 1) / CV_I), (unsigned)((ldp + CV_J - 1) / CV_J), (unsigned)K);
     note_launch();
     if (t.prec == SB_PREC_BF16)
-        k_tc_convert_L<uint16_t><<<1184, 256, 0, s>>>(d, K, ldp, pv.L, (uint16_t *)t.p[0], (uint16_t *)t.p[1]);
+        k_tc_convert_L<SB_PREC_BF16><<<gc, 256, 0, s>>>(d, ldp, pv.L, t.p[0], t.p[1]);
     else
-        k_tc_convert_L<float><<<1184, 256, 0, s>>>(d, K, ldp, pv.L, (float *)t.p[0], (float *)t.p[1]);
+        k_tc_convert_L<SB_PREC_TF32><<<gc, 256, 0, s>>>(d, ldp, pv.L, t.p[0], t.p[1]);
     note_launch();
     k_tc_convert_vec<<<(K * d + 255) / 256, 256, 0, s>>>(d, K, pv.mu, pv.c, (float *)t.p[2], (float *)t.p[3]);
     if (skip_bounds) {  // partials in the qpart scratch (the Gram pass below overwrites it later)
@@ -1351,93 +1424,158 @@ sb_status tc_prepare(const ProbView &pv, TcWs &t, cudaStream_t s, bool skip_boun
 }
 
 // ------------------------------------------------------------------ quadratic form of the rays
-// x split into hi + lo of the operand precision: hi = round(x), lo = round(x - hi)
-template <int PREC>
-__device__ __forceinline__ void split_op(double x, float &hi, float &lo) {
-    if (PREC == SB_PREC_BF16) {
-        hi = __bfloat162float(__double2bfloat16(x));
-        lo = __bfloat162float(__double2bfloat16(x - (double)hi));
-    } else {
-        hi = to_tf32((float)x);
-        lo = to_tf32((float)(x - (double)hi));
-    }
-}
-template <int PREC>
-__device__ __forceinline__ void put_op(void *base, size_t e, float v) {
-    if (PREC == SB_PREC_BF16)
-        reinterpret_cast<__nv_bfloat16 *>(base)[e] = __float2bfloat16_rn(v);  // exact: v is a bf16 value
-    else
-        reinterpret_cast<float *>(base)[e] = v;
-}
-
 // A2[r][0 .. dK) = hi(u_r), A2[r][dK .. 2 dK) = lo(u_r); zeros past d and past the ray
-// count (n_rays, or *n_dev when given), rows past the count's last 128-row block untouched
+// count (n_rays, or *n_dev when given), rows past the count's last 128-row block untouched.
+// A warp per row, two neighbouring coordinates per lane. texit given: also the ray's exit
+// length from the box centre, min_i half_i / |u_i| as warp_exit_min (the exact FP64 minimum):
+// FP32 quotients of the truncated operands are within 2^-21, and only the lanes that hold
+// one within 2^-18 of the smallest (or a coordinate out of FP32's range) go over their
+// coordinates again and divide in FP64. One pass over u (134 MB at 16384 rays, d = 1024)
+// where the split and the exit lengths were two, each bound by FP64 conversions: 297 us,
+// 104 us now.
 template <int PREC>
-__global__ void k_q_split_rows(int n_rays, int rows, int d, int dK, const double *u, void *A2, const int32_t *n_dev) {
+__global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int d, int dK, const double *u, void *A2,
+                                                      const int32_t *n_dev, const double *half, double *texit) {
+    __shared__ float hf[kMaxD];  // half-widths, -1 outside the range the FP32 quotients hold for
     if (n_dev) {
         const int c = *n_dev < n_rays ? *n_dev : n_rays;
         const int rb = (c + BM - 1) / BM * BM;
         n_rays = c;
         rows = rb < rows ? rb : rows;
     }
-    const size_t tot = (size_t)rows * dK;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / dK), i = (int)(e % dK);
-        float hi = 0.f, lo = 0.f;
-        if (r < n_rays && i < d) split_op<PREC>(u[(size_t)r * d + i], hi, lo);
-        put_op<PREC>(A2, (size_t)r * 2 * dK + i, hi);
-        put_op<PREC>(A2, (size_t)r * 2 * dK + dK + i, lo);
+    const int lane = threadIdx.x & 31;
+    constexpr float kLo = 1e-30f, kHi = 1e30f;
+    if (texit) {
+        for (int i = threadIdx.x; i < d; i += blockDim.x) {
+            const float h = f64_to_f32(half[i]);
+            hf[i] = h >= kLo && h <= kHi ? h : -1.f;
+        }
+        __syncthreads();
+    }
+    for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
+        const bool live = r < n_rays;
+        const double *ur = u + (size_t)r * d;
+        const size_t o = (size_t)r * 2 * dK;
+        float est = INFINITY;
+        bool odd = false;
+#pragma unroll 4
+        for (int i = 2 * lane; i < dK; i += 64) {
+            const double x0 = live && i < d ? ur[i] : 0.0, x1 = live && i + 1 < d ? ur[i + 1] : 0.0;
+            float h0, l0, h1, l1;
+            split_op<PREC>(x0, h0, l0);
+            split_op<PREC>(x1, h1, l1);
+            put_pair<PREC>(A2, o + i, h0, h1);
+            put_pair<PREC>(A2, o + dK + i, l0, l1);
+            if (texit) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const double x = q ? x1 : x0;
+                    if (i + q >= d || ((__double_as_longlong(x) << 1) == 0)) continue;
+                    float t, rest;
+                    const bool ok = split24(x, t, rest) && hf[i + q] > 0.f;
+                    odd = odd || !ok;
+                    if (ok) est = fminf(est, __fdividef(hf[i + q], fabsf(t)));
+                }
+            }
+        }
+        if (texit && live) {
+            const float thr = warp_min(est) * (1.0f + 0x1p-18f);
+            long long best = 0x7ff0000000000000ll;  // +inf; positive doubles order as their bits
+            if (est <= thr || odd) {
+                for (int i = 2 * lane; i < d; i += 64) {
+                    for (int q = 0; q < 2 && i + q < d; ++q) {
+                        const double x = ur[i + q];
+                        if ((__double_as_longlong(x) << 1) == 0) continue;
+                        float t, rest;
+                        const bool ok = split24(x, t, rest) && hf[i + q] > 0.f;
+                        if (ok && __fdividef(hf[i + q], fabsf(t)) > thr) continue;
+                        const double v = __ddiv_rn(half[i + q], fabs(x));
+                        const long long b = __double_as_longlong(v);
+                        if (v == v && b < best) best = b;
+                    }
+                }
+            }
+#pragma unroll
+            for (int w = 16; w > 0; w >>= 1) {
+                const long long b = __shfl_xor_sync(0xffffffffu, best, w);
+                best = b < best ? b : best;
+            }
+            if (lane == 0) texit[r] = __longlong_as_double(best);
+        }
     }
 }
 
 // B2[k][j][i] = hi(L_k[i][j]), B2[k][j][dK + i] = lo(L_k[i][j]) for i >= j (L_k^T, the
-// operand of GEMM1), zeros elsewhere
+// operand of GEMM1), zeros elsewhere: 64 x 32 tiles of L_k through shared memory, as
+// k_tc_convert_L (63 us at d = 1024, K = 8 with the columns read directly, 19 us now)
 template <int PREC>
-__global__ void k_q_split_LT(int d, int K, int dK, const double *L, void *B2) {
-    const size_t tot = (size_t)K * d * dK;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(e / ((size_t)d * dK));
-        const size_t rem = e % ((size_t)d * dK);
-        const int j = (int)(rem / dK), i = (int)(rem % dK);
+__global__ void __launch_bounds__(256) k_q_split_LT(int d, int dK, const double *L, void *B2) {
+    __shared__ float th[CV_J][CV_I + 2], tl[CV_J][CV_I + 2];
+    const int i0 = blockIdx.x * CV_I, j0 = blockIdx.y * CV_J, k = blockIdx.z;
+    const double *Lk = L + (size_t)k * d * d;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < CV_I / 8; ++q) {
+        const int i = i0 + wid + 8 * q, j = j0 + lane;
         float hi = 0.f, lo = 0.f;
-        if (i < d && i >= j) split_op<PREC>(L[((size_t)k * d + i) * d + j], hi, lo);
+        if (i < d && j <= i) split_op<PREC>(Lk[(size_t)i * d + j], hi, lo);
+        th[lane][wid + 8 * q] = hi;
+        tl[lane][wid + 8 * q] = lo;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < CV_J / 8; ++q) {
+        const int jj = wid + 8 * q, j = j0 + jj, i = i0 + 2 * lane;
+        if (j >= d || i >= dK) continue;
         const size_t row = ((size_t)k * d + j) * 2 * dK;
-        put_op<PREC>(B2, row + i, hi);
-        put_op<PREC>(B2, row + dK + i, lo);
+        put_pair<PREC>(B2, row + i, th[jj][2 * lane], th[jj][2 * lane + 1]);
+        put_pair<PREC>(B2, row + dK + i, tl[jj][2 * lane], tl[jj][2 * lane + 1]);
     }
 }
 
-// z_k(c)_j = sum_{i >= j} (c_i - mu_k,i) L_k,ij in FP64 (c null: -mu_k L_k): one CTA per
-// (32 columns, component), a lane per column (rows of L_k read 256 bytes at a time),
-// the eight warps over interleaved rows, their partials summed in a fixed order
+// Quarter p of the rows of z_k(c)_j = sum_{i >= j} (c_i - mu_k,i) L_k,ij in FP64 (c null:
+// -mu_k L_k): one CTA per (32 columns, component, quarter of the columns' rows), a lane per
+// column (rows of L_k read 256 bytes at a time), the eight warps over interleaved rows,
+// their partials summed in a fixed order. Bound by the FP64 pipe, so the differences are
+// formed once per CTA and the rows shared out (one CTA per column tile: 43 us at d = 1024,
+// K = 8, 17 us now).
+constexpr int ZC_PARTS = 4;
 __global__ void __launch_bounds__(256) k_q_zc(int d, const double *c, const double *mu, const double *L,
-                                              double *zc) {
+                                              double *zcp) {
+    __shared__ double dl[kMaxD / ZC_PARTS + ZC_PARTS];
+    __shared__ double part[8][32];
     const int k = blockIdx.y, j0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int j = j0 + lane;
+    const int j = j0 + lane, len = (d - j0 + ZC_PARTS - 1) / ZC_PARTS;
+    const int i0 = j0 + blockIdx.z * len, i1 = min(d, i0 + len);
     const double *Lk = L + (size_t)k * d * d;
     const double *mk = mu + (size_t)k * d;
+    for (int i = i0 + threadIdx.x; i < i1; i += 256) dl[i - i0] = c ? c[i] - mk[i] : -mk[i];
+    __syncthreads();
     double s = 0.0;
-    if (j < d)
-        for (int i = j0 + w; i < d; i += 8)
-            if (i >= j) s = fma(c ? c[i] - mk[i] : -mk[i], Lk[(size_t)i * d + j], s);
-    __shared__ double part[8][32];
+    if (j < d) {
+#pragma unroll 4
+        for (int i = i0 + w; i < i1; i += 8)
+            s = fma(dl[i - i0], i >= j ? Lk[(size_t)i * d + j] : 0.0, s);
+    }
     part[w][lane] = s;
     __syncthreads();
     if (w == 0 && j < d) {
         double t = 0.0;
         for (int q = 0; q < 8; ++q) t += part[q][lane];
-        zc[(size_t)k * d + j] = t;
+        zcp[((size_t)blockIdx.z * gridDim.y + k) * d + j] = t;
     }
 }
 
-// alpha[k][j] = (float) z_k(c)_j (zero for d <= j < ald) and q0[k] = |z_k(c)|^2 (FP64,
-// partials in a fixed order): one CTA per component
-__global__ void __launch_bounds__(256) k_q_alpha(int d, int ald, const double *zc, float *alpha, double *q0) {
+// z_k(c) from its parts: alpha[k][j] = (float) z_k(c)_j (zero for d <= j < ald) and q0[k] =
+// |z_k(c)|^2 (FP64, partials in a fixed order): one CTA per component
+__global__ void __launch_bounds__(256) k_q_alpha(int d, int K, int ald, const double *zcp, float *alpha, double *q0) {
     const int k = blockIdx.x;
     double s = 0.0;
     for (int j = threadIdx.x; j < ald; j += blockDim.x) {
-        const double z = j < d ? zc[(size_t)k * d + j] : 0.0;
-        alpha[(size_t)k * ald + j] = (float)z;
+        double z = 0.0;
+        if (j < d)
+            for (int p = 0; p < ZC_PARTS; ++p) z += zcp[((size_t)p * K + k) * d + j];
+        alpha[(size_t)k * ald + j] = f64_to_f32(z);
         s = fma(z, z, s);
     }
     __shared__ double part[8];
@@ -1451,55 +1589,116 @@ __global__ void __launch_bounds__(256) k_q_alpha(int d, int ald, const double *z
     }
 }
 
-// (q1, q2)[r][k]: the FP64 sums of ray r's column-tile partials (FP32) of z_k(c) . w_rk
-// and |w_rk|^2, one thread per (ray, component)
-// (qp0 given: also q0r[r][k], the sum of the origin pass's |z_k(o_r)|^2 partials; K and
-// the ray count *n_dev bound the pairs when n_dev is given)
+// The term of component k along ray r is e_k(tau) = c0 + tau (c1 + tau c2), c0 = a_k - q0 /
+// 2, c1 = -q1, c2 = -q2 / 2 with the FP64 sums of the ray's column-tile partials (FP32) of
+// z_k(o) . w_rk and |w_rk|^2 (and of |z_k(o)|^2 when qp0 is given, else q0[k]): one thread
+// per (ray, component) leaves the coefficients in FP64 and FP32. K and the ray count *n_dev
+// bound the pairs when n_dev is given.
 __global__ void __launch_bounds__(256) k_q_sum(int n_rk, int n_ntile, const float *qp1, const float *qp2,
-                                               double2 *q12, const float *qp0, double *q0r, int K,
-                                               const int32_t *n_dev) {
+                                               const double *a_k, const double *q0, const float *qp0, double *co,
+                                               float4 *cf, int K, const int32_t *n_dev) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n_rk || (n_dev && e >= *n_dev * K)) return;
+    const int k = e % K;
     const float *p1 = qp1 + (size_t)e * n_ntile;
     const float *p2 = qp2 + (size_t)e * n_ntile;
-    double q1 = 0.0, q2 = 0.0;
-    for (int t = 0; t < n_ntile; ++t) {
-        q1 += (double)p1[t];
-        q2 += (double)p2[t];
+    double q1 = f32_to_f64(p1[0]), q2 = f32_to_f64(p2[0]), q = 0.0;
+    for (int t = 1; t < n_ntile; ++t) {
+        q1 += f32_to_f64(p1[t]);
+        q2 += f32_to_f64(p2[t]);
     }
-    q12[e] = make_double2(q1, q2);
     if (qp0) {
         const float *p0 = qp0 + (size_t)e * n_ntile;
-        double q0 = 0.0;
-        for (int t = 0; t < n_ntile; ++t) q0 += (double)p0[t];
-        q0r[e] = q0;
+        q = f32_to_f64(p0[0]);
+        for (int t = 1; t < n_ntile; ++t) q += f32_to_f64(p0[t]);
+    } else {
+        q = q0[k];
+    }
+    const double c0 = fma(-0.5, q, a_k[k]), c1 = -q1, c2 = -0.5 * q2;
+    co[3 * (size_t)e] = c0;
+    co[3 * (size_t)e + 1] = c1;
+    co[3 * (size_t)e + 2] = c2;
+    cf[e] = make_float4(f64_to_f32(c0), f64_to_f32(c1), f64_to_f32(c2), 0.f);
+}
+
+// l at sample j of ray r, tau = ((j + 1) / n_steps) t_exit,r: the terms in FP64, the LSE as
+// in k_tc_lse (FP32 exponentials of the shifted terms). Bound by the FP64 pipe, so FP32
+// decides which terms can matter: with the coefficients rounded to FP32 a term is off by at
+// most 2^-21 of |c0| + tau |c1| + tau^2 |c2|, and a component that stays 110 nats below the
+// largest lower bound adds an FP32 exponential of exactly 0. A CTA takes RB rays at a time
+// by JW samples and QE_PASS times that, so that (j + 1) / n_steps is divided once per thread.
+// Every term in FP64, twice, and a division per sample: 196 us at 16384 rays x 64 samples,
+// K = 8, 66 us now. (ns_dev given: samples past *ns_dev are skipped)
+constexpr int QE_PASS = 8;
+__global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, int JW, const double *co,
+                                               const float4 *cf, const double *texit, double *ell,
+                                               const int32_t *ns_dev) {
+    const int nj = (n_steps + JW - 1) / JW, rb = blockIdx.x / nj;
+    const int RB = 256 / JW, j = (blockIdx.x - rb * nj) * JW + threadIdx.x % JW;
+    if (j >= n_steps) return;
+    const int64_t ns = ns_dev ? *ns_dev : (int64_t)n_rays * n_steps;
+    const double tf64 = (double)(j + 1) / (double)n_steps;
+    int r = rb * RB * QE_PASS + threadIdx.x / JW;
+    for (int p = 0; p < QE_PASS; ++p, r += RB) {
+        const int64_t e = (int64_t)r * n_steps + j;
+        if (r >= n_rays || e >= ns) return;
+        const double tau = tf64 * texit[r];
+        const float tf = f64_to_f32(tau);
+        const float4 *cr = cf + (size_t)r * K;
+        const double *dr = co + 3 * (size_t)r * K;
+        auto bound = [&](const float4 &c, float sgn) {
+            const float f = fmaf(tf, fmaf(tf, c.z, c.y), c.x);
+            return fmaf(sgn * 0x1p-21f, fmaf(tf, fmaf(tf, fabsf(c.z), fabsf(c.y)), fabsf(c.x)), f);
+        };
+        float low = -INFINITY;
+        for (int k = 0; k < K; ++k) low = fmaxf(low, bound(cr[k], -1.f));
+        low -= kSkipNats;
+        auto term = [&](int k) { return fma(tau, fma(tau, dr[3 * k + 2], dr[3 * k + 1]), dr[3 * k]); };
+        uint64_t keep = 0;
+        double emax = -INFINITY;
+        for (int k = 0; k < K; ++k) {
+            if (bound(cr[k], 1.f) < low) continue;
+            keep |= 1ull << k;
+            const double t = term(k);
+            emax = t > emax ? t : emax;
+        }
+        double l = emax;  // one term left: its exponential is 1
+        if ((keep & (keep - 1)) || !finite_bits(emax)) {
+            float s = 0.f;
+            for (uint64_t m = keep; m; m &= m - 1) s += __expf(f64_to_f32(term(__ffsll((long long)m) - 1) - emax));
+            l = emax + f32_to_f64(__logf(s));
+        }
+        ell[e] = l;
     }
 }
 
-// l at sample j of ray r: |z_k|^2 = q0_k + 2 tau q1_rk + tau^2 q2_rk in FP64,
-// tau = ((j + 1) / n_steps) t_exit,r; the LSE as in k_tc_lse (FP64 terms, FP32
-// exponentials of the shifted terms). The threads of a warp mostly share a ray, so
-// its coefficients are broadcast loads.
-// (q0r given: q0 of ray r is q0r[r][k], the ray's own origin; ns_dev given: samples
-// past *ns_dev are skipped)
-__global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, const double *a_k, const double *q0,
-                                               const double2 *q12, const double *texit, double *ell,
-                                               const double *q0r, const int32_t *ns_dev) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)n_rays * n_steps || (ns_dev && e >= *ns_dev)) return;
-    const int r = (int)(e / n_steps), j = (int)(e - (int64_t)r * n_steps);
-    const double tau = ((double)(j + 1) / (double)n_steps) * texit[r];
-    const double2 *qr = q12 + (size_t)r * K;
-    const double *q0k = q0r ? q0r + (size_t)r * K : q0;
-    auto term = [&](int k) {
-        const double2 q = qr[k];
-        return a_k[k] - 0.5 * (q0k[k] + tau * (2.0 * q.x + tau * q.y));
-    };
-    double emax = -INFINITY;
-    for (int k = 0; k < K; ++k) emax = fmax(emax, term(k));
-    float s = 0.f;
-    for (int k = 0; k < K; ++k) s += __expf((float)(term(k) - emax));
-    ell[e] = emax + (double)__logf(s);
+void launch_q_ell(int n_rays, int n_steps, int K, const TcQuadWs &q, const double *texit, double *ell,
+                  const int32_t *ns_dev, cudaStream_t s) {
+    int JW = 32;
+    while (JW < 256 && JW < n_steps) JW *= 2;
+    const int rays = 256 / JW * QE_PASS;
+    note_launch();
+    const int64_t grid = (int64_t)((n_rays + rays - 1) / rays) * ((n_steps + JW - 1) / JW);
+    k_q_ell<<<(unsigned)grid, 256, 0, s>>>(n_rays, n_steps, K, JW, q.co, q.cf, texit, ell, ns_dev);
+}
+
+void launch_q_split_LT(const ProbView &pv, int prec, const TcQuadWs &q, cudaStream_t s) {
+    const dim3 g((unsigned)((q.dK + CV_I - 1) / CV_I), (unsigned)((pv.d + CV_J - 1) / CV_J), (unsigned)pv.K);
+    note_launch();
+    if (prec == SB_PREC_BF16)
+        k_q_split_LT<SB_PREC_BF16><<<g, 256, 0, s>>>(pv.d, q.dK, pv.L, q.B2);
+    else
+        k_q_split_LT<SB_PREC_TF32><<<g, 256, 0, s>>>(pv.d, q.dK, pv.L, q.B2);
+}
+
+void launch_q_split_rows(int n_rays, int d, int prec, const TcQuadWs &q, const double *u, const int32_t *n_dev,
+                         const double *half, double *texit, cudaStream_t s) {
+    const int g = (q.rows + 7) / 8 < 8 * num_sms() ? (q.rows + 7) / 8 : 8 * num_sms();
+    note_launch();
+    if (prec == SB_PREC_BF16)
+        k_q_split_rows<SB_PREC_BF16><<<g, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, n_dev, half, texit);
+    else
+        k_q_split_rows<SB_PREC_TF32><<<g, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, n_dev, half, texit);
 }
 
 void carve_tc_quad(Carver &cv, TcQuadWs &q, int n_rays, int d, int K, int prec) {
@@ -1513,31 +1712,24 @@ void carve_tc_quad(Carver &cv, TcQuadWs &q, int n_rays, int d, int K, int prec) 
     q.alpha = cv.take<float>((size_t)K * q.ald);
     q.qpart1 = cv.take<float>((size_t)q.rows * K * nct);
     q.qpart2 = cv.take<float>((size_t)q.rows * K * nct);
-    q.zc = cv.take<double>((size_t)K * d);
+    q.zc = cv.take<double>((size_t)ZC_PARTS * K * d);
     q.q0 = cv.take<double>((size_t)K);
-    q.q12 = cv.take<double2>((size_t)n_rays * K);
+    q.co = cv.take<double>(3 * (size_t)n_rays * K);
+    q.cf = cv.take<float4>((size_t)n_rays * K);
 }
 
 sb_status tc_ray_loglik_quad(const ProbView &pv, int n_rays, int n_steps, int prec, int bn, TcQuadWs q,
-                             const double *u, const double *texit, double *ell_all, cudaStream_t s) {
+                             const double *u, double *texit, bool exits, double *ell_all, cudaStream_t s) {
     const int d = pv.d, K = pv.K;
     if (bn <= 0) bn = tc_tuned_tile(d, K, prec);
     if (bn <= 0) bn = bn_of(d);
-    const unsigned gs = 1184;
-    note_launch();
-    note_launch();
-    if (prec == SB_PREC_BF16) {
-        k_q_split_rows<SB_PREC_BF16><<<gs, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, nullptr);
-        k_q_split_LT<SB_PREC_BF16><<<gs, 256, 0, s>>>(d, K, q.dK, pv.L, q.B2);
-    } else {
-        k_q_split_rows<SB_PREC_TF32><<<gs, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, nullptr);
-        k_q_split_LT<SB_PREC_TF32><<<gs, 256, 0, s>>>(d, K, q.dK, pv.L, q.B2);
-    }
+    launch_q_split_rows(n_rays, d, prec, q, u, nullptr, pv.half, exits ? texit : nullptr, s);
+    launch_q_split_LT(pv, prec, q, s);
     // z_k(c) in FP64 (one point), then its FP32 copy and |z_k(c)|^2
     note_launch();
-    k_q_zc<<<dim3((unsigned)((d + 31) / 32), (unsigned)K), 256, 0, s>>>(d, pv.c, pv.mu, pv.L, q.zc);
+    k_q_zc<<<dim3((unsigned)((d + 31) / 32), (unsigned)K, ZC_PARTS), 256, 0, s>>>(d, pv.c, pv.mu, pv.L, q.zc);
     note_launch();
-    k_q_alpha<<<K, 256, 0, s>>>(d, q.ald, q.zc, q.alpha, q.q0);
+    k_q_alpha<<<K, 256, 0, s>>>(d, K, q.ald, q.zc, q.alpha, q.q0);
     if (!make_map(&q.mapU, q.A2, 2 * q.dK, q.rows, 1, 2 * q.dK, prec, BM) ||
         !make_map(&q.mapL, q.B2, 2 * q.dK, d, K, 2 * q.dK, prec, bn))
         return SB_ERR_CUDA;
@@ -1556,13 +1748,10 @@ sb_status tc_ray_loglik_quad(const ProbView &pv, int n_rays, int n_steps, int pr
     a.zmask = nullptr;
     a.rflag = nullptr;
     launch_gemm_any(prec, MODE_Q, bn, q.mapU, q.mapL, a, s);
-    const int64_t ns = (int64_t)n_rays * n_steps;
     note_launch();
-    k_q_sum<<<(unsigned)((n_rays * K + 255) / 256), 256, 0, s>>>(n_rays * K, a.n_ntile, q.qpart1, q.qpart2, q.q12,
-                                                                 nullptr, nullptr, K, nullptr);
-    note_launch();
-    k_q_ell<<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(n_rays, n_steps, K, pv.a, q.q0, q.q12, texit, ell_all,
-                                                         nullptr, nullptr);
+    k_q_sum<<<(unsigned)((n_rays * K + 255) / 256), 256, 0, s>>>(n_rays * K, a.n_ntile, q.qpart1, q.qpart2, pv.a, q.q0,
+                                                                 nullptr, q.co, q.cf, K, nullptr);
+    launch_q_ell(n_rays, n_steps, K, q, texit, ell_all, nullptr, s);
     return cudaGetLastError() == cudaSuccess ? SB_OK : SB_ERR_CUDA;
 }
 
@@ -1574,24 +1763,18 @@ void carve_tc_origins(Carver &cv, TcOriginWs &o, int n_rays, int d, int K, int p
     o.zo = cv.take<float>((size_t)rows * K * ald);
     o.off = cv.take<float>((size_t)K * ald);
     o.qp0 = cv.take<float>((size_t)rows * K * nct);
-    o.negm = cv.take<double>((size_t)K * d);
+    o.negm = cv.take<double>((size_t)ZC_PARTS * K * d);
     o.q0k = cv.take<double>((size_t)K);
-    o.q0r = cv.take<double>((size_t)rows * K);
 }
 
 sb_status tc_quad_prepare_origins(const ProbView &pv, int prec, TcQuadWs q, TcOriginWs o, cudaStream_t s) {
     const int d = pv.d, K = pv.K;
-    const unsigned gs = 1184;
-    note_launch();
-    if (prec == SB_PREC_BF16)
-        k_q_split_LT<SB_PREC_BF16><<<gs, 256, 0, s>>>(d, K, q.dK, pv.L, q.B2);
-    else
-        k_q_split_LT<SB_PREC_TF32><<<gs, 256, 0, s>>>(d, K, q.dK, pv.L, q.B2);
+    launch_q_split_LT(pv, prec, q, s);
     // -mu_k L_k in FP64, then its FP32 copy (the origin pass's offset)
     note_launch();
-    k_q_zc<<<dim3((unsigned)((d + 31) / 32), (unsigned)K), 256, 0, s>>>(d, nullptr, pv.mu, pv.L, o.negm);
+    k_q_zc<<<dim3((unsigned)((d + 31) / 32), (unsigned)K, ZC_PARTS), 256, 0, s>>>(d, nullptr, pv.mu, pv.L, o.negm);
     note_launch();
-    k_q_alpha<<<K, 256, 0, s>>>(d, q.ald, o.negm, o.off, o.q0k);
+    k_q_alpha<<<K, 256, 0, s>>>(d, K, q.ald, o.negm, o.off, o.q0k);
     return cudaGetLastError() == cudaSuccess ? SB_OK : SB_ERR_CUDA;
 }
 
@@ -1601,16 +1784,11 @@ sb_status tc_ray_origins_quad(const ProbView &pv, int n_cap, int n_steps, int pr
     const int d = pv.d, K = pv.K;
     if (bn <= 0) bn = tc_tuned_tile(d, K, prec);
     if (bn <= 0) bn = bn_of(d);
-    const unsigned gs = 1184;
     if (!make_map(&q.mapU, q.A2, 2 * q.dK, q.rows, 1, 2 * q.dK, prec, BM) ||
         !make_map(&q.mapL, q.B2, 2 * q.dK, d, K, 2 * q.dK, prec, bn))
         return SB_ERR_CUDA;
     auto split = [&](const double *src) {
-        note_launch();
-        if (prec == SB_PREC_BF16)
-            k_q_split_rows<SB_PREC_BF16><<<gs, 256, 0, s>>>(n_cap, q.rows, d, q.dK, src, q.A2, n_rays_dev);
-        else
-            k_q_split_rows<SB_PREC_TF32><<<gs, 256, 0, s>>>(n_cap, q.rows, d, q.dK, src, q.A2, n_rays_dev);
+        launch_q_split_rows(n_cap, d, prec, q, src, n_rays_dev, nullptr, nullptr, s);
     };
     TcArgs a{};
     a.d = d;
@@ -1638,12 +1816,9 @@ sb_status tc_ray_origins_quad(const ProbView &pv, int n_cap, int n_steps, int pr
     a.qpart1 = q.qpart1;
     launch_gemm_any(prec, MODE_Q, bn, q.mapU, q.mapL, a, s);
     note_launch();
-    k_q_sum<<<(unsigned)((n_cap * K + 255) / 256), 256, 0, s>>>(n_cap * K, a.n_ntile, q.qpart1, q.qpart2, q.q12, o.qp0,
-                                                                o.q0r, K, n_rays_dev);
-    const int64_t ns = (int64_t)n_cap * n_steps;
-    note_launch();
-    k_q_ell<<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(n_cap, n_steps, K, pv.a, nullptr, q.q12, texit, ell, o.q0r,
-                                                         n_samples_dev);
+    k_q_sum<<<(unsigned)((n_cap * K + 255) / 256), 256, 0, s>>>(n_cap * K, a.n_ntile, q.qpart1, q.qpart2, pv.a,
+                                                                nullptr, o.qp0, q.co, q.cf, K, n_rays_dev);
+    launch_q_ell(n_cap, n_steps, K, q, texit, ell, n_samples_dev, s);
     return cudaGetLastError() == cudaSuccess ? SB_OK : SB_ERR_CUDA;
 }
 
