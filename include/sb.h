@@ -118,9 +118,8 @@ size_t sb_workspace_bytes(const sb_problem *prob, const sb_config *cfg);
  * allocation, or a plugin that may not call cudaMalloc). There is no
  * counterpart in the paper. Same arguments and results as sb_loglik minus
  * ws/ws_bytes: the scratch is a 32 MiB array inside this library, held by
- * every GPU that loads it until the process exits. Requests whose
- * sb_loglik_workspace_bytes exceed 32 MiB return SB_ERR_WORKSPACE before any
- * launch. Every call made outside a stream capture looks up this device's
+ * every GPU that loads it until the process exits. Requests that need more
+ * than 32 MiB return SB_ERR_WORKSPACE before any launch. Every call made outside a stream capture looks up this device's
  * address of the array (so the first call on a device must come before any
  * capture; a capture reuses the last address looked up). With SB_PREC_BF16 /
  * SB_PREC_TF32, the first call per (d, K, prec) in a process also runs the
@@ -137,7 +136,9 @@ sb_status sb_loglik_noalloc(const sb_problem *prob, int32_t prec, const double *
  * `stream`, returns it as sb_check does, and clears it. */
 sb_status sb_loglik_noalloc_check(void *stream);
 
-/* Bytes of scratch sb_loglik needs for n points at precision prec. */
+/* Bytes of scratch sb_loglik takes for n points at precision prec (FP64: with the row lists
+ * of its grouped evaluation; a workspace without room for them is accepted too, and every
+ * component is then evaluated in full, with the same results). */
 size_t sb_loglik_workspace_bytes(const sb_problem *prob, int32_t prec, int32_t n);
 
 /*

@@ -8,31 +8,102 @@
 // The Gaussian-mixture likelihood is the paper's problem statement (Sec. 3.2);
 // the analytic gradient replaces its finite differences (App. A.4.1).
 //
-// Tiling: 64 points x 64 output coordinates per CTA, reduction chunks of 16,
-// 256 threads with a 4x4 register tile each. Only the triangle that L_k
-// occupies is visited: the z GEMM for output column block [j0, j0+64) reads
-// rows i >= j0 of L_k; the gradient GEMM for output block [i0, i0+64) reads
-// columns j < i0 + 64. FP64 throughput bounds this path; it exists as the
-// exact reference path and the plain-FP64 comparator of the tensor-core path.
+// FP64 throughput bounds this path (an SM takes one FP64 warp instruction per 19 cycles); it
+// exists as the exact reference path and the plain-FP64 comparator of the tensor-core path.
+//
+// Tiling: 8 R points x 64 output coordinates per CTA (R = 4; R = 1 for the short row lists
+// below, whose few tiles would otherwise be the launch's tail), reduction chunks of 16, 128
+// threads with an R x 4 register tile each (columns tx + 16 c). Only the
+// triangle that L_k occupies is visited: the z GEMM for output column block [j0, j0 + 64)
+// reads rows i >= j0 of L_k, the gradient GEMM for output block [i0, i0 + 64) columns j < i0 +
+// 64, and inside a diagonal block the 16-column groups that lie wholly outside the
+// triangle are left out (6 of 16).
+//
+// Grouped evaluation (K >= 2, more than one column block, and enough rows): the last column
+// block of every z_k, the cheapest, gives part of |z_k|^2; the row's component with the largest
+// a_k - |part|^2 / 2 leads and is finished first; another component is finished only when it
+// could still come within kSkipNats64 nats of the leading term. exp() of the difference is
+// exactly 0 in FP64 otherwise, so neither l, r nor grad l depends on the rest of its z_k.
+// Rows are listed per component, so the tiles hold rows that need the same L_k, and the
+// gradient runs over the components with r != 0 only. Each sum keeps the order of the full
+// evaluation, so the results are the same bits. l and grad l at 4096 points, d = 256, K = 4:
+// 3227 us -> 819 us (the FP64 pipe's floor for every component in full is 2.0 ms).
 #include "sb_internal.cuh"
 #include "sb_small_f64.cuh"
+
+#include <type_traits>
 
 namespace sb {
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16;
+constexpr int BM = 32, BN = 64, BK = 16;  // BM: rows of an R = 4 tile
+constexpr int NT = 128;                   // threads of a tile
+constexpr int kGroupMinRows = 256;     // fewer rows: the grouping's launches cost more than they save
+constexpr double kSkipNats64 = 800.0;  // exp(x) is 0 in FP64 below -745.2
 
 enum { SRC_GATHER = 0, SRC_RAYS = 1 };
 
 __device__ __forceinline__ int rows_of(const LikF64Args &a) { return a.n_rows_dev ? *a.n_rows_dev : a.n_rows; }
 
-template <int SRC, bool STORE_Z>
-__global__ void __launch_bounds__(256) k_zgemm_f64(LikF64Args a) {
+// Row lists of the grouped evaluation, in the caller's integer scratch a.grp.
+struct Lists {
+    int32_t *lead;           // [n] leading component
+    int32_t *l1, *l2, *lg;   // [K][n] rows led by k; rows that need k besides; rows with r_k = 1 alone
+    int32_t *lm;             // [n] rows with several r != 0
+    int32_t *c1, *c2, *cg, *cm;  // their lengths [K], [K], [K], [1]
+    uint64_t *mask;          // [n] components evaluated in full
+};
+__host__ __device__ inline Lists lists_of(int32_t *p, int n, int K) {
+    Lists L;
+    L.mask = reinterpret_cast<uint64_t *>(p);  // 256-byte aligned
+    p += 2 * (size_t)n;
+    L.c1 = p;
+    L.c2 = p + K;
+    L.cg = p + 2 * K;
+    L.cm = p + 3 * K;
+    p += 3 * K + 1;
+    L.lead = p;
+    L.l1 = p + n;
+    L.l2 = L.l1 + (size_t)K * n;
+    L.lg = L.l2 + (size_t)K * n;
+    L.lm = L.lg + (size_t)K * n;
+    return L;
+}
+
+// The (component, first list entry) of row tile t over lists of lengths cnt[0 .. K), or
+// k = -1 past the last tile.
+template <int ROWS>
+__device__ __forceinline__ int list_tile(const int32_t *cnt, int K, int t, int &r0) {
+    for (int k = 0; k < K; ++k) {
+        const int nt = (cnt[k] + ROWS - 1) / ROWS;
+        if (t < nt) {
+            r0 = t * ROWS;
+            return k;
+        }
+        t -= nt;
+    }
+    return -1;
+}
+
+// z of one tile: 8 R rows x columns [64 jt, 64 jt + 64) of component k. LISTED: the rows are
+// entries of the list of k (row tile from cnt), else rows 8 R blockIdx.x .. of all rows.
+// jt = jt0 + blockIdx.y (ascending: the longest column block first).
+// Returns false past the last tile.
+template <int SRC, bool STORE_Z, bool LISTED, int R>
+__device__ __forceinline__ bool z_tile(const LikF64Args &a, int tile, int jt0, const int32_t *list,
+                                       const int32_t *cnt) {
+    constexpr int BM = 8 * R;
     const int n_rows = rows_of(a);
-    const int n0 = blockIdx.x * BM;
-    if (n0 >= n_rows) return;
-    const int jt = blockIdx.y, j0 = jt * BN, k = blockIdx.z;
     const int d = a.d, K = a.K, nJT = (d + BN - 1) / BN;
+    int k = blockIdx.z, n0 = tile * BM, n_end = n_rows;
+    if (LISTED) {
+        k = list_tile<BM>(cnt, K, tile, n0);
+        if (k < 0) return false;
+        n_end = cnt[k];
+        list += (size_t)k * a.n_rows;
+    }
+    if (n0 >= n_end) return false;
+    const int jt = jt0 + blockIdx.y, j0 = jt * BN;
     const double *Lk = a.L + (size_t)k * d * d;
     const double *mk = a.mu + (size_t)k * d;
 
@@ -44,8 +115,8 @@ __global__ void __launch_bounds__(256) k_zgemm_f64(LikF64Args a) {
 
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     if (tid < BM) {
-        const int n = n0 + tid;
-        const bool valid = n < n_rows;
+        const bool valid = n0 + tid < n_end;
+        const int n = valid ? (LISTED ? list[n0 + tid] : n0 + tid) : 0;
         if (SRC == SRC_GATHER) {
             const int w = valid ? (a.rows ? a.rows[n] : n) : 0;
             s_src[tid] = a.X + (size_t)w * d;
@@ -63,16 +134,17 @@ __global__ void __launch_bounds__(256) k_zgemm_f64(LikF64Args a) {
     }
     __syncthreads();
 
-    double acc[4][4];
+    double acc[R][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = 0.0;
 
-    for (int i0 = (j0 / BK) * BK; i0 < d; i0 += BK) {
+    auto chunk = [&](int i0, auto NC) {  // the first NC column groups
+        constexpr int nc = decltype(NC)::value;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + 256 * q;
+        for (int q = 0; q < BM * BK / NT; ++q) {
+            const int e = tid + NT * q;
             const int row = e >> 4, kk = e & 15, i = i0 + kk;
             double v = 0.0;
             if (s_out[row] >= 0 && i < d) {
@@ -87,30 +159,35 @@ __global__ void __launch_bounds__(256) k_zgemm_f64(LikF64Args a) {
             As[kk][row] = v;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + 256 * q;
+        for (int q = 0; q < BN * BK / NT; ++q) {
+            const int e = tid + NT * q;
             const int kk = e >> 6, col = e & 63, i = i0 + kk, j = j0 + col;
             Bs[kk][col] = (i < d && j < d && j <= i) ? Lk[(size_t)i * d + j] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            double av[4], bv[4];
+            double av[R], bv[nc];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) av[r] = As[kk][ty + 16 * r];
+            for (int r = 0; r < R; ++r) av[r] = As[kk][ty + 8 * r];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
+            for (int c = 0; c < nc; ++c) bv[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
+                for (int c = 0; c < nc; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
         }
         __syncthreads();
-    }
+    };
+    // the diagonal block: rows i of chunk q meet the column groups c <= q only
+    chunk(j0, std::integral_constant<int, 1>());
+    if (j0 + BK < d) chunk(j0 + BK, std::integral_constant<int, 2>());
+    if (j0 + 2 * BK < d) chunk(j0 + 2 * BK, std::integral_constant<int, 3>());
+    for (int i0 = j0 + 3 * BK; i0 < d; i0 += BK) chunk(i0, std::integral_constant<int, 4>());
 
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int row = ty + 16 * r;
+    for (int r = 0; r < R; ++r) {
+        const int row = ty + 8 * r;
         const int out = s_out[row];
         double q = 0.0;
 #pragma unroll
@@ -131,75 +208,218 @@ __global__ void __launch_bounds__(256) k_zgemm_f64(LikF64Args a) {
             }
         }
     }
+    return true;
 }
 
-// Per point: l = LSE_k (a_k - q_k/2) and the responsibilities r_k.
-__global__ void __launch_bounds__(256) k_lse_f64(LikF64Args a) {
+template <int SRC, bool STORE_Z>
+__global__ void __launch_bounds__(NT) k_zgemm_f64(LikF64Args a, int jt0) {
+    z_tile<SRC, STORE_Z, false, 4>(a, blockIdx.x, jt0, nullptr, nullptr);
+}
+// The lists' lengths are known on the device only: CTAs go from tile to tile.
+template <bool STORE_Z, int R>
+__global__ void __launch_bounds__(NT) k_zgemm_f64_listed(LikF64Args a, const int32_t *list, const int32_t *cnt) {
+    for (int t = blockIdx.x; z_tile<SRC_GATHER, STORE_Z, true, R>(a, t, 0, list, cnt); t += gridDim.x)
+        __syncthreads();  // the shared tiles are free for the next one
+}
+
+// The row's place in per-component lists: one atomic per warp and component (the order
+// inside a list does not reach the results, which are stored by row).
+__device__ __forceinline__ void append(bool put, int k, int n, int K, int cap, int32_t *list, int32_t *cnt) {
+    const int lane = threadIdx.x & 31;
+    for (int c = 0; c < K; ++c) {
+        const unsigned m = __ballot_sync(0xffffffffu, put && k == c);
+        if (!m) continue;
+        int base = 0;
+        if (lane == __ffs(m) - 1) base = atomicAdd(&cnt[c], __popc(m));
+        base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
+        if ((m >> lane) & 1u) list[(size_t)c * cap + base + __popc(m & ((1u << lane) - 1u))] = n;
+    }
+}
+
+__device__ __forceinline__ int out_row(const LikF64Args &a, int n) {
+    return a.out_by_walker ? (a.rows ? a.rows[n] : n) : n;
+}
+
+// The leading component of each row from the last column block's part of |z_k|^2.
+__global__ void __launch_bounds__(128) k_grp_lead(LikF64Args a, Lists L) {
     const int n_rows = rows_of(a);
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= n_rows) return;
     const int K = a.K, nJT = (a.d + BN - 1) / BN;
-    const int out = a.out_by_walker ? (a.rows ? a.rows[n] : n) : n;
-    double e[kMaxK];
-    double emax = -INFINITY;
-    for (int k = 0; k < K; ++k) {
-        const double *qp = a.qpart + ((size_t)out * K + k) * nJT;
-        double q = 0.0;
-        for (int t = 0; t < nJT; ++t) q += qp[t];
-        e[k] = a.a[k] - 0.5 * q;
-        emax = fmax(emax, e[k]);
+    int lead = 0;
+    if (n < n_rows) {
+        const double *qp = a.qpart + (size_t)out_row(a, n) * K * nJT + nJT - 1;
+        double top = -INFINITY;
+        for (int k = 0; k < K; ++k) {
+            const double e = fma(-0.5, qp[(size_t)k * nJT], a.a[k]);
+            if (e > top) {
+                top = e;
+                lead = k;
+            }
+        }
+        L.lead[n] = lead;
     }
-    double ssum = 0.0;
-    for (int k = 0; k < K; ++k) ssum += exp(e[k] - emax);
-    const double ell = emax + log(ssum);
-    a.ell[out] = a.ell_sign * ell;
-    if (a.R)
-        for (int k = 0; k < K; ++k) a.R[(size_t)out * K + k] = exp(e[k] - emax) / ssum;
+    append(n < n_rows, lead, n, K, a.n_rows, L.l1, L.c1);
 }
 
-// grad: out[n][i] = sign * sum_k sum_{j<=i} r_nk z_nk[j] L_k[i][j]  (= -sign * grad l)
-__global__ void __launch_bounds__(256) k_ggemm_f64(LikF64Args a) {
+// The components a row needs besides its leading one (see the header).
+__global__ void __launch_bounds__(128) k_grp_need(LikF64Args a, Lists L) {
     const int n_rows = rows_of(a);
-    const int n0 = blockIdx.x * BM;
-    if (n0 >= n_rows) return;
-    const int i0 = blockIdx.y * BN;
-    const int d = a.d, K = a.K;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int K = a.K, nJT = (a.d + BN - 1) / BN;
+    uint64_t mask = 0;
+    if (n < n_rows) {
+        const double *qp = a.qpart + (size_t)out_row(a, n) * K * nJT;
+        const int j = L.lead[n];
+        double q = 0.0;
+        for (int t = 0; t < nJT; ++t) q += qp[(size_t)j * nJT + t];
+        const double low = (a.a[j] - 0.5 * q) - kSkipNats64;
+        for (int k = 0; k < K; ++k) {
+            const double ql = qp[(size_t)k * nJT + nJT - 1];
+            const bool skip = k != j && finite_bits(ql) && fma(-0.5 * (1.0 - 1e-10), ql, a.a[k]) < low;
+            if (!skip) mask |= 1ull << k;
+        }
+        L.mask[n] = mask;
+        mask &= ~(1ull << j);
+    }
+    for (int k = 0; k < K; ++k) append((mask >> k) & 1ull, k, n, K, a.n_rows, L.l2 + 0, L.c2);
+}
 
-    __shared__ double As[BK][BM + 1];
-    __shared__ double Bs[BK][BN + 1];
-    __shared__ int s_out[BM];
+// Per point: l = LSE_k (a_k - q_k/2) and the responsibilities r_k. GROUPED: over the
+// components evaluated in full (the others add exact zeros), and with a.G also the
+// gradient's row lists.
+template <bool GROUPED>
+__global__ void __launch_bounds__(128) k_lse_f64(LikF64Args a, Lists L) {
+    const int n_rows = rows_of(a);
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int K = a.K, nJT = (a.d + BN - 1) / BN;
+    int one = -1;
+    bool multi = false;
+    if (n < n_rows) {
+        const int out = out_row(a, n);
+        const uint64_t mask = GROUPED ? L.mask[n] : ~0ull;
+        const double *qr = a.qpart + (size_t)out * K * nJT;
+        auto term = [&](int k) {
+            const double *qp = qr + (size_t)k * nJT;
+            double q = 0.0;
+            for (int t = 0; t < nJT; ++t) q += qp[t];
+            return a.a[k] - 0.5 * q;
+        };
+        const int k1 = GROUPED ? __ffsll((long long)mask) - 1 : 0;
+        if (GROUPED && (mask & (mask - 1)) == 0 && finite_bits(term(k1))) {
+            // one component left: its exponential, and the sum, are 1
+            a.ell[out] = a.ell_sign * term(k1);
+            if (a.R)
+                for (int k = 0; k < K; ++k) a.R[(size_t)out * K + k] = k == k1 ? 1.0 : 0.0;
+            one = k1;
+        } else {
+            double e[kMaxK];
+            double emax = -INFINITY;
+            for (int k = 0; k < K; ++k) {
+                if (GROUPED && !((mask >> k) & 1ull)) continue;
+                e[k] = term(k);
+                emax = fmax(emax, e[k]);
+            }
+            double ssum = 0.0;
+            for (int k = 0; k < K; ++k) {
+                if (GROUPED && !((mask >> k) & 1ull)) continue;
+                e[k] = exp(e[k] - emax);
+                ssum += e[k];
+            }
+            a.ell[out] = a.ell_sign * (emax + log(ssum));
+            int cnt = 0;
+            if (a.R)
+                for (int k = 0; k < K; ++k) {
+                    const double r = GROUPED && !((mask >> k) & 1ull) ? 0.0 : e[k] / ssum;
+                    a.R[(size_t)out * K + k] = r;
+                    if (r != 0.0) {
+                        ++cnt;
+                        one = r == 1.0 ? k : -2;
+                    }
+                }
+            multi = cnt != 1 || one < 0;
+        }
+    }
+    if (GROUPED && a.G) {
+        append(n < n_rows && !multi, one, n, K, a.n_rows, L.lg, L.cg);
+        append(multi, 0, n, 1, a.n_rows, L.lm, L.cm);
+    }
+}
+
+// grad: out[n][i] = sign * sum_k sum_{j<=i} r_nk z_nk[j] L_k[i][j]  (= -sign * grad l).
+// ROWS_ALL: every row and component; ROWS_ONE: the rows of the list of each component,
+// whose r is 1 there and 0 elsewhere; ROWS_MULTI: the listed rows, components with r = 0 left out.
+enum { ROWS_ALL = 0, ROWS_ONE = 1, ROWS_MULTI = 2 };
+template <int MODE, int R>
+struct GradTile {
+    static constexpr int BM = 8 * R;
+    double As[BK][BM + 1];
+    double Bs[BK][BN + 1];
+    int s_out[BM];
+};
+template <int MODE, int R>
+__device__ __forceinline__ bool grad_tile(const LikF64Args &a, int tile, const int32_t *list, const int32_t *cnt,
+                                          GradTile<MODE, R> &sm) {
+    constexpr int BM = 8 * R;
+    auto &As = sm.As;
+    auto &Bs = sm.Bs;
+    auto &s_out = sm.s_out;
+    const int d = a.d, K = a.K;
+    int n0 = tile * BM, n_end = rows_of(a), k_lo = 0, k_hi = K;
+    if (MODE == ROWS_ONE) {
+        k_lo = list_tile<BM>(cnt, K, tile, n0);
+        if (k_lo < 0) return false;
+        k_hi = k_lo + 1;
+        n_end = cnt[k_lo];
+        list += (size_t)k_lo * a.n_rows;
+    } else if (MODE == ROWS_MULTI) {
+        n_end = *cnt;
+    }
+    if (n0 >= n_end) return false;
+    const int i0 = (gridDim.y - 1 - blockIdx.y) * BN;  // the longest column range first
+
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     if (tid < BM) {
-        const int n = n0 + tid;
-        s_out[tid] = n < n_rows ? (a.out_by_walker ? (a.rows ? a.rows[n] : n) : n) : -1;
+        const bool valid = n0 + tid < n_end;
+        s_out[tid] = valid ? out_row(a, MODE == ROWS_ALL ? n0 + tid : list[n0 + tid]) : -1;
     }
     __syncthreads();
 
-    double acc[4][4];
+    double acc[R][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = 0.0;
 
-    const int jmax = min(d, i0 + BN);
-    for (int k = 0; k < K; ++k) {
+    for (int k = k_lo; k < k_hi; ++k) {
+        if (MODE == ROWS_MULTI) {
+            const bool on = tid < BM && s_out[tid] >= 0 && a.R[(size_t)s_out[tid] * K + k] != 0.0;
+            if (!__syncthreads_or(on)) continue;
+        }
         const double *Lk = a.L + (size_t)k * d * d;
-        for (int j0 = 0; j0 < jmax; j0 += BK) {
+        auto chunk = [&](int j0, auto C0) {  // the column groups from C0 on
+            constexpr int c0 = decltype(C0)::value;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int e = tid + 256 * q;
+            for (int q = 0; q < BM * BK / NT; ++q) {
+                const int e = tid + NT * q;
                 const int row = e >> 4, kk = e & 15, j = j0 + kk;
                 const int out = s_out[row];
                 double v = 0.0;
-                if (out >= 0 && j < d) v = a.R[(size_t)out * K + k] * a.Z[((size_t)out * K + k) * d + j];
+                if (out >= 0 && j < d) {
+                    if (MODE == ROWS_ONE) {
+                        v = a.Z[((size_t)out * K + k) * d + j];
+                    } else {
+                        const double r = a.R[(size_t)out * K + k];
+                        if (MODE == ROWS_ALL || r != 0.0) v = r * a.Z[((size_t)out * K + k) * d + j];
+                    }
+                }
                 As[kk][row] = v;
             }
             {
-                // 64 columns (rows i of L_k) x 16 j: each thread loads 4 consecutive j of one row
-                const int col = tid >> 2, kq = (tid & 3) * 4;
+                // 64 columns (rows i of L_k) x 16 j: each thread loads 8 consecutive j of one row
+                const int col = tid >> 1, kq = (tid & 1) * 8;
                 const int i = i0 + col;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
+                for (int t = 0; t < 8; ++t) {
                     const int j = j0 + kq + t;
                     Bs[kq + t][col] = (i < d && j < d && j <= i) ? Lk[(size_t)i * d + j] : 0.0;
                 }
@@ -207,28 +427,51 @@ __global__ void __launch_bounds__(256) k_ggemm_f64(LikF64Args a) {
             __syncthreads();
 #pragma unroll
             for (int kk = 0; kk < BK; ++kk) {
-                double av[4], bv[4];
+                double av[R], bv[4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) av[r] = As[kk][ty + 16 * r];
+                for (int r = 0; r < R; ++r) av[r] = As[kk][ty + 8 * r];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
+                for (int c = c0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
+                for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
+                    for (int c = c0; c < 4; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
             }
             __syncthreads();
-        }
+        };
+        for (int j0 = 0; j0 <= i0 && j0 < d; j0 += BK) chunk(j0, std::integral_constant<int, 0>());
+        // the rest of the diagonal block: columns j of chunk q reach the rows of groups c >= q only
+        if (i0 + BK < d) chunk(i0 + BK, std::integral_constant<int, 1>());
+        if (i0 + 2 * BK < d) chunk(i0 + 2 * BK, std::integral_constant<int, 2>());
+        if (i0 + 3 * BK < d) chunk(i0 + 3 * BK, std::integral_constant<int, 3>());
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int out = s_out[ty + 16 * r];
+    for (int r = 0; r < R; ++r) {
+        const int out = s_out[ty + 8 * r];
         if (out < 0) continue;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const int i = i0 + tx + 16 * c;
             if (i < d) a.G[(size_t)out * d + i] = a.grad_sign * acc[r][c];
         }
+    }
+    return true;
+}
+__global__ void __launch_bounds__(NT) k_ggemm_f64(LikF64Args a) {
+    __shared__ GradTile<ROWS_ALL, 4> sm;
+    grad_tile<ROWS_ALL, 4>(a, blockIdx.x, nullptr, nullptr, sm);
+}
+// The gradient of the grouped evaluation: first the tiles of the rows with several
+// components (8 rows each: up to K times as long as the others'), on n_multi CTAs.
+__global__ void __launch_bounds__(NT) k_ggemm_f64_grouped(LikF64Args a, Lists L, int n_multi) {
+    __shared__ union {
+        GradTile<ROWS_MULTI, 1> m;
+        GradTile<ROWS_ONE, 4> o;
+    } sm;
+    if ((int)blockIdx.x < n_multi) {
+        for (int t = blockIdx.x; grad_tile<ROWS_MULTI, 1>(a, t, L.lm, L.cm, sm.m); t += n_multi) __syncthreads();
+    } else {
+        grad_tile<ROWS_ONE, 4>(a, blockIdx.x - n_multi, L.lg, L.cg, sm.o);
     }
 }
 // ------------------------------------------------------------------ few points (GEMV shape)
@@ -387,58 +630,91 @@ __global__ void __launch_bounds__(256) k_few_g(LikF64Args a) {
 
 size_t lik_f64_qpart_elems(int d, int K, int rows) { return (size_t)rows * K * ((d + BN - 1) / BN); }
 
-void launch_lik_f64_z(const LikF64Args &a, cudaStream_t s) {
-    if (a.n_rows <= 0) return;
-    dim3 g((a.n_rows + BM - 1) / BM, (a.d + BN - 1) / BN, a.K);
+size_t lik_f64_group_elems(int K, int rows) { return 4 * (size_t)rows + 3 * (size_t)K * rows + 3 * (size_t)K + 4; }
+
+namespace {
+template <int SRC, bool STORE_Z>
+void z_all(const LikF64Args &a, int jt0, int njt, cudaStream_t s) {
+    const dim3 g((a.n_rows + BM - 1) / BM, njt, a.K);
     ProfScope prof(PROF_F64_Z, s);
     note_launch();
-    k_zgemm_f64<SRC_GATHER, true><<<g, 256, 0, s>>>(a);
+    k_zgemm_f64<SRC, STORE_Z><<<g, NT, 0, s>>>(a, jt0);
+}
+
+// The listed rows (at most `total` over the K lists, whose last tiles may be short).
+template <bool STORE_Z, int R>
+void z_listed(const LikF64Args &a, int njt, const int32_t *list, const int32_t *cnt, long long total,
+              cudaStream_t s) {
+    const long long tiles = total / (8 * R) + a.K;
+    ProfScope prof(PROF_F64_Z, s);
+    note_launch();
+    k_zgemm_f64_listed<STORE_Z, R><<<dim3((unsigned)(tiles < 1216 ? tiles : 1216), njt), NT, 0, s>>>(a, list, cnt);
+}
+
+// l (and grad l when a.G is given) in groups of rows per component.
+template <bool GRAD>
+void points_grouped(const LikF64Args &a, cudaStream_t s) {
+    const int n = a.n_rows, K = a.K, nJT = (a.d + BN - 1) / BN;
+    const Lists L = lists_of(a.grp, n, K);
+    cudaMemsetAsync(L.c1, 0, sizeof(int32_t) * (3 * K + 1), s);
+    const unsigned gr = (unsigned)((n + 127) / 128);
+    z_all<SRC_GATHER, GRAD>(a, nJT - 1, 1, s);
+    note_launch();
+    k_grp_lead<<<gr, 128, 0, s>>>(a, L);
+    z_listed<GRAD, 4>(a, nJT - 1, L.l1, L.c1, n, s);
+    note_launch();
+    k_grp_need<<<gr, 128, 0, s>>>(a, L);
+    z_listed<GRAD, 1>(a, nJT - 1, L.l2, L.c2, (long long)(K - 1) * n, s);
+    note_launch();
+    k_lse_f64<true><<<gr, 128, 0, s>>>(a, L);
+    if (!GRAD) return;
+    ProfScope prof(PROF_F64_GRAD, s);
+    note_launch();
+    const int n_multi = (n + 7) / 8 < 608 ? (n + 7) / 8 : 608;
+    // unused shared memory holds an SM to two CTAs, so that the tiles, up to nJT times
+    // different in length, are dealt out as SMs come free (all resident at once: 484 us at
+    // 4096 points, d = 256, K = 4, 304 us so; 287 us of FP64 instructions)
+    constexpr int kPad = 96 * 1024;
+    static const cudaError_t pad_set =
+        cudaFuncSetAttribute(k_ggemm_f64_grouped, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad);
+    k_ggemm_f64_grouped<<<dim3(n_multi + n / BM + K, nJT), NT, pad_set == cudaSuccess ? kPad : 0, s>>>(a, L, n_multi);
+}
+}  // namespace
+
+void launch_lik_f64_z(const LikF64Args &a, cudaStream_t s) {
+    if (a.n_rows <= 0) return;
+    z_all<SRC_GATHER, true>(a, 0, (a.d + BN - 1) / BN, s);
 }
 
 void launch_lik_f64_rays(const LikF64Args &a, cudaStream_t s) {
     if (a.n_rows <= 0) return;
     if (small_f64_fits(a.d, a.K, 0)) return launch_small_points_f64(a, true, s);
-    dim3 g((a.n_rows + BM - 1) / BM, (a.d + BN - 1) / BN, a.K);
-    {
-        ProfScope prof(PROF_F64_Z, s);
-        note_launch();
-        k_zgemm_f64<SRC_RAYS, false><<<g, 256, 0, s>>>(a);
-    }
+    z_all<SRC_RAYS, false>(a, 0, (a.d + BN - 1) / BN, s);
     note_launch();
-    k_lse_f64<<<(a.n_rows + 255) / 256, 256, 0, s>>>(a);
+    k_lse_f64<false><<<(a.n_rows + 127) / 128, 128, 0, s>>>(a, Lists{});
 }
 
-void launch_lik_f64_points(const LikF64Args &a, bool want_grad, cudaStream_t s) {
-    if (a.n_rows <= 0) return;
-    if (small_f64_fits(a.d, a.K, 0)) {
-        LikF64Args b = a;
-        if (!want_grad) b.G = nullptr;
-        return launch_small_points_f64(b, false, s);
-    }
-    dim3 g((a.n_rows + BM - 1) / BM, (a.d + BN - 1) / BN, a.K);
-    if (want_grad) {
-        {
-            ProfScope prof(PROF_F64_Z, s);
-            note_launch();
-            k_zgemm_f64<SRC_GATHER, true><<<g, 256, 0, s>>>(a);
-        }
-        note_launch();
-        k_lse_f64<<<(a.n_rows + 255) / 256, 256, 0, s>>>(a);
-        dim3 g2((a.n_rows + BM - 1) / BM, (a.d + BN - 1) / BN);
-        {
-            ProfScope prof(PROF_F64_GRAD, s);
-            note_launch();
-            k_ggemm_f64<<<g2, 256, 0, s>>>(a);
-        }
-    } else {
-        {
-            ProfScope prof(PROF_F64_Z, s);
-            note_launch();
-            k_zgemm_f64<SRC_GATHER, false><<<g, 256, 0, s>>>(a);
-        }
-        note_launch();
-        k_lse_f64<<<(a.n_rows + 255) / 256, 256, 0, s>>>(a);
-    }
+// Routes: small problems whole in shared memory (small_f64.cu); several components over
+// several column blocks and at least kGroupMinRows rows in groups per component (when the
+// caller gives the scratch); else every row and component.
+void launch_lik_f64_points(const LikF64Args &a0, bool want_grad, cudaStream_t s) {
+    if (a0.n_rows <= 0) return;
+    LikF64Args a = a0;
+    if (!want_grad) a.G = nullptr;
+    if (small_f64_fits(a.d, a.K, 0)) return launch_small_points_f64(a, false, s);
+    const int nJT = (a.d + BN - 1) / BN;
+    if (a.grp && a.K >= 2 && nJT >= 2 && a.n_rows >= kGroupMinRows)
+        return want_grad ? points_grouped<true>(a, s) : points_grouped<false>(a, s);
+    if (want_grad)
+        z_all<SRC_GATHER, true>(a, 0, nJT, s);
+    else
+        z_all<SRC_GATHER, false>(a, 0, nJT, s);
+    note_launch();
+    k_lse_f64<false><<<(a.n_rows + 127) / 128, 128, 0, s>>>(a, Lists{});
+    if (!want_grad) return;
+    ProfScope prof(PROF_F64_GRAD, s);
+    note_launch();
+    k_ggemm_f64<<<dim3((a.n_rows + BM - 1) / BM, nJT), NT, 0, s>>>(a);
 }
 
 }  // namespace sb
@@ -454,7 +730,7 @@ void launch_lik_f64_few(const LikF64Args &a, bool want_grad, cudaStream_t s) {
         k_few_z<<<dim3(nJT, a.K, cb), 256, 0, s>>>(a);
     }
     note_launch();
-    k_lse_f64<<<(a.n_rows + 255) / 256, 256, 0, s>>>(a);
+    k_lse_f64<false><<<(a.n_rows + 127) / 128, 128, 0, s>>>(a, Lists{});
     if (want_grad) {
         ProfScope prof(PROF_F64_GRAD, s);
         note_launch();

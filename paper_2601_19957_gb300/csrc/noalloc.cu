@@ -48,7 +48,7 @@ sb_status scratch_address(cudaStream_t s, void **out) {
 
 extern "C" sb_status sb_loglik_noalloc(const sb_problem *prob, int32_t prec, const double *x, int32_t n, double *ell,
                                        double *grad, void *stream) {
-    const size_t need = sb_loglik_workspace_bytes(prob, prec, n);
+    const size_t need = sb::loglik_bytes(prob, prec, n, false);  // without the optional row lists
     if (need == 0) return SB_ERR_INVALID_ARG;
     if (need > kScratchBytes) return SB_ERR_WORKSPACE;
     void *ws = nullptr;

@@ -172,6 +172,7 @@ struct RefineWs {
     int32_t *act_tmp;       // [N] scratch of the grouped compaction (mixed path)
     int32_t *act_cnt;       // its per-CTA bucket counts
     double *qpart, *Z, *R;  // FP64 evaluation
+    int32_t *grp;           // its row lists
     TcWs tc;                // mixed-precision evaluation
 };
 
@@ -235,6 +236,7 @@ void carve_refine(Carver &cv, RefineWs<T> &r, int n, int d, int K, int m, bool f
         r.qpart = cv.take<double>(lik_f64_qpart_elems(d, K, n));
         r.Z = cv.take<double>((size_t)n * K * d);
         r.R = cv.take<double>((size_t)n * K);
+        r.grp = cv.take<int32_t>(lik_f64_group_elems(K, n));
     } else {
         carve_tc(cv, r.tc, n, d, K, prec);
         r.act_tmp = cv.take<int32_t>((size_t)n);
@@ -410,6 +412,7 @@ void eval_round<double>(const ProbView &pv, const sb_config *c, const RefineWs<d
     a.qpart = r.qpart;
     a.Z = r.Z;
     a.R = r.R;
+    a.grp = r.grp;
     a.ell = r.lb.FT;
     a.ell_sign = -1.0;  // f = -l
     a.G = r.lb.GT;
@@ -837,7 +840,9 @@ extern "C" sb_status sb_evidence_host(const sb_problem *hp, const sb_config *c, 
 }
 
 // ------------------------------------------------------------------ batched log-likelihood
-extern "C" size_t sb_loglik_workspace_bytes(const sb_problem *p, int32_t prec, int32_t n) {
+// lists: with the row lists of the FP64 path's grouped evaluation. A workspace without
+// room for them is accepted, and every row and component is then evaluated.
+size_t sb::loglik_bytes(const sb_problem *p, int32_t prec, int32_t n, bool lists) {
     if (check_problem(p) != SB_OK || n < 1) return 0;
     Carver cv(nullptr);
     cv.take<WsHeader>(1);
@@ -846,6 +851,7 @@ extern "C" size_t sb_loglik_workspace_bytes(const sb_problem *p, int32_t prec, i
         cv.take<double>(lik_f64_qpart_elems(p->d, p->K, n));
         cv.take<double>((size_t)n * p->K * p->d);
         cv.take<double>((size_t)n * p->K);
+        if (lists) cv.take<int32_t>(lik_f64_group_elems(p->K, n));
     } else if (prec == SB_PREC_TF32 || prec == SB_PREC_BF16) {
         TcWs t;
         carve_tc(cv, t, n, p->d, p->K, prec);
@@ -858,6 +864,10 @@ extern "C" size_t sb_loglik_workspace_bytes(const sb_problem *p, int32_t prec, i
     return cv.bytes();
 }
 
+extern "C" size_t sb_loglik_workspace_bytes(const sb_problem *p, int32_t prec, int32_t n) {
+    return sb::loglik_bytes(p, prec, n, true);
+}
+
 extern "C" sb_status sb_loglik(const sb_problem *p, int32_t prec, const double *x, int32_t n, double *ell,
                                double *grad, void *ws, size_t ws_bytes, void *stream) {
     sb_status st = check_problem(p);
@@ -865,7 +875,7 @@ extern "C" sb_status sb_loglik(const sb_problem *p, int32_t prec, const double *
     if (!x || !ell || !ws || n < 1) return SB_ERR_INVALID_ARG;
     if (prec < SB_PREC_FP64 || prec > SB_PREC_BF16) return SB_ERR_INVALID_ARG;
     if (prec != SB_PREC_FP64 && !tc_available(prec)) return SB_ERR_UNSUPPORTED;
-    if (ws_bytes < sb_loglik_workspace_bytes(p, prec, n)) return SB_ERR_WORKSPACE;
+    if (ws_bytes < sb::loglik_bytes(p, prec, n, false)) return SB_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Carver cv(ws);
     WsHeader *hdr = cv.take<WsHeader>(1);
@@ -885,6 +895,8 @@ extern "C" sb_status sb_loglik(const sb_problem *p, int32_t prec, const double *
         double *qpart = cv.take<double>(lik_f64_qpart_elems(p->d, p->K, n));
         double *Z = cv.take<double>((size_t)n * p->K * p->d);
         double *R = cv.take<double>((size_t)n * p->K);
+        int32_t *grp = ws_bytes < sb::loglik_bytes(p, prec, n, true) ? nullptr
+                                                                     : cv.take<int32_t>(lik_f64_group_elems(p->K, n));
         // setup needs c/half/logV/wmax only for box work; give it scratch inside Z (overwritten later)
         pv.c = Z;
         pv.half = Z + p->d;
@@ -897,10 +909,16 @@ extern "C" sb_status sb_loglik(const sb_problem *p, int32_t prec, const double *
         la.qpart = qpart;
         la.Z = Z;
         la.R = R;
+        la.grp = grp;
         la.ell = ell;
         la.G = grad;
         la.out_by_walker = 0;
-        launch_lik_f64_points(la, grad != nullptr, s);
+        // a few points of a problem too large for small_f64.cu leave most SMs without a
+        // 32-row tile: the matrix-vector kernels spread them over (column block, component)
+        if (n <= 64 && !small_f64_fits(p->d, p->K, 0))
+            launch_lik_f64_few(la, grad != nullptr, s);
+        else
+            launch_lik_f64_points(la, grad != nullptr, s);
     } else {
         TcWs t;
         carve_tc(cv, t, n, p->d, p->K, prec);
@@ -1142,6 +1160,7 @@ sb_status run_chisao(const Prelude &P, const sb_config *c, const sb_chisao_confi
         a.qpart = r.qpart;
         a.Z = r.Z;
         a.R = r.R;
+        a.grp = r.grp;
         a.ell = w.ellg;
         a.G = w.G;
         a.out_by_walker = 1;

@@ -210,6 +210,9 @@ struct ProbView {
     int32_t *status;
 };
 
+// Bytes sb_loglik needs (lists: with its optional row lists, what the query returns).
+size_t loglik_bytes(const sb_problem *p, int32_t prec, int32_t n, bool lists);
+
 // Host-side count of kernel launches issued by the library (diagnostics).
 void note_launch(int64_t n = 1);
 
@@ -264,10 +267,12 @@ struct LikF64Args {
     double *G;                // [out_rows][d] gradient (sign applied)
     double grad_sign;
     int out_by_walker;        // 1: outputs indexed by rows[n]; 0: by n
+    int32_t *grp;             // scratch of the grouped evaluation (lik_f64_group_elems), may be null
 };
 void launch_lik_f64_rays(const LikF64Args &a, cudaStream_t s);                 // values at ray samples
 void launch_lik_f64_points(const LikF64Args &a, bool want_grad, cudaStream_t s);// values (+grads) at points
 size_t lik_f64_qpart_elems(int d, int K, int rows);
+size_t lik_f64_group_elems(int K, int rows);  // int32 elements of LikF64Args::grp
 // z_nk = L_k^T (x_n - mu_k) stored in Z (and the |z|^2 partials in qpart) for gathered rows, no l.
 void launch_lik_f64_z(const LikF64Args &a, cudaStream_t s);
 // Same outputs for a handful of points (GEMV-shaped work split; n_rows is the capacity).
