@@ -49,6 +49,7 @@ struct TcQuadWs {
     double *zc, *q0;                 // parts of z_k(c) [.][K][d], [K] |z_k(c)|^2
     double *co;                      // [n_rays][K][3] coefficients of e_k in tau (FP64)
     float4 *cf;                      // [n_rays][K] the same in FP32
+    int32_t *arg;                    // [n_rays] coordinate of a ray's exit
     int rows, dK, ald;
     CUtensorMap mapU, mapL;
 };

@@ -1424,19 +1424,57 @@ sb_status tc_prepare(const ProbView &pv, TcWs &t, cudaStream_t s, bool skip_boun
 }
 
 // ------------------------------------------------------------------ quadratic form of the rays
+// Two neighbouring elements split and stored at the even index e of the hi part (the lo
+// part follows dK elements on); returns |x| rounded down to FP32 (0 for x = 0, -1 where the
+// FP32 route does not hold).
+template <int PREC>
+__device__ __forceinline__ void split_store(void *A2, size_t e, int dK, double x0, double x1, float &m0, float &m1) {
+    float t0, t1, r0, r1;
+    const bool ok = split24(x0, t0, r0) & split24(x1, t1, r1);
+    m0 = fabsf(t0);
+    m1 = fabsf(t1);
+    bool mid = !ok;
+    if (PREC == SB_PREC_BF16) {
+        // the dropped bits as a sticky last bit: rounding t to 8 bits is then rounding x
+        const uint32_t s0 = __float_as_uint(t0) | (r0 != 0.f ? 1u : 0u), s1 = __float_as_uint(t1) | (r1 != 0.f ? 1u : 0u);
+        const uint32_t hi = pack_bf16x2(__uint_as_float(s0), __uint_as_float(s1));
+        const float l0 = (t0 - __uint_as_float(hi << 16)) + r0, l1 = (t1 - __uint_as_float(hi & 0xffff0000u)) + r1;
+        mid = mid || (__float_as_uint(l0) & 0xffffu) == 0x8000u || (__float_as_uint(l1) & 0xffffu) == 0x8000u;
+        if (!mid) {
+            reinterpret_cast<uint32_t *>(A2)[e / 2] = hi;
+            reinterpret_cast<uint32_t *>(A2)[(e + dK) / 2] = pack_bf16x2(l0, l1);
+        }
+    } else {
+        mid = true;
+    }
+    if (mid) {
+        float h0, h1, l0, l1;
+        split_op<PREC>(x0, h0, l0);
+        split_op<PREC>(x1, h1, l1);
+        put_pair<PREC>(A2, e, h0, h1);
+        put_pair<PREC>(A2, e + dK, l0, l1);
+        if (!ok) {
+            if (!split24(x0, t0, r0)) m0 = -1.f;
+            if (!split24(x1, t1, r1)) m1 = -1.f;
+        }
+    }
+}
+
 // A2[r][0 .. dK) = hi(u_r), A2[r][dK .. 2 dK) = lo(u_r); zeros past d and past the ray
 // count (n_rays, or *n_dev when given), rows past the count's last 128-row block untouched.
-// A warp per row, two neighbouring coordinates per lane. texit given: also the ray's exit
-// length from the box centre, min_i half_i / |u_i| as warp_exit_min (the exact FP64 minimum):
-// FP32 quotients of the truncated operands are within 2^-21, and only the lanes that hold
-// one within 2^-18 of the smallest (or a coordinate out of FP32's range) go over their
-// coordinates again and divide in FP64. One pass over u (134 MB at 16384 rays, d = 1024)
-// where the split and the exit lengths were two, each bound by FP64 conversions: 297 us,
-// 104 us now.
+// A warp per row, two neighbouring coordinates per lane. arg given: also what k_q_exit needs
+// for the ray's exit length from the box centre, min_i half_i / |u_i| as warp_exit_min (the
+// exact FP64 minimum): FP32 quotients of the truncated operands are within 2^-21, so when a
+// single one lies within 2^-18 of the smallest, its index is left in arg and one FP64
+// division per ray remains; otherwise (or with a coordinate out of FP32's range) the lanes
+// concerned go over their coordinates and divide here (arg -1). One pass over u (134 MB at
+// 16384 rays, d = 1024) where the split and the exit lengths were two, each bound by FP64
+// conversions: 297 us, 59 us now.
 template <int PREC>
 __global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int d, int dK, const double *u, void *A2,
-                                                      const int32_t *n_dev, const double *half, double *texit) {
-    __shared__ float hf[kMaxD];  // half-widths, -1 outside the range the FP32 quotients hold for
+                                                      const int32_t *n_dev, const double *half, double *texit,
+                                                      int32_t *arg) {
+    __shared__ float hf[kMaxD + 1];  // half-widths, -1 outside the range the FP32 quotients hold for
     if (n_dev) {
         const int c = *n_dev < n_rays ? *n_dev : n_rays;
         const int rb = (c + BM - 1) / BM * BM;
@@ -1445,7 +1483,7 @@ __global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int 
     }
     const int lane = threadIdx.x & 31;
     constexpr float kLo = 1e-30f, kHi = 1e30f;
-    if (texit) {
+    if (arg) {
         for (int i = threadIdx.x; i < d; i += blockDim.x) {
             const float h = f64_to_f32(half[i]);
             hf[i] = h >= kLo && h <= kHi ? h : -1.f;
@@ -1457,52 +1495,71 @@ __global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int 
         const double *ur = u + (size_t)r * d;
         const size_t o = (size_t)r * 2 * dK;
         float est = INFINITY;
+        int at = -1, close = 0;  // the lane's smallest quotient, and whether another is near it
         bool odd = false;
-#pragma unroll 4
         for (int i = 2 * lane; i < dK; i += 64) {
             const double x0 = live && i < d ? ur[i] : 0.0, x1 = live && i + 1 < d ? ur[i + 1] : 0.0;
-            float h0, l0, h1, l1;
-            split_op<PREC>(x0, h0, l0);
-            split_op<PREC>(x1, h1, l1);
-            put_pair<PREC>(A2, o + i, h0, h1);
-            put_pair<PREC>(A2, o + dK + i, l0, l1);
-            if (texit) {
+            float m0, m1;
+            split_store<PREC>(A2, o + i, dK, x0, x1, m0, m1);
+            if (arg) {
+                odd = odd || m0 < 0.f || m1 < 0.f;
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    const double x = q ? x1 : x0;
-                    if (i + q >= d || ((__double_as_longlong(x) << 1) == 0)) continue;
-                    float t, rest;
-                    const bool ok = split24(x, t, rest) && hf[i + q] > 0.f;
-                    odd = odd || !ok;
-                    if (ok) est = fminf(est, __fdividef(hf[i + q], fabsf(t)));
-                }
-            }
-        }
-        if (texit && live) {
-            const float thr = warp_min(est) * (1.0f + 0x1p-18f);
-            long long best = 0x7ff0000000000000ll;  // +inf; positive doubles order as their bits
-            if (est <= thr || odd) {
-                for (int i = 2 * lane; i < d; i += 64) {
-                    for (int q = 0; q < 2 && i + q < d; ++q) {
-                        const double x = ur[i + q];
-                        if ((__double_as_longlong(x) << 1) == 0) continue;
-                        float t, rest;
-                        const bool ok = split24(x, t, rest) && hf[i + q] > 0.f;
-                        if (ok && __fdividef(hf[i + q], fabsf(t)) > thr) continue;
-                        const double v = __ddiv_rn(half[i + q], fabs(x));
-                        const long long b = __double_as_longlong(v);
-                        if (v == v && b < best) best = b;
+                    const float m = q ? m1 : m0;
+                    if (m > 0.f) {
+                        const float h = hf[i + q], e = __fdividef(h, m);
+                        odd = odd || h < 0.f;
+                        if (e <= est * (1.0f + 0x1p-17f)) close = e * (1.0f + 0x1p-17f) < est ? 0 : close + (at >= 0);
+                        if (e < est) {
+                            est = e;
+                            at = i + q;
+                        }
                     }
                 }
             }
+        }
+        if (arg && live) {
+            const float thr = warp_min(est) * (1.0f + 0x1p-18f);
+            const unsigned near = __ballot_sync(0xffffffffu, est <= thr);
+            const bool tie = __any_sync(0xffffffffu, odd || (est <= thr && (close || at < 0)));
+            if (__popc(near) == 1 && !tie) {
+                if (est <= thr) arg[r] = at;
+            } else {
+                long long best = 0x7ff0000000000000ll;  // +inf; positive doubles order as their bits
+                if (est <= thr || odd) {
+                    for (int i = 2 * lane; i < d; i += 64) {
+                        for (int q = 0; q < 2 && i + q < d; ++q) {
+                            const double x = ur[i + q];
+                            if ((__double_as_longlong(x) << 1) == 0) continue;
+                            float t, rest;
+                            const bool ok = split24(x, t, rest) && hf[i + q] > 0.f;
+                            if (ok && __fdividef(hf[i + q], fabsf(t)) > thr) continue;
+                            const double v = __ddiv_rn(half[i + q], fabs(x));
+                            const long long b = __double_as_longlong(v);
+                            if (v == v && b < best) best = b;
+                        }
+                    }
+                }
 #pragma unroll
-            for (int w = 16; w > 0; w >>= 1) {
-                const long long b = __shfl_xor_sync(0xffffffffu, best, w);
-                best = b < best ? b : best;
+                for (int w = 16; w > 0; w >>= 1) {
+                    const long long b = __shfl_xor_sync(0xffffffffu, best, w);
+                    best = b < best ? b : best;
+                }
+                if (lane == 0) {
+                    texit[r] = __longlong_as_double(best);
+                    arg[r] = -1;
+                }
             }
-            if (lane == 0) texit[r] = __longlong_as_double(best);
         }
     }
+}
+// The exit lengths whose coordinate is known: 32 divisions per warp instead of one.
+__global__ void __launch_bounds__(256) k_q_exit(int n_rays, int d, const double *u, const double *half,
+                                                const int32_t *arg, double *texit) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n_rays) return;
+    const int i = arg[r];
+    if (i >= 0) texit[r] = __ddiv_rn(half[i], fabs(u[(size_t)r * d + i]));
 }
 
 // B2[k][j][i] = hi(L_k[i][j]), B2[k][j][dK + i] = lo(L_k[i][j]) for i >= j (L_k^T, the
@@ -1628,7 +1685,7 @@ __global__ void __launch_bounds__(256) k_q_sum(int n_rk, int n_ntile, const floa
 // largest lower bound adds an FP32 exponential of exactly 0. A CTA takes RB rays at a time
 // by JW samples and QE_PASS times that, so that (j + 1) / n_steps is divided once per thread.
 // Every term in FP64, twice, and a division per sample: 196 us at 16384 rays x 64 samples,
-// K = 8, 66 us now. (ns_dev given: samples past *ns_dev are skipped)
+// K = 8, 28 us now. (ns_dev given: samples past *ns_dev are skipped)
 constexpr int QE_PASS = 8;
 __global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, int JW, const double *co,
                                                const float4 *cf, const double *texit, double *ell,
@@ -1655,17 +1712,16 @@ __global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, i
         low -= kSkipNats;
         auto term = [&](int k) { return fma(tau, fma(tau, dr[3 * k + 2], dr[3 * k + 1]), dr[3 * k]); };
         uint64_t keep = 0;
-        double emax = -INFINITY;
-        for (int k = 0; k < K; ++k) {
-            if (bound(cr[k], 1.f) < low) continue;
-            keep |= 1ull << k;
-            const double t = term(k);
-            emax = t > emax ? t : emax;
-        }
+        for (int k = 0; k < K; ++k) keep |= (uint64_t)(bound(cr[k], 1.f) < low ? 0 : 1) << k;
+        // each lane its own kept terms (neighbouring samples may keep different ones; one
+        // loop over the components would take each of them for the whole warp)
+        uint64_t m = keep & (keep - 1);
+        double emax = term(__ffsll((long long)keep) - 1);
         double l = emax;  // one term left: its exponential is 1
-        if ((keep & (keep - 1)) || !finite_bits(emax)) {
+        if (m || !finite_bits(emax)) {
+            for (; m; m &= m - 1) emax = fmax(emax, term(__ffsll((long long)m) - 1));
             float s = 0.f;
-            for (uint64_t m = keep; m; m &= m - 1) s += __expf(f64_to_f32(term(__ffsll((long long)m) - 1) - emax));
+            for (m = keep; m; m &= m - 1) s += __expf(f64_to_f32(term(__ffsll((long long)m) - 1) - emax));
             l = emax + f32_to_f64(__logf(s));
         }
         ell[e] = l;
@@ -1695,10 +1751,15 @@ void launch_q_split_rows(int n_rays, int d, int prec, const TcQuadWs &q, const d
                          const double *half, double *texit, cudaStream_t s) {
     const int g = (q.rows + 7) / 8 < 8 * num_sms() ? (q.rows + 7) / 8 : 8 * num_sms();
     note_launch();
+    int32_t *arg = texit ? q.arg : nullptr;
     if (prec == SB_PREC_BF16)
-        k_q_split_rows<SB_PREC_BF16><<<g, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, n_dev, half, texit);
+        k_q_split_rows<SB_PREC_BF16><<<g, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, n_dev, half, texit, arg);
     else
-        k_q_split_rows<SB_PREC_TF32><<<g, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, n_dev, half, texit);
+        k_q_split_rows<SB_PREC_TF32><<<g, 256, 0, s>>>(n_rays, q.rows, d, q.dK, u, q.A2, n_dev, half, texit, arg);
+    if (texit) {
+        note_launch();
+        k_q_exit<<<(unsigned)((n_rays + 255) / 256), 256, 0, s>>>(n_rays, d, u, half, q.arg, texit);
+    }
 }
 
 void carve_tc_quad(Carver &cv, TcQuadWs &q, int n_rays, int d, int K, int prec) {
@@ -1716,6 +1777,7 @@ void carve_tc_quad(Carver &cv, TcQuadWs &q, int n_rays, int d, int K, int prec) 
     q.q0 = cv.take<double>((size_t)K);
     q.co = cv.take<double>(3 * (size_t)n_rays * K);
     q.cf = cv.take<float4>((size_t)n_rays * K);
+    q.arg = cv.take<int32_t>((size_t)n_rays);
 }
 
 sb_status tc_ray_loglik_quad(const ProbView &pv, int n_rays, int n_steps, int prec, int bn, TcQuadWs q,
