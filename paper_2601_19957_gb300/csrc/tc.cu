@@ -98,6 +98,9 @@ struct TcArgs {
     float *qzout;
     const float *qoff;
     int qalpha_rows;
+    int nt0, nts;       // GEMM1: column tiles nt0 .. nt0 + nts - 1 only (nts 0: all); n_ntile counts those
+    bool mask_exact;    // zmask: a block without any set component is left out whole
+    double *G64;        // GEMM2: grad l = -G in FP64 instead of G
 };
 
 // ------------------------------------------------------------------ PTX helpers
@@ -191,11 +194,11 @@ struct TileInfo {
 // Components with r_nk > 0 at some row of row block mb (all when no flags are
 // given); a block with none keeps component 0 (non-finite or empty rows). One bit
 // per component (K <= 64).
-__device__ __forceinline__ uint64_t block_kmask(const uint32_t *rflag, int mb, int K) {
+__device__ __forceinline__ uint64_t block_kmask(const uint32_t *rflag, int mb, int K, bool exact = false) {
     uint64_t m = 0;
     for (int k = 0; k < K; ++k)
         if (!rflag || rflag[(size_t)mb * K + k]) m |= 1ull << k;
-    return m ? m : 1ull;
+    return m || exact ? m : 1ull;
 }
 
 // Component of GEMM2 chunk q: the (q / c_hi)-th set bit of the tile's mask.
@@ -208,9 +211,9 @@ __device__ __forceinline__ int chunk_component(const TileInfo &ti, int q) {
 
 template <int MODE, int BN, int KC>
 __device__ __forceinline__ TileInfo decode_tile(int t, int d, int K, const uint32_t *rflag, const int *glist,
-                                                int n_mblk) {
+                                                int n_mblk, int nct, int nt0, bool exact) {
+    // nct: column tiles per group, from tile nt0 on
     TileInfo ti;
-    const int nct = (d + BN - 1) / BN;
     if (glist) t = glist[t / nct] * nct + t % nct;  // compacted store-pass schedule
     ti.kmask = 0;
     ti.skip = false;
@@ -233,7 +236,7 @@ __device__ __forceinline__ TileInfo decode_tile(int t, int d, int K, const uint3
     } else {
         // column tiles of one (row block, component) are adjacent in the schedule, so
         // CTAs that run together gather the same x rows (served from L2)
-        ti.nt = t % nct;
+        ti.nt = nt0 + t % nct;
         ti.k = (t / nct) % K;
         ti.mb = t / (K * nct);
         ti.c_lo = (ti.nt * BN) / KC;
@@ -243,7 +246,8 @@ __device__ __forceinline__ TileInfo decode_tile(int t, int d, int K, const uint3
         // store pass (flags given): only the (block, component) pairs GEMM2 reads;
         // |z|^2 pass (mask given): only the pairs k_tc_need keeps (already the case
         // for a compacted schedule)
-        if (MODE != MODE_G && rflag && !glist) ti.skip = !((block_kmask(rflag, ti.mb, K) >> ti.k) & 1ull);
+        if (MODE != MODE_G && rflag && !glist)
+            ti.skip = !((block_kmask(rflag, ti.mb, K, exact) >> ti.k) & 1ull);
     }
     return ti;
 }
@@ -289,7 +293,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
     const int d = a.d, K = a.K;
     const int n_rows = a.n_rows_dev ? *a.n_rows_dev : a.n_rows_max;
     const int n_mblk = (n_rows + BM - 1) / BM;
-    const int nct = (d + BN - 1) / BN;
+    const int nct = MODE != MODE_G && a.nts ? a.nts : (d + BN - 1) / BN;
     int n_tiles = (MODE == MODE_G) ? n_mblk * nct : n_mblk * nct * K;
     // Store pass: the (row block, component) groups GEMM2 reads, compacted in
     // order, so that the round-robin deal spreads the work that remains (a
@@ -304,7 +308,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
         __syncthreads();
         for (int g0 = 0; g0 < n_groups; g0 += (int)blockDim.x) {
             const int g = g0 + (int)threadIdx.x;
-            const bool act = g < n_groups && ((block_kmask(gmask, g / K, K) >> (g % K)) & 1ull);
+            const bool act = g < n_groups && ((block_kmask(gmask, g / K, K, a.mask_exact) >> (g % K)) & 1ull);
             const unsigned bal = __ballot_sync(0xffffffffu, act);
             if (lane == 0) s_wcnt[warp] = __popc(bal);
             __syncthreads();
@@ -356,7 +360,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
             uint32_t inflight_phase[8];
             int n_inflight = 0;
             for (int it = 0, t = tile_of(0, gsz); t < n_tiles && !*s_abort; t = tile_of(++it, gsz)) {
-                const TileInfo ti = decode_tile<MODE, BN, KC>(t, d, K, MODE == MODE_G ? a.rflag : gmask, glist, n_mblk);
+                const TileInfo ti = decode_tile<MODE, BN, KC>(t, d, K, MODE == MODE_G ? a.rflag : gmask, glist, n_mblk, nct,
+                                                              a.nt0, a.mask_exact);
                 if (ti.skip) continue;
                 bool ok = true;
                 for (int q = 0; q < ti.nchunks; ++q) {
@@ -418,7 +423,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
             uint32_t acc_phase = 0;
             bool issued = false;
             for (int it = 0, t = tile_of(0, gsz); t < n_tiles && !*s_abort; t = tile_of(++it, gsz)) {
-                const TileInfo ti = decode_tile<MODE, BN, KC>(t, d, K, MODE == MODE_G ? a.rflag : gmask, glist, n_mblk);
+                const TileInfo ti = decode_tile<MODE, BN, KC>(t, d, K, MODE == MODE_G ? a.rflag : gmask, glist, n_mblk, nct,
+                                                              a.nt0, a.mask_exact);
                 if (ti.skip) continue;
                 if (!bwait(&tempty[acc], acc_phase ^ 1, s_abort)) break;
                 tc_fence_after();
@@ -465,7 +471,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
         int acc = 0;
         uint32_t acc_phase = 0;
         for (int it = 0, t = tile_of(0, gsz); t < n_tiles && !warp_aborted(s_abort); t = tile_of(++it, gsz)) {
-            const TileInfo ti = decode_tile<MODE, BN, KC>(t, d, K, MODE == MODE_G ? a.rflag : gmask, glist, n_mblk);
+            const TileInfo ti = decode_tile<MODE, BN, KC>(t, d, K, MODE == MODE_G ? a.rflag : gmask, glist, n_mblk, nct,
+                                                              a.nt0, a.mask_exact);
             if (ti.skip) continue;
             if (!warp_bwait(&tfull[acc], acc_phase, s_abort)) break;
             tc_fence_after();
@@ -495,7 +502,24 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
                 SB_TMEM_LD32(taddr + c0, v);
                 const int col = ti.nt * BN + c0;
                 if (MODE == MODE_G) {
-                    if (valid && col < d) {
+                    if (valid && col < d && a.G64) {
+                        // grad l = -G, widened on the integer units; 32-byte stores when the rows allow
+                        double *g = a.G64 + (size_t)w_out * d + col;
+                        if ((d & 3) == 0 && col + 32 <= d && (reinterpret_cast<uintptr_t>(a.G64) & 31) == 0) {
+#pragma unroll
+                            for (int e = 0; e < 32; e += 4)  // a whole 32-byte sector per store
+                                asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(g + e),
+                                             "d"(f32_to_f64(-__uint_as_float(v[e]))),
+                                             "d"(f32_to_f64(-__uint_as_float(v[e + 1]))),
+                                             "d"(f32_to_f64(-__uint_as_float(v[e + 2]))),
+                                             "d"(f32_to_f64(-__uint_as_float(v[e + 3])))
+                                             : "memory");
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (col + e < d) g[e] = f32_to_f64(-__uint_as_float(v[e]));
+                        }
+                    } else if (valid && col < d) {
                         float *g = a.G + (size_t)w_out * d + col;
                         if ((d & 3) == 0 && col + 32 <= d) {
 #pragma unroll
@@ -575,7 +599,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
                 }
             }
             if (MODE != MODE_G && !scaled && valid) {
-                a.qpart[((size_t)n * K + ti.k) * a.n_ntile + ti.nt] = q2;
+                a.qpart[((size_t)n * K + ti.k) * a.n_ntile + ti.nt - a.nt0] = q2;
                 if (MODE == MODE_Q && a.qpart1) a.qpart1[((size_t)n * K + ti.k) * a.n_ntile + ti.nt] = q1;
             }
             tc_fence_before();
@@ -601,7 +625,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
 // LSE over components from the FP32 |z|^2 partials: e_k and the maximum in
 // FP64, exp/log of the shifted values (in [0, 1] and [1, K]) in FP32, whose
 // absolute error stays below the FP32 resolution of the outputs.
-// mode 0: walkers (FT[act[n]] = -l, R); mode 2: points (ell[n] = l, R). Both raise
+// mode 0: walkers (FT[act[n]] = -l, R); mode 2: points (ell[act[n]] = l, R). Both raise
 // rflag[block][k] when some row of the 128-row block has r_nk > 0 (GEMM2 and the scaling
 // pass skip the other (block, component) pairs, whose terms are exactly zero).
 // Bound by the FP64 pipe (one warp instruction per 19 cycles and SM): each e_k is formed
@@ -702,7 +726,7 @@ __global__ void __launch_bounds__(LSE_ROWS) k_tc_lse(int mode, int K, int n_ntil
     if (mode == 0)
         FT[act ? act[n] : n] = f64_to_f32(-l);
     else
-        ell[n] = l;
+        ell[act ? act[n] : n] = l;
 }
 
 // GEMM2's A operand from the stored z: for every (128-row block, component) pair whose
@@ -891,46 +915,66 @@ __global__ void __launch_bounds__(256) k_tc_lnorm_gram(int d, int K, int k0, int
 }
 
 // A operand of GEMM1: A1[k][n][i] = round(x_n[i] - mu_k[i]) formed in FP32; x_n is a
-// walker row (through the active list).
+// row of X (through the list act when given), FP32 walkers or the caller's FP64 points
+// (rounded to FP32 on the integer units as they are read).
 // Rows from n_rows up to the next multiple of 128 and columns >= d are zeroed.
-// One thread per (row, 16-byte column group): x is formed once and the thread
-// writes that column group for every component.
-template <int PREC>
-__global__ void __launch_bounds__(256) k_tc_center(int d, int K, int rows_cap, int ldp, const int32_t *n_rows_dev,
-                                                   int n_rows_max, const int32_t *act, const float *X, int ld,
-                                                   const float *mu32, void *A1, const uint32_t *zmask) {
+// One thread per (row, 16-byte column group from group cg0 on): x is formed once and the
+// thread writes that column group for every component. vec: X allows 16-byte loads.
+template <int PREC, typename T>
+__global__ void __launch_bounds__(256) k_tc_center(int d, int K, int rows_cap, int ldp, int cg0,
+                                                   const int32_t *n_rows_dev, int n_rows_max, const int32_t *act,
+                                                   const T *X, bool vec_ok, const float *mu32, void *A1,
+                                                   const uint32_t *zmask, bool mask_exact) {
     constexpr int VE = (PREC == SB_PREC_BF16) ? 8 : 4;  // elements per 16-byte store
     const int n_rows = n_rows_dev ? *n_rows_dev : n_rows_max;
     int rows_pad = (n_rows + BM - 1) / BM * BM;
     if (rows_pad > rows_cap) rows_pad = rows_cap;
-    const int ncg = ldp / VE;
+    const int ncg = ldp / VE - cg0;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = e / ncg, cg = e - n * ncg;
+    const int n = e / ncg, cg = cg0 + e - n * ncg;
     if (n >= rows_pad) return;
+    const uint64_t km = zmask ? block_kmask(zmask, n / BM, K, mask_exact) : ~0ull;  // pairs the |z|^2 pass visits
+    if (!km) return;
     const int i0 = cg * VE;
     const bool live = n < n_rows;
-    const bool vec = ((d & 3) == 0) && i0 + VE <= d;
+    const bool vec = vec_ok && i0 + VE <= d;
     float x[VE];
 #pragma unroll
     for (int q = 0; q < VE; ++q) x[q] = 0.f;
     if (live) {
-        const float *xr = X + (size_t)(act ? act[n] : n) * ld;
-        if (vec && (ld & 3) == 0) {
+        const T *xr = X + (size_t)(act ? act[n] : n) * d;
+        if (vec) {
+            if constexpr (sizeof(T) == 4) {
 #pragma unroll
-            for (int q = 0; q < VE; q += 4) {
-                const float4 t = *reinterpret_cast<const float4 *>(xr + i0 + q);
-                x[q] = t.x;
-                x[q + 1] = t.y;
-                x[q + 2] = t.z;
-                x[q + 3] = t.w;
+                for (int q = 0; q < VE; q += 4) {
+                    const float4 t = *reinterpret_cast<const float4 *>(xr + i0 + q);
+                    x[q] = t.x;
+                    x[q + 1] = t.y;
+                    x[q + 2] = t.z;
+                    x[q + 3] = t.w;
+                }
+            } else {
+                double2 t[VE / 2];
+#pragma unroll
+                for (int q = 0; q < VE / 2; ++q) t[q] = reinterpret_cast<const double2 *>(xr + i0)[q];
+#pragma unroll
+                for (int q = 0; q < VE / 2; ++q) {
+                    x[2 * q] = f64_to_f32(t[q].x);
+                    x[2 * q + 1] = f64_to_f32(t[q].y);
+                }
             }
         } else {
 #pragma unroll
             for (int q = 0; q < VE; ++q)
-                if (i0 + q < d) x[q] = xr[i0 + q];
+                if (i0 + q < d) {
+                    if constexpr (sizeof(T) == 4)
+                        x[q] = xr[i0 + q];
+                    else
+                        x[q] = f64_to_f32(xr[i0 + q]);
+                }
         }
     }
-    const uint64_t km = zmask ? block_kmask(zmask, n / BM, K) : ~0ull;  // pairs the |z|^2 pass visits
+    const bool vmu = (d & 3) == 0 && i0 + VE <= d;
     for (int k = 0; k < K; ++k) {
         if (!((km >> k) & 1ull)) continue;
         float v[VE];
@@ -938,7 +982,7 @@ __global__ void __launch_bounds__(256) k_tc_center(int d, int K, int rows_cap, i
         for (int q = 0; q < VE; ++q) v[q] = 0.f;
         if (live) {
             const float *mk = mu32 + (size_t)k * d;
-            if (vec) {
+            if (vmu) {
 #pragma unroll
                 for (int q = 0; q < VE; q += 4) {
                     const float4 m4 = *reinterpret_cast<const float4 *>(mk + i0 + q);
@@ -963,6 +1007,105 @@ __global__ void __launch_bounds__(256) k_tc_center(int d, int K, int rows_cap, i
         } else {
             *reinterpret_cast<float4 *>(reinterpret_cast<float *>(A1) + o) =
                 make_float4(to_tf32(v[0]), to_tf32(v[1]), to_tf32(v[2]), to_tf32(v[3]));
+        }
+    }
+}
+
+// ------------------------------------------------------------------ component screen of a point set
+// The first points of a call come in any order, so every 128-row block would need every
+// component. From the last column tile of each z_k (the cheapest: its rows of the triangle
+// are the shortest) a point's leading component is guessed, points are listed by it, and
+// GEMM1 runs over the leading components; another component follows only where its term,
+// bounded by that tile's part of |z_k|^2, comes within kSkipNats of the leading one. The
+// FP32 exponential of the others is exactly 0, so the results are the same bits. Points
+// that will need several components (far from every mode the leading term itself is low)
+// are listed apart, so that the others' blocks keep to one: that guess takes the whole
+// |z|^2 as the last tile's part scaled by the coordinates.
+//
+// lead[n] (+ K when several components look needed) and the length of each list (hist,
+// zeroed before)
+__global__ void __launch_bounds__(256) k_tc_lead(int n_rows, int K, float scale, const float *qs, const double *a_k,
+                                                 int32_t *lead, int32_t *hist) {
+    __shared__ int h[2 * kMaxK];
+    __shared__ float a[kMaxK];
+    for (int k = threadIdx.x; k < 2 * K; k += blockDim.x) h[k] = 0;
+    for (int k = threadIdx.x; k < K; k += blockDim.x) a[k] = f64_to_f32(a_k[k]);
+    __syncthreads();
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n < n_rows) {
+        const float *q = qs + (size_t)n * K;
+        float top = -INFINITY;
+        int j = 0;
+        for (int k = 0; k < K; ++k) {
+            const float e = fmaf(-0.5f, q[k], a[k]);
+            if (e > top) {
+                top = e;
+                j = k;
+            }
+        }
+        const float low = fmaf(-0.5f * scale, q[j], a[j]) - kSkipNats;
+        bool more = false;
+        for (int k = 0; k < K; ++k) more = more || (k != j && !(fmaf(-0.5f, q[k], a[k]) < low));
+        if (more) j += K;
+        lead[n] = j;
+        atomicAdd(&h[j], 1);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < 2 * K; k += blockDim.x)
+        if (h[k]) atomicAdd(&hist[k], h[k]);
+}
+// act: the points grouped by list (the order inside a list does not reach the results,
+// which are stored by point), lead[n] reduced to the component; zmask[block][k]: the blocks
+// that hold a point led by k, or one that looked to need several. cursor zeroed before.
+__global__ void __launch_bounds__(256) k_tc_place(int n_rows, int K, int32_t *lead, const int32_t *hist,
+                                                  int32_t *cursor, int32_t *act, uint32_t *zmask) {
+    __shared__ int h[2 * kMaxK], base[2 * kMaxK], start[2 * kMaxK + 1];
+    for (int k = threadIdx.x; k < 2 * K; k += blockDim.x) h[k] = 0;
+    if (threadIdx.x == 0) {
+        start[0] = 0;
+        for (int k = 0; k < 2 * K; ++k) start[k + 1] = start[k] + hist[k];
+    }
+    __syncthreads();
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = n < n_rows ? lead[n] : 0;
+    const int at = n < n_rows ? atomicAdd(&h[j], 1) : 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < 2 * K; k += blockDim.x) base[k] = h[k] ? atomicAdd(&cursor[k], h[k]) : 0;
+    __syncthreads();
+    if (n < n_rows) {
+        act[start[j] + base[j] + at] = n;
+        if (j >= K) lead[n] = j - K;
+    }
+    const int n_mblk = (n_rows + BM - 1) / BM;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_mblk * K; e += gridDim.x * blockDim.x) {
+        const int mb = e / K, k = e - mb * K;
+        const bool own = start[k] < (mb + 1) * BM && start[k + 1] > mb * BM && start[k] < start[k + 1];
+        zmask[e] = own || (start[K] < n_rows && start[K] < (mb + 1) * BM) ? 1u : 0u;
+    }
+}
+// more[block][k]: the pairs the leading pass left out that some point of the block still
+// needs; zmask gains them.
+__global__ void __launch_bounds__(BM) k_tc_more(int n_rows, int K, int n_ntile, const int32_t *act, const int32_t *lead,
+                                                const float *qpart, const float *qs, const double *a_k,
+                                                uint32_t *zmask, uint32_t *more) {
+    const int p = blockIdx.x * BM + threadIdx.x;
+    const bool valid = p < n_rows;
+    const int n = valid ? act[p] : 0, j = valid ? lead[n] : 0;
+    double low = 0.0;
+    if (valid) {
+        const float *qp = qpart + ((size_t)p * K + j) * n_ntile;
+        double q = f32_to_f64(qp[0]);
+        for (int t = 1; t < n_ntile; ++t) q += f32_to_f64(qp[t]);
+        low = fma(-0.5, q, a_k[j]) - (double)(kSkipNats + 1.0f);
+    }
+    for (int k = 0; k < K; ++k) {
+        const bool in = zmask[(size_t)blockIdx.x * K + k] != 0u;
+        bool need = valid && !in;
+        if (need) need = !(fma(-0.5, f32_to_f64(qs[(size_t)n * K + k]), a_k[k]) < low);
+        const int any = __syncthreads_or(need);
+        if (threadIdx.x == 0) {
+            more[(size_t)blockIdx.x * K + k] = any ? 1u : 0u;
+            if (any) zmask[(size_t)blockIdx.x * K + k] = 1u;
         }
     }
 }
@@ -1069,21 +1212,9 @@ __global__ void k_tc_convert_vec(int d, int K, const double *mu, const double *c
     }
 }
 
-__global__ void k_tc_points_in(int n, int d, const double *x, float *X) {
-    const size_t tot = (size_t)n * d;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x)
-        X[e] = (float)x[e];
-}
-
 __global__ void k_tc_to_f32(size_t n, const double *x, float *y) {
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-        y[e] = (float)x[e];
-}
-
-__global__ void k_tc_points_out(int n, int d, const float *G, double *grad) {
-    const size_t tot = (size_t)n * d;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x)
-        grad[e] = -(double)G[e];  // G holds grad f = -grad l
+        y[e] = f64_to_f32(x[e]);
 }
 
 // ------------------------------------------------------------------ host side
@@ -1184,20 +1315,22 @@ void launch_gemm_any(int prec, int mode, int bn, const CUtensorMap &mapA, const 
     }
 }
 
+template <typename T>
 void launch_center(const TcWs &t, int d, int K, const int32_t *n_rows_dev, int n_rows_max, const int32_t *act,
-                   const float *X, cudaStream_t s, const uint32_t *zmask = nullptr) {
-    const int ldp = ldp_of(d, t.prec);
-    const int ncg = ldp / (t.prec == SB_PREC_BF16 ? 8 : 4);
+                   const T *X, cudaStream_t s, const uint32_t *zmask = nullptr, bool mask_exact = false, int col0 = 0) {
+    const int ldp = ldp_of(d, t.prec), ve = t.prec == SB_PREC_BF16 ? 8 : 4;
+    const int cg0 = col0 / ve, ncg = ldp / ve - cg0;
     int rows = (n_rows_max + BM - 1) / BM * BM;
     if (rows > (int)t.rows) rows = (int)t.rows;
+    const bool vec = d % (sizeof(T) == 4 ? 4 : 2) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     const dim3 grid((unsigned)(((long long)rows * ncg + 255) / 256));
     note_launch();
     if (t.prec == SB_PREC_BF16)
-        k_tc_center<SB_PREC_BF16><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, n_rows_dev, n_rows_max, act, X, d,
-                                                      (const float *)t.p[2], t.p[9], zmask);
+        k_tc_center<SB_PREC_BF16, T><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, cg0, n_rows_dev, n_rows_max, act, X,
+                                                          vec, (const float *)t.p[2], t.p[9], zmask, mask_exact);
     else
-        k_tc_center<SB_PREC_TF32><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, n_rows_dev, n_rows_max, act, X, d,
-                                                      (const float *)t.p[2], t.p[9], zmask);
+        k_tc_center<SB_PREC_TF32, T><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, cg0, n_rows_dev, n_rows_max, act, X,
+                                                          vec, (const float *)t.p[2], t.p[9], zmask, mask_exact);
 }
 
 size_t lse_smem(int K) {
@@ -1930,31 +2063,68 @@ sb_status tc_loglik_points(const ProbView &pv, const sb_config *c, const TcWs &t
                            float *g, double *ell, double *grad, cudaStream_t s) {
     (void)c;
     (void)f;
-    float *X = (float *)t.p[7];
-    float *G = g ? g : (float *)t.p[8];
-    note_launch();
-    k_tc_points_in<<<(unsigned)(((size_t)n * pv.d + 255) / 256 < 4096 ? ((size_t)n * pv.d + 255) / 256 : 4096), 256,
-                     0, s>>>(n, pv.d, x, X);
+    (void)g;
+    const int d = pv.d, K = pv.K;
     TcArgs a = base_args(pv, t);
     a.n_rows_max = n;
     a.prof = PROF_TC_Z_WALKERS;
-    launch_center(t, pv.d, pv.K, nullptr, n, nullptr, X, s);
-    // with the gradient, GEMM1 also stores z (the A operand of GEMM2 once scaled by r)
+    const int mode = grad ? MODE_ZW : MODE_ZR;  // with the gradient GEMM1 also stores z
+    int32_t *act = nullptr;
+    uint32_t *zmask = nullptr;
     a.rflag = nullptr;
-    launch_gemm_any(t.prec, grad ? MODE_ZW : MODE_ZR, t.bn, t.mapA1, t.mapT, a, s);
+    // The screen's eight launches take about 60 us at 16384 points; it pays when the flops
+    // it can spare, K - 1 of K components' GEMM1 less the last column tile of each, are worth
+    // about 40 us at the rate of these kernels, 1 PFLOP/s in BF16 (GEMM2 spares as many).
+    // d = 1024, K = 8, 16384 points, BF16 with the gradient: 365 us, 560 without.
+    const int nct = a.n_ntile, kc = t.prec == SB_PREC_BF16 ? 64 : 32;
+    int chunks = 0;
+    for (int nt = 0; nt < nct; ++nt) chunks += (d + kc - 1) / kc - nt * t.bn / kc;
+    const double last = (double)((d + kc - 1) / kc - (nct - 1) * t.bn / kc) / chunks;
+    const double spared = (double)n * d * (d + 1) * (K * (1.0 - last) - 1.0) * (t.prec == SB_PREC_BF16 ? 1.0 : 2.0);
+    if (nct >= 2 && spared >= 4.0e10) {
+        float *qs = (float *)t.p[11];
+        int32_t *lead = (int32_t *)t.p[13], *hist = (int32_t *)t.p[14];
+        uint32_t *more = (uint32_t *)t.p[10];  // rflag's place, which k_tc_lse writes later
+        act = (int32_t *)t.p[12];
+        zmask = (uint32_t *)t.p[16];
+        SB_CUDA_TRY(cudaMemsetAsync(hist, 0, 4 * sizeof(int32_t) * kMaxK, s));
+        launch_center(t, d, K, nullptr, n, nullptr, x, s, nullptr, false, (nct - 1) * t.bn);
+        TcArgs b = a;
+        b.nt0 = nct - 1;
+        b.nts = b.n_ntile = 1;
+        b.qpart = qs;
+        launch_gemm_any(t.prec, MODE_ZR, t.bn, t.mapA1, t.mapT, b, s);
+        const unsigned gn = (unsigned)((n + 255) / 256), gb = (unsigned)((n + BM - 1) / BM);
+        note_launch(2);
+        k_tc_lead<<<gn, 256, 0, s>>>(n, K, (float)d / (float)(d - (nct - 1) * t.bn), qs, pv.a, lead, hist);
+        k_tc_place<<<gn, 256, 0, s>>>(n, K, lead, hist, hist + 2 * kMaxK, act, zmask);
+        launch_center(t, d, K, nullptr, n, act, x, s, zmask);
+        a.zmask = zmask;
+        launch_gemm_any(t.prec, mode, t.bn, t.mapA1, t.mapT, a, s);
+        note_launch();
+        k_tc_more<<<gb, BM, 0, s>>>(n, K, a.n_ntile, act, lead, a.qpart, qs, pv.a, zmask, more);
+        launch_center(t, d, K, nullptr, n, act, x, s, more, true);
+        a.zmask = more;
+        a.mask_exact = true;
+        launch_gemm_any(t.prec, mode, t.bn, t.mapA1, t.mapT, a, s);
+        a.zmask = nullptr;
+        a.mask_exact = false;
+    } else {
+        launch_center(t, d, K, nullptr, n, nullptr, x, s);
+        launch_gemm_any(t.prec, mode, t.bn, t.mapA1, t.mapT, a, s);
+    }
     a.rflag = (const uint32_t *)t.p[10];  // written for every block by k_tc_lse
     note_launch();
-    k_tc_lse<<<(n + LSE_ROWS - 1) / LSE_ROWS, LSE_ROWS, lse_smem(pv.K), s>>>(2, pv.K, a.n_ntile, nullptr, n, nullptr, a.qpart, pv.a,
-                                             (float *)t.p[6], nullptr, ell, (uint32_t *)t.p[10], nullptr, nullptr,
-                                             nullptr, nullptr);
+    k_tc_lse<<<(n + LSE_ROWS - 1) / LSE_ROWS, LSE_ROWS, lse_smem(K), s>>>(2, K, a.n_ntile, nullptr, n, act, a.qpart,
+                                                                         pv.a, (float *)t.p[6], nullptr, ell,
+                                                                         (uint32_t *)t.p[10], zmask, nullptr, nullptr,
+                                                                         nullptr);
     if (grad) {
         launch_scale_z(pv, t, nullptr, n, s);
         a.prof = -1;
-        a.G = G;
+        a.act = act;
+        a.G64 = grad;
         launch_gemm_any(t.prec, MODE_G, t.bn, t.mapZ, t.mapB, a, s);
-        note_launch();
-        k_tc_points_out<<<(unsigned)(((size_t)n * pv.d + 255) / 256 < 4096 ? ((size_t)n * pv.d + 255) / 256 : 4096),
-                          256, 0, s>>>(n, pv.d, G, grad);
     }
     return cudaGetLastError() == cudaSuccess ? SB_OK : SB_ERR_CUDA;
 }
