@@ -17,9 +17,7 @@
 //  * log Z_k = l(x*) + (d/2) log 2pi - sum_i log C_ii (Sec. 3.7.1 with the
 //    whitening identity of App. A.8) and log Z = LSE_k log Z_k - log V
 //    (Sec. 3.7.3, App. A.10, Sec. 3.2).
-#include <vector>
 
-#include "sb_graph.cuh"
 #include "sb_laplace.cuh"
 
 namespace sb {
@@ -367,66 +365,114 @@ __global__ void __launch_bounds__(256) k_hessian(int d, int K, const double *P, 
 // launch latency: 96 dependent launches per factorisation at d = 1024). Blocks written
 // by one CTA are read by others after a barrier, so every read of H bypasses L1.
 //
-// Diagonal block factor, 256 threads, one barrier per column. Step j updates the
-// trailing lower triangle with the unscaled pivot column, a_ik -= a_ij a_kj / a_jj
-// (= L_ij L_kj), every thread taking 1 / a_jj itself; column j is final after
-// step j (later steps touch only columns > j), so the columns are scaled by
-// 1 / sqrt(a_jj) once at the end. A pivot <= 0 (not positive definite) sets the
-// candidate's info flag (read by every CTA after the next barrier).
+// The factorisation is a chain through the diagonal blocks, and on it every FP64
+// instruction of a warp costs 64 cycles (the pipe's rate per scheduler), so the diagonal
+// step is built from as few as possible.
 constexpr int CF_THREADS = 256;
-__device__ void potrf_block(int d, int kb, double *A, int32_t *info_c) {
+
+// 1 / p: an FP32 reciprocal of the mantissa (within 2^-22) with the negated exponent, then one
+// third-order step r + r (e + e^2), e = 1 - p r (error e^3 < 2^-66 before rounding): three
+// dependent FP64 instructions instead of a division's.
+__device__ __forceinline__ double recip(double p) {
+    const uint32_t hi = (uint32_t)__double2hiint(p), e = (hi >> 20) & 0x7ffu;
+    if (e - 64u > 1918u) return 1.0 / p;  // near the ends of the range
+    const float m = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | ((uint32_t)__double2loint(p) >> 29));
+    const uint32_t u = __float_as_uint(__frcp_rn(m));  // in (1/2, 1]: exponent 126 or 127
+    const double r = __hiloint2double((int)((hi & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + ((1919u - e) << 20))),
+                                      (int)(u << 29));
+    const double d = fma(-p, r, 1.0);
+    return fma(r, fma(d, d, d), r);
+}
+
+// Diagonal block kb: A[kb][kb] -= A[kb][kb-1] A[kb][kb-1]^T (upd, the trailing update of the
+// step before), then its factor. Threads 0..127 hold the block in registers: lane = row i,
+// warp q the columns q, q + 4, ... Step j: the owner warp of column j publishes it unscaled
+// and as the multipliers a_ij / a_jj, one barrier of the four warps, and every warp updates
+// its later columns, a_ik -= (a_ij / a_jj) a_kj. Columns are scaled by 1 / sqrt(a_jj) at the
+// end, all square roots at once. A pivot <= 0 (not positive definite) sets the candidate's
+// info flag (read by every CTA after the next barrier).
+__device__ void diag_block(int d, int kb, bool upd, double *A, int32_t *info_c) {
     __shared__ double a[NB][NB + 1];
-    const int o = kb * NB;
-    for (int e = threadIdx.x; e < NB * NB; e += CF_THREADS) {
+    __shared__ double pa[NB][NB + 1];
+    __shared__ double col[2][NB], mul[2][NB], piv[NB];
+    __shared__ int s_bad;
+    const int o = kb * NB, tid = threadIdx.x;
+    for (int e = tid; e < NB * NB; e += CF_THREADS) {
         const int i = e / NB, j = e % NB;
         a[i][j] = (o + i < d && o + j < d) ? __ldcg(&A[(size_t)(o + i) * d + o + j])
                                            : (i == j ? 1.0 : 0.0);  // identity padding
+        if (upd) pa[i][j] = o + i < d ? __ldcg(&A[(size_t)(o + i) * d + o - NB + j]) : 0.0;
     }
+    if (tid == 0) s_bad = 0;
     __syncthreads();
-    bool bad = false;
-    for (int j = 0; j < NB; ++j) {
-        const double p = a[j][j];
-        if (!(p > 0.0)) {
-            bad = true;
-            break;
-        }
-        const double ip = 1.0 / p;
-        const int m = NB - 1 - j;
-        for (int e = threadIdx.x; e < m * (m + 1) / 2; e += CF_THREADS) {
-            // e -> (ii >= kk) in the packed lower triangle of the trailing block
-            int ii = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-            while (ii * (ii + 1) / 2 > e) --ii;
-            while ((ii + 1) * (ii + 2) / 2 <= e) ++ii;
-            const int kk = e - ii * (ii + 1) / 2;
-            const int i = j + 1 + ii, k = j + 1 + kk;
-            a[i][k] -= a[i][j] * a[k][j] * ip;
+    if (upd) {
+        // the 528 entries of the lower triangle over the threads
+        for (int e = tid; e < NB * (NB + 1) / 2; e += CF_THREADS) {
+            int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+            while (i * (i + 1) / 2 > e) --i;
+            while ((i + 1) * (i + 2) / 2 <= e) ++i;
+            const int j = e - i * (i + 1) / 2;
+            double s = 0.0;
+#pragma unroll
+            for (int q = 0; q < NB; ++q) s = fma(pa[i][q], pa[j][q], s);
+            a[i][j] -= s;
         }
         __syncthreads();
     }
-    if (bad) {
-        if (threadIdx.x == 0) *info_c = 1;
+    if (tid < 128) {
+        const int i = tid & 31, q = tid >> 5;
+        double x[NB / 4];
+#pragma unroll
+        for (int t = 0; t < NB / 4; ++t) x[t] = i >= 4 * t + q ? a[i][4 * t + q] : 0.0;
+#pragma unroll
+        for (int t0 = 0; t0 < NB / 4; ++t0) {
+            for (int qo = 0; qo < 4; ++qo) {
+                const int j = 4 * t0 + qo, sl = j & 1;
+                if (q == qo) {
+                    const double p = __shfl_sync(0xffffffffu, x[t0], j);
+                    if (i == 0) {
+                        piv[j] = p;
+                        if (__double_as_longlong(p) <= 0 || p != p) s_bad = 1;
+                    }
+                    col[sl][i] = x[t0];
+                    mul[sl][i] = x[t0] * recip(p);
+                }
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                const double m = mul[sl][i];
+                // the column the next step needs comes first
+#pragma unroll
+                for (int t = 0; t < NB / 4; ++t)
+                    if (t > t0 || (t == t0 && q > qo)) x[t] = fma(-m, col[sl][4 * t + q], x[t]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < NB / 4; ++t)
+            if (i >= 4 * t + q) a[i][4 * t + q] = x[t];
+    }
+    __syncthreads();
+    if (s_bad) {
+        if (tid == 0) *info_c = 1;
         __syncthreads();
         return;
     }
-    for (int e = threadIdx.x; e < NB * NB; e += CF_THREADS) {
+    if (tid < NB) col[0][tid] = rsqrt(piv[tid]);
+    __syncthreads();
+    for (int e = tid; e < NB * NB; e += CF_THREADS) {
         const int i = e / NB, j = e % NB;
-        if (o + i < d && o + j < d && j <= i) {
-            const double r = rsqrt(a[j][j]);
-            A[(size_t)(o + i) * d + o + j] = i == j ? a[j][j] * r : a[i][j] * r;
-        }
+        if (o + i < d && o + j < d && j <= i) A[(size_t)(o + i) * d + o + j] = a[i][j] * col[0][j];
     }
-    __syncthreads();  // the shared block is free for the next item
+    __syncthreads();  // the shared blocks are free for the next item
 }
 
-// Panel: A[ib][kb] <- A[ib][kb] L_kk^{-T}. Threads 0..127: thread (r, part) holds row r's
-// columns part, part + 4, ... in registers; per column j the owner scales by
-// 1 / L_jj (reciprocals taken once, in parallel) and publishes it, then every
-// thread updates its later columns. One barrier per column (every thread of the
-// CTA takes part in them); the FP64 updates are spread over four warps.
-constexpr int TRSM_THREADS = 128;
-__device__ void trsm_block(int d, int kb, int ib, double *A) {
+// Panel: rows r0 .. r0 + 15 of column block kb, A <- A L_kk^{-T}. Threads 0..127: thread
+// (row, part) holds the row's columns part, part + 8, ...; per column j the owner scales by
+// 1 / L_jj (reciprocals taken once, in parallel) and publishes it, then every thread
+// updates its later columns, two on average (16 rows, not 32, because a warp instruction
+// takes its 64 cycles whatever the lanes: eight parts a row halve the chain).
+constexpr int TRSM_THREADS = 128, TRSM_ROWS = 16;
+__device__ void trsm_block(int d, int kb, int r0, double *A) {
     __shared__ double l[NB][NB + 1];
-    __shared__ double xs[NB][NB + 1];
+    __shared__ double xs[TRSM_ROWS][NB + 1];
     __shared__ double inv[NB];
     const int o = kb * NB;
     for (int e = threadIdx.x; e < NB * NB; e += CF_THREADS) {
@@ -434,33 +480,33 @@ __device__ void trsm_block(int d, int kb, int ib, double *A) {
         l[i][j] = (o + i < d && o + j < d) ? __ldcg(&A[(size_t)(o + i) * d + o + j]) : (i == j ? 1.0 : 0.0);
     }
     __syncthreads();
-    const bool act = threadIdx.x < TRSM_THREADS;
-    if (threadIdx.x < NB) inv[threadIdx.x] = 1.0 / l[threadIdx.x][threadIdx.x];
-    const int r = threadIdx.x & (NB - 1), part = (threadIdx.x >> 5) & 3;
-    const int row = ib * NB + r;
-    double x[NB / 4];
+    if (threadIdx.x < NB) inv[threadIdx.x] = recip(l[threadIdx.x][threadIdx.x]);
+    const int r = threadIdx.x & (TRSM_ROWS - 1), part = threadIdx.x / TRSM_ROWS;  // parts 0..7
+    const int row = r0 + r;
+    double x[NB / 8];
+    if (threadIdx.x < TRSM_THREADS)
 #pragma unroll
-    for (int q = 0; q < NB / 4; ++q) {
-        const int j = part + 4 * q;
-        x[q] = (act && row < d && o + j < d) ? __ldcg(&A[(size_t)row * d + o + j]) : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-        if (act && part == (j & 3)) {
-            x[j >> 2] *= inv[j];
-            xs[r][j] = x[j >> 2];
+        for (int q = 0; q < NB / 8; ++q) {
+            const int j = part + 8 * q;
+            x[q] = (row < d && o + j < d) ? __ldcg(&A[(size_t)row * d + o + j]) : 0.0;
         }
-        __syncthreads();
-        const double xj = xs[r][j];
+    __syncthreads();
+    if (threadIdx.x < TRSM_THREADS) {
 #pragma unroll
-        for (int q = 0; q < NB / 4; ++q)
-            if (part + 4 * q > j) x[q] -= xj * l[part + 4 * q][j];
-    }
-    if (act) {
+        for (int j = 0; j < NB; ++j) {
+            if (part == (j & 7)) {
+                x[j >> 3] *= inv[j];
+                xs[r][j] = x[j >> 3];
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            const double xj = xs[r][j];
 #pragma unroll
-        for (int q = 0; q < NB / 4; ++q) {
-            const int j = part + 4 * q;
+            for (int q = 0; q < NB / 8; ++q)
+                if (part + 8 * q > j) x[q] = fma(-xj, l[part + 8 * q][j], x[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < NB / 8; ++q) {
+            const int j = part + 8 * q;
             if (row < d && o + j < d) A[(size_t)row * d + o + j] = x[q];
         }
     }
@@ -502,23 +548,35 @@ __device__ __forceinline__ bool chol_live(int c, const int32_t *onehot, const in
 __global__ void __launch_bounds__(CF_THREADS) k_chol_coop(int d, double *H, const int32_t *n_c,
                                                          const int32_t *onehot, int32_t *info, uint32_t *bar,
                                                          int32_t *err) {
-    // the candidate count is the same value in every CTA, so all CTAs reach every barrier
+    // the candidate count is the same value in every CTA, so all CTAs reach every
+    // barrier; none is needed when every candidate is one-hot
     const int nc = *n_c;
+    if (onehot) {
+        bool any = false;
+        for (int c = 0; c < nc && !any; ++c) any = onehot[c] < 0;
+        if (!any) return;
+    }
     const int nblk = (d + NB - 1) / NB;
-    for (int kb = 0; kb < nblk; ++kb) {
-        for (int c = blockIdx.x; c < nc; c += gridDim.x)
-            if (chol_live(c, onehot, info)) potrf_block(d, kb, H + (size_t)c * d * d, info + c);
-        if (!grid_barrier(bar, gridDim.x, err)) return;
+    for (int c = blockIdx.x; c < nc; c += gridDim.x)
+        if (chol_live(c, onehot, info)) diag_block(d, 0, false, H + (size_t)c * d * d, info + c);
+    if (!grid_barrier(bar, gridDim.x, err)) return;
+    for (int kb = 0; kb + 1 < nblk; ++kb) {
         const int rest = nblk - kb - 1;
-        if (rest == 0) break;
-        for (int it = blockIdx.x; it < nc * rest; it += gridDim.x) {
-            const int c = it / rest;
-            if (chol_live(c, onehot, info)) trsm_block(d, kb, kb + 1 + it % rest, H + (size_t)c * d * d);
+        for (int it = blockIdx.x; it < nc * 2 * rest; it += gridDim.x) {
+            const int c = it / (2 * rest);
+            if (chol_live(c, onehot, info))
+                trsm_block(d, kb, (kb + 1) * NB + (it % (2 * rest)) * TRSM_ROWS, H + (size_t)c * d * d);
         }
         if (!grid_barrier(bar, gridDim.x, err)) return;
-        const int tri = rest * (rest + 1) / 2;  // trailing blocks (ii >= jj) per candidate
-        for (int it = blockIdx.x; it < nc * tri; it += gridDim.x) {
-            const int c = it / tri, e = it - c * tri;
+        // the next diagonal block of every candidate is updated and factored at once, by
+        // the first CTAs; the other trailing blocks (ii >= jj, ii > 0) go to the rest
+        for (int c = blockIdx.x; c < nc; c += gridDim.x)
+            if (chol_live(c, onehot, info)) diag_block(d, kb + 1, true, H + (size_t)c * d * d, info + c);
+        const int tri = rest * (rest + 1) / 2 - 1;
+        const int skip = (int)gridDim.x > 2 * nc ? nc : 0;  // CTAs that only factor in this phase
+        const int b = (int)blockIdx.x - skip, nb = (int)gridDim.x - skip;
+        for (int it = b; b >= 0 && it < nc * tri; it += nb) {
+            const int c = it / tri, e = it - c * tri + 1;
             if (!chol_live(c, onehot, info)) continue;
             int ii = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
             while (ii * (ii + 1) / 2 > e) --ii;
@@ -530,25 +588,63 @@ __global__ void __launch_bounds__(CF_THREADS) k_chol_coop(int d, double *H, cons
     }
 }
 
+// The inverses of the factors' 32 x 32 diagonal blocks, for the solves: the strictly lower
+// part of a block's inverse, transposed, goes into the strictly upper part of the block,
+// which nothing else uses. A CTA per (block, candidate), a warp per four columns, lanes over
+// rows.
+__global__ void __launch_bounds__(256) k_chol_dinv(int d, double *H, const int32_t *n_c, const int32_t *info) {
+    __shared__ double Cs[NB][NB + 1];
+    __shared__ double inv[NB];
+    const int c = blockIdx.y, r0 = blockIdx.x * NB;
+    if (c >= *n_c || info[c]) return;
+    double *C = H + (size_t)c * d * d;
+    for (int e = threadIdx.x; e < NB * NB; e += 256) {
+        const int i = r0 + e / NB, j = r0 + e % NB;
+        Cs[e / NB][e % NB] = i < d && j <= i ? C[(size_t)i * d + j] : (i == j ? 1.0 : 0.0);
+    }
+    __syncthreads();
+    if (threadIdx.x < NB) inv[threadIdx.x] = recip(Cs[threadIdx.x][threadIdx.x]);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = lane == wid * 4 + q ? 1.0 : 0.0;
+    for (int i = wid * 4; i < NB; ++i) {  // rows above the warp's columns stay zero
+        const double v = lane > i ? Cs[lane][i] : 0.0, iv = inv[i];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double xi = __shfl_sync(0xffffffffu, b[q], i) * iv;
+            b[q] = lane == i ? xi : fma(-v, xi, b[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int j = r0 + wid * 4 + q, i = r0 + lane;
+        if (i < d && i > j) C[(size_t)j * d + i] = b[q];
+    }
+}
+
 // Solve (C C^T) delta = g for each candidate still polishing and the model
 // increase g^T delta / 2 (cooperative launch, one bounded grid barrier per 32-row
 // block and direction). The grid is split into slots of Gc CTAs (Gc from the
 // candidate count on the device, 1 to 16); slot j serves candidates j, j + slots,
 // ... in turn, and CTA q of a slot owns the row blocks J with J % Gc == q of each.
 // Forward (C y = g): in step I the owner of block I (already updated by every
-// earlier step, by itself) solves the diagonal block and publishes y_I; after the
-// barrier every owner subtracts C_JI y_I from its blocks J > I. The owner of block
-// I + 1 has then finished block I + 1's last update before it solves it in step
+// earlier step, by itself) multiplies it by the inverse of the diagonal block (k_chol_dinv) and
+// publishes y_I; after the barrier every owner subtracts C_JI y_I from its blocks J > I. The
+// owner of block I + 1 has then finished block I + 1's last update before it solves it in step
 // I + 1, so one barrier per step suffices. Backward (C^T delta = y) mirrors it
 // with (C^T)_JI = (C_IJ)^T for J < I. The right-hand side lives in delta[c]
-// (global, read past L1 after barriers).
+// (global, read past L1 after barriers). Both products are 32 x 32 by a vector: lane = row,
+// warp w the columns 4 w .. 4 w + 3, the eight partial sums added in order; the matrix is
+// read into shared memory before the barrier it does not depend on. (A substitution per
+// block was 32 dependent steps, 375 us per solve of four candidates at d = 512; 253 now.)
 constexpr int CS_THREADS = 256;
 __global__ void __launch_bounds__(CS_THREADS) k_chol_solve_coop(int d, const double *H, const double *g,
                                                                 const int32_t *n_c, const int32_t *info,
                                                                 const uint8_t *active, double *delta, double *pred,
                                                                 uint32_t *bar, int32_t *err) {
-    __shared__ double Dg[32][33];
-    __shared__ double dinv[32];
+    __shared__ double M[32][33];
     __shared__ double xs[32];
     __shared__ double part[8];
     __shared__ double red[8][33];
@@ -572,93 +668,80 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_solve_coop(int d, const dou
                 y[i] = g[(size_t)c * d + i];
     }
     __syncthreads();
-    // the owner's diagonal solve of block I of candidate c (lower: forward; upper: with C^T)
-    auto diag = [&](int c, int I, bool upper) {
-        const double *C = H + (size_t)c * d * d;
-        double *y = delta + (size_t)c * d;
-        const int r0 = I * 32, rows = min(32, d - r0);
+    // M = the inverse of diagonal block I (upper: its transpose): the strictly lower part from
+    // above the diagonal of the block, the diagonal as reciprocals
+    auto load_dinv = [&](const double *C, int I, bool upper) {
+        const int r0 = I * 32;
+        __syncthreads();
         for (int e = threadIdx.x; e < 32 * 32; e += CS_THREADS) {
             const int i = e / 32, j = e % 32;
-            Dg[i][j] = (i < rows && j < rows) ? C[(size_t)(r0 + i) * d + r0 + j] : (i == j ? 1.0 : 0.0);
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) dinv[threadIdx.x] = 1.0 / Dg[threadIdx.x][threadIdx.x];
-        __syncthreads();
-        if (wid == 0) {
-            double v = lane < rows ? __ldcg(y + r0 + lane) : 0.0;
-            if (!upper) {
-                for (int i = 0; i < 32; ++i) {
-                    const double yi = __shfl_sync(0xffffffffu, v, i) * dinv[i];
-                    if (lane == i) v = yi;
-                    if (lane > i) v -= Dg[lane][i] * yi;
-                }
-            } else {
-                for (int i = 31; i >= 0; --i) {
-                    const double xi = __shfl_sync(0xffffffffu, v, i) * dinv[i];
-                    if (lane == i) v = xi;
-                    if (lane < i) v -= Dg[i][lane] * xi;
-                }
+            const bool in = r0 + i < d && r0 + j < d;
+            if (j > i) {
+                const double v = in ? C[(size_t)(r0 + i) * d + r0 + j] : 0.0;  // (block^-1)[j][i]
+                M[upper ? i : j][upper ? j : i] = v;
+                M[upper ? j : i][upper ? i : j] = 0.0;
+            } else if (i == j) {
+                M[i][i] = in ? recip(C[(size_t)(r0 + i) * d + r0 + i]) : 1.0;
             }
-            if (lane < rows) y[r0 + lane] = v;
         }
-        __threadfence();
-        __syncthreads();
     };
-    // forward
-    for (int I = 0; I < nb; ++I) {
-        if (I % Gc == q)
-            for (int c = c0; c < ncand; c += slots)
-                if (live(c)) diag(c, I, false);
-        if (!grid_barrier(bar, gridDim.x, err)) return;
-        const int r0 = I * 32, rows = min(32, d - r0);
-        for (int c = c0; c < ncand; c += slots) {
-            if (!live(c)) continue;
-            const double *C = H + (size_t)c * d * d;
-            double *y = delta + (size_t)c * d;
-            if (threadIdx.x < 32) xs[threadIdx.x] = threadIdx.x < rows ? __ldcg(y + r0 + threadIdx.x) : 0.0;
-            __syncthreads();
-            // y_J -= C_JI y_I for owned J > I: warp per output row
-            for (int J = I + 1; J < nb; ++J) {
-                if (J % Gc != q) continue;
-                const int j0 = J * 32, jr = min(32, d - j0);
-                for (int rr = wid; rr < jr; rr += CS_THREADS / 32) {
-                    const double a = lane < rows ? C[(size_t)(j0 + rr) * d + r0 + lane] * xs[lane] : 0.0;
-                    const double sum = warp_sum(a);
-                    if (lane == 0) y[j0 + rr] -= sum;
-                }
-            }
-            __syncthreads();
+    // M = block C_JI (rows of J), or for the backward pass (C_IJ)^T
+    auto load_block = [&](const double *C, int J, int I, bool upper) {
+        const int j0 = J * 32, i0 = I * 32;
+        __syncthreads();
+        for (int e = threadIdx.x; e < 32 * 32; e += CS_THREADS) {
+            const int i = e / 32, j = e % 32;
+            if (!upper)
+                M[i][j] = j0 + i < d && i0 + j < d ? C[(size_t)(j0 + i) * d + i0 + j] : 0.0;
+            else
+                M[j][i] = i0 + i < d && j0 + j < d ? C[(size_t)(i0 + i) * d + j0 + j] : 0.0;
         }
-    }
-    // backward
-    for (int I = nb - 1; I >= 0; --I) {
-        if (I % Gc == q)
-            for (int c = c0; c < ncand; c += slots)
-                if (live(c)) diag(c, I, true);
-        if (!grid_barrier(bar, gridDim.x, err)) return;
-        const int r0 = I * 32, rows = min(32, d - r0);
-        for (int c = c0; c < ncand; c += slots) {
-            if (!live(c)) continue;
-            const double *C = H + (size_t)c * d * d;
-            double *y = delta + (size_t)c * d;
-            if (threadIdx.x < 32) xs[threadIdx.x] = threadIdx.x < rows ? __ldcg(y + r0 + threadIdx.x) : 0.0;
-            __syncthreads();
-            // y_J -= (C_IJ)^T x_I for owned J < I: thread per output column j (coalesced rows of C)
-            for (int J = 0; J < I; ++J) {
-                if (J % Gc != q) continue;
-                const int j0 = J * 32;
-                // 8 warps split the 32 rows of block I; lane = column j
-                double a = 0.0;
-                for (int i = wid; i < rows; i += CS_THREADS / 32) a += C[(size_t)(r0 + i) * d + j0 + lane] * xs[i];
-                red[wid][lane] = a;
-                __syncthreads();
-                if (wid == 0) {
-                    double t = 0.0;
-                    for (int w = 0; w < CS_THREADS / 32; ++w) t += red[w][lane];
-                    y[j0 + lane] -= t;
+    };
+    // the product M x (x: 32 entries of y from x0, zero past d) in warp 0's lanes
+    auto apply = [&](const double *y, int x0) {
+        if (threadIdx.x < 32) xs[threadIdx.x] = x0 + (int)threadIdx.x < d ? __ldcg(y + x0 + threadIdx.x) : 0.0;
+        __syncthreads();
+        double s = M[lane][4 * wid] * xs[4 * wid];
+#pragma unroll
+        for (int t = 1; t < 4; ++t) s = fma(M[lane][4 * wid + t], xs[4 * wid + t], s);
+        red[wid][lane] = s;
+        __syncthreads();
+        if (wid != 0) return 0.0;
+        const double s01 = red[0][lane] + red[1][lane], s23 = red[2][lane] + red[3][lane];
+        const double s45 = red[4][lane] + red[5][lane], s67 = red[6][lane] + red[7][lane];
+        return (s01 + s23) + (s45 + s67);
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        const bool upper = pass == 1;
+        for (int st = 0; st < nb; ++st) {
+            const int I = upper ? nb - 1 - st : st, r0 = I * 32;
+            if (I % Gc == q)
+                for (int c = c0; c < ncand; c += slots) {
+                    if (!live(c)) continue;
+                    double *y = delta + (size_t)c * d;
+                    load_dinv(H + (size_t)c * d * d, I, upper);
+                    __syncthreads();
+                    const double v = apply(y, r0);
+                    if (wid == 0 && r0 + lane < d) y[r0 + lane] = v;
+                    __threadfence();
                 }
-                __syncthreads();
+            // the first block this CTA updates after the barrier
+            const int J0 = upper ? q : I + 1 + ((q - (I + 1)) % Gc + Gc) % Gc;
+            const bool any = c0 < ncand && (upper ? J0 < I : J0 < nb);
+            if (any && live(c0)) load_block(H + (size_t)c0 * d * d, J0, I, upper);
+            if (!grid_barrier(bar, gridDim.x, err)) return;
+            for (int c = c0; any && c < ncand; c += slots) {
+                if (!live(c)) continue;
+                const double *C = H + (size_t)c * d * d;
+                double *y = delta + (size_t)c * d;
+                for (int J = J0; upper ? J < I : J < nb; J += Gc) {
+                    if (c != c0 || J != J0) load_block(C, J, I, upper);
+                    __syncthreads();
+                    const double v = apply(y, r0);
+                    if (wid == 0 && J * 32 + lane < d) y[J * 32 + lane] -= v;
+                }
             }
+            __syncthreads();
         }
     }
     if (!grid_barrier(bar, gridDim.x, err)) return;
@@ -941,18 +1024,6 @@ void launch_precision_needed(int d, int K, const double *L, const double *R, con
     k_precision<<<g, 256, 0, s>>>(d, L, P, need);
 }
 
-// Condition of the blocked factorisation: some live candidate is not one-hot.
-__global__ void k_chol_needed(cudaGraphConditionalHandle h, const int32_t *n_c, const int32_t *onehot) {
-    __shared__ int any;
-    if (threadIdx.x == 0) any = 0;
-    __syncthreads();
-    const int nc = *n_c;
-    for (int c = threadIdx.x; c < nc; c += blockDim.x)
-        if (onehot[c] < 0) any = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) cudaGraphSetConditional(h, any ? 1u : 0u);
-}
-
 int laplace_sms();
 
 void launch_hessian_chol(int d, int K, int cap, const double *L, const double *P, const double *Z, const double *R,
@@ -977,33 +1048,7 @@ void launch_hessian_chol(int d, int K, int cap, const double *L, const double *P
         note_launch();
         cudaLaunchCooperativeKernel((const void *)k_chol_coop, dim3(G), dim3(CF_THREADS), args, 0, fs);
     };
-    // in a graph, the factorisation is the body of an IF node that runs only when some
-    // live candidate is not one-hot (its launches would otherwise all be idle CTAs)
-    if (onehot && stream_capturing(s)) {
-        const sb_status st = capture_if(
-            s,
-            [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
-                note_launch();
-                k_chol_needed<<<1, 256, 0, cs>>>(h, n_c, onehot);
-            },
-            factor);
-        if (st == SB_OK) return;
-        // the node could not be added: factor unconditionally (a capture left broken by
-        // the failure reports it when it ends)
-    } else if (onehot && !stream_capturing(s)) {
-        // eager mode (host reads allowed): the same decision on the host, so that an
-        // all-one-hot candidate set launches no idle factorisation kernels either
-        int32_t nc = 0;
-        std::vector<int32_t> oh((size_t)cap);
-        if (cudaMemcpyAsync(&nc, n_c, sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-            cudaMemcpyAsync(oh.data(), onehot, sizeof(int32_t) * (size_t)cap, cudaMemcpyDeviceToHost, s) ==
-                cudaSuccess &&
-            cudaStreamSynchronize(s) == cudaSuccess) {
-            bool any = false;
-            for (int c = 0; c < nc && c < cap; ++c) any = any || oh[(size_t)c] < 0;
-            if (!any) return;
-        }
-    }
+    // (the kernel leaves at once when every live candidate is one-hot)
     factor(s);
 }
 
@@ -1017,13 +1062,15 @@ int laplace_sms() {
     return n;
 }
 
-void launch_chol_solve_coop(int d, int cap, const double *H, const double *g, const int32_t *n_c, const int32_t *info,
+void launch_chol_solve_coop(int d, int cap, double *H, const double *g, const int32_t *n_c, const int32_t *info,
                             const uint8_t *active, double *delta, double *pred, uint32_t *bar, int32_t *err,
                             cudaStream_t s) {
     // one CTA per SM at most (a cooperative grid must be co-resident), up to 16 per
     // candidate of the cap; the kernel divides them among the live candidates
     int G = laplace_sms();
     if (G > 16 * cap) G = 16 * cap;
+    note_launch();
+    k_chol_dinv<<<dim3((d + NB - 1) / NB, cap), 256, 0, s>>>(d, H, n_c, info);
     cudaMemsetAsync(bar, 0, 2 * sizeof(uint32_t), s);
     void *args[] = {&d, &H, &g, &n_c, &info, &active, &delta, &pred, &bar, &err};
     note_launch();

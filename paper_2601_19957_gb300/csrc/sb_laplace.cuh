@@ -39,7 +39,7 @@ void launch_hessian_chol(int d, int K, int cap, const double *L, const double *P
 // co-resident CTAs (cooperative launch, one bounded grid barrier per 32-row block
 // and direction; at most one per SM and 16 per candidate of the cap, divided among
 // the *n_c candidates on the device).
-void launch_chol_solve_coop(int d, int cap, const double *H, const double *g, const int32_t *n_c, const int32_t *info,
+void launch_chol_solve_coop(int d, int cap, double *H, const double *g, const int32_t *n_c, const int32_t *info,
                             const uint8_t *active, double *delta, double *pred, uint32_t *bar, int32_t *err,
                             cudaStream_t s);
 // *n_eff = *n_reps when *n_live > 0 (or n_live is null), else 0: the candidate count the
