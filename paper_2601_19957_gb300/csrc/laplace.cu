@@ -37,7 +37,7 @@ constexpr int NB = 32;  // Cholesky block
 //      it, CTA 0 records it;
 //   4. every CTA tests its unassigned points against the representative,
 //      one warp per point: coalesced 32-coordinate slices, leaving at the
-//      first coordinate farther than tau (a warp vote).
+//      first four that hold a coordinate farther than tau (a warp vote).
 // A slot is rewritten two rounds later, after every CTA has passed the
 // barrier of the round in between, so it is never overwritten while read.
 // The barrier wait is bounded: on timeout the CTA flags SB_DEV_TIMEOUT and
@@ -75,9 +75,24 @@ __device__ bool grid_barrier(uint32_t *bar, uint32_t n_blocks, int32_t *err) {
     return s_ok != 0;
 }
 
-// (l, index) order of the greedy: larger l first, ties to the lower index; index < 0 is "none".
-__device__ __forceinline__ bool dd_better(double l, int i, double bl, int bi) {
+// (l, index) order of the greedy: larger l first, ties to the lower index; index < 0 is
+// "none". l is compared as order-preserving integers (the FP64 pipe takes 64 cycles per
+// warp instruction and scheduler, and a round compares along several reductions).
+__device__ __forceinline__ bool dd_better(uint64_t l, int i, uint64_t bl, int bi) {
     return i >= 0 && (bi < 0 || l > bl || (l == bl && i < bi));
+}
+__device__ __forceinline__ uint64_t dd_key(double l) {  // -0 and +0 alike
+    return ordered_bits((__double_as_longlong(l) << 1) == 0 ? 0.0 : l);
+}
+
+// |x - b| > tau, decided in FP32 on the rounded operands unless the difference lies within
+// their rounding of tau, where FP64 decides (a call: inlined it would be predicated).
+static __device__ __noinline__ bool dd_far_exact(double x, double b, double tau) { return fabs(x - b) > tau; }
+__device__ __forceinline__ bool dd_far(double x, double b, float bf, double tau, float tf) {
+    const float xf = f64_to_f32(x), df = fabsf(xf - bf), err = (fabsf(xf) + fabsf(bf)) * 0x1p-23f;
+    if (df - err > tf * (1.0f + 0x1p-20f)) return true;
+    if (df + err < tf * (1.0f - 0x1p-20f)) return false;
+    return dd_far_exact(x, b, tau);
 }
 
 __global__ void __launch_bounds__(DD_THREADS) k_dedup(int n, int d, const double *X, const double *ell,
@@ -85,8 +100,9 @@ __global__ void __launch_bounds__(DD_THREADS) k_dedup(int n, int d, const double
                                                       const double *wmax, int cap, int32_t *reps, int32_t *n_reps,
                                                       uint8_t *assigned, double *part_l, int32_t *part_i,
                                                       uint32_t *bar, int32_t *err) {
-    extern __shared__ double s_xb[];  // [d] the round's representative
-    __shared__ double s_l[DD_THREADS / 32];
+    extern __shared__ double s_xb[];  // [d] the round's representative, then the same in FP32
+    float *s_xf = reinterpret_cast<float *>(s_xb + d);
+    __shared__ uint64_t s_l[DD_THREADS / 32];
     __shared__ int s_i[DD_THREADS / 32];
     __shared__ int s_best;
     const int G = gridDim.x;
@@ -94,29 +110,20 @@ __global__ void __launch_bounds__(DD_THREADS) k_dedup(int n, int d, const double
     const int w0 = blockIdx.x * per, w1 = min(n, w0 + per);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double tau = tau_scale * wmax[0];
+    const float tf = f64_to_f32(tau);
+    uint64_t *part_k = reinterpret_cast<uint64_t *>(part_l);
     for (int w = w0 + threadIdx.x; w < w1; w += DD_THREADS) {
-        bool el = isfinite(ell[w]);
+        bool el = finite_bits(ell[w]);
         if (status && status[w] == SB_WALKER_NONFINITE) el = false;
         if (keep_in && !keep_in[w]) el = false;
         assigned[w] = el ? 0 : 1;
     }
     __syncthreads();
-    int count = 0;
-    for (int round = 0;; ++round) {
-        // 1. this CTA's best unassigned point
-        double bl = -INFINITY;
-        int bi = -1;
-        for (int w = w0 + threadIdx.x; w < w1; w += DD_THREADS) {
-            if (assigned[w]) continue;
-            const double l = ell[w];
-            if (bi < 0 || l > bl) {  // strided ascending: the first seen has the lower index
-                bl = l;
-                bi = w;
-            }
-        }
+    // the best of a warp's lanes, then of the CTA's warps (in every thread)
+    auto cta_best = [&](uint64_t &bl, int &bi) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const double ol = __shfl_xor_sync(0xffffffffu, bl, o);
+            const uint64_t ol = __shfl_xor_sync(0xffffffffu, bl, o);
             const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
             if (dd_better(ol, oi, bl, bi)) {
                 bl = ol;
@@ -128,58 +135,53 @@ __global__ void __launch_bounds__(DD_THREADS) k_dedup(int n, int d, const double
             s_i[wid] = bi;
         }
         __syncthreads();
+        bl = 0;
+        bi = -1;
+        for (int q = 0; q < DD_THREADS / 32; ++q)
+            if (dd_better(s_l[q], s_i[q], bl, bi)) {
+                bl = s_l[q];
+                bi = s_i[q];
+            }
+        __syncthreads();
+    };
+    int count = 0;
+    for (int round = 0;; ++round) {
+        // 1. this CTA's best unassigned point
+        uint64_t bl = 0;
+        int bi = -1;
+        for (int w = w0 + threadIdx.x; w < w1; w += DD_THREADS) {
+            if (assigned[w]) continue;
+            const uint64_t l = dd_key(ell[w]);
+            if (bi < 0 || l > bl) {  // strided ascending: the first seen has the lower index
+                bl = l;
+                bi = w;
+            }
+        }
+        cta_best(bl, bi);
         const int slot = (round & 1) * G;
         if (threadIdx.x == 0) {
-            double b = -INFINITY;
-            int ib = -1;
-            for (int q = 0; q < DD_THREADS / 32; ++q)
-                if (dd_better(s_l[q], s_i[q], b, ib)) {
-                    b = s_l[q];
-                    ib = s_i[q];
-                }
-            part_l[slot + blockIdx.x] = b;
-            part_i[slot + blockIdx.x] = ib;
+            part_k[slot + blockIdx.x] = bl;
+            part_i[slot + blockIdx.x] = bi;
         }
         // 2.
         if (!grid_barrier(bar, (uint32_t)G, err)) break;
         // 3. the global best from the partials (read past L1: written by other CTAs)
-        bl = -INFINITY;
+        bl = 0;
         bi = -1;
         for (int q = threadIdx.x; q < G; q += DD_THREADS) {
-            const double l = __ldcg(part_l + slot + q);
+            const uint64_t l = __ldcg(reinterpret_cast<const unsigned long long *>(part_k + slot + q));
             const int i = __ldcg(part_i + slot + q);
             if (dd_better(l, i, bl, bi)) {
                 bl = l;
                 bi = i;
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double ol = __shfl_xor_sync(0xffffffffu, bl, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (dd_better(ol, oi, bl, bi)) {
-                bl = ol;
-                bi = oi;
-            }
-        }
-        __syncthreads();  // s_l / s_i of step 1 fully consumed
-        if (lane == 0) {
-            s_l[wid] = bl;
-            s_i[wid] = bi;
-        }
-        __syncthreads();
+        cta_best(bl, bi);
         if (threadIdx.x == 0) {
-            double b = -INFINITY;
-            int ib = -1;
-            for (int q = 0; q < DD_THREADS / 32; ++q)
-                if (dd_better(s_l[q], s_i[q], b, ib)) {
-                    b = s_l[q];
-                    ib = s_i[q];
-                }
-            s_best = ib;
-            if (ib >= 0) {
-                if (ib >= w0 && ib < w1) assigned[ib] = 1;
-                if (blockIdx.x == 0 && count < cap) reps[count] = ib;
+            s_best = bi;
+            if (bi >= 0) {
+                if (bi >= w0 && bi < w1) assigned[bi] = 1;
+                if (blockIdx.x == 0 && count < cap) reps[count] = bi;
             }
         }
         __syncthreads();
@@ -189,15 +191,29 @@ __global__ void __launch_bounds__(DD_THREADS) k_dedup(int n, int d, const double
         if (count >= cap) break;
         // 4. L-infinity test of this CTA's unassigned points against the representative
         const double *xb = X + (size_t)best * d;
-        for (int i = threadIdx.x; i < d; i += DD_THREADS) s_xb[i] = xb[i];
+        for (int i = threadIdx.x; i < d; i += DD_THREADS) {
+            s_xb[i] = xb[i];
+            s_xf[i] = f64_to_f32(xb[i]);
+        }
         __syncthreads();
         for (int w = w0 + wid; w < w1; w += DD_THREADS / 32) {
             if (assigned[w]) continue;
             const double *xw = X + (size_t)w * d;
             bool within = true;
-            for (int i0 = 0; i0 < d; i0 += 32) {
-                const int i = i0 + lane;
-                const bool far = i < d && fabs(xw[i] - s_xb[i]) > tau;
+            for (int i0 = 0; i0 < d; i0 += 128) {
+                // four slices in flight; the walk leaves at the first that holds a far coordinate
+                double v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int i = i0 + 32 * q + lane;
+                    v[q] = i < d ? xw[i] : 0.0;
+                }
+                bool far = false;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int i = i0 + 32 * q + lane;
+                    far = far || (i < d && dd_far(v[q], s_xb[i], s_xf[i], tau, tf));
+                }
                 if (__any_sync(0xffffffffu, far)) {
                     within = false;
                     break;
@@ -978,7 +994,7 @@ __global__ void __launch_bounds__(1024) k_laplace_final(int d, const double *XC,
 void launch_dedup(int n, int d, const double *X, const double *ell, const int8_t *status, const uint8_t *keep,
                   double tau_scale, const double *wmax, int cap, int32_t *reps, int32_t *n_reps, uint8_t *assigned,
                   const DedupScratch &sc, cudaStream_t s) {
-    // one CTA per 128 points up to one per SM (kept small so that concurrent
+    // one CTA per 32 points up to one per SM (kept small so that concurrent
     // solves on other streams can still be co-resident)
     static const int sms = [] {  // thread-safe one-time query (batched solves use several host threads)
         int dev = 0, n = 0;
@@ -986,7 +1002,7 @@ void launch_dedup(int n, int d, const double *X, const double *ell, const int8_t
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         return n > 0 ? n : 1;
     }();
-    int G = (n + 127) / 128;
+    int G = (n + 31) / 32;
     if (G > sms) G = sms;
     if (G > kDedupMaxGrid) G = kDedupMaxGrid;
     if (G < 1) G = 1;
@@ -995,7 +1011,8 @@ void launch_dedup(int n, int d, const double *X, const double *ell, const int8_t
                     const_cast<double **>(&sc.part_l), const_cast<int32_t **>(&sc.part_i),
                     const_cast<uint32_t **>(&sc.bar), const_cast<int32_t **>(&sc.err)};
     note_launch();
-    cudaLaunchCooperativeKernel((const void *)k_dedup, dim3(G), dim3(DD_THREADS), args, sizeof(double) * d, s);
+    cudaLaunchCooperativeKernel((const void *)k_dedup, dim3(G), dim3(DD_THREADS), args,
+                                (sizeof(double) + sizeof(float)) * d, s);
 }
 
 void launch_gather_rows(int d, int cap, const double *X, const int32_t *idx, const int32_t *n_idx, double *out,
