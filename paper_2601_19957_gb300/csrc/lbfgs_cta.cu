@@ -39,23 +39,26 @@ namespace sb {
 
 namespace {
 
+// CT: threads per walker, eight coordinates each, so CT = 32, 64 and 128 serve d <= 256, 512
+// and 1024. A visit is a chain of phases whose length hardly depends on d, so what counts is
+// the walkers per SM: threads past d would only repeat the chain (with 128 threads for every
+// d a batch of 64 problems with d <= 512 took 234 ms, 186 with the width that fits d).
 template <int CT>
 struct Cfg {
     static constexpr int NW = CT / 32;            // warps per walker
-    static constexpr int VPT = kMaxD / (4 * CT);  // float4 groups per thread
-    static constexpr int MINB = 4;                // CTAs per SM
+    static constexpr int VPT = 2;                 // float4 groups per thread
+    static constexpr int MAXD = 4 * VPT * CT;     // largest d
+    static constexpr int MINB = 512 / CT;         // CTAs per SM (registers)
     // ring of the stored pairs: DB slots of PGB pairs (one 8-column tensor-core tile
-    // of s, y vectors), each stored row up to kMaxD bf16 coordinates plus 16 bytes:
+    // of s, y vectors), each stored row up to MAXD bf16 coordinates plus 16 bytes:
     // row r of a slot starts 16 r bytes further into the 128-byte bank window than
     // row 0, so the same 16-byte chunk of the 8 rows falls in 8 different bank groups
     static constexpr int PGB = 4;
     static constexpr int DB = 3;
-    static constexpr int ROW_B = kMaxD * 2 + 16;
+    static constexpr int ROW_B = MAXD * 2 + 16;
     static constexpr int SLOT_B = 2 * PGB * ROW_B;
     static constexpr int RING_B = DB * SLOT_B;
 };
-
-constexpr int kCT = 128;  // threads per walker used by the solver
 
 // Vector accesses need 16-byte aligned rows: d % 4 == 0 (rows start at multiples of d).
 __device__ __forceinline__ float4 ld4(const float *p, int i0, int d) {
@@ -394,8 +397,8 @@ __device__ __forceinline__ uint64_t new_mm(const Lay<CT> &L, float *myy, float *
 // it. Results in cw, ca and sh.gamma.
 template <int CT>
 __device__ __forceinline__ void solve_mm(Shared<CT> &sh, const Lay<CT> &L, int c, int cn, float *mri, int m, int head) {
-    const int G = c <= CT / 4 ? 4 : (c <= CT / 2 ? 2 : 1);  // threads per entry
-    const int i = (int)threadIdx.x / G, p = (int)threadIdx.x % G;
+    const int G = c <= 32 ? 4 : (c <= 64 ? 2 : 1);  // threads per entry (the same for every CT)
+    const int p = (int)threadIdx.x % G, E = CT / G;  // E entries at a time
     const int LD = L.ld;
     float *RI = L.RI();
     const float *YY = L.YY();
@@ -409,21 +412,23 @@ __device__ __forceinline__ void solve_mm(Shared<CT> &sh, const Lay<CT> &L, int c
     };
     if (cn >= 0) {
         const float dn = nr[cn];
-        float t = 0.f;
-        if (i < cn)
-            for (int k = i + p; k < cn; k += G) t += RI[i * LD + k] * nr[k];
-        t = gsum(t);
-        if (p == 0 && i <= cn) {
-            const float v = i == cn ? 1.f / dn : -t / dn;
-            RI[i * LD + cn] = v;
-            int si = head + i, sc = head + cn;
-            if (si >= m) si -= m;
-            if (sc >= m) sc -= m;
-            mri[(size_t)si * m + sc] = v;
+        for (int i = (int)threadIdx.x / G, b = 0; b <= cn; b += E, i += E) {
+            float t = 0.f;
+            if (i < cn)
+                for (int k = i + p; k < cn; k += G) t += RI[i * LD + k] * nr[k];
+            t = gsum(t);
+            if (p == 0 && i <= cn) {
+                const float v = i == cn ? 1.f / dn : -t / dn;
+                RI[i * LD + cn] = v;
+                int si = head + i, sc = head + cn;
+                if (si >= m) si -= m;
+                if (sc >= m) sc -= m;
+                mri[(size_t)si * m + sc] = v;
+            }
         }
         __syncthreads();
     }
-    {
+    for (int i = (int)threadIdx.x / G, b = 0; b < c; b += E, i += E) {
         float t = 0.f;
         if (i < c)
             for (int k = i + p; k < c; k += G) t += RI[i * LD + k] * u1[k];
@@ -433,7 +438,7 @@ __device__ __forceinline__ void solve_mm(Shared<CT> &sh, const Lay<CT> &L, int c
     __syncthreads();
     const float gam = dg[c - 1] / YY[(c - 1) * LD + (c - 1)];
     if (threadIdx.x == 0) sh.gamma = gam;
-    {
+    for (int i = (int)threadIdx.x / G, b = 0; b < c; b += E, i += E) {
         float t = 0.f;
         if (i < c)
             for (int j = p; j < c; j += G) t += YY[i * LD + j] * cw[j];
@@ -441,7 +446,7 @@ __device__ __forceinline__ void solve_mm(Shared<CT> &sh, const Lay<CT> &L, int c
         if (p == 0 && i < c) tv[i] = dg[i] * cw[i] + gam * t - gam * u2[i];
     }
     __syncthreads();
-    {
+    for (int i = (int)threadIdx.x / G, b = 0; b < c; b += E, i += E) {
         float t = 0.f;
         if (i < c)
             for (int k = p; k <= i; k += G) t += RI[k * LD + i] * tv[k];
@@ -1024,24 +1029,43 @@ void launch_lbfgs_compact_by_key(const LbfgsArgs<float> &a, int n, int64_t *n_ev
 
 bool lbfgs_compact_by_key_fits(int n) { return n >= 0 && n < (1 << kPackShift); }
 
-void launch_lbfgs_step_cta(const LbfgsArgs<float> &a, int n, float *MRI, float *MYY, int num_sms, cudaStream_t s) {
-    ProfScope prof(PROF_LBFGS_STEP, s);
+namespace {
+template <int CT, bool EVEN>
+void launch_step(const LbfgsArgs<float> &a, int n, float *MRI, float *MYY, int num_sms, cudaStream_t s) {
     const int count_bytes = prof_class_on(PROF_LBFGS_STEP) ? 1 : 0;
-    int grid = num_sms * Cfg<kCT>::MINB;
-    if (grid > n) grid = n > 0 ? n : 1;
-    const size_t dyn = (size_t)Cfg<kCT>::RING_B + sizeof(float) * mm_floats<kCT>(a.m);
+    const size_t dyn = (size_t)Cfg<CT>::RING_B + sizeof(float) * mm_floats<CT>(a.m);
     static std::once_flag once;  // batched solves launch from several host threads
     std::call_once(once, [] {
-        const size_t most = (size_t)Cfg<kCT>::RING_B + sizeof(float) * mm_floats<kCT>(kMaxM);
-        cudaFuncSetAttribute(k_lbfgs_cta<kCT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
-        cudaFuncSetAttribute(k_lbfgs_cta<kCT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        const size_t most = (size_t)Cfg<CT>::RING_B + sizeof(float) * mm_floats<CT>(kMaxM);
+        cudaFuncSetAttribute(k_lbfgs_cta<CT, EVEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     });
+    // as many CTAs as stay resident: each goes from walker to walker
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_lbfgs_cta<CT, EVEN>, CT, dyn) != cudaSuccess || per < 1)
+        per = 1;
+    int grid = num_sms * per;
+    if (grid > n) grid = n > 0 ? n : 1;
     note_launch();
+    k_lbfgs_cta<CT, EVEN><<<grid, CT, dyn, s>>>(a, MRI, MYY, count_bytes);
+}
+template <int CT>
+void launch_step_ct(const LbfgsArgs<float> &a, int n, float *MRI, float *MYY, int num_sms, cudaStream_t s) {
     // d a multiple of 8 (one whole 16-byte chunk per thread or none): no per-element bounds
-    if (a.d % (4 * Cfg<kCT>::VPT) == 0)
-        k_lbfgs_cta<kCT, true><<<grid, kCT, dyn, s>>>(a, MRI, MYY, count_bytes);
+    if (a.d % (4 * Cfg<CT>::VPT) == 0)
+        launch_step<CT, true>(a, n, MRI, MYY, num_sms, s);
     else
-        k_lbfgs_cta<kCT, false><<<grid, kCT, dyn, s>>>(a, MRI, MYY, count_bytes);
+        launch_step<CT, false>(a, n, MRI, MYY, num_sms, s);
+}
+}  // namespace
+
+void launch_lbfgs_step_cta(const LbfgsArgs<float> &a, int n, float *MRI, float *MYY, int num_sms, cudaStream_t s) {
+    ProfScope prof(PROF_LBFGS_STEP, s);
+    if (a.d <= Cfg<32>::MAXD)
+        launch_step_ct<32>(a, n, MRI, MYY, num_sms, s);
+    else if (a.d <= Cfg<64>::MAXD)
+        launch_step_ct<64>(a, n, MRI, MYY, num_sms, s);
+    else
+        launch_step_ct<128>(a, n, MRI, MYY, num_sms, s);
 }
 
 double lbfgs_bytes_take() {
