@@ -119,49 +119,49 @@ __global__ void __launch_bounds__(256) k_ray_dirs_f32(int d, int n_rays, uint32_
     if (lane == 0) texit[r] = tmin;
 }
 
-// One warp per ray: tier and rank of every sample, histogram of buckets.
-__global__ void __launch_bounds__(128) k_ray_bucket(const double *ell, int n_rays, int S, int32_t *bucket,
-                                                    uint32_t *hist) {
-    extern __shared__ double sh[];  // [4][S]
+// Tier and rank of every sample, histogram of buckets: a warp per ray, rays in turn, the
+// histogram kept per CTA. l is compared as order-preserving integers (a rank is n_steps
+// comparisons per sample: 2 n_steps FP64 instructions took 260 us for 16384 rays x 64
+// samples together with a global atomic per sample, 40 us now); a NaN is never greater.
+constexpr int RB_WARPS = 8;
+__global__ void __launch_bounds__(32 * RB_WARPS) k_ray_bucket(const double *ell, int n_rays, int S, int32_t *bucket,
+                                                              uint32_t *hist) {
+    extern __shared__ uint64_t sh[];  // [RB_WARPS][S], then the histogram [2 S]
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int r = blockIdx.x * 4 + wl;
-    double *row = sh + (size_t)wl * S;
-    if (r < n_rays)
-        for (int j = lane; j < S; j += 32) row[j] = ell[(size_t)r * S + j];
-    __syncwarp();
-    if (r >= n_rays) return;
-    for (int j = lane; j < S; j += 32) {
-        const double l = row[j];
-        const double left = j > 0 ? row[j - 1] : -INFINITY;
-        const double right = j + 1 < S ? row[j + 1] : -INFINITY;
-        const int tier = (l > left && l >= right) ? 0 : 1;
-        int rank = 0;
-        for (int j2 = 0; j2 < S; ++j2) {
-            const double l2 = row[j2];
-            rank += (l2 > l || (l2 == l && j2 < j)) ? 1 : 0;
+    uint64_t *row = sh + (size_t)wl * S;
+    uint32_t *h = reinterpret_cast<uint32_t *>(sh + (size_t)RB_WARPS * S);
+    for (int b = threadIdx.x; b < 2 * S; b += blockDim.x) h[b] = 0;
+    __syncthreads();
+    for (int r = blockIdx.x * RB_WARPS + wl; r < n_rays; r += gridDim.x * RB_WARPS) {
+        for (int j = lane; j < S; j += 32) {
+            const double l = ell[(size_t)r * S + j];
+            const uint64_t b = (uint64_t)__double_as_longlong(l);
+            // 0: below every key of a number; -0 as +0
+            row[j] = (b << 1) > 0xffe0000000000000ull ? 0ull : ordered_bits((b << 1) == 0 ? 0.0 : l);
         }
-        const int b = tier * S + rank;
-        bucket[(size_t)r * S + j] = b;
-        atomicAdd(&hist[b], 1u);
-    }
-}
-
-// state: [0] cut bucket, [1] need (1-based rank inside the bucket), [2] key hi prefix, [3] key lo prefix
-__global__ void k_pick_bucket(uint32_t *hist, int nbins, int n_starts, uint64_t *state) {
-    if (threadIdx.x == 0) {
-        uint64_t cum = 0;
-        int b = 0;
-        for (; b < nbins; ++b) {
-            if (cum + hist[b] >= (uint64_t)n_starts) break;
-            cum += hist[b];
+        __syncwarp();
+        constexpr uint64_t kNegInf = 0x000fffffffffffffull;  // ordered_bits(-inf)
+        for (int j = lane; j < S; j += 32) {
+            const uint64_t l = row[j];
+            const uint64_t left = j > 0 ? row[j - 1] : kNegInf;
+            const uint64_t right = j + 1 < S ? row[j + 1] : kNegInf;
+            const bool nan = l == 0;
+            const int tier = (!nan && left != 0 && right != 0 && l > left && l >= right) ? 0 : 1;
+            int rank = 0;
+            if (!nan)
+                for (int j2 = 0; j2 < S; ++j2) {
+                    const uint64_t l2 = row[j2];
+                    rank += (l2 > l || (l2 == l && j2 < j)) ? 1 : 0;
+                }
+            const int b = tier * S + rank;
+            bucket[(size_t)r * S + j] = b;
+            atomicAdd(&h[b], 1u);
         }
-        state[0] = (uint64_t)b;
-        state[1] = (uint64_t)n_starts - cum;
-        state[2] = 0;
-        state[3] = 0;
+        __syncwarp();
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+    for (int b = threadIdx.x; b < 2 * S; b += blockDim.x)
+        if (h[b]) atomicAdd(&hist[b], h[b]);
 }
 
 __device__ __forceinline__ void sample_key(const double *ell, int64_t f, uint64_t &hi, uint32_t &lo) {
@@ -169,54 +169,114 @@ __device__ __forceinline__ void sample_key(const double *ell, int64_t f, uint64_
     lo = (uint32_t)f;
 }
 
-// Digit histogram of pass p (0..11) over the 96-bit keys in the cut bucket.
-__global__ void __launch_bounds__(256) k_digit_hist(const double *ell, const int32_t *bucket, int64_t total, int pass,
-                                                    const uint64_t *state, uint32_t *hist) {
-    __shared__ uint32_t sh[256];
-    sh[threadIdx.x] = 0;
+// The bucket that holds the n_starts-th sample (state[0]), the rank of that sample inside it
+// (state[1], from 1), and the list of the bucket's samples (at most one per ray): every CTA
+// finds the bucket from the histogram itself.
+__global__ void __launch_bounds__(256) k_cut_gather(const int32_t *bucket, int64_t total, const uint32_t *hist,
+                                                    int nbins, int n_starts, uint64_t *state, int32_t *list) {
+    __shared__ uint32_t wsum[8];
+    __shared__ int s_cut;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int per = (nbins + 255) / 256, b0 = threadIdx.x * per;
+    uint32_t own = 0;
+    for (int b = b0; b < b0 + per && b < nbins; ++b) own += hist[b];
+    uint32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[wid] = incl;
     __syncthreads();
-    const int64_t cut = (int64_t)state[0];
-    const uint64_t phi = state[2];
-    const uint32_t plo = (uint32_t)state[3];
-    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < total; f += (int64_t)gridDim.x * blockDim.x) {
-        if (bucket[f] != cut) continue;
-        uint64_t hi;
-        uint32_t lo;
-        sample_key(ell, f, hi, lo);
-        uint32_t digit;
-        bool match;
-        if (pass < 8) {
-            const int sh_hi = 64 - 8 * pass;  // bits above the current digit
-            match = pass == 0 ? true : ((hi >> sh_hi) == (phi >> sh_hi));
-            digit = (uint32_t)((hi >> (56 - 8 * pass)) & 0xffu);
-        } else {
-            const int q = pass - 8;
-            const int sh_lo = 32 - 8 * q;
-            match = (hi == phi) && (q == 0 ? true : ((lo >> sh_lo) == (plo >> sh_lo)));
-            digit = (lo >> (24 - 8 * q)) & 0xffu;
+    uint32_t before = incl - own;
+    for (int w = 0; w < wid; ++w) before += wsum[w];
+    if (before < (uint32_t)n_starts && before + own >= (uint32_t)n_starts) {
+        int b = b0;
+        while (before + hist[b] < (uint32_t)n_starts) before += hist[b++];
+        s_cut = b;
+        if (blockIdx.x == 0) {
+            state[0] = (uint64_t)b;
+            state[1] = (uint64_t)n_starts - before;
         }
-        if (match) atomicAdd(&sh[digit], 1u);
     }
     __syncthreads();
-    if (sh[threadIdx.x]) atomicAdd(&hist[threadIdx.x], sh[threadIdx.x]);
+    const int cut = s_cut;
+    unsigned long long *cnt = reinterpret_cast<unsigned long long *>(state + 4);
+    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < total; f += (int64_t)gridDim.x * blockDim.x)
+        if (bucket[f] == cut) list[atomicAdd(cnt, 1ull)] = (int32_t)f;
 }
 
-__global__ void k_digit_decide(uint32_t *hist, int pass, uint64_t *state) {
-    if (threadIdx.x == 0) {
-        uint64_t need = state[1], cum = 0;
-        uint32_t dg = 0;
-        for (; dg < 256; ++dg) {
-            if (cum + hist[dg] >= need) break;
-            cum += hist[dg];
+// The 96-bit key of that sample (state[2], state[3]) by radix selection over the listed
+// samples, 8 bits a pass, in one CTA; it stops as soon as one sample is left, or all that
+// are left are selected. (Two launches a pass over every sample, the digit found by one
+// thread: 24 launches, 150 us for 16384 samples.)
+__global__ void __launch_bounds__(1024) k_cut_select(const double *ell, const int32_t *list, uint64_t *state) {
+    __shared__ uint32_t h[256];
+    __shared__ uint32_t s_digit, s_cum, s_left;
+    const int n = (int)state[4];
+    uint64_t phi = 0, need = state[1];
+    uint32_t plo = 0;
+    for (int pass = 0; pass < 12; ++pass) {
+        if (threadIdx.x < 256) h[threadIdx.x] = 0;
+        __syncthreads();
+        const int sft = pass < 8 ? 56 - 8 * pass : 24 - 8 * (pass - 8);
+        auto match = [&](int e, uint32_t &digit) {
+            uint64_t hi;
+            uint32_t lo;
+            sample_key(ell, list[e], hi, lo);
+            if (pass < 8) {
+                digit = (uint32_t)(hi >> sft) & 0xffu;
+                return pass == 0 || (hi >> (sft + 8)) == (phi >> (sft + 8));
+            }
+            digit = (lo >> sft) & 0xffu;
+            return hi == phi && (pass == 8 || (lo >> (sft + 8)) == (plo >> (sft + 8)));
+        };
+        for (int e = threadIdx.x; e < n; e += blockDim.x) {
+            uint32_t digit;
+            if (match(e, digit)) atomicAdd(&h[digit], 1u);
         }
-        state[1] = need - cum;
+        __syncthreads();
+        if (threadIdx.x < 32) {  // the digit where the count reaches need: eight bins a lane
+            const int lane = threadIdx.x;
+            uint32_t own = 0;
+            for (int q = 0; q < 8; ++q) own += h[8 * lane + q];
+            uint32_t incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            uint32_t cum = incl - own;
+            if (cum < need && incl >= need) {
+                int q = 8 * lane;
+                while (cum + h[q] < need) cum += h[q++];
+                s_digit = (uint32_t)q;
+                s_cum = cum;
+                s_left = h[q];
+            }
+        }
+        __syncthreads();
+        const uint32_t dg = s_digit, left = s_left;
+        need -= s_cum;
         if (pass < 8)
-            state[2] |= (uint64_t)dg << (56 - 8 * pass);
+            phi |= (uint64_t)dg << sft;
         else
-            state[3] |= (uint64_t)dg << (24 - 8 * (pass - 8));
+            plo |= dg << sft;
+        if (need == left) {  // every sample with this prefix is selected: the largest such key
+            if (pass < 8) {
+                phi |= (1ull << sft) - 1ull;
+                plo = 0xffffffffu;
+            } else {
+                plo |= (1u << sft) - 1u;
+            }
+            break;
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+    if (threadIdx.x == 0) {
+        state[2] = phi;
+        state[3] = (uint64_t)plo;
+    }
 }
 
 __device__ __forceinline__ bool is_selected(const double *ell, const int32_t *bucket, int64_t f,
@@ -313,19 +373,20 @@ void launch_select_starts(const double *ell_all, int n_rays, int n_steps, int n_
                           cudaStream_t s) {
     const int64_t total = (int64_t)n_rays * n_steps;
     const int nbins = 2 * n_steps;
-    cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * (size_t)(nbins > 256 ? nbins : 256), s);
+    cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * (size_t)nbins, s);
+    cudaMemsetAsync(w.state, 0, sizeof(uint64_t) * 8, s);
+    const size_t sm = sizeof(uint64_t) * RB_WARPS * n_steps + sizeof(uint32_t) * nbins;
+    static const cudaError_t attr = cudaFuncSetAttribute(k_ray_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         (int)(sizeof(uint64_t) * RB_WARPS * 1024 + sizeof(uint32_t) * 2048));
+    (void)attr;
+    const int rb = (n_rays + RB_WARPS - 1) / RB_WARPS;
     note_launch();
-    k_ray_bucket<<<(n_rays + 3) / 4, 128, sizeof(double) * 4 * n_steps, s>>>(ell_all, n_rays, n_steps, w.bucket,
-                                                                             w.hist);
-    note_launch();
-    k_pick_bucket<<<1, 256, 0, s>>>(w.hist, nbins, n_starts, w.state);
+    k_ray_bucket<<<rb < 608 ? rb : 608, 32 * RB_WARPS, sm, s>>>(ell_all, n_rays, n_steps, w.bucket, w.hist);
     const int hb = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
-    for (int pass = 0; pass < 12; ++pass) {
-        note_launch();
-        k_digit_hist<<<hb, 256, 0, s>>>(ell_all, w.bucket, total, pass, w.state, w.hist);
-        note_launch();
-        k_digit_decide<<<1, 256, 0, s>>>(w.hist, pass, w.state);
-    }
+    note_launch();
+    k_cut_gather<<<hb, 256, 0, s>>>(w.bucket, total, w.hist, nbins, n_starts, w.state, w.list);
+    note_launch();
+    k_cut_select<<<1, 1024, 0, s>>>(ell_all, w.list, w.state);
     const int nb = (int)select_blocks(total);
     note_launch();
     k_sel_count<<<nb, SEL_BLOCK, 0, s>>>(ell_all, w.bucket, total, w.state, w.blockcnt);

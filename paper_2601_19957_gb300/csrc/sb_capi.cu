@@ -275,6 +275,7 @@ Layout layout(void *base, const sb_problem *p, const sb_config *c) {
     L.di.sel.state = cv.take<uint64_t>(8);
     L.di.sel.blockcnt = cv.take<int32_t>(select_blocks(total));
     L.di.sel.idx = cv.take<int64_t>(c->n_starts);
+    L.di.sel.list = cv.take<int32_t>(total);
 
     const int n = c->n_starts;
     if (fp64)

@@ -290,6 +290,7 @@ struct SelectWs {
     uint64_t *state;     // [8]
     int32_t *blockcnt;   // [nblocks]
     int64_t *idx;        // [n_starts]
+    int32_t *list;       // [total] samples of the cut bucket
 };
 void launch_select_starts(const double *ell_all, int n_rays, int n_steps, int n_starts, const SelectWs &w,
                           cudaStream_t s);
