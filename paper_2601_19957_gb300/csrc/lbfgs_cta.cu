@@ -1008,6 +1008,64 @@ __global__ void __launch_bounds__(kCkThreads) k_compact_place(int32_t *act, int3
     }
 }
 
+// The same for a list that one CTA holds in registers (kCkThreads kCompactE entries), in one
+// launch: a short round is bound by the rate at which its kernels start.
+__global__ void __launch_bounds__(kCkThreads) k_compact_one(const WalkerState<float> *st, int32_t *act, int32_t *n_act,
+                                                            int64_t *n_evals, const int32_t *key, int K) {
+    constexpr int NW = kCkThreads / 32;
+    __shared__ int wtot[NW][kSortBuckets], start[kSortBuckets + 1];
+    const int prev = *n_act, nb = K + 1;
+    const int E = compact_E(prev, 1);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int s0 = (int)threadIdx.x * E;
+    int w[kCompactE];
+    uint32_t pk[kCompactE];
+#pragma unroll
+    for (int e = 0; e < kCompactE; ++e) w[e] = (e < E && s0 + e < prev) ? act[s0 + e] : -1;
+#pragma unroll
+    for (int e = 0; e < kCompactE; ++e) {
+        const bool run = w[e] >= 0 && st[w[e]].status == SB_WALKER_RUNNING;
+        const int k = w[e] >= 0 ? key[w[e]] : -1;
+        const int b = (k >= 0 && k < K) ? k : K;
+        pk[e] = run ? ((uint32_t)b << kPackShift) | (uint32_t)w[e] : kPackDrop;
+    }
+    for (int b = lane; b < nb; b += 32) wtot[wid][b] = 0;
+    __syncwarp();
+    const uint64_t wpres = warp_buckets(pk, E, nb);
+    for (uint64_t m = wpres; m; m &= m - 1) {
+        const int b = __ffsll((long long)m) - 1;
+        const int sum = __reduce_add_sync(0xffffffffu, count_bucket(pk, E, b));
+        if (lane == 0) wtot[wid][b] = sum;
+    }
+    __syncthreads();  // every entry is read before any is written
+    if (wid == 0) {
+        int carry = 0;
+        for (int b0 = 0; b0 < nb; b0 += 32) {
+            const int b = b0 + lane;
+            int tot = 0;
+            if (b < nb)
+                for (int q = 0; q < NW; ++q) tot += wtot[q][b];
+            const int incl = warp_incl_scan(tot);
+            if (b < nb) start[b] = carry + incl - tot;
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) {
+            *n_act = carry;
+            if (n_evals) *n_evals += prev;
+        }
+    }
+    __syncthreads();
+    for (uint64_t m = wpres; m; m &= m - 1) {
+        const int b = __ffsll((long long)m) - 1;
+        const int n_b = count_bucket(pk, E, b);
+        int pos = start[b] + warp_incl_scan(n_b) - n_b;
+        for (int q = 0; q < wid; ++q) pos += wtot[q][b];
+#pragma unroll
+        for (int e = 0; e < kCompactE; ++e)
+            if (e < E && (pk[e] >> kPackShift) == (uint32_t)b) act[pos++] = (int32_t)(pk[e] & ((1u << kPackShift) - 1u));
+    }
+}
+
 }  // namespace
 
 int lbfgs_compact_blocks(int n) {
@@ -1020,6 +1078,11 @@ size_t lbfgs_compact_cnt_elems(int n) { return (size_t)lbfgs_compact_blocks(n) *
 
 void launch_lbfgs_compact_by_key(const LbfgsArgs<float> &a, int n, int64_t *n_evals, const int32_t *key, int K,
                                  int32_t *tmp, int32_t *cnt, cudaStream_t s) {
+    if (n <= kCkThreads * kCompactE) {
+        note_launch();
+        k_compact_one<<<1, kCkThreads, 0, s>>>(a.st, a.act, a.n_act, n_evals, key, K);
+        return;
+    }
     const int G = lbfgs_compact_blocks(n);
     note_launch();
     k_compact_count<<<G, kCkThreads, 0, s>>>(a.st, a.act, a.n_act, key, K, reinterpret_cast<uint32_t *>(tmp), cnt);
