@@ -20,6 +20,13 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, int64_t *round, int pe
     cudaGraphSetConditional(h, (active && r < cap) ? 1u : 0u);
 }
 
+__global__ void k_newton_cond(cudaGraphConditionalHandle h, const int32_t *n_eff, int32_t *step, int max_steps) {
+    if (threadIdx.x != 0) return;
+    const int s = *step + 1;
+    *step = s;
+    cudaGraphSetConditional(h, (*n_eff > 0 && s < max_steps) ? 1u : 0u);
+}
+
 // Streams of this host thread, one per device: bodies of conditional nodes, and the
 // library's own captures of calls made outside a capture.
 cudaStream_t thread_stream(int which) {
@@ -121,6 +128,12 @@ void launch_loop_cond(cudaGraphConditionalHandle h, int64_t *round, int per_batc
                       const int32_t *n_act, int32_t *err, cudaStream_t s) {
     note_launch();
     k_loop_cond<<<1, 32, 0, s>>>(h, round, per_batch, cap_rounds, n_act, err);
+}
+
+void launch_newton_cond(cudaGraphConditionalHandle h, const int32_t *n_eff, int32_t *step, int max_steps,
+                        cudaStream_t s) {
+    note_launch();
+    k_newton_cond<<<1, 32, 0, s>>>(h, n_eff, step, max_steps);
 }
 
 }  // namespace sb

@@ -187,6 +187,7 @@ struct LaplaceWs {
     int32_t *n_live;           // candidates still moving in a Newton step
     int32_t *onehot;           // [cap] component k when a candidate's responsibilities are one-hot, else -1
     int32_t *n_eff;            // candidates a Newton step's evaluations run on (0 once none moves)
+    int32_t *step;             // Newton steps taken (graph mode's loop)
 };
 
 struct EvidenceWs {
@@ -299,6 +300,7 @@ Layout layout(void *base, const sb_problem *p, const sb_config *c) {
     la.n_live = cv.take<int32_t>(1);
     la.onehot = cv.take<int32_t>(cap);
     la.n_eff = cv.take<int32_t>(1);
+    la.step = cv.take<int32_t>(1);
     la.XC = cv.take<double>((size_t)cap * d);
     la.LC = cv.take<double>(cap);
     la.GC = cv.take<double>((size_t)cap * d);
@@ -554,33 +556,51 @@ sb_status run_laplace(const ProbView &pv, const sb_config *c, const Layout &L, c
     // stage can sit in a captured graph.
     SB_CUDA_TRY(cudaMemsetAsync(la.active, 1, cap, s));
     // l, grad l, H and its Cholesky factor at every candidate (of the first *nc)
-    auto eval_full = [&](const int32_t *nc) {
-        f64_points(pv, la.XC, nullptr, nc, cap, la.qpart, la.Z, la.R, la.LC, la.GC, s);
-        launch_onehot(K, la.R, nc, cap, la.onehot, s);
-        launch_precision_needed(d, K, pv.L, la.R, nc, la.p_done, la.p_need, la.P, s, la.onehot);
-        launch_hessian_chol(d, K, cap, pv.L, la.P, la.Z, la.R, la.GC, nc, la.GK, la.H, la.info, la.dd_bar, pv.status, s,
-                            la.onehot);
+    auto eval_full = [&](const int32_t *nc, cudaStream_t es) {
+        f64_points(pv, la.XC, nullptr, nc, cap, la.qpart, la.Z, la.R, la.LC, la.GC, es);
+        launch_onehot(K, la.R, nc, cap, la.onehot, es);
+        launch_precision_needed(d, K, pv.L, la.R, nc, la.p_done, la.p_need, la.P, es, la.onehot);
+        launch_hessian_chol(d, K, cap, pv.L, la.P, la.Z, la.R, la.GC, nc, la.GK, la.H, la.info, la.dd_bar, pv.status,
+                            es, la.onehot);
     };
-    eval_full(la.n_reps);
+    eval_full(la.n_reps, s);
     // Newton polish, newton_steps steps; a step's evaluations run on n_eff candidates,
     // which drops to zero once no candidate's Newton step is above the convergence
     // threshold (the rest of the polish is then empty launches)
     launch_set_eff(la.n_eff, la.n_reps, nullptr, s);
-    for (int step = 0; step < c->newton_steps; ++step) {
+    auto newton_step = [&](cudaStream_t ns) -> sb_status {
         launch_chol_solve_coop(d, cap, la.H, la.GC, la.n_eff, la.info, la.active, la.delta, la.pred, la.dd_bar,
-                               pv.status, s);
-        SB_CUDA_TRY(cudaMemsetAsync(la.n_live, 0, sizeof(int32_t), s));
+                               pv.status, ns);
+        SB_CUDA_TRY(cudaMemsetAsync(la.n_live, 0, sizeof(int32_t), ns));
         launch_newton_ls(d, cap, 0, la.n_eff, la.info, la.active, la.searching, la.halvings, la.t, la.XC, la.LC,
-                         la.delta, la.XN, la.LN, la.pred, la.n_live, s);
-        launch_set_eff(la.n_eff, la.n_reps, la.n_live, s);
-        f64_points(pv, la.XN, nullptr, la.n_eff, cap, la.qpart, nullptr, nullptr, la.LN, nullptr, s);
+                         la.delta, la.XN, la.LN, la.pred, la.n_live, ns);
+        launch_set_eff(la.n_eff, la.n_reps, la.n_live, ns);
+        f64_points(pv, la.XN, nullptr, la.n_eff, cap, la.qpart, nullptr, nullptr, la.LN, nullptr, ns);
         launch_newton_ls(d, cap, 1, la.n_eff, la.info, la.active, la.searching, la.halvings, la.t, la.XC, la.LC,
-                         la.delta, la.XN, la.LN, la.pred, la.n_live, s);
-        launch_ls_batch_setup(d, cap, la.n_eff, la.searching, la.XC, la.delta, la.XN2, la.rows2, la.n_rows2, s);
+                         la.delta, la.XN, la.LN, la.pred, la.n_live, ns);
+        launch_ls_batch_setup(d, cap, la.n_eff, la.searching, la.XC, la.delta, la.XN2, la.rows2, la.n_rows2, ns);
         f64_points(pv, la.XN2, la.rows2, la.n_rows2, cap * (kHalvings - 1), la.qpart2, nullptr, nullptr, la.LN2,
-                   nullptr, s);
-        launch_ls_batch_decide(d, cap, la.n_eff, la.searching, la.active, la.XC, la.LC, la.XN2, la.LN2, s);
-        eval_full(la.n_eff);
+                   nullptr, ns);
+        launch_ls_batch_decide(d, cap, la.n_eff, la.searching, la.active, la.XC, la.LC, la.XN2, la.LN2, ns);
+        eval_full(la.n_eff, ns);
+        return SB_OK;
+    };
+    if (stream_capturing(s) && c->newton_steps > 1) {
+        // in a graph, a WHILE node ends the polish after the step in which no candidate
+        // moved, instead of launching the remaining steps empty (24 launches each)
+        SB_CUDA_TRY(cudaMemsetAsync(la.step, 0, sizeof(int32_t), s));
+        const sb_status st = capture_while(s, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
+            const sb_status r = newton_step(bs);
+            if (r != SB_OK) return r;
+            launch_newton_cond(h, la.n_eff, la.step, c->newton_steps, bs);
+            return cudaGetLastError() == cudaSuccess ? SB_OK : SB_ERR_CUDA;
+        });
+        if (st != SB_OK) return st;
+    } else {
+        for (int step = 0; step < c->newton_steps; ++step) {
+            const sb_status st = newton_step(s);
+            if (st != SB_OK) return st;
+        }
     }
     SB_CUDA_TRY(cudaMemsetAsync(la.keep, 0, cap, s));
     launch_cand_stats(d, cap, la.XC, la.LC, la.GC, la.H, la.info, pv.lo, pv.hi, c->eps_grad, la.n_reps, la.keep,

@@ -116,4 +116,9 @@ sb_status run_graph_or_direct(cudaStream_t s, const GraphKey &key, F enqueue) {
 void launch_loop_cond(cudaGraphConditionalHandle h, int64_t *round, int per_batch, int64_t cap_rounds,
                       const int32_t *n_act, int32_t *err, cudaStream_t s);
 
+// Sets the WHILE condition of the Newton polish: another step while some candidate moved
+// (*n_eff > 0) and fewer than max_steps were taken (*step counts them).
+void launch_newton_cond(cudaGraphConditionalHandle h, const int32_t *n_eff, int32_t *step, int max_steps,
+                        cudaStream_t s);
+
 }  // namespace sb
