@@ -33,7 +33,9 @@
 // exactly 0) H = P_k and C = L_k, so W L_k = L_k^-T: tr(W P_k) = d and lower[W L_k] =
 // diag(1 / L_ii), with no GEMM. Products with P_k are formed as L_k (L_k^T v); P_k itself
 // is built only for the Hessian of a mode that is not one-hot. Nothing is read back to
-// the host: every skip is decided from R and the one-hot flag on the device.
+// the host: every skip is decided from R and the one-hot flag on the device. Modes go
+// through the kernels in groups (adj_group), since one mode's factor, inverse and vector
+// steps leave most of the chip idle; their shares are added to dmu and dL in mode order.
 //
 // The bound is the FP64 pipe (one warp instruction per 19 cycles and SM): per mode K d^3 /
 // 3 fused multiply-adds in the two GEMMs, d^3 / 6 each in the factor and its inverse.
@@ -86,6 +88,8 @@ __global__ void __launch_bounds__(256) k_inv_diag(int d, const double *C, double
     __shared__ double Cs[TB][TB + 1];
     __shared__ double inv[TB];
     const int r0 = blockIdx.x * TB;
+    C += (size_t)blockIdx.y * d * d;  // mode
+    Ci += (size_t)blockIdx.y * d * d;
     for (int e = threadIdx.x; e < TB * TB; e += 256) {
         const int i = r0 + e / TB, j = r0 + e % TB;
         Cs[e / TB][e % TB] = i < d && j <= i ? C[(size_t)i * d + j] : (i == j ? 1.0 : 0.0);
@@ -114,11 +118,15 @@ __global__ void __launch_bounds__(256) k_inv_diag(int d, const double *C, double
 }
 
 // One level of the merge [A 0; B D]^-1 = [A^-1 0; -D^-1 B A^-1, D^-1] for every pair of
-// blocks of s rows (blockIdx.z): pass 0 T = B A^-1, pass 1 Ci = -D^-1 T.
+// blocks of s rows and mode (blockIdx.z): pass 0 T = B A^-1, pass 1 Ci = -D^-1 T.
 template <int PASS>
 __global__ void __launch_bounds__(256) k_inv_merge(int d, int s, const double *C, double *Ci, double *T) {
     __shared__ TileBuf sm;
-    const int p0 = blockIdx.z * 2 * s, q0 = p0 + s;  // first rows of the A and the D block
+    const int pairs = (d + 2 * s - 1) / (2 * s), mo = blockIdx.z / pairs;
+    C += (size_t)mo * d * d;
+    Ci += (size_t)mo * d * d;
+    T += (size_t)mo * d * d;
+    const int p0 = (blockIdx.z % pairs) * 2 * s, q0 = p0 + s;  // first rows of the A and the D block
     const int i0 = q0 + blockIdx.y * TB, j0 = p0 + blockIdx.x * TB;
     if (i0 >= d) return;
     double acc[2][2] = {};
@@ -142,12 +150,12 @@ __global__ void __launch_bounds__(256) k_inv_merge(int d, int s, const double *C
         }
 }
 
-void launch_tri_inverse(int d, const double *C, double *Ci, double *T, cudaStream_t st) {
+void launch_tri_inverse(int d, int nm, const double *C, double *Ci, double *T, cudaStream_t st) {
     note_launch();
-    k_inv_diag<<<(d + TB - 1) / TB, 256, 0, st>>>(d, C, Ci);
+    k_inv_diag<<<dim3((d + TB - 1) / TB, nm), 256, 0, st>>>(d, C, Ci);
     for (int s = TB; s < d; s *= 2) {
         const int pairs = (d + 2 * s - 1) / (2 * s);
-        const dim3 g(s / TB, s / TB, pairs);
+        const dim3 g(s / TB, s / TB, pairs * nm);
         note_launch();
         k_inv_merge<0><<<g, 256, 0, st>>>(d, s, C, Ci, T);
         note_launch();
@@ -176,8 +184,11 @@ __global__ void __launch_bounds__(256) k_adj_X(int d, const double *Ci, const do
                                                const int32_t *onehot, double *X, double *trp) {
     __shared__ TileBuf sm;
     __shared__ double sh[8];
-    const int k = blockIdx.y;
-    if (!needs_product(R, onehot, k)) return;
+    const int k = blockIdx.y, mo = blockIdx.z, K = gridDim.y;
+    if (!needs_product(R + (size_t)mo * K, onehot + mo, k)) return;
+    Ci += (size_t)mo * d * d;
+    X += (size_t)mo * K * d * d;
+    trp += (size_t)mo * K * gridDim.x;
     int I, J;
     tile_from(blockIdx.x, (d + TB - 1) / TB, I, J);
     const int i0 = I * TB, j0 = J * TB;
@@ -213,88 +224,135 @@ __global__ void __launch_bounds__(256) k_adj_X(int d, const double *Ci, const do
 // dL_k += pi lower[ eps (diag(1/L) - delta z^T) - gam z^T - delta u^T - r W L_k ] with u =
 // L^T gam and the tile of W L_k = C^-T X_k formed here (at a one-hot mode lower[W L_k] =
 // diag(1 / L_ii)).
-__global__ void __launch_bounds__(256) k_adj_dL(int d, const double *pi, const double *R, const double *eps,
+__global__ void __launch_bounds__(256) k_adj_dL(int d, int nm, const double *pi, const double *R, const double *eps,
                                                 const int32_t *onehot, const double *L, const double *x,
                                                 const double *mu, const double *Z, const double *gam,
                                                 const double *U, const double *Ci, const double *X, double *dL) {
     __shared__ TileBuf sm;
-    const int k = blockIdx.y;
-    const double rk = R[k];
-    if (rk == 0.0) return;
+    const int k = blockIdx.y, K = gridDim.y;
     int I, J;
-    tile_from(blockIdx.x, (d + TB - 1) / TB, I, J);
+    tile_from(gridDim.x - 1 - blockIdx.x, (d + TB - 1) / TB, I, J);  // here the top rows are the longest
     const int i0 = I * TB, j0 = J * TB;
-    const double *Lk = L + (size_t)k * d * d, *Xk = X + (size_t)k * d * d;
-    const bool oh = onehot[0] >= 0;
-    double acc[2][2] = {};
-    if (!oh)
-        tile_gemm(
-            sm, i0, d, acc,
-            [&](int r, int l) { return l < d && i0 + r <= l ? Ci[(size_t)l * d + i0 + r] : 0.0; },
-            [&](int l, int c) { return l < d && j0 + c < d ? Xk[(size_t)l * d + j0 + c] : 0.0; });
+    const double *Lk = L + (size_t)k * d * d;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const double p = pi[0], ek = eps[k];
+    double sum[2][2];
 #pragma unroll
     for (int r = 0; r < 2; ++r)
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
-            if (i >= d || j > i) continue;
-            const size_t e = (size_t)i * d + j, kd = (size_t)k * d;
-            const double di = x[i] - mu[kd + i], zj = Z[kd + j];
-            const double wl = oh ? (i == j ? 1.0 / Lk[e] : 0.0) : acc[r][c];
-            double v = -ek * di * zj - gam[kd + i] * zj - di * U[kd + j] - rk * wl;
-            if (i == j) v += ek / Lk[e];
-            dL[(size_t)k * d * d + e] += p * v;
+            sum[r][c] = i < d && j <= i ? dL[(size_t)k * d * d + (size_t)i * d + j] : 0.0;
+        }
+    for (int mo = 0; mo < nm; ++mo) {
+        const size_t mk = (size_t)mo * K + k, kd = mk * d;
+        const double rk = R[mk];
+        if (rk == 0.0) continue;
+        const double *Cm = Ci + (size_t)mo * d * d, *Xk = X + mk * d * d;
+        const bool oh = onehot[mo] >= 0;
+        double acc[2][2] = {};
+        if (!oh)
+            tile_gemm(
+                sm, i0, d, acc,
+                [&](int r, int l) { return l < d && i0 + r <= l ? Cm[(size_t)l * d + i0 + r] : 0.0; },
+                [&](int l, int c) { return l < d && j0 + c < d ? Xk[(size_t)l * d + j0 + c] : 0.0; });
+        const double p = pi[mo], ek = eps[mk];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+                if (i >= d || j > i) continue;
+                const size_t e = (size_t)i * d + j;
+                const double di = x[(size_t)mo * d + i] - mu[(size_t)k * d + i], zj = Z[kd + j];
+                const double wl = oh ? (i == j ? 1.0 / Lk[e] : 0.0) : acc[r][c];
+                double v = -ek * di * zj - gam[kd + i] * zj - di * U[kd + j] - rk * wl;
+                if (i == j) v += ek / Lk[e];
+                sum[r][c] += p * v;
+            }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+            if (i < d && j <= i) dL[(size_t)k * d * d + (size_t)i * d + j] = sum[r][c];
         }
 }
 
 // ------------------------------------------------------------------ per-mode vector algebra
-// Vectors are rows of [nv][d]. Rows of V: 0 .. K-1 = g_k (active only, else 0), K = gbar.
+// Vectors are rows of [mode][nv][d]. Rows of V: 0 .. K-1 = g_k (active only, else 0), K = gbar.
 __global__ void k_pack_rhs(int d, int K, const double *GK, const double *gbar, const double *R, double *V) {
-    const int c = blockIdx.y;
+    const int c = blockIdx.y, mo = blockIdx.z;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < d) V[(size_t)c * d + i] = c < K ? (R[c] != 0.0 ? GK[(size_t)c * d + i] : 0.0) : gbar[i];
+    if (i >= d) return;
+    double v = gbar[(size_t)mo * d + i];
+    if (c < K) v = R[(size_t)mo * K + c] != 0.0 ? GK[((size_t)mo * K + c) * d + i] : 0.0;
+    V[((size_t)mo * (K + 1) + c) * d + i] = v;
 }
 
-// y_c = T_c v_c for a lower triangular matrix T (T_c = T + c tstride), a warp per row.
-// R given: vectors c < K with R[c] == 0 are skipped.
-// dmu given: dmu_c += pi (-eps_c g_c + y_c) instead of storing y_c.
-__global__ void __launch_bounds__(256) k_adj_lower(int d, const double *T, size_t tstride, const double *V,
-                                                   const double *R, int K, double *Y, const double *pi,
-                                                   const double *eps, const double *GK, double *dmu) {
-    const int c = blockIdx.y;
-    if (R && c < K && R[c] == 0.0) return;
+// Where a vector kernel finds its operands: matrix T + mode tm + vector tc, vectors
+// V + mode vm + vector d (skipped where R[mode rm + c] == 0, c < K).
+struct VecArgs {
+    const double *T;
+    size_t tm, tc;
+    const double *V;
+    size_t vm;
+    const double *R;
+    int K;
+    double *Y;
+    size_t ym;
+};
+
+// y = T v for a lower triangular matrix, a warp per row; vector c = blockIdx.y, mode blockIdx.z.
+__global__ void __launch_bounds__(256) k_adj_lower(int d, VecArgs a) {
+    const int c = blockIdx.y, mo = blockIdx.z;
+    if (a.R && c < a.K && a.R[(size_t)mo * a.K + c] == 0.0) return;
     const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= d) return;
-    const double *row = T + c * tstride + (size_t)i * d, *v = V + (size_t)c * d;
+    const double *row = a.T + mo * a.tm + c * a.tc + (size_t)i * d, *v = a.V + mo * a.vm + (size_t)c * d;
     double s = 0.0;
 #pragma unroll 4
     for (int j = lane; j <= i; j += 32) s = fma(row[j], v[j], s);
     s = warp_sum(s);
-    if (lane != 0) return;
-    const size_t o = (size_t)c * d + i;
-    if (dmu)
-        dmu[o] += pi[0] * (-eps[c] * GK[o] + s);
-    else
-        Y[o] = s;
+    if (lane == 0) a.Y[mo * a.ym + (size_t)c * d + i] = s;
 }
 
-// y_c = T_c^T v_c (v_c = diff - v_c when diff is given): a CTA per 32 columns, a lane per column, the eight warps
-// over interleaved rows, partials summed in a fixed order.
-__global__ void __launch_bounds__(256) k_adj_upper(int d, const double *T, size_t tstride, const double *V,
-                                                   const double *diff, const double *R, int K, double *Y) {
+// dmu_k += pi (-eps_k g_k + y_k) with y_k = L_k u_k, the group's modes in turn: a warp per (i, k).
+__global__ void __launch_bounds__(256) k_adj_dmu(int d, int nm, const double *L, const double *U, const double *R,
+                                                 const double *pi, const double *eps, const double *GK, double *dmu) {
+    const int k = blockIdx.y, K = gridDim.y;
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= d) return;
+    const double *row = L + (size_t)k * d * d + (size_t)i * d;
+    double sum = dmu[(size_t)k * d + i];
+    for (int mo = 0; mo < nm; ++mo) {
+        const size_t mk = (size_t)mo * K + k;
+        if (R[mk] == 0.0) continue;
+        const double *v = U + mk * d;
+        double s = 0.0;
+#pragma unroll 4
+        for (int j = lane; j <= i; j += 32) s = fma(row[j], v[j], s);
+        s = warp_sum(s);
+        sum += pi[mo] * (-eps[mk] * GK[mk * d + i] + s);
+    }
+    if (lane == 0) dmu[(size_t)k * d + i] = sum;
+}
+
+// y = T^T v (diff: v = gbar row - v, the row K of the same mode): a CTA per 32 columns, a lane per column, the eight
+// warps over interleaved rows, partials summed in a fixed order.
+__global__ void __launch_bounds__(256) k_adj_upper(int d, VecArgs a, bool diff) {
     __shared__ double part[8][32];
-    const int c = blockIdx.y;
-    if (R && c < K && R[c] == 0.0) return;
+    const int c = blockIdx.y, mo = blockIdx.z;
+    if (a.R && c < a.K && a.R[(size_t)mo * a.K + c] == 0.0) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, j0 = blockIdx.x * 32, j = j0 + lane;
-    const double *Tc = T + c * tstride, *v = V + (size_t)c * d;
+    const double *Tc = a.T + mo * a.tm + c * a.tc, *v = a.V + mo * a.vm + (size_t)c * d;
+    const double *w = a.V + mo * a.vm + (size_t)a.K * d;
     double s = 0.0;
     if (j < d) {
 #pragma unroll 4
         for (int i = j0 + wid; i < d; i += 8) {
             const double t = i >= j ? Tc[(size_t)i * d + j] : 0.0;
-            s = fma(t, diff ? diff[i] - v[i] : v[i], s);
+            s = fma(t, diff ? w[i] - v[i] : v[i], s);
         }
     }
     part[wid][lane] = s;
@@ -302,12 +360,12 @@ __global__ void __launch_bounds__(256) k_adj_upper(int d, const double *T, size_
     if (wid == 0 && j < d) {
         double t = 0.0;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) t += part[w][lane];
-        Y[(size_t)c * d + j] = t;
+        for (int q = 0; q < 8; ++q) t += part[q][lane];
+        a.Y[mo * a.ym + (size_t)c * d + j] = t;
     }
 }
 
-// One CTA of 1024 threads: given WV (rows W g_0 .. W g_{K-1}, W gbar) and the partials of
+// One CTA of 1024 threads per mode: given WV (rows W g_0 .. W g_{K-1}, W gbar) and the partials of
 // tr(W P_k), form t (stage 0), or with Wt known form eps and gam (stage 1). A warp per
 // component for the inner products.
 __global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, int n_part, const double *R,
@@ -315,9 +373,23 @@ __global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, int
                                                     const double *WV, const double *trp, const double *PY,
                                                     const double *Wt, double *t_out, double *eps, double *gam) {
     __shared__ double s_beta[kMaxK];
+    const int mo = blockIdx.x;
+    R += (size_t)mo * K;
+    GK += (size_t)mo * K * d;
+    gbar += (size_t)mo * d;
+    WV += (size_t)mo * (K + 1) * d;
+    trp += (size_t)mo * K * n_part;
+    PY += (size_t)mo * K * d;
+    if (stage == 0) {
+        t_out += (size_t)mo * d;
+    } else {
+        Wt += (size_t)mo * d;
+        eps += (size_t)mo * K;
+        gam += (size_t)mo * K * d;
+    }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double *Wg = WV + (size_t)K * d;  // W gbar
-    const bool oh = onehot[0] >= 0;
+    const bool oh = onehot[mo] >= 0;
     for (int k = wid; k < K; k += 32) {
         double beta = 0.0;
         if (R[k] != 0.0) {
@@ -377,64 +449,77 @@ __global__ void k_softmax_pi(int n, const double *logZk, double g, double *pi) {
 
 }  // namespace
 
+// Modes a group holds: four matrices of each kind, fewer with many components (X_k).
+static int adj_group(int K) {
+    const int g = 32 / K;
+    return g < 1 ? 1 : (g > 4 ? 4 : g);
+}
+
 void adjoint_carve(Carver &cv, AdjWs &w, int d, int K) {
-    const int nJT = (d + 63) / 64, nt = (d + TB - 1) / TB;
-    w.P = cv.take<double>((size_t)K * d * d);
-    w.H = cv.take<double>((size_t)d * d);
-    w.Ci = cv.take<double>((size_t)d * d);
-    w.T2 = cv.take<double>((size_t)d * d);
-    w.X = cv.take<double>((size_t)K * d * d);
-    w.trp = cv.take<double>((size_t)K * nt * (nt + 1) / 2);
-    w.Z = cv.take<double>((size_t)K * d);
-    w.R = cv.take<double>((size_t)K);
-    w.qpart = cv.take<double>((size_t)K * nJT);
-    w.gbar = cv.take<double>(d);
-    w.ell = cv.take<double>(1);
-    w.GK = cv.take<double>((size_t)K * d);
-    w.V = cv.take<double>((size_t)d * (K + 1));
-    w.Y = cv.take<double>((size_t)d * (K + 1));
-    w.WV = cv.take<double>((size_t)d * (K + 1));
-    w.T = cv.take<double>(d);
-    w.eps = cv.take<double>(K);
-    w.gam = cv.take<double>((size_t)K * d);
-    w.U = cv.take<double>((size_t)K * d);
-    w.PY = cv.take<double>((size_t)K * d);
+    const size_t nJT = (d + 63) / 64, nt = (d + TB - 1) / TB, dd = (size_t)d * d, g = adj_group(K);
+    w.P = cv.take<double>(K * dd);
+    w.H = cv.take<double>(g * dd);
+    w.Ci = cv.take<double>(g * dd);
+    w.T2 = cv.take<double>(g * dd);
+    w.X = cv.take<double>(g * K * dd);
+    w.trp = cv.take<double>(g * K * nt * (nt + 1) / 2);
+    w.Z = cv.take<double>(g * K * d);
+    w.R = cv.take<double>(g * K);
+    w.qpart = cv.take<double>(g * K * nJT);
+    w.gbar = cv.take<double>(g * d);
+    w.ell = cv.take<double>(g);
+    w.GK = cv.take<double>(g * K * d);
+    w.V = cv.take<double>(g * d * (K + 1));
+    w.Y = cv.take<double>(g * d * (K + 1));
+    w.WV = cv.take<double>(g * d * (K + 1));
+    w.T = cv.take<double>(g * d);
+    w.eps = cv.take<double>(g * K);
+    w.gam = cv.take<double>(g * K * d);
+    w.U = cv.take<double>(g * K * d);
+    w.PY = cv.take<double>(g * K * d);
     w.pi = cv.take<double>(kMaxAdjModes);
-    w.info = cv.take<int32_t>(1);
-    w.one = cv.take<int32_t>(1);
-    w.onehot = cv.take<int32_t>(1);
+    w.info = cv.take<int32_t>(g);
+    w.count = cv.take<int32_t>(1);
+    w.onehot = cv.take<int32_t>(g);
     w.p_done = cv.take<int32_t>(kMaxK);
     w.p_need = cv.take<int32_t>(kMaxK);
     w.bar = cv.take<uint32_t>(2);
 }
 
-__global__ void k_set_one(int32_t *p) {
-    if (threadIdx.x == 0) *p = 1;
+__global__ void k_set_count(int32_t *p, int v) {
+    if (threadIdx.x == 0) *p = v;
 }
 
 sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, const double *logZk, int n_modes,
                       double grad_logZ, double *dmu, double *dL, cudaStream_t s) {
-    const int d = pv.d, K = pv.K;
+    const int d = pv.d, K = pv.K, group = adj_group(K);
     if (n_modes < 1 || n_modes > kMaxAdjModes) return SB_ERR_INVALID_ARG;
     SB_CUDA_TRY(cudaMemsetAsync(dmu, 0, sizeof(double) * K * d, s));
     SB_CUDA_TRY(cudaMemsetAsync(dL, 0, sizeof(double) * (size_t)K * d * d, s));
     SB_CUDA_TRY(cudaMemsetAsync(w.p_done, 0, sizeof(int32_t) * kMaxK, s));
     note_launch();
-    k_set_one<<<1, 32, 0, s>>>(w.one);
-    note_launch();
     k_softmax_pi<<<1, 32, 0, s>>>(n_modes, logZk, grad_logZ, w.pi);
     const int nt = (d + TB - 1) / TB, tiles = nt * (nt + 1) / 2;
     const unsigned rows8 = (unsigned)((d + 7) / 8), cols32 = (unsigned)((d + 31) / 32);
-    const size_t dd = (size_t)d * d;
-    // W v for the rows of V [nv][d] (rows c < nk with R[c] == 0 skipped: their V is zero and unread)
-    auto apply_W = [&](int nv, const double *V, double *out, const double *R, int nk) {
-        note_launch(2);
-        k_adj_lower<<<dim3(rows8, nv), 256, 0, s>>>(d, w.Ci, 0, V, R, nk, w.Y, nullptr, nullptr, nullptr, nullptr);
-        k_adj_upper<<<dim3(cols32, nv), 256, 0, s>>>(d, w.Ci, 0, w.Y, nullptr, R, nk, out);
-    };
-    for (int mo = 0; mo < n_modes; ++mo) {
-        const double *x = modes + (size_t)mo * d;
-        const double *pi = w.pi + mo;
+    const size_t dd = (size_t)d * d, dK = (size_t)d * K, dV = (size_t)d * (K + 1);
+    // unused shared memory holds an SM to two CTAs of the GEMMs, so that their tiles, up to
+    // nt times different in length, are dealt out as SMs come free (d = 512, K = 4: 390 us per
+    // mode with every tile resident at once, 206 so)
+    constexpr int kPad = 80 * 1024;
+    SB_CUDA_TRY(cudaFuncSetAttribute(k_adj_X, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad));
+    SB_CUDA_TRY(cudaFuncSetAttribute(k_adj_dL, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad));
+    for (int m0 = 0; m0 < n_modes; m0 += group) {
+        const int nm = n_modes - m0 < group ? n_modes - m0 : group;
+        const double *x = modes + (size_t)m0 * d;
+        const double *pi = w.pi + m0;
+        note_launch();
+        k_set_count<<<1, 32, 0, s>>>(w.count, nm);
+        // W v for the nv vectors per mode of V (stride vm; those with R == 0 skipped, zero and unread)
+        auto apply_W = [&](int nv, const double *V, size_t vm, double *out, size_t om, const double *R) {
+            note_launch(2);
+            k_adj_lower<<<dim3(rows8, nv, nm), 256, 0, s>>>(d, VecArgs{w.Ci, dd, 0, V, vm, R, K, w.Y, dV});
+            k_adj_upper<<<dim3(cols32, nv, nm), 256, 0, s>>>(d, VecArgs{w.Ci, dd, 0, w.Y, dV, R, K, out, om}, false);
+        };
         // l, grad l, z_k, r_k at x (FP64 likelihood kernels), then g_k, H and H = C C^T
         // (at a one-hot mode C = L_k is copied, as in the Laplace stage), C^-1
         LikF64Args la{};
@@ -444,7 +529,7 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
         la.L = pv.L;
         la.a = pv.a;
         la.X = x;
-        la.n_rows = 1;
+        la.n_rows = nm;
         la.qpart = w.qpart;
         la.Z = w.Z;
         la.R = w.R;
@@ -454,38 +539,38 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
         la.grad_sign = -1.0;
         la.out_by_walker = 0;
         launch_lik_f64_few(la, true, s);
-        launch_onehot(K, w.R, w.one, 1, w.onehot, s);
-        launch_precision_needed(d, K, pv.L, w.R, w.one, w.p_done, w.p_need, w.P, s, w.onehot);
-        launch_hessian_chol(d, K, 1, pv.L, w.P, w.Z, w.R, w.gbar, w.one, w.GK, w.H, w.info, w.bar, pv.status, s,
+        launch_onehot(K, w.R, w.count, nm, w.onehot, s);
+        launch_precision_needed(d, K, pv.L, w.R, w.count, w.p_done, w.p_need, w.P, s, w.onehot);
+        launch_hessian_chol(d, K, nm, pv.L, w.P, w.Z, w.R, w.gbar, w.count, w.GK, w.H, w.info, w.bar, pv.status, s,
                             w.onehot);
-        launch_tri_inverse(d, w.H, w.Ci, w.T2, s);
+        launch_tri_inverse(d, nm, w.H, w.Ci, w.T2, s);
         // W [g_0 .. g_{K-1}, gbar]; X_k = C^-1 L_k and tr(W P_k)
         note_launch();
-        k_pack_rhs<<<dim3((d + 255) / 256, K + 1), 256, 0, s>>>(d, K, w.GK, w.gbar, w.R, w.V);
-        apply_W(K + 1, w.V, w.WV, w.R, K);
+        k_pack_rhs<<<dim3((d + 255) / 256, K + 1, nm), 256, 0, s>>>(d, K, w.GK, w.gbar, w.R, w.V);
+        apply_W(K + 1, w.V, dV, w.WV, dV, w.R);
         note_launch();
-        k_adj_X<<<dim3(tiles, K), 256, 0, s>>>(d, w.Ci, pv.L, w.R, w.onehot, w.X, w.trp);
+        k_adj_X<<<dim3(tiles, K, nm), 256, kPad, s>>>(d, w.Ci, pv.L, w.R, w.onehot, w.X, w.trp);
         // P_k (W gbar - W g_k) = L_k (L_k^T (W gbar - W g_k))
         note_launch(2);
-        k_adj_upper<<<dim3(cols32, K), 256, 0, s>>>(d, pv.L, dd, w.WV, w.WV + (size_t)K * d, w.R, K, w.U);
-        k_adj_lower<<<dim3(rows8, K), 256, 0, s>>>(d, pv.L, dd, w.U, w.R, K, w.PY, nullptr, nullptr, nullptr,
-                                                   nullptr);
-        // t = grad_x log det H, then v = W t (into V's first row), then c, eps_k, gam_k
+        k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.WV, dV, w.R, K, w.U, dK}, true);
+        k_adj_lower<<<dim3(rows8, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.U, dK, w.R, K, w.PY, dK});
+        // t = grad_x log det H, then v = W t (into V), then c, eps_k, gam_k
         note_launch();
-        k_adj_stage<<<1, 1024, 0, s>>>(0, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, nullptr, w.T,
-                                       nullptr, nullptr);
-        apply_W(1, w.T, w.V, nullptr, 0);
+        k_adj_stage<<<nm, 1024, 0, s>>>(0, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, nullptr, w.T,
+                                        nullptr, nullptr);
+        apply_W(1, w.T, d, w.V, d, nullptr);
         note_launch();
-        k_adj_stage<<<1, 1024, 0, s>>>(1, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, w.V, nullptr,
-                                       w.eps, w.gam);
+        k_adj_stage<<<nm, 1024, 0, s>>>(1, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, w.V, nullptr,
+                                        w.eps, w.gam);
         // u_k = L_k^T gam_k, dmu_k += pi (-eps_k g_k + L_k u_k), dL_k
         note_launch(3);
-        k_adj_upper<<<dim3(cols32, K), 256, 0, s>>>(d, pv.L, dd, w.gam, nullptr, w.R, K, w.U);
-        k_adj_lower<<<dim3(rows8, K), 256, 0, s>>>(d, pv.L, dd, w.U, w.R, K, nullptr, pi, w.eps, w.GK, dmu);
-        k_adj_dL<<<dim3(tiles, K), 256, 0, s>>>(d, pi, w.R, w.eps, w.onehot, pv.L, x, pv.mu, w.Z, w.gam, w.U, w.Ci,
-                                                w.X, dL);
+        k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.gam, dK, w.R, K, w.U, dK}, false);
+        k_adj_dmu<<<dim3(rows8, K), 256, 0, s>>>(d, nm, pv.L, w.U, w.R, pi, w.eps, w.GK, dmu);
+        k_adj_dL<<<dim3(tiles, K), 256, kPad, s>>>(d, nm, pi, w.R, w.eps, w.onehot, pv.L, x, pv.mu, w.Z, w.gam, w.U,
+                                                   w.Ci, w.X, dL);
     }
     SB_CUDA_TRY(cudaGetLastError());
+    SB_CUDA_TRY(cudaStreamSynchronize(s));  // the call returns with its results written
     return SB_OK;
 }
 

@@ -10,11 +10,12 @@ namespace sb {
 constexpr int kMaxAdjModes = 1024;
 
 struct AdjWs {
-    double *P, *H, *Ci, *T2, *X, *trp;  // P_k, H (its factor C), C^-1, merge scratch, C^-1 L_k, |X_k|^2 partials
+    // per mode of a group, but for P_k: H (its factor C), C^-1, merge scratch, C^-1 L_k, |X_k|^2 partials
+    double *P, *H, *Ci, *T2, *X, *trp;
     double *Z, *R, *qpart, *gbar, *ell, *GK;
     double *V, *Y, *WV;  // [K + 1][d]: right-hand sides, C^-1 V, W V
     double *T, *eps, *gam, *U, *PY, *pi;
-    int32_t *info, *one, *onehot, *p_done, *p_need;
+    int32_t *info, *count, *onehot, *p_done, *p_need;
     uint32_t *bar;  // grid-barrier state of the cooperative factorisation
 };
 
