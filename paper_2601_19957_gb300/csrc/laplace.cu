@@ -241,7 +241,8 @@ __global__ void __launch_bounds__(256) k_gather_rows(int d, const double *X, con
 // bounds the FP64 critical path when only a few components are formed.
 constexpr int PT = 32;
 __global__ void __launch_bounds__(256) k_precision(int d, const double *L, double *P, const int32_t *need) {
-    const int k = blockIdx.z, i0 = blockIdx.y * PT, j0 = blockIdx.x * PT;
+    // the longest tiles (large j0) first
+    const int k = blockIdx.z, i0 = (gridDim.x - 1 - blockIdx.x) * PT, j0 = (gridDim.y - 1 - blockIdx.y) * PT;
     if (j0 > i0) return;
     if (need && !need[k]) return;
     const double *Lk = L + (size_t)k * d * d;
@@ -1021,10 +1022,13 @@ void launch_gather_rows(int d, int cap, const double *X, const int32_t *idx, con
     k_gather_rows<<<cap, 256, 0, s>>>(d, X, idx, n_idx, out, ell, ell_out);
 }
 
-void launch_precision(int d, int K, const double *L, double *P, cudaStream_t s) {
-    dim3 g((d + PT - 1) / PT, (d + PT - 1) / PT, K);
-    note_launch();
-    k_precision<<<g, 256, 0, s>>>(d, L, P, nullptr);
+// Unused shared memory that holds an SM to three CTAs of k_precision, so that its tiles, up to
+// d / 32 times different in length, are dealt out as SMs come free (four P_k at d = 512: 371 us
+// with every tile resident at once, 274 so).
+static int precision_pad() {
+    constexpr int kPad = 60 * 1024;
+    return cudaFuncSetAttribute(k_precision, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad) == cudaSuccess ? kPad
+                                                                                                               : 0;
 }
 
 void launch_onehot(int K, const double *R, const int32_t *n_c, int cap, int32_t *onehot, cudaStream_t s) {
@@ -1038,7 +1042,7 @@ void launch_precision_needed(int d, int K, const double *L, const double *R, con
     k_precision_need<<<1, kMaxK, 0, s>>>(K, R, n_c, onehot, done, need);
     dim3 g((d + PT - 1) / PT, (d + PT - 1) / PT, K);
     note_launch();
-    k_precision<<<g, 256, 0, s>>>(d, L, P, need);
+    k_precision<<<g, 256, precision_pad(), s>>>(d, L, P, need);
 }
 
 int laplace_sms();

@@ -19,7 +19,6 @@ void launch_dedup(int n, int d, const double *X, const double *ell, const int8_t
                   const DedupScratch &sc, cudaStream_t s);
 void launch_gather_rows(int d, int cap, const double *X, const int32_t *idx, const int32_t *n_idx, double *out,
                         const double *ell, double *ell_out, cudaStream_t s);
-void launch_precision(int d, int K, const double *L, double *P, cudaStream_t s);
 // P_k only for the components with r != 0 at some live candidate that are not
 // formed yet (done[K] is cleared by the caller before the first call).
 // onehot[c] = k when candidate c's responsibilities R[c] are exactly one-hot at k
