@@ -406,6 +406,106 @@ __global__ void __launch_bounds__(32 * kMaxWarps) k_small_points(LikF64Args a, i
     }
 }
 
+// A point per CTA, for fewer points than SMs: a warp per component forms z_k (32 lanes), one warp
+// the LSE, and the gradient's 32-row slots go to a warp each, so the four schedulers share
+// one point's FP64 instructions. Sums in the same order as in evaluate(). l and grad l at
+// one point, d = 64, K = 4: 41 us a call with a warp per point,
+// 24 so (the kernel itself 19).
+inline size_t point_doubles(int d, int K) { return problem_doubles(d, K) + (size_t)(K + kMaxWarps) * d + 2 * (size_t)K; }
+template <int VPL>
+__global__ void __launch_bounds__(32 * kMaxWarps) k_small_point(LikF64Args a) {
+    extern __shared__ double sh[];
+    __shared__ unsigned long long s_odd;  // components whose z is not finite throughout
+    __shared__ double s_ell;
+    __shared__ unsigned long long s_act;  // components that add to grad l
+    __shared__ int s_one;
+    const int n_rows = a.n_rows_dev ? *a.n_rows_dev : a.n_rows, n = blockIdx.x;
+    if (n >= n_rows) return;
+    const int d = a.d, K = a.K, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nv = (d + 31) / 32;
+    const size_t T = tri(d);
+    const int w = a.rows ? a.rows[n] : n, out = a.out_by_walker ? w : n;
+    if (threadIdx.x == 0) s_odd = 0ull;
+    const SmallProb P = load_problem(d, K, a.L, a.mu, a.a, sh);
+    double *zs = sh + problem_doubles(d, K), *buf = zs + (size_t)K * d + (size_t)warp * d;
+    double *es = zs + (size_t)(K + kMaxWarps) * d, *ex = es + K;
+    const double *X = a.X + (size_t)w * d;
+    for (int k = warp; k < K; k += kMaxWarps) {
+        const double *mk = P.mus + (size_t)k * d;
+        __syncwarp();
+        for (int i = lane; i < d; i += 32) buf[i] = sub_rn(X[i], mk[i]);
+        __syncwarp();
+        double z[VPL];
+        bool odd = false;
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            z[v] = v < nv ? z_column<32>(P.Ls + k * T, buf, d, v, lane) : 0.0;
+            if (lane + 32 * v < d) zs[(size_t)k * d + lane + 32 * v] = z[v];
+            odd = odd || !finite_bits(z[v]);
+        }
+        const double q = norm2<32, VPL>(z);
+        if (lane == 0) es[k] = P.as[k] - 0.5 * q;
+        if (__any_sync(0xffffffffu, odd) && lane == 0) atomicOr(&s_odd, 1ull << k);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double emax = -INFINITY;
+        for (int k = 0; k < K; ++k) emax = fmax(emax, es[k]);
+        // the components whose exponential is not certain to be 0
+        uint64_t keep = 0;
+        for (int k0 = 0; k0 < K; k0 += 32) {
+            const bool far = k0 + lane >= K || es[k0 + lane] < emax - kSkipNats64;
+            keep |= (uint64_t)(~__ballot_sync(0xffffffffu, far)) << k0;
+        }
+        if (__popcll(keep) == 1 && finite_bits(emax)) {
+            if (lane == 0) {
+                s_ell = emax;
+                s_act = keep | s_odd;
+                s_one = s_odd == 0ull;
+            }
+            for (int k = lane; k < K; k += 32) ex[k] = (keep >> k) & 1ull ? 1.0 : 0.0;
+        } else {
+            for (int k = lane; k < K; k += 32) ex[k] = exp(es[k] - emax);
+            __syncwarp();
+            double t = 0.0;
+            for (int k = 0; k < K; ++k) t += ex[k];
+            const double l = emax + log(t);
+            __syncwarp();
+            uint64_t act = 0;
+            for (int k0 = 0; k0 < K; k0 += 32) {
+                const int k = k0 + lane;
+                const double r = k < K ? ex[k] / t : 0.0;
+                if (k < K) ex[k] = r;
+                act |= (uint64_t)__ballot_sync(0xffffffffu, k < K && r != 0.0) << k0;
+            }
+            if (lane == 0) {
+                s_ell = l;
+                s_act = act | s_odd;
+                s_one = 0;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) a.ell[out] = a.ell_sign * s_ell;
+    if (!a.G) return;
+    const uint64_t act = s_act;
+    if (!s_one) {  // r z in place
+        for (uint64_t m = act; m; m &= m - 1) {
+            const int k = __ffsll((long long)m) - 1;
+            for (int j = threadIdx.x; j < d; j += blockDim.x) zs[(size_t)k * d + j] = mul_rn(ex[k], zs[(size_t)k * d + j]);
+        }
+        __syncthreads();
+    }
+    for (int v = warp; v < nv; v += kMaxWarps) {
+        double g = 0.0;
+        for (uint64_t m = act; m; m &= m - 1) {
+            const int k = __ffsll((long long)m) - 1;
+            g = g_row<32>(P.Ls + k * T, zs + (size_t)k * d, d, v, lane, g);
+        }
+        const int i = lane + 32 * v;
+        if (i < d) a.G[(size_t)out * d + i] = a.grad_sign * g;
+    }
+}
+
 // ------------------------------------------------------------------ L-BFGS (see lbfgs.cu)
 template <int LPW, int VPL>
 __global__ void __launch_bounds__(32 * kMaxWarps) k_small_refine(ProbView pv, LbfgsArgs<double> a,
@@ -777,8 +877,20 @@ void launch_small_refine_f64(const ProbView &pv, const LbfgsArgs<double> &a, con
 
 void launch_small_points_f64(const LikF64Args &a, bool rays, cudaStream_t s) {
     if (a.n_rows <= 0) return;
-    const Shape sp = shape_for(a.d, a.K, 0, a.n_rows);
     ProfScope prof(PROF_F64_Z, s);
+    const size_t pt = sizeof(double) * point_doubles(a.d, a.K);
+    if (!rays && a.n_rows <= sm_count() && pt <= (size_t)kSmemMax) {
+        auto launch = [&](auto VP) {
+            auto *k = k_small_point<decltype(VP)::value>;
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+            note_launch();
+            k<<<a.n_rows, 32 * kMaxWarps, pt, s>>>(a);
+        };
+        if (a.d <= 32) return launch(std::integral_constant<int, 1>());
+        if (a.d <= 64) return launch(std::integral_constant<int, 2>());
+        return launch(std::integral_constant<int, 4>());
+    }
+    const Shape sp = shape_for(a.d, a.K, 0, a.n_rows);
     with_variant(a.d, sp.lpw, [&](auto LP, auto VP) {
         auto *k = rays ? k_small_points<decltype(LP)::value, decltype(VP)::value, true>
                        : k_small_points<decltype(LP)::value, decltype(VP)::value, false>;
