@@ -1467,7 +1467,10 @@ float time_tile(const ProbView &pv, TcWs &t, int bn, cudaStream_t s) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return -1.f;
     float best = -1.f;
-    for (int rep = 0; rep < 3; ++rep) {
+    // the best of six: one launch varies by 2 %, and a width within 3 % of another that wins by
+    // chance changes the order of the |z|^2 partial sums from one process to the next (of two
+    // launches d = 300, K = 3 in TF32 gave 128 or 256 columns)
+    for (int rep = 0; rep < 7; ++rep) {
         cudaEventRecord(e0, s);
         launch_gemm_any(u.prec, MODE_ZW, bn, u.mapA1, u.mapT, a, s);
         launch_gemm_any(u.prec, MODE_G, bn, u.mapZ, u.mapB, a, s);
