@@ -29,6 +29,11 @@
 // solve), so the SM is kept busy by several walkers at once: CT threads per
 // walker, thread t owning the 8 consecutive coordinates from 8 t (one 16-byte
 // chunk of a stored bf16 row).
+//
+// What bounds it at d = 1024, m = 20: HBM for the pairs (4.9 of 6.8 TB/s) and the
+// instructions of a visit, 2890 per warp. They were 4570 with the pairs walked in
+// the order of their age (a wrap test per row and per entry of the m x m state), one
+// FMA per coordinate and a shuffle tree per reduced value: 8192 walkers 235 us, 197 so.
 #include <cuda_bf16.h>
 
 #include <mutex>
@@ -102,10 +107,6 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src) {
 // step). Inner products, R and Y^T Y are formed from the stored (rounded)
 // vectors, so the direction applies the exact L-BFGS matrix of the pairs as
 // stored.
-__device__ __forceinline__ float4 round_bf16(float4 v) {
-    return make_float4(__bfloat162float(__float2bfloat16_rn(v.x)), __bfloat162float(__float2bfloat16_rn(v.y)),
-                       __bfloat162float(__float2bfloat16_rn(v.z)), __bfloat162float(__float2bfloat16_rn(v.w)));
-}
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t *>(&h);
@@ -114,6 +115,18 @@ __device__ __forceinline__ float4 unpack4(uint32_t lo, uint32_t hi) {
     const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162 *>(&lo);
     const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162 *>(&hi);
     return make_float4(__low2float(a), __high2float(a), __low2float(b), __high2float(b));
+}
+
+__device__ __forceinline__ uint64_t dup2(float c) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(c));
+    return r;
+}
+// acc += c x for the two bf16 of one word, exactly widened
+__device__ __forceinline__ void fma_bf16x2(uint64_t &acc, uint64_t c, uint32_t x) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(x << 16), "r"(x & 0xffff0000u));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(c), "l"(v));
 }
 
 template <int N>
@@ -215,257 +228,276 @@ __device__ __forceinline__ Vec<CT> subv(const Vec<CT> &a, const Vec<CT> &b) {
         r.v[q] = make_float4(a.v[q].x - b.v[q].x, a.v[q].y - b.v[q].y, a.v[q].z - b.v[q].z, a.v[q].w - b.v[q].w);
     return r;
 }
+// bits of the largest |a_i|: 0x7f800000 and more when some a_i is infinite or NaN
 template <int CT>
-__device__ __forceinline__ bool finitev(const Vec<CT> &a) {
-    bool f = true;
+__device__ __forceinline__ uint32_t absmax_bits(const Vec<CT> &a) {
+    uint32_t m = 0;
+    auto up = [&](float v) { m = max(m, __float_as_uint(v) & 0x7fffffffu); };
 #pragma unroll
-    for (int q = 0; q < Cfg<CT>::VPT; ++q)
-        f = f && isfinite(a.v[q].x) && isfinite(a.v[q].y) && isfinite(a.v[q].z) && isfinite(a.v[q].w);
-    return f;
-}
-template <int CT>
-__device__ __forceinline__ float absmaxv(const Vec<CT> &a) {
-    float m = 0.f;
-#pragma unroll
-    for (int q = 0; q < Cfg<CT>::VPT; ++q)
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(a.v[q].x), fabsf(a.v[q].y)), fmaxf(fabsf(a.v[q].z), fabsf(a.v[q].w))));
+    for (int q = 0; q < Cfg<CT>::VPT; ++q) {
+        up(a.v[q].x);
+        up(a.v[q].y);
+        up(a.v[q].z);
+        up(a.v[q].w);
+    }
     return m;
 }
-
-// Sum of NV per-thread values over the CTA; every thread gets the totals.
-// One barrier: callers alternate between two scratch buffers, so a buffer is
-// never rewritten before every thread has read it (the next call's barrier
-// orders it).
-template <int CT, int NV>
-__device__ __forceinline__ void block_sum(float (&v)[NV], float *sh) {
-    static_assert(NV <= 32, "block_sum scratch holds 32 values per warp");
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = warp_sum(v[j]);
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < NV; ++j) sh[wid * NV + j] = v[j];
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        float t = 0.f;
-#pragma unroll
-        for (int q = 0; q < Cfg<CT>::NW; ++q) t += sh[q * NV + j];
-        v[j] = t;
-    }
+template <int CT>
+__device__ __forceinline__ uint4 pack_bf16(const Vec<CT> &v) {
+    return make_uint4(pack2(v.v[0].x, v.v[0].y), pack2(v.v[0].z, v.v[0].w), pack2(v.v[1].x, v.v[1].y),
+                      pack2(v.v[1].z, v.v[1].w));
+}
+template <int CT>
+__device__ __forceinline__ Vec<CT> unpack_bf16(uint4 p) {
+    Vec<CT> r;
+    r.v[0] = unpack4(p.x, p.y);
+    r.v[1] = unpack4(p.z, p.w);
+    return r;
 }
 
-// NV sums and one maximum over the CTA with a single barrier; every thread gets all.
-template <int CT, int NV>
-__device__ __forceinline__ void block_sum_max(float (&v)[NV], float &mx, float *sh) {
-    static_assert(NV + 1 <= 32, "scratch holds 32 values per warp");
+// Sums of per-thread values over the CTA; every thread gets the totals. One barrier:
+// callers alternate between two scratch buffers, so a buffer is never rewritten before
+// every thread has read it (the next call's barrier orders it). Several values share the
+// shuffles: each step that halves the lanes of a value halves the values of a lane too.
+template <int CT>
+__device__ __forceinline__ float2 block_sum2(float a, float b, float4 *sh) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool hi = lane & 16;
+    float v = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
 #pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = warp_sum(v[j]);
-    mx = warp_max(mx);
-    if (lane == 0) {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) sh[wid * 32 + j] = v[j];
-        sh[wid * 32 + NV] = mx;
-    }
+    for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 15) == 0) reinterpret_cast<float *>(sh + wid)[lane >> 4] = v;
     __syncthreads();
+    float2 t = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        float t = 0.f;
-#pragma unroll
-        for (int q = 0; q < Cfg<CT>::NW; ++q) t += sh[q * 32 + j];
-        v[j] = t;
+    for (int q = 0; q < Cfg<CT>::NW; ++q) {
+        const float2 u = *reinterpret_cast<const float2 *>(sh + q);
+        t.x += u.x;
+        t.y += u.y;
     }
-    float m = sh[NV];
+    return t;
+}
+// three sums and the largest of mx
+template <int CT>
+__device__ __forceinline__ float3 block_sum3_max(float a, float b, float c, uint32_t &mx, float4 *sh) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool b4 = lane & 16, b3 = lane & 8;
+    const float ab = (b4 ? b : a) + __shfl_xor_sync(0xffffffffu, b4 ? a : b, 16);
+    c += __shfl_xor_sync(0xffffffffu, c, 16);
+    float v = (b3 ? c : ab) + __shfl_xor_sync(0xffffffffu, b3 ? ab : c, 8);
 #pragma unroll
-    for (int q = 1; q < Cfg<CT>::NW; ++q) m = fmaxf(m, sh[q * 32 + NV]);
-    mx = m;
+    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    // lane 0 holds a, 16 b, 8 c; lane 24 writes the maximum
+    if ((lane & 7) == 0)
+        reinterpret_cast<float *>(sh + wid)[lane == 24 ? 3 : b3 ? 2 : b4 ? 1 : 0] = lane == 24 ? __uint_as_float(mx) : v;
+    __syncthreads();
+    float3 t = make_float3(0.f, 0.f, 0.f);
+    mx = 0;
+#pragma unroll
+    for (int q = 0; q < Cfg<CT>::NW; ++q) {
+        const float4 u = sh[q];
+        t.x += u.x;
+        t.y += u.y;
+        t.z += u.z;
+        mx = max(mx, __float_as_uint(u.w));
+    }
+    return t;
 }
 
-// The dynamic shared memory of the step kernel: the pair ring (Cfg RING_B bytes),
-// then R^-1 and Y^T Y (logical order, stride ld), pass 1's per-warp partial sums and
-// the m-vectors S^T g, Y^T g, the direction's coefficients a, w, D = diag(S^T Y) and
-// the new pair's column of R. Addresses are formed from the array and m (registers),
-// not kept in shared memory, so that no access waits on a pointer load.
+// The dynamic shared memory of the step kernel: the pair ring (Cfg RING_B bytes), pass 2's
+// coefficient pairs, R^-1 and Y^T Y (row stride ld), pass 1's per-warp partial sums and the
+// m-vectors S^T g, Y^T g, w, D = diag(S^T Y) and the new pair's column of R. Addresses are
+// formed from the array and m (registers), not kept in shared memory, so that no access
+// waits on a pointer load.
 extern __shared__ __align__(16) float4 lb_dyn[];
 __device__ __forceinline__ unsigned char *ring_base() { return reinterpret_cast<unsigned char *>(lb_dyn); }
 
-// Odd row stride of the m x m matrices: their rows and their columns are both
-// free of shared-memory bank conflicts.
-__host__ __device__ __forceinline__ int mm_ld(int m) { return (m & 1) ? m + 2 : m + 1; }
-// Pass 1's partial sums per ring group and warp: three rows (g, y_new, s_new) x
-// the group's 2 PGB vectors.
+// Row stride of the m x m matrices: as in HBM (one linear copy) unless m is a multiple of 8,
+// whose rows would share banks.
+__host__ __device__ __forceinline__ int mm_ld(int m) { return (m & 7) ? m : m + 4; }
+// Pass 1's partial sums per ring group and warp: two rows (g, y_new) x the group's 2 PGB
+// vectors.
 template <int CT>
 __host__ __device__ __forceinline__ int p1_floats(int m) {
-    return (m + Cfg<CT>::PGB - 1) / Cfg<CT>::PGB * Cfg<CT>::NW * 3 * 2 * Cfg<CT>::PGB;
+    return (m + Cfg<CT>::PGB - 1) / Cfg<CT>::PGB * Cfg<CT>::NW * 2 * 2 * Cfg<CT>::PGB;
 }
-// Floats of the dynamic area after the ring: R^-1, Y^T Y, pass 1's sums and the
-// six m-vectors (u1, u2, ca, cw, dg, nr).
+// Floats of the dynamic area after the ring.
 template <int CT>
 __host__ __device__ __forceinline__ int mm_floats(int m) {
-    return 2 * m * mm_ld(m) + p1_floats<CT>(m) + 6 * m;
+    return 2 * m * mm_ld(m) + p1_floats<CT>(m) + 7 * m;
 }
 template <int CT>
 struct Lay {
     int m, ld;
     __device__ __forceinline__ explicit Lay(int m_) : m(m_), ld(mm_ld(m_)) {}
-    __device__ __forceinline__ float *RI() const { return reinterpret_cast<float *>(ring_base() + Cfg<CT>::RING_B); }
+    __device__ __forceinline__ float2 *cf() const { return reinterpret_cast<float2 *>(ring_base() + Cfg<CT>::RING_B); }
+    // 16-byte aligned when m is even
+    __device__ __forceinline__ float *RI() const { return reinterpret_cast<float *>(cf() + m); }
     __device__ __forceinline__ float *YY() const { return RI() + m * ld; }
     __device__ __forceinline__ float *p1() const { return YY() + m * ld; }
     __device__ __forceinline__ float *u1() const { return p1() + p1_floats<CT>(m); }
     __device__ __forceinline__ float *u2() const { return u1() + m; }
-    __device__ __forceinline__ float *ca() const { return u2() + m; }
-    __device__ __forceinline__ float *cw() const { return ca() + m; }
+    __device__ __forceinline__ float *nr() const { return u2() + m; }
+    __device__ __forceinline__ float *cw() const { return nr() + m; }
     __device__ __forceinline__ float *dg() const { return cw() + m; }
-    __device__ __forceinline__ float *nr() const { return dg() + m; }
 };
 
 template <int CT>
 struct Shared {
-    float red2[2][Cfg<CT>::NW * 32];  // reduction scratch, used alternately (see block_sum)
-    float gamma;
-    uint4 zero16;  // a zero row for the unused rows of the tensor-core operand
+    float4 red2[2][Cfg<CT>::NW];  // reduction scratch, used alternately (see block_sum2)
+    uint4 zero16;                 // a zero row for the unused rows of the tensor-core operand
 };
 
-// The m x m state of a walker, slot-indexed in HBM (logical pair i sits in slot
-// (head + i) mod m): R^-1, the inverse of R = upper(S^T Y) (entries i <= j), Y^T Y,
-// and D_i = s_i . y_i (in rho). R^-1 is kept instead of R because the history
-// changes only by appending a pair (one new column of R^-1, a triangular
-// matvec) and dropping the oldest (the inverse of R's trailing block is the
-// trailing block of R^-1), so the direction needs matvecs, not substitutions.
+// The m x m state of a walker, indexed by the slots the pairs sit in (as the ring below and
+// both passes are: the pairs enter only sums, so their order does not matter, and slots
+// 0 .. count - 1 are one contiguous piece): R^-1, the inverse of R = upper(S^T Y), with
+// zeros below its diagonal in the pairs' order of age, Y^T Y, and D_i = s_i . y_i (in
+// rho). R^-1 is kept instead of R because the history changes only by appending a pair
+// (one new column of R^-1, a triangular matvec) and dropping the oldest (the inverse of
+// R's trailing block is the trailing block of R^-1), so the direction needs matvecs, not
+// substitutions.
 //
-// Copies the walker's R^-1, Y^T Y and D into shared memory in logical order as
-// 4-byte asynchronous copies (one copy group, waited for before the solve); the new
-// pair's row and column (logical cn, or -1) are skipped: pass 1 supplies them.
+// Starts the copies of the walker's R^-1, Y^T Y and D into shared memory (one copy group,
+// waited for before the solve). What it reads of the new pair's row and column is old;
+// new_mm and the solve write those.
 template <int CT>
 __device__ __forceinline__ void fetch_mm(const Lay<CT> &L, const float *mri, const float *myy, const float *dw,
-                                         int count, int m, int head, int cn) {
+                                         int count, int m) {
     float *RI = L.RI(), *YY = L.YY(), *dg = L.dg();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = wid; i < count; i += Cfg<CT>::NW) {
-        if (i == cn) continue;
-        int si = head + i;
-        if (si >= m) si -= m;
-        for (int j = lane; j < count; j += 32) {
-            if (j == cn) continue;
-            int sj = head + j;
-            if (sj >= m) sj -= m;
-            if (j >= i) cp_async4(RI + i * L.ld + j, mri + (size_t)si * m + sj);
-            cp_async4(YY + i * L.ld + j, myy + (size_t)si * m + sj);
+    const int t = threadIdx.x;
+    if (m & 1) {
+        for (int e = t; e < count * m; e += CT) {
+            cp_async4(RI + e, mri + e);
+            cp_async4(YY + e, myy + e);
         }
-        if (lane == 0) cp_async4(dg + i, dw + si);
-    }
-}
-// The new pair's part of the state from pass 1: Y^T Y's row and column (y_i .
-// y_new) into shared memory and HBM, R's new column (s_i . y_new, the last entry
-// being D_new) into nr and D_new into dg and HBM. R^-1's new column is
-// formed by the solver. Returns the bytes of m x m state moved this visit.
-template <int CT, typename P1>
-__device__ __forceinline__ uint64_t new_mm(const Lay<CT> &L, float *myy, float *dw, int count, int m, int head, int cn,
-                                           P1 p1sum) {
-    if (cn >= 0) {
-        float *YY = L.YY(), *nr = L.nr(), *dg = L.dg();
-        for (int e = threadIdx.x; e < 2 * count - 1; e += CT) {
-            // e < count: column cn, row e; else row cn, column e - count
-            const int i = e < count ? e : cn, j = e < count ? cn : e - count;
-            const float yy = p1sum(4, e < count ? i : j);
-            int si = head + i, sj = head + j;
-            if (si >= m) si -= m;
-            if (sj >= m) sj -= m;
-            myy[(size_t)si * m + sj] = yy;
-            YY[i * L.ld + j] = yy;
-            if (e < count) {
-                const float r = p1sum(2, i);
-                nr[i] = r;
-                if (i == cn) {
-                    dg[cn] = r;
-                    dw[si] = r;
-                }
+    } else if (m & 7) {  // m^2 is a multiple of 4: the last chunk stays inside
+#pragma unroll 1
+        for (int e = 4 * t; e < count * m; e += 4 * CT) {
+            cp_async16(RI + e, mri + e);
+            cp_async16(YY + e, myy + e);
+        }
+    } else {
+        for (int i = t >> 5; i < count; i += Cfg<CT>::NW)
+            for (int j = 4 * (t & 31); j < m; j += 128) {
+                cp_async16(RI + i * L.ld + j, mri + i * m + j);
+                cp_async16(YY + i * L.ld + j, myy + i * m + j);
             }
+    }
+    for (int i = t; i < count; i += CT) cp_async4(dg + i, dw + i);
+}
+// Pass 1's totals (the warps' sums in warp order): u1 = S^T g, u2 = Y^T g and, when a pair
+// was appended (slot sc), its column of R (s_i . y_new, into nr; D_new into dg and HBM) and
+// its row and column of Y^T Y (shared memory and HBM). R^-1's new column is formed by the
+// solver. Returns the algorithmic bytes of m x m state of this visit.
+template <int CT>
+__device__ __forceinline__ uint64_t new_mm(const Lay<CT> &L, float *myy, float *dw, int count, int m, int sc) {
+    constexpr int PG = Cfg<CT>::PGB, NW = Cfg<CT>::NW;
+    const float *p1 = L.p1();
+    const int n = (sc >= 0 ? 4 : 2) * count;
+#pragma unroll 1
+    for (int e = threadIdx.x; e < n; e += CT) {
+        // role: 0 s.g, 1 y.g, 2 s.y_new, 3 y.y_new
+        const int role = (e >= count) + (e >= 2 * count) + (e >= 3 * count), i = e - role * count;
+        const float *src = p1 + ((i / PG) * NW * 2 + (role >> 1)) * (2 * PG) + 2 * (i % PG) + (role & 1);
+        float v = 0.f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) v += src[q * 2 * 2 * PG];
+        if (role < 3) {
+            L.u1()[role * m + i] = v;  // u1, u2, nr
+            if (role == 2 && i == sc) L.dg()[sc] = dw[sc] = v;
+        } else {
+            L.YY()[i * L.ld + sc] = L.YY()[sc * L.ld + i] = v;
+            myy[i * m + sc] = myy[sc * m + i] = v;
         }
     }
     const uint64_t c = count;
-    return (c * (c + 1) / 2 + c * c + c) * 4 + (cn >= 0 ? (uint64_t)(3 * c) * 4 : 0);
+    return (c * (c + 1) / 2 + c * c + c) * 4 + (sc >= 0 ? (uint64_t)(3 * c) * 4 : 0);
 }
 
-// The m x m part, on the whole CTA, with R^-1 in shared memory: the new column
-// of R^-1 when a pair was appended (logical cn; RI_i,cn = -(sum_{i<=k<cn} RI_ik
-// R_k,cn) / D_cn, RI_cn,cn = 1 / D_cn, also written to HBM), then w = R^-1 u1,
-// gamma = D_c-1 / (y^T y)_c-1, tv = D w + gamma Y^T Y w - gamma u2 and
-// a = R^-T tv. Each entry is a dot product over G threads (strided terms, then a
-// fixed-order shuffle sum), one barrier between the stages. Every thread calls
-// it. Results in cw, ca and sh.gamma.
+// The m x m part, on the whole CTA, with R^-1 in shared memory: when a pair was appended
+// (slot sc) R^-1's new column, v_i = -(sum_k RI_ik R_k,sc) / D_sc, v_sc = 1 / D_sc, and its
+// row, zero elsewhere (also written to HBM); w = R^-1 u1 (the new column's term added
+// apart), gamma = D / (y^T y) of the newest pair (slot sn), tv = D w + gamma Y^T Y w -
+// gamma u2 and a = R^-T tv. Each entry is a dot product over G threads (strided terms,
+// then a fixed-order shuffle sum), one barrier between the stages. Every thread calls it.
+// Leaves (-a_i, gamma w_i) in cf; returns gamma.
 template <int CT>
-__device__ __forceinline__ void solve_mm(Shared<CT> &sh, const Lay<CT> &L, int c, int cn, float *mri, int m, int head) {
-    const int G = c <= 32 ? 4 : (c <= 64 ? 2 : 1);  // threads per entry (the same for every CT)
-    const int p = (int)threadIdx.x % G, E = CT / G;  // E entries at a time
+__device__ __forceinline__ float solve_mm(const Lay<CT> &L, int c, int sc, int sn, float *mri, int m) {
+    const int lg = c <= 32 ? 2 : (c <= 64 ? 1 : 0), G = 1 << lg;  // threads per entry (the same for every CT)
+    const int p = (int)threadIdx.x & (G - 1), i0 = (int)threadIdx.x >> lg, E = CT >> lg;  // E entries at a time
     const int LD = L.ld;
     float *RI = L.RI();
     const float *YY = L.YY();
     float *tv = L.p1();  // pass 1's partial sums are consumed before the solve
     const float *nr = L.nr(), *u1 = L.u1(), *u2 = L.u2(), *dg = L.dg();
-    float *cw = L.cw(), *ca = L.ca();
+    float *cw = L.cw();
     auto gsum = [&](float v) {  // every lane calls it: full-warp shuffles
         if (G >= 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
         if (G >= 4) v += __shfl_xor_sync(0xffffffffu, v, 2);
         return v;
     };
-    if (cn >= 0) {
-        const float dn = nr[cn];
-        for (int i = (int)threadIdx.x / G, b = 0; b <= cn; b += E, i += E) {
-            float t = 0.f;
-            if (i < cn)
-                for (int k = i + p; k < cn; k += G) t += RI[i * LD + k] * nr[k];
-            t = gsum(t);
-            if (p == 0 && i <= cn) {
-                const float v = i == cn ? 1.f / dn : -t / dn;
-                RI[i * LD + cn] = v;
-                int si = head + i, sc = head + cn;
-                if (si >= m) si -= m;
-                if (sc >= m) sc -= m;
-                mri[(size_t)si * m + sc] = v;
+#pragma unroll 1
+    for (int i = i0, b = 0; b < c; b += E, i += E) {
+        float t = 0.f, r = 0.f;
+        if (i < c && i != sc) {
+#pragma unroll 1
+            for (int k = p; k < c; k += G) {
+                const float ri = RI[i * LD + k];
+                if (k != sc) {  // the slot's old column
+                    t = fmaf(ri, u1[k], t);
+                    if (sc >= 0) r = fmaf(ri, nr[k], r);
+                }
             }
         }
-        __syncthreads();
-    }
-    for (int i = (int)threadIdx.x / G, b = 0; b < c; b += E, i += E) {
-        float t = 0.f;
-        if (i < c)
-            for (int k = i + p; k < c; k += G) t += RI[i * LD + k] * u1[k];
         t = gsum(t);
+        if (sc >= 0) {
+            r = gsum(r);
+            if (p == 0 && i < c) {
+                const float dn = nr[sc], v = i == sc ? 1.f / dn : -r / dn;
+                t = fmaf(v, u1[sc], t);
+                RI[i * LD + sc] = v;
+                mri[i * m + sc] = v;
+                if (i != sc) {
+                    RI[sc * LD + i] = 0.f;
+                    mri[sc * m + i] = 0.f;
+                }
+            }
+        }
         if (p == 0 && i < c) cw[i] = t;
     }
     __syncthreads();
-    const float gam = dg[c - 1] / YY[(c - 1) * LD + (c - 1)];
-    if (threadIdx.x == 0) sh.gamma = gam;
-    for (int i = (int)threadIdx.x / G, b = 0; b < c; b += E, i += E) {
+    const float gam = dg[sn] / YY[sn * LD + sn];
+#pragma unroll 1
+    for (int i = i0, b = 0; b < c; b += E, i += E) {
         float t = 0.f;
         if (i < c)
-            for (int j = p; j < c; j += G) t += YY[i * LD + j] * cw[j];
+#pragma unroll 1
+            for (int j = p; j < c; j += G) t = fmaf(YY[i * LD + j], cw[j], t);
         t = gsum(t);
         if (p == 0 && i < c) tv[i] = dg[i] * cw[i] + gam * t - gam * u2[i];
     }
     __syncthreads();
-    for (int i = (int)threadIdx.x / G, b = 0; b < c; b += E, i += E) {
+#pragma unroll 1
+    for (int i = i0, b = 0; b < c; b += E, i += E) {
         float t = 0.f;
         if (i < c)
-            for (int k = p; k <= i; k += G) t += RI[k * LD + i] * tv[k];
+#pragma unroll 1
+            for (int k = p; k < c; k += G) t = fmaf(RI[k * LD + i], tv[k], t);
         t = gsum(t);
-        if (p == 0 && i < c) ca[i] = t;
+        if (p == 0 && i < c) L.cf()[i] = make_float2(-t, gam * cw[i]);
     }
+    __syncthreads();
+    return gam;
 }
 
 using bf16 = __nv_bfloat16;
 
-// Stores this thread's chunk of a history row (values already bf16; coordinates past
-// d are zero in the vector): 8 consecutive coordinates, one 16-byte store, for every
-// chunk inside the row pitch.
-template <int CT>
-__device__ __forceinline__ void store_hist(const Vec<CT> &v, bf16 *row, int ldh) {
-    const int e0 = Vec<CT>::i0(0);
-    if (e0 >= ldh) return;
-    *reinterpret_cast<uint4 *>(row + e0) = make_uint4(pack2(v.v[0].x, v.v[0].y), pack2(v.v[0].z, v.v[0].w),
-                                                      pack2(v.v[1].x, v.v[1].y), pack2(v.v[1].z, v.v[1].w));
+// Stores this thread's chunk of a history row (coordinates past d are zero in the vector):
+// 8 consecutive coordinates, one 16-byte store, for every chunk inside the row pitch.
+__device__ __forceinline__ void store_hist(uint4 v, bf16 *row, int ldh) {
+    const int e0 = 8 * (int)threadIdx.x;
+    if (e0 < ldh) *reinterpret_cast<uint4 *>(row + e0) = v;
 }
 
 // The ring the stored pairs stream through (Cfg: DB slots of PGB pairs; row 2 q + v of
@@ -478,8 +510,9 @@ template <int CT>
 struct Ring {
     static constexpr int PG = Cfg<CT>::PGB, D = Cfg<CT>::DB;
     static_assert(Cfg<CT>::VPT == 2, "one 16-byte bf16 chunk (8 coordinates) per stored vector and thread");
-    int ldh, m, head, J, cn;  // row pitch, history size, first slot, pairs in the ring, new pair (or -1)
+    int ldh, J, cn;  // row pitch, pairs (slots 0 .. J - 1), slot of the new pair (or -1)
     const bf16 *S, *Y;
+    uint4 s_new, y_new;
 
     __device__ __forceinline__ unsigned char *row(int sl, int r) const {
         return ring_base() + sl * Cfg<CT>::SLOT_B + r * Cfg<CT>::ROW_B;
@@ -488,26 +521,30 @@ struct Ring {
     __device__ __forceinline__ uint4 *chunk(int sl, int r) const {
         return reinterpret_cast<uint4 *>(row(sl, r)) + threadIdx.x;
     }
-    // Group k (logical pairs k PG .. k PG + PG - 1 below J; none for k < 0) into slot sl.
-    // The visit's new pair comes from registers (s_new, y_new), not HBM.
-    __device__ __forceinline__ void issue(int k, int sl, const Vec<CT> &s_new, const Vec<CT> &y_new) const {
+    // Group k (slots k PG .. k PG + PG - 1 below J; none for k < 0) into ring slot sl. The
+    // visit's new pair comes from registers (s_new, y_new), not HBM.
+    __device__ __forceinline__ void issue(int k, int sl) const {
         const int e0 = Vec<CT>::i0(0);
         if (k >= 0 && e0 < ldh) {
+            const int j0 = k * PG;
+            const bf16 *s = S + (size_t)(j0 * ldh + e0), *y = Y + (size_t)(j0 * ldh + e0);
+            if (j0 + PG <= J && (unsigned)(cn - j0) >= (unsigned)PG) {
 #pragma unroll
-            for (int q = 0; q < PG; ++q) {
-                const int j = k * PG + q;
-                if (j >= J) break;
-                if (j == cn) {
-                    *chunk(sl, 2 * q) = make_uint4(pack2(s_new.v[0].x, s_new.v[0].y), pack2(s_new.v[0].z, s_new.v[0].w),
-                                                   pack2(s_new.v[1].x, s_new.v[1].y), pack2(s_new.v[1].z, s_new.v[1].w));
-                    *chunk(sl, 2 * q + 1) = make_uint4(pack2(y_new.v[0].x, y_new.v[0].y), pack2(y_new.v[0].z, y_new.v[0].w),
-                                                       pack2(y_new.v[1].x, y_new.v[1].y), pack2(y_new.v[1].z, y_new.v[1].w));
-                    continue;
+                for (int q = 0; q < PG; ++q, s += ldh, y += ldh) {
+                    cp_async16(chunk(sl, 2 * q), s);
+                    cp_async16(chunk(sl, 2 * q + 1), y);
                 }
-                int slot = head + j;
-                if (slot >= m) slot -= m;
-                cp_async16(chunk(sl, 2 * q), S + (size_t)slot * ldh + e0);
-                cp_async16(chunk(sl, 2 * q + 1), Y + (size_t)slot * ldh + e0);
+            } else {
+#pragma unroll 1
+                for (int q = 0; q < PG && j0 + q < J; ++q, s += ldh, y += ldh) {
+                    if (j0 + q == cn) {
+                        *chunk(sl, 2 * q) = s_new;
+                        *chunk(sl, 2 * q + 1) = y_new;
+                    } else {
+                        cp_async16(chunk(sl, 2 * q), s);
+                        cp_async16(chunk(sl, 2 * q + 1), y);
+                    }
+                }
             }
         }
         cp_async_commit();
@@ -517,31 +554,35 @@ struct Ring {
         cp_async_wait<D - 1>();
         __syncwarp();
     }
-    // this thread's coordinates of pair q of slot sl
-    __device__ __forceinline__ void fetch(int sl, int q, Vec<CT> &sv, Vec<CT> &yv) const {
+    // p += c.x s + c.y y for pair q of ring slot sl, on this thread's coordinates
+    __device__ __forceinline__ void add(int sl, int q, float2 c, uint64_t (&p)[4]) const {
         const uint4 a4 = *chunk(sl, 2 * q), b4 = *chunk(sl, 2 * q + 1);
-        sv.v[0] = unpack4(a4.x, a4.y);
-        sv.v[1] = unpack4(a4.z, a4.w);
-        yv.v[0] = unpack4(b4.x, b4.y);
-        yv.v[1] = unpack4(b4.z, b4.w);
+        const uint64_t cs = dup2(c.x), cy = dup2(c.y);
+        fma_bf16x2(p[0], cs, a4.x);
+        fma_bf16x2(p[1], cs, a4.y);
+        fma_bf16x2(p[2], cs, a4.z);
+        fma_bf16x2(p[3], cs, a4.w);
+        fma_bf16x2(p[0], cy, b4.x);
+        fma_bf16x2(p[1], cy, b4.y);
+        fma_bf16x2(p[2], cy, b4.z);
+        fma_bf16x2(p[3], cy, b4.w);
     }
 };
 
-// Direction for walker state st (count pairs from ring slot head). When
-// new_slot >= 0 the pair in that slot was stored this visit (the newest, logical
-// index count - 1; s_new, y_new) and its column of R, row and column of Y^T Y
-// come from the same pass. Writes P and the unit trial X + P; updates st.dphi /
+// Direction for walker state st (pairs in slots 0 .. count - 1). When sc >= 0 the pair in
+// that slot was stored this visit (s_new, y_new) and its column of R, row and column of
+// Y^T Y come from the same pass. Writes P and the unit trial X + P; updates st.dphi /
 // alpha / bt and possibly resets the history (steepest descent when p is not a
 // descent direction). Returns the algorithmic bytes moved.
 //
-// Pass 1 streams the pairs oldest first; at its end the ring holds the newest
-// min(groups, DB) groups, so pass 2 walks the groups newest first: those are read
-// where they are, and each slot it frees is refilled with the group DB older (the
-// same slot, g mod DB), the only ones read from HBM (L2) again.
+// Pass 1 streams the slots upwards; at its end the ring holds the last min(groups, DB)
+// groups, so pass 2 walks the groups downwards: those are read where they are, and each
+// ring slot it frees is refilled with the group DB below (the same ring slot, g mod DB), the
+// only ones read from HBM (L2) again.
 template <int CT, bool EVEN>
-__device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<float> &st, int new_slot,
-                              const Vec<CT> &g_in, const Vec<CT> &x_in, const Vec<CT> &s_new, const Vec<CT> &y_new,
-                              float *MRI, float *MYY, Shared<CT> &sh, const Lay<CT> &L, int &par) {
+__device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<float> &st, int sc, const Vec<CT> &g_in,
+                              const Vec<CT> &x_in, uint4 s_new, uint4 y_new, float *MRI, float *MYY, Shared<CT> &sh,
+                              const Lay<CT> &L, int &par) {
     using RG = Ring<CT>;
     constexpr int PG = RG::PG, D = RG::D, NW = Cfg<CT>::NW;
     const int d = a.d, m = a.m, ldh = hist_ld(d);
@@ -554,20 +595,18 @@ __device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<floa
     // instead of being held through it
     Vec<CT> g = g_in, x = x_in;
     if (count > 0) {
-        const bool added = new_slot >= 0;
-        const int cn = added ? count - 1 : -1;
-        const RG ring{ldh, m, st.head, count, cn, reinterpret_cast<const bf16 *>(a.S) + (size_t)w * m * ldh,
-                      reinterpret_cast<const bf16 *>(a.Y) + (size_t)w * m * ldh};
+        const RG ring{ldh, count, sc, reinterpret_cast<const bf16 *>(a.S) + (size_t)w * m * ldh,
+                      reinterpret_cast<const bf16 *>(a.Y) + (size_t)w * m * ldh, s_new, y_new};
         const int ng = (count + PG - 1) / PG;
         float *mri_w = MRI + (size_t)w * m * m, *myy_w = MYY + (size_t)w * m * m, *dw = a.rho + (size_t)w * m;
-#pragma unroll 1
-        for (int k = 0; k < D - 1; ++k) ring.issue(k, k, s_new, y_new);
+#pragma unroll
+        for (int k = 0; k < D - 1; ++k) ring.issue(k, k);
         float *p1 = L.p1();
         {
             // Pass 1 on the tensor cores: per warp (its 256 coordinates, 16 k-steps of
             // 16) and group (8 stored vectors s_0 y_0 .. s_3 y_3 as the columns of B),
-            // D = A B with the rows of A = (g_hi, g_mid, g_lo, y_new, s_new, 0 ..) at the
-            // same coordinates. The A fragments are staged once through this warp's
+            // D = A B with the rows of A = (g_hi, g_mid, g_lo, y_new, 0 ..) at the same
+            // coordinates. The A fragments are staged once through this warp's
             // own chunks of ring slot D - 1 (free until group D - 1 is issued into it).
             {
                 float hi[8], mi[8], lo[8];
@@ -580,19 +619,15 @@ __device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<floa
                     make_uint4(pack2(mi[0], mi[1]), pack2(mi[2], mi[3]), pack2(mi[4], mi[5]), pack2(mi[6], mi[7]));
                 *ring.chunk(D - 1, 2) =
                     make_uint4(pack2(lo[0], lo[1]), pack2(lo[2], lo[3]), pack2(lo[4], lo[5]), pack2(lo[6], lo[7]));
-                // s_new, y_new are bf16 values already (the pair as stored): exact
-                *ring.chunk(D - 1, 3) = make_uint4(pack2(y_new.v[0].x, y_new.v[0].y), pack2(y_new.v[0].z, y_new.v[0].w),
-                                                   pack2(y_new.v[1].x, y_new.v[1].y), pack2(y_new.v[1].z, y_new.v[1].w));
-                *ring.chunk(D - 1, 4) = make_uint4(pack2(s_new.v[0].x, s_new.v[0].y), pack2(s_new.v[0].z, s_new.v[0].w),
-                                                   pack2(s_new.v[1].x, s_new.v[1].y), pack2(s_new.v[1].z, s_new.v[1].w));
+                *ring.chunk(D - 1, 3) = y_new;  // as stored
             }
             __syncwarp();
             const int mi8 = lane >> 3, ri8 = lane & 7;  // ldmatrix: matrix and row this lane addresses
+            const int u0 = 16 * (32 * wid + 2 * (mi8 >> 1) + (mi8 & 1));  // its byte in the row at k-step 0
             uint32_t af[16][2];                         // A fragments (a0, a2) per k-step
 #pragma unroll
             for (int c = 0; c < 16; c += 2) {
-                const int u = 32 * wid + 2 * (c + (mi8 >> 1)) + (mi8 & 1);  // chunk (thread) index
-                const void *src = ri8 < 5 ? (const void *)(ring.row(D - 1, ri8) + 16 * u) : (const void *)&sh.zero16;
+                const void *src = ri8 < 4 ? (const void *)(ring.row(D - 1, ri8) + u0 + 32 * c) : (const void *)&sh.zero16;
                 uint32_t r[4];
                 ldsm_x4(r, src);
                 af[c][0] = r[0];
@@ -604,116 +639,106 @@ __device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<floa
             nk = nk < 0 ? 0 : (nk > 16 ? 16 : nk);
             const int gid = lane >> 2, tig = lane & 3;
             __syncwarp();
-            fetch_mm<CT>(L, mri_w, myy_w, dw, count, m, st.head, cn);
-            ring.issue(D - 1, D - 1, s_new, y_new);
+            fetch_mm<CT>(L, mri_w, myy_w, dw, count, m);
+            ring.issue(D - 1, D - 1);
+            int sl = 0;
+#pragma unroll 1
             for (int k = 0; k < ng; ++k) {
-                const int sl = k % D;
                 ring.wait();
                 // B rows: the group's 8 stored vectors (pair n / 2, s or y); the k-steps
                 // accumulate into four independent sets (k-step mod 4), summed after, so
                 // that the MMAs are not one dependent chain
                 float a4[4][4] = {};
+                const unsigned char *br = ring.row(sl, ri8) + u0;
+                auto step = [&](int c) {
+                    uint32_t b[4];
+                    ldsm_x4(b, br + 32 * c);
+                    mma_rows8(a4[c & 3], af[c][0], af[c][1], b[0], b[1]);
+                    mma_rows8(a4[(c + 1) & 3], af[c + 1][0], af[c + 1][1], b[2], b[3]);
+                };
+                if (nk == 16) {
 #pragma unroll
-                for (int c = 0; c < 16; c += 2) {
-                    if (c < nk) {
-                        uint32_t b[4];
-                        ldsm_x4(b, ring.row(sl, ri8) + 16 * (32 * wid + 2 * (c + (mi8 >> 1)) + (mi8 & 1)));
-                        mma_rows8(a4[c & 3], af[c][0], af[c][1], b[0], b[1]);
-                        if (c + 1 < nk) mma_rows8(a4[(c + 1) & 3], af[c + 1][0], af[c + 1][1], b[2], b[3]);
-                    }
+                    for (int c = 0; c < 16; c += 2) step(c);
+                } else {
+                    // past d both operands are zero
+#pragma unroll
+                    for (int c = 0; c < 16; c += 2)
+                        if (c < nk) step(c);
                 }
-                float acc[4];
+                float acc[2];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) acc[e] = (a4[0][e] + a4[1][e]) + (a4[2][e] + a4[3][e]);
+                for (int e = 0; e < 2; ++e) acc[e] = (a4[0][e] + a4[1][e]) + (a4[2][e] + a4[3][e]);
                 // g . v = (g_hi + g_mid) . v + g_lo . v from rows 0, 1, 2
                 const float h0 = __shfl_down_sync(0xffffffffu, acc[0], 4);
                 const float l0 = __shfl_down_sync(0xffffffffu, acc[0], 8);
                 const float h1 = __shfl_down_sync(0xffffffffu, acc[1], 4);
                 const float l1 = __shfl_down_sync(0xffffffffu, acc[1], 8);
-                const int r = gid == 0 ? 0 : gid == 3 ? 1 : gid == 4 ? 2 : -1;
-                if (r >= 0 && tig < PG) {
+                if (gid == 0 || gid == 3) {
                     const float2 o = gid == 0 ? make_float2((acc[0] + h0) + l0, (acc[1] + h1) + l1)
                                               : make_float2(acc[0], acc[1]);
-                    *reinterpret_cast<float2 *>(p1 + ((k * NW + wid) * 3 + r) * (2 * PG) + 2 * tig) = o;
+                    *reinterpret_cast<float2 *>(p1 + ((k * NW + wid) * 2 + (gid != 0)) * (2 * PG) + 2 * tig) = o;
                 }
                 __syncwarp();  // the warp has read the group before its slot is refilled
-                ring.issue(k + D < ng ? k + D : -1, sl, s_new, y_new);
+                ring.issue(k + D < ng ? k + D : -1, sl);
+                sl = sl == D - 1 ? 0 : sl + 1;
             }
         }
         cp_async_wait<0>();  // the m x m state
         __syncthreads();
-        // product k of logical pair i (k: 0 s.g, 1 y.g, 2 s.y_new, 3 s_new.y, 4 y.y_new):
-        // the warps' totals summed in warp order
-        auto p1sum = [&](int k, int i) {
-            // rows (g, y_new, s_new) x columns (s_q, y_q) of the group's warp totals
-            constexpr int rk[5] = {0, 0, 1, 2, 1}, ck[5] = {0, 1, 0, 1, 1};
-            const float *src = p1 + ((i / PG) * NW * 3 + rk[k]) * (2 * PG) + 2 * (i % PG) + ck[k];
-            float t = 0.f;
-#pragma unroll
-            for (int q = 0; q < NW; ++q) t += src[q * 3 * 2 * PG];
-            return t;
-        };
-        {
-            float *u1 = L.u1(), *u2 = L.u2();
-            for (int e = threadIdx.x; e < 2 * count; e += CT) {
-                if (e < count)
-                    u1[e] = p1sum(0, e);
-                else
-                    u2[e - count] = p1sum(1, e - count);
-            }
-        }
-        bytes += new_mm<CT>(L, myy_w, dw, count, m, st.head, cn, p1sum);
+        bytes += new_mm<CT>(L, myy_w, dw, count, m, sc);
         g.template load<EVEN>(a.G + (size_t)w * d, d);
         x.template load<EVEN>(a.X + (size_t)w * d, d);
         __syncthreads();
-        solve_mm<CT>(sh, L, count, cn, mri_w, m, st.head);
-        __syncthreads();
-        // pass 2: p = -gamma g - S a + gamma Y w, the groups newest first
-        const float gam = sh.gamma;
-        p.zero();
-        axpyv(-gam, g, p);
-        const int r0 = ng > D ? ng - D : 0;  // groups below r0 are no longer in the ring
-        const float *ca = L.ca(), *cw = L.cw();
-        for (int k = ng - 1; k >= 0; --k) {
-            const int sl = k % D;
-            if (k < r0) ring.wait();
+        int sn = st.head + count - 1;  // the newest pair's slot
+        if (sn >= m) sn -= m;
+        const float gam = solve_mm<CT>(L, count, sc, sn, mri_w, m);
+        // pass 2: p = -gamma g - S a + gamma Y w, the groups downwards
+        uint64_t p2[4];
 #pragma unroll
-            for (int q = 0; q < PG; ++q) {
-                const int i = k * PG + q;
-                if (i < count) {
-                    Vec<CT> s4, y4;
-                    ring.fetch(sl, q, s4, y4);
-                    axpyv(-ca[i], s4, p);
-                    axpyv(gam * cw[i], y4, p);
-                }
+        for (int q = 0; q < 2; ++q) {
+            const float4 t = make_float4(-gam * g.v[q].x, -gam * g.v[q].y, -gam * g.v[q].z, -gam * g.v[q].w);
+            asm("mov.b64 %0, {%1, %2};" : "=l"(p2[2 * q]) : "f"(t.x), "f"(t.y));
+            asm("mov.b64 %0, {%1, %2};" : "=l"(p2[2 * q + 1]) : "f"(t.z), "f"(t.w));
+        }
+        const int r0 = ng > D ? ng - D : 0;  // groups below r0 are no longer in the ring
+        const float2 *cf = L.cf();
+        int sl = (ng - 1) % D;
+#pragma unroll 1
+        for (int k = ng - 1; k >= 0; --k) {
+            if (k < r0) ring.wait();
+            const int n = count - k * PG;
+            if (n >= PG) {
+#pragma unroll
+                for (int q = 0; q < PG; ++q) ring.add(sl, q, cf[k * PG + q], p2);
+            } else {
+#pragma unroll 1
+                for (int q = 0; q < n; ++q) ring.add(sl, q, cf[k * PG + q], p2);
             }
-            ring.issue(k - D, sl, s_new, y_new);  // this thread's own chunks, just read
+            ring.issue(k - D, sl);  // this thread's own chunks, just read
+            sl = sl == 0 ? D - 1 : sl - 1;
         }
         cp_async_wait<0>();  // (only empty groups remain) the ring is free for the next walker
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(p.v[q].x), "=f"(p.v[q].y) : "l"(p2[2 * q]));
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(p.v[q].z), "=f"(p.v[q].w) : "l"(p2[2 * q + 1]));
+        }
         // the two-loop recursion's history traffic: each pair read in both passes
         bytes += (uint64_t)4 * count * d * sizeof(bf16);
     }
-    float dp[2];  // grad f . p and |p|^2
-    if (count > 0) {
-        dp[0] = dotv(g, p);
-        dp[1] = dotv(p, p);
-        block_sum<CT, 2>(dp, sh.red2[par++ & 1]);
-    }
-    if (count == 0 || !(dp[0] < 0.f)) {
+    float2 dp = make_float2(0.f, 0.f);  // grad f . p and |p|^2
+    if (count > 0) dp = block_sum2<CT>(dotv(g, p), dotv(p, p), sh.red2[par++ & 1]);
+    if (count == 0 || !(dp.x < 0.f)) {
         st.count = 0;
         st.head = 0;
-        float gg[1] = {dotv(g, g)};
-        block_sum<CT, 1>(gg, sh.red2[par++ & 1]);
-        const float gn = sqrtf(gg[0]);
+        const float gn = sqrtf(block_sum2<CT>(dotv(g, g), 0.f, sh.red2[par++ & 1]).x);
 #pragma unroll
         for (int q = 0; q < Cfg<CT>::VPT; ++q)
             p.v[q] = make_float4(-g.v[q].x / gn, -g.v[q].y / gn, -g.v[q].z / gn, -g.v[q].w / gn);
-        dp[0] = dotv(g, p);
-        dp[1] = dotv(p, p);
-        block_sum<CT, 2>(dp, sh.red2[par++ & 1]);
+        dp = block_sum2<CT>(dotv(g, p), dotv(p, p), sh.red2[par++ & 1]);
     }
-    st.dphi = dp[0];
-    st.pn = sqrtf(dp[1]);
+    st.dphi = dp.x;
+    st.pn = sqrtf(dp.y);
     st.alpha = 1.f;
     st.bt = 0;
     p.template store<EVEN>(a.P + (size_t)w * d, d);
@@ -758,23 +783,19 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
         xt.template load<EVEN>(a.XT + (size_t)w * d, d);
         gt.template load<EVEN>(a.GT + (size_t)w * d, d);
         bytes += (uint64_t)16 * d + 4 + 2 * sizeof(WalkerState<float>);
-        // finiteness of the trial gradient, the candidate pair's inner products and
-        // max |grad| at the trial, all in one reduction
-        Vec<CT> s4 = subv(xt, x), y4 = subv(gt, g);
-#pragma unroll
-        for (int q = 0; q < Cfg<CT>::VPT; ++q) {  // the pair as it will be stored
-            s4.v[q] = round_bf16(s4.v[q]);
-            y4.v[q] = round_bf16(y4.v[q]);
+        // finiteness of the trial gradient, the candidate pair (as it will be stored) and its
+        // inner products, and max |grad| at the trial, all in one reduction
+        const uint4 s_new = pack_bf16<CT>(subv(xt, x)), y_new = pack_bf16<CT>(subv(gt, g));
+        uint32_t gm_bits = absmax_bits<CT>(gt);
+        float3 r3;
+        {
+            const Vec<CT> s4 = unpack_bf16<CT>(s_new), y4 = unpack_bf16<CT>(y_new);
+            r3 = block_sum3_max<CT>(dotv(s4, s4), dotv(y4, y4), dotv(s4, y4), gm_bits, sh.red2[par++ & 1]);
         }
-        float r4[4] = {finitev(gt) ? 0.f : 1.f, dotv(s4, s4), dotv(y4, y4), dotv(s4, y4)};
-        float gm = absmaxv(gt);
-        block_sum_max<CT, 4>(r4, gm, sh.red2[par++ & 1]);
-        const bool finite = isfinite(ft) && r4[0] == 0.f;
+        const bool finite = isfinite(ft) && gm_bits < 0x7f800000u;
+        const float gm = __uint_as_float(gm_bits);
         bool newiter = false;
         int new_slot = -1;
-        Vec<CT> s_new, y_new;
-        s_new.zero();
-        y_new.zero();
         if (st.phase == 0) {
             x = xt;
             g = gt;
@@ -788,21 +809,19 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
             else
                 newiter = true;
         } else if (finite && ft <= st.f + (a.c1 * st.alpha) * st.dphi) {
-            if (r4[3] > 1e-10f * sqrtf(r4[1]) * sqrtf(r4[2])) {
+            if (r3.z > 1e-10f * sqrtf(r3.x) * sqrtf(r3.y)) {
                 int slot;
                 if (st.count < m) {
-                    slot = (st.head + st.count) % m;
+                    slot = st.count;  // the slots fill upwards from 0
                     ++st.count;
                 } else {
                     slot = st.head;
-                    st.head = (st.head + 1) % m;
+                    st.head = slot + 1 == m ? 0 : slot + 1;
                 }
-                store_hist<CT>(s4, reinterpret_cast<bf16 *>(a.S) + ((size_t)w * m + slot) * ldh, ldh);
-                store_hist<CT>(y4, reinterpret_cast<bf16 *>(a.Y) + ((size_t)w * m + slot) * ldh, ldh);
+                store_hist(s_new, reinterpret_cast<bf16 *>(a.S) + ((size_t)w * m + slot) * ldh, ldh);
+                store_hist(y_new, reinterpret_cast<bf16 *>(a.Y) + ((size_t)w * m + slot) * ldh, ldh);
                 bytes += (uint64_t)2 * d * sizeof(bf16);
                 new_slot = slot;
-                s_new = s4;
-                y_new = y4;
             }
             st.flat = (ft >= st.f) ? st.flat + 1 : 0;
             x = xt;
