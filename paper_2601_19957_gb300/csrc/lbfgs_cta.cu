@@ -134,6 +134,8 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Four 8 x 8 bf16 matrices from shared memory; lane l gives the address of row
 // l % 8 of matrix l / 8 (16 bytes) and receives row l / 4, columns 2 (l % 4),
 // 2 (l % 4) + 1 of each matrix.
@@ -358,9 +360,8 @@ struct Shared {
 // R's trailing block is the trailing block of R^-1), so the direction needs matvecs, not
 // substitutions.
 //
-// Starts the copies of the walker's R^-1, Y^T Y and D into shared memory (one copy group,
-// waited for before the solve). What it reads of the new pair's row and column is old;
-// new_mm and the solve write those.
+// Starts the copies of the walker's R^-1, Y^T Y and D into shared memory (waited for before
+// the solve). A new pair's row and column are written by new_mm and the solve.
 template <int CT>
 __device__ __forceinline__ void fetch_mm(const Lay<CT> &L, const float *mri, const float *myy, const float *dw,
                                          int count, int m) {
@@ -513,6 +514,7 @@ struct Ring {
     int ldh, J, cn;  // row pitch, pairs (slots 0 .. J - 1), slot of the new pair (or -1)
     const bf16 *S, *Y;
     uint4 s_new, y_new;
+    bool known;  // s_new and y_new are (before the trial is judged only the slot is)
 
     __device__ __forceinline__ unsigned char *row(int sl, int r) const {
         return ring_base() + sl * Cfg<CT>::SLOT_B + r * Cfg<CT>::ROW_B;
@@ -538,8 +540,10 @@ struct Ring {
 #pragma unroll 1
                 for (int q = 0; q < PG && j0 + q < J; ++q, s += ldh, y += ldh) {
                     if (j0 + q == cn) {
-                        *chunk(sl, 2 * q) = s_new;
-                        *chunk(sl, 2 * q + 1) = y_new;
+                        if (known) {
+                            *chunk(sl, 2 * q) = s_new;
+                            *chunk(sl, 2 * q + 1) = y_new;
+                        }
                     } else {
                         cp_async16(chunk(sl, 2 * q), s);
                         cp_async16(chunk(sl, 2 * q + 1), y);
@@ -548,6 +552,25 @@ struct Ring {
             }
         }
         cp_async_commit();
+    }
+    // The first D - 1 groups after the trial is judged: the new pair's row, or, when its slot sp
+    // keeps its old pair, that row.
+    __device__ __forceinline__ void settle(int sp) const {
+        if (sp >= (D - 1) * PG) return;
+        const int sl = sp / PG, q = sp % PG, e0 = Vec<CT>::i0(0);
+        if (cn == sp) {
+            if (e0 < ldh) {
+                *chunk(sl, 2 * q) = s_new;
+                *chunk(sl, 2 * q + 1) = y_new;
+            }
+        } else if (sp < J) {
+            if (e0 < ldh) {
+                cp_async16(chunk(sl, 2 * q), S + (size_t)(sp * ldh + e0));
+                cp_async16(chunk(sl, 2 * q + 1), Y + (size_t)(sp * ldh + e0));
+            }
+            cp_async_commit();
+            cp_async_wait<0>();
+        }
     }
     // the group issued D - 1 issues ago has landed, and is visible to the warp
     __device__ __forceinline__ void wait() const {
@@ -569,23 +592,24 @@ struct Ring {
     }
 };
 
-// Direction for walker state st (pairs in slots 0 .. count - 1). When sc >= 0 the pair in
-// that slot was stored this visit (s_new, y_new) and its column of R, row and column of
-// Y^T Y come from the same pass. Writes P and the unit trial X + P; updates st.dphi /
-// alpha / bt and possibly resets the history (steepest descent when p is not a
-// descent direction). Returns the algorithmic bytes moved.
+// Direction for walker state st (pairs in slots 0 .. count - 1). When sc = ring.cn >= 0 the
+// pair in that slot was stored this visit and its column of R, row and column of
+// Y^T Y come from the same pass. sp: the slot the caller left out when it started the first
+// D - 1 groups. Writes P and the unit trial X + P; updates st.dphi / alpha / bt and possibly
+// resets the history (steepest descent when p is not a descent direction). Returns the
+// algorithmic bytes moved.
 //
 // Pass 1 streams the slots upwards; at its end the ring holds the last min(groups, DB)
 // groups, so pass 2 walks the groups downwards: those are read where they are, and each
 // ring slot it frees is refilled with the group DB below (the same ring slot, g mod DB), the
 // only ones read from HBM (L2) again.
 template <int CT, bool EVEN>
-__device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<float> &st, int sc, const Vec<CT> &g_in,
-                              const Vec<CT> &x_in, uint4 s_new, uint4 y_new, float *MRI, float *MYY, Shared<CT> &sh,
+__device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<float> &st, int sp, const Vec<CT> &g_in,
+                              const Vec<CT> &x_in, const Ring<CT> &ring, float *mri_w, float *myy_w, Shared<CT> &sh,
                               const Lay<CT> &L, int &par) {
     using RG = Ring<CT>;
     constexpr int PG = RG::PG, D = RG::D, NW = Cfg<CT>::NW;
-    const int d = a.d, m = a.m, ldh = hist_ld(d);
+    const int d = a.d, m = a.m;
     const int count = st.count;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint64_t bytes = 0;
@@ -595,12 +619,10 @@ __device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<floa
     // instead of being held through it
     Vec<CT> g = g_in, x = x_in;
     if (count > 0) {
-        const RG ring{ldh, count, sc, reinterpret_cast<const bf16 *>(a.S) + (size_t)w * m * ldh,
-                      reinterpret_cast<const bf16 *>(a.Y) + (size_t)w * m * ldh, s_new, y_new};
         const int ng = (count + PG - 1) / PG;
-        float *mri_w = MRI + (size_t)w * m * m, *myy_w = MYY + (size_t)w * m * m, *dw = a.rho + (size_t)w * m;
-#pragma unroll
-        for (int k = 0; k < D - 1; ++k) ring.issue(k, k);
+        const int sc = ring.cn;
+        float *dw = a.rho + (size_t)w * m;
+        ring.settle(sp);
         float *p1 = L.p1();
         {
             // Pass 1 on the tensor cores: per warp (its 256 coordinates, 16 k-steps of
@@ -619,7 +641,7 @@ __device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<floa
                     make_uint4(pack2(mi[0], mi[1]), pack2(mi[2], mi[3]), pack2(mi[4], mi[5]), pack2(mi[6], mi[7]));
                 *ring.chunk(D - 1, 2) =
                     make_uint4(pack2(lo[0], lo[1]), pack2(lo[2], lo[3]), pack2(lo[4], lo[5]), pack2(lo[6], lo[7]));
-                *ring.chunk(D - 1, 3) = y_new;  // as stored
+                *ring.chunk(D - 1, 3) = ring.y_new;  // as stored; zero when there is none
             }
             __syncwarp();
             const int mi8 = lane >> 3, ri8 = lane & 7;  // ldmatrix: matrix and row this lane addresses
@@ -639,7 +661,6 @@ __device__ uint64_t direction(const LbfgsArgs<float> &a, int w, WalkerState<floa
             nk = nk < 0 ? 0 : (nk > 16 ? 16 : nk);
             const int gid = lane >> 2, tig = lane & 3;
             __syncwarp();
-            fetch_mm<CT>(L, mri_w, myy_w, dw, count, m);
             ring.issue(D - 1, D - 1);
             int sl = 0;
 #pragma unroll 1
@@ -783,6 +804,17 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
         xt.template load<EVEN>(a.XT + (size_t)w * d, d);
         gt.template load<EVEN>(a.GT + (size_t)w * d, d);
         bytes += (uint64_t)16 * d + 4 + 2 * sizeof(WalkerState<float>);
+        // Most trials are accepted with a new pair, so the first groups of the history and
+        // the m x m state are started before the trial is judged, all but the slot the
+        // pair would take (sp); they land while the vectors are read and reduced.
+        const int sp = st.count < m ? st.count : st.head;
+        Ring<CT> ring{ldh, sp < st.count ? st.count : sp + 1, sp, reinterpret_cast<const bf16 *>(a.S) + (size_t)w * m * ldh,
+                      reinterpret_cast<const bf16 *>(a.Y) + (size_t)w * m * ldh, make_uint4(0u, 0u, 0u, 0u),
+                      make_uint4(0u, 0u, 0u, 0u), false};
+        float *mri_w = MRI + (size_t)w * m * m, *myy_w = MYY + (size_t)w * m * m;
+#pragma unroll
+        for (int k = 0; k < Cfg<CT>::DB - 1; ++k) ring.issue(k, k);
+        fetch_mm<CT>(L, mri_w, myy_w, a.rho + (size_t)w * m, st.count, m);  // joins the next copy group
         // finiteness of the trial gradient, the candidate pair (as it will be stored) and its
         // inner products, and max |grad| at the trial, all in one reduction
         const uint4 s_new = pack_bf16<CT>(subv(xt, x)), y_new = pack_bf16<CT>(subv(gt, g));
@@ -795,7 +827,8 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
         const bool finite = isfinite(ft) && gm_bits < 0x7f800000u;
         const float gm = __uint_as_float(gm_bits);
         bool newiter = false;
-        int new_slot = -1;
+        ring.known = true;
+        ring.cn = -1;
         if (st.phase == 0) {
             x = xt;
             g = gt;
@@ -821,8 +854,11 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
                 store_hist(s_new, reinterpret_cast<bf16 *>(a.S) + ((size_t)w * m + slot) * ldh, ldh);
                 store_hist(y_new, reinterpret_cast<bf16 *>(a.Y) + ((size_t)w * m + slot) * ldh, ldh);
                 bytes += (uint64_t)2 * d * sizeof(bf16);
-                new_slot = slot;
+                ring.s_new = s_new;
+                ring.y_new = y_new;
+                ring.cn = slot;
             }
+            ring.J = st.count;
             st.flat = (ft >= st.f) ? st.flat + 1 : 0;
             x = xt;
             g = gt;
@@ -845,7 +881,7 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
                 st.count = 0;
                 st.head = 0;
                 st.attempt = 1;
-                bytes += direction<CT, EVEN>(a, w, st, -1, g, x, s_new, y_new, MRI, MYY, sh, L, par);
+                bytes += direction<CT, EVEN>(a, w, st, sp, g, x, ring, mri_w, myy_w, sh, L, par);
                 dnext = st.pn + alpha0 * pn0;  // from the old trial back to x, then out
             } else {
                 st.status = SB_WALKER_STALLED;
@@ -860,7 +896,7 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
                 st.status = SB_WALKER_MAXITER;
             } else {
                 st.attempt = 0;
-                bytes += direction<CT, EVEN>(a, w, st, new_slot, g, x, s_new, y_new, MRI, MYY, sh, L, par);
+                bytes += direction<CT, EVEN>(a, w, st, sp, g, x, ring, mri_w, myy_w, sh, L, par);
                 dnext = st.pn;  // x is this visit's trial
             }
         }
@@ -868,6 +904,7 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
             a.st[w] = st;
             if (a.dist && dnext >= 0.f) a.dist[w] = dnext * 1.0001f;  // margin for the rounding of |p|
         }
+        cp_async_wait_all();  // what a rejected or last trial did not use
         // No barrier before the next walker: a thread's ring chunks are read by
         // other lanes only in pass 1, behind warp barriers, and every copy group has
         // completed. The reduction scratch alternates, and every other shared array
