@@ -33,7 +33,7 @@
 // What bounds it at d = 1024, m = 20: HBM for the pairs (4.9 of 6.8 TB/s) and the
 // instructions of a visit, 2890 per warp. They were 4570 with the pairs walked in
 // the order of their age (a wrap test per row and per entry of the m x m state), one
-// FMA per coordinate and a shuffle tree per reduced value: 8192 walkers 235 us, 197 so.
+// FMA per coordinate and a shuffle tree per reduced value: 8192 walkers 235 us, 195 so.
 #include <cuda_bf16.h>
 
 #include <mutex>
@@ -823,6 +823,14 @@ __global__ void __launch_bounds__(CT, Cfg<CT>::MINB) k_lbfgs_cta(LbfgsArgs<float
         {
             const Vec<CT> s4 = unpack_bf16<CT>(s_new), y4 = unpack_bf16<CT>(y_new);
             r3 = block_sum3_max<CT>(dotv(s4, s4), dotv(y4, y4), dotv(s4, y4), gm_bits, sh.red2[par++ & 1]);
+        }
+        if (EVEN && n + (int)gridDim.x < n_act && threadIdx.x < 4) {
+            // the next walker's vectors into L2 (rows are whole 32-byte pieces); its pairs are
+            // too many for that (the solve 147 -> 157 ms with them, 132.5 -> 131.2 without)
+            const float *v = threadIdx.x == 0 ? a.X : threadIdx.x == 1 ? a.G : threadIdx.x == 2 ? a.XT : a.GT;
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(v + (size_t)w_next * d),
+                         "r"((uint32_t)d * 4u)
+                         : "memory");
         }
         const bool finite = isfinite(ft) && gm_bits < 0x7f800000u;
         const float gm = __uint_as_float(gm_bits);
