@@ -26,19 +26,17 @@
 // tr(W P_k) = <W L_k, L_k>_F. Components with r_k == 0 contribute exactly zero
 // and are skipped. H is recomputed at every mode (not stored by the forward),
 // factored H = C C^T, and C^-1 is formed once (its 32 x 32 diagonal blocks by
-// substitution, then pairs of blocks merged level by level), so that everything with W =
-// C^-T C^-1 is a product over all components at once: X_k = C^-1 L_k (lower triangular),
-// tr(W P_k) = |X_k|_F^2, the lower triangle of W L_k = C^-T X_k (added to dL_k as it
-// leaves the GEMM), and W v = C^-T (C^-1 v). At a one-hot mode (r_k = 1, the other r
+// substitution, then pairs of blocks merged level by level) for the vectors, W v = C^-T (C^-1
+// v); W L_k comes from triangular solves (k_adj_solve says why). At a one-hot mode (r_k = 1, the other r
 // exactly 0) H = P_k and C = L_k, so W L_k = L_k^-T: tr(W P_k) = d and lower[W L_k] =
-// diag(1 / L_ii), with no GEMM. Products with P_k are formed as L_k (L_k^T v); P_k itself
+// diag(1 / L_ii), with no solve. Products with P_k are formed as L_k (L_k^T v); P_k itself
 // is built only for the Hessian of a mode that is not one-hot. Nothing is read back to
 // the host: every skip is decided from R and the one-hot flag on the device. Modes go
 // through the kernels in groups (adj_group), since one mode's factor, inverse and vector
 // steps leave most of the chip idle; their shares are added to dmu and dL in mode order.
 //
 // The bound is the FP64 pipe (one warp instruction per 19 cycles and SM): per mode K d^3 /
-// 3 fused multiply-adds in the two GEMMs, d^3 / 6 each in the factor and its inverse.
+// 3 fused multiply-adds in the two solves, d^3 / 6 each in the factor and its inverse.
 #include "sb_adjoint.cuh"
 
 namespace sb {
@@ -168,115 +166,211 @@ __device__ __forceinline__ bool needs_product(const double *R, const int32_t *on
     return R[k] != 0.0 && onehot[0] < 0;
 }
 
-// Tile (I, J <= I) of the lower triangle from a flat index, the longest (J far left of a
-// low row) first.
-__device__ __forceinline__ void tile_from(int t, int nt, int &I, int &J) {
-    const int e = nt * (nt + 1) / 2 - 1 - t;
-    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-    while (i * (i + 1) / 2 > e) --i;
-    while ((i + 1) * (i + 2) / 2 <= e) ++i;
-    I = i;
-    J = i - (e - i * (i + 1) / 2);
+// W L_k = C^-T (C^-1 L_k) by triangular solves, rows from each column's own block down (the
+// lower triangle is all that is used).
+// One CTA takes 16 columns of one component and mode through both solves: per 32-row block
+// the products with the blocks solved before are subtracted one after the other (each summed
+// from zero), then the diagonal block is solved by substitution. Near a one-hot mode
+// eps / L_ii - r (W L_k)_ii and its off-diagonal part cancel to about r_j of another
+// component, 1e-5 to 1e-8 of the terms, so the rounding of these solves shows in dL_k: the
+// products with an explicit C^-1 take as long at d = 512, but their dL lies up to 1.5e-9 of
+// its norm from that of the solves.
+// Bound by the FP64 pipe: two outputs per thread; in the substitution a warp takes two columns,
+// lane = (column, row of a half block), 80 warp instructions instead of 128 with a row per
+// lane. 16 columns, not 32, because the first column tile is the longest chain of all, and
+// two CTAs per SM (unused shared memory), so that the chains, which differ in length by nb
+// squared, are dealt out as SMs come free, the longest first. d = 512, K = 4, four modes:
+// 2.0 ms (2.06 for the two products).
+constexpr int SC = 16;  // columns per CTA
+__global__ void __launch_bounds__(256) k_adj_solve(int d, int K, const double *C, const double *L, const double *R,
+                                                   const int32_t *onehot, double *X) {
+    __shared__ double As[TB][TB + 1];
+    __shared__ double Xs[TB][SC + 1];
+    __shared__ double Bs[TB][SC + 1];
+    __shared__ double inv[TB];
+    const int k = blockIdx.x % K, mo = blockIdx.x / K;
+    if (!needs_product(R + (size_t)mo * K, onehot + mo, k)) return;
+    C += (size_t)mo * d * d;
+    X += ((size_t)mo * K + k) * d * d;
+    const double *Lk = L + (size_t)k * d * d;
+    const int c0 = blockIdx.y * SC, I0 = c0 / TB, nb = (d + TB - 1) / TB;
+    const int tid = threadIdx.x, tc = tid & (SC - 1), tr = tid / SC;  // rows tr and tr + 16
+    const int lane = tid & 31, wid = tid >> 5;
+    // the block (I, J) of C, or of C^T for upper, into registers: A[i][q] of the product;
+    // and rows of X block J
+    auto load = [&](int I, int J, bool upper, double (&a)[4], double (&x)[2]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int r = (tid >> 5) + 8 * e;
+            const int gi = (upper ? J : I) * TB + r, gj = (upper ? I : J) * TB + lane;
+            a[e] = gi < d && gj < d ? C[(size_t)gi * d + gj] : 0.0;
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int gr = J * TB + tr + 16 * e;
+            x[e] = gr < d && c0 + tc < d ? X[(size_t)gr * d + c0 + tc] : 0.0;
+        }
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        const bool upper = pass;
+        for (int s = I0; s < nb; ++s) {
+            const int I = upper ? nb - 1 - (s - I0) : s, step = upper ? -1 : 1;
+            double b[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int gi = I * TB + tr + 16 * e, gc = c0 + tc;
+                b[e] = 0.0;
+                if (gi < d && gc < d) b[e] = upper ? X[(size_t)gi * d + gc] : gc <= gi ? Lk[(size_t)gi * d + gc] : 0.0;
+            }
+            double dinv = 1.0;
+            if (wid == 0 && I * TB + lane < d) dinv = 1.0 / C[(size_t)(I * TB + lane) * (d + 1)];
+            double a[4], x[2];
+            int J = upper ? nb - 1 : I0;
+            if (J != I) load(I, J, upper, a, x);
+            for (; J != I; J += step) {
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int r = (tid >> 5) + 8 * e;
+                    As[upper ? lane : r][upper ? r : lane] = a[e];
+                }
+                Xs[tr][tc] = x[0];
+                Xs[tr + 16][tc] = x[1];
+                __syncthreads();
+                if (J + step != I) load(I, J + step, upper, a, x);
+                double acc[2] = {};
+#pragma unroll
+                for (int q = 0; q < TB; ++q) {
+                    const double xq = Xs[q][tc];
+                    acc[0] = fma(As[tr][q], xq, acc[0]);
+                    acc[1] = fma(As[tr + 16][q], xq, acc[1]);
+                }
+                b[0] -= acc[0];
+                b[1] -= acc[1];
+            }
+            // the diagonal block (identity past d)
+            __syncthreads();
+            for (int e = tid; e < TB * TB; e += 256) {
+                const int r = e / TB, c = e % TB, gi = I * TB + r, gj = I * TB + c;
+                const double v = gi < d && gj < d ? C[(size_t)gi * d + gj] : r == c ? 1.0 : 0.0;
+                As[upper ? c : r][upper ? r : c] = v;
+            }
+            if (wid == 0) inv[lane] = dinv;
+            Bs[tr][tc] = b[0];
+            Bs[tr + 16][tc] = b[1];
+            __syncthreads();
+            {
+                const int col = 2 * wid + (lane >> 4), r = lane & 15, base = lane & 16;
+                double lo = Bs[r][col], hi = Bs[r + 16][col];  // rows r and r + 16
+                if (!upper) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const double xi = __shfl_sync(0xffffffffu, lo, base | i) * inv[i];
+                        const double t = fma(-As[r][i], xi, lo);
+                        lo = r == i ? xi : r > i ? t : lo;
+                        hi = fma(-As[r + 16][i], xi, hi);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const double xi = __shfl_sync(0xffffffffu, hi, base | i) * inv[i + 16];
+                        const double t = fma(-As[r + 16][i + 16], xi, hi);
+                        hi = r == i ? xi : r > i ? t : hi;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 15; i >= 0; --i) {
+                        const double xi = __shfl_sync(0xffffffffu, hi, base | i) * inv[i + 16];
+                        const double t = fma(-As[r + 16][i + 16], xi, hi);
+                        hi = r == i ? xi : r < i ? t : hi;
+                        lo = fma(-As[r][i + 16], xi, lo);
+                    }
+#pragma unroll
+                    for (int i = 15; i >= 0; --i) {
+                        const double xi = __shfl_sync(0xffffffffu, lo, base | i) * inv[i];
+                        const double t = fma(-As[r][i], xi, lo);
+                        lo = r == i ? xi : r < i ? t : lo;
+                    }
+                }
+                Bs[r][col] = lo;
+                Bs[r + 16][col] = hi;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int gi = I * TB + tr + 16 * e, gc = c0 + tc;
+                const double v = Bs[tr + 16 * e][tc];
+                if (gi < d && gc < d) X[(size_t)gi * d + gc] = v;
+            }
+            __syncthreads();  // the rows are written before a later block reads them
+        }
+    }
 }
 
-// X_k = C^-1 L_k (lower triangular) and the tile's share of |X_k|_F^2 = tr(W P_k).
-__global__ void __launch_bounds__(256) k_adj_X(int d, const double *Ci, const double *L, const double *R,
-                                               const int32_t *onehot, double *X, double *trp) {
-    __shared__ TileBuf sm;
+// tr(W P_k) = <W L_k, L_k>_F over the lower triangle, a CTA per component and mode. About d in
+// size, and at the mode's own component eps_k is what remains of it after the cancellation
+// above, so it is one sum in a fixed order, 130 us at d = 512.
+__global__ void __launch_bounds__(256) k_adj_trace(int d, int K, const double *X, const double *L, const double *R,
+                                                   const int32_t *onehot, double *tr) {
     __shared__ double sh[8];
-    const int k = blockIdx.y, mo = blockIdx.z, K = gridDim.y;
+    const int k = blockIdx.x % K, mo = blockIdx.x / K;
     if (!needs_product(R + (size_t)mo * K, onehot + mo, k)) return;
-    Ci += (size_t)mo * d * d;
-    X += (size_t)mo * K * d * d;
-    trp += (size_t)mo * K * gridDim.x;
-    int I, J;
-    tile_from(blockIdx.x, (d + TB - 1) / TB, I, J);
-    const int i0 = I * TB, j0 = J * TB;
-    const double *Lk = L + (size_t)k * d * d;
-    double acc[2][2] = {};
-    tile_gemm(
-        sm, j0, min(d, i0 + TB), acc,
-        [&](int r, int l) { return i0 + r < d && l <= i0 + r ? Ci[(size_t)(i0 + r) * d + l] : 0.0; },
-        [&](int l, int c) { return l < d && j0 + c <= l ? Lk[(size_t)l * d + j0 + c] : 0.0; });
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double ss = 0.0;
+    X += ((size_t)mo * K + k) * d * d;
+    L += (size_t)k * d * d;
+    constexpr int kBatch = 32;  // loads in flight per thread and matrix
+    const int di = 256 / d, dj = 256 % d;
+    int i = threadIdx.x / d, j = threadIdx.x % d;
+    double s = 0.0;
+    while (i < d) {
+        double a[kBatch], b[kBatch];
+        bool in[kBatch];
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
-            if (i < d && j < d) {
-                const double v = j <= i ? acc[r][c] : 0.0;
-                X[((size_t)k * d + i) * d + j] = v;
-                ss = fma(v, v, ss);
+        for (int q = 0; q < kBatch; ++q) {
+            in[q] = i < d && j <= i;
+            a[q] = in[q] ? X[(size_t)i * d + j] : 0.0;
+            b[q] = in[q] ? L[(size_t)i * d + j] : 0.0;
+            i += di;
+            j += dj;
+            if (j >= d) {
+                j -= d;
+                ++i;
             }
         }
-    ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ss;
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q)
+            if (__any_sync(__activemask(), in[q])) s = in[q] ? fma(a[q], b[q], s) : s;
+    }
+    __syncwarp();
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
         for (int w = 0; w < 8; ++w) t += sh[w];
-        trp[(size_t)k * gridDim.x + blockIdx.x] = t;
+        tr[blockIdx.x] = t;
     }
 }
 
 // dL_k += pi lower[ eps (diag(1/L) - delta z^T) - gam z^T - delta u^T - r W L_k ] with u =
-// L^T gam and the tile of W L_k = C^-T X_k formed here (at a one-hot mode lower[W L_k] =
-// diag(1 / L_ii)).
+// L^T gam (at a one-hot mode lower[W L_k] = diag(1 / L_ii)), the modes in order.
 __global__ void __launch_bounds__(256) k_adj_dL(int d, int nm, const double *pi, const double *R, const double *eps,
                                                 const int32_t *onehot, const double *L, const double *x,
                                                 const double *mu, const double *Z, const double *gam,
-                                                const double *U, const double *Ci, const double *X, double *dL) {
-    __shared__ TileBuf sm;
-    const int k = blockIdx.y, K = gridDim.y;
-    int I, J;
-    tile_from(gridDim.x - 1 - blockIdx.x, (d + TB - 1) / TB, I, J);  // here the top rows are the longest
-    const int i0 = I * TB, j0 = J * TB;
-    const double *Lk = L + (size_t)k * d * d;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double sum[2][2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
-            sum[r][c] = i < d && j <= i ? dL[(size_t)k * d * d + (size_t)i * d + j] : 0.0;
-        }
+                                                const double *U, const double *X, double *dL) {
+    const int k = blockIdx.z, K = gridDim.z, i = blockIdx.y, j = blockIdx.x * 256 + threadIdx.x;
+    if (j > i) return;
+    const size_t e = (size_t)i * d + j, ek = (size_t)k * d * d + e;
+    double sum = dL[ek];
     for (int mo = 0; mo < nm; ++mo) {
         const size_t mk = (size_t)mo * K + k, kd = mk * d;
         const double rk = R[mk];
         if (rk == 0.0) continue;
-        const double *Cm = Ci + (size_t)mo * d * d, *Xk = X + mk * d * d;
-        const bool oh = onehot[mo] >= 0;
-        double acc[2][2] = {};
-        if (!oh)
-            tile_gemm(
-                sm, i0, d, acc,
-                [&](int r, int l) { return l < d && i0 + r <= l ? Cm[(size_t)l * d + i0 + r] : 0.0; },
-                [&](int l, int c) { return l < d && j0 + c < d ? Xk[(size_t)l * d + j0 + c] : 0.0; });
-        const double p = pi[mo], ek = eps[mk];
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
-                if (i >= d || j > i) continue;
-                const size_t e = (size_t)i * d + j;
-                const double di = x[(size_t)mo * d + i] - mu[(size_t)k * d + i], zj = Z[kd + j];
-                const double wl = oh ? (i == j ? 1.0 / Lk[e] : 0.0) : acc[r][c];
-                double v = -ek * di * zj - gam[kd + i] * zj - di * U[kd + j] - rk * wl;
-                if (i == j) v += ek / Lk[e];
-                sum[r][c] += p * v;
-            }
+        const double ep = eps[mk], di = x[(size_t)mo * d + i] - mu[(size_t)k * d + i], zj = Z[kd + j];
+        const double wl = onehot[mo] >= 0 ? (i == j ? 1.0 / L[ek] : 0.0) : X[mk * d * d + e];
+        double v = -ep * di * zj - gam[kd + i] * zj - di * U[kd + j] - rk * wl;
+        if (i == j) v += ep / L[ek];
+        sum += pi[mo] * v;
     }
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
-            if (i < d && j <= i) dL[(size_t)k * d * d + (size_t)i * d + j] = sum[r][c];
-        }
+    dL[ek] = sum;
 }
 
 // ------------------------------------------------------------------ per-mode vector algebra
@@ -365,10 +459,10 @@ __global__ void __launch_bounds__(256) k_adj_upper(int d, VecArgs a, bool diff) 
     }
 }
 
-// One CTA of 1024 threads per mode: given WV (rows W g_0 .. W g_{K-1}, W gbar) and the partials of
+// One CTA of 1024 threads per mode: given WV (rows W g_0 .. W g_{K-1}, W gbar) and
 // tr(W P_k), form t (stage 0), or with Wt known form eps and gam (stage 1). A warp per
 // component for the inner products.
-__global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, int n_part, const double *R,
+__global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, const double *R,
                                                     const int32_t *onehot, const double *GK, const double *gbar,
                                                     const double *WV, const double *trp, const double *PY,
                                                     const double *Wt, double *t_out, double *eps, double *gam) {
@@ -378,7 +472,7 @@ __global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, int
     GK += (size_t)mo * K * d;
     gbar += (size_t)mo * d;
     WV += (size_t)mo * (K + 1) * d;
-    trp += (size_t)mo * K * n_part;
+    trp += (size_t)mo * K;
     PY += (size_t)mo * K * d;
     if (stage == 0) {
         t_out += (size_t)mo * d;
@@ -394,17 +488,15 @@ __global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, int
         double beta = 0.0;
         if (R[k] != 0.0) {
             const double *gk = GK + (size_t)k * d, *wgk = WV + (size_t)k * d;
-            double a1 = 0.0, a2 = 0.0, tr = 0.0;
+            double a1 = 0.0, a2 = 0.0;
             for (int i = lane; i < d; i += 32) {
                 a1 = fma(gk[i], wgk[i], a1);  // g_k^T W g_k
                 // gbar^T W g_k, or c^T g_k with c = -W gbar - W t / 2
                 a2 = stage == 0 ? fma(gbar[i], wgk[i], a2) : fma(fma(-0.5, Wt[i], -Wg[i]), gk[i], a2);
             }
-            if (!oh)
-                for (int q = lane; q < n_part; q += 32) tr += trp[(size_t)k * n_part + q];
             a1 = warp_sum(a1);
             a2 = warp_sum(a2);
-            tr = oh ? (double)d : warp_sum(tr);
+            const double tr = oh ? (double)d : trp[k];
             beta = stage == 0 ? (tr - a1 + 2.0 * a2) : (-0.5 * (tr - a1) + a2);
         }
         if (lane == 0) s_beta[k] = beta;
@@ -462,7 +554,7 @@ void adjoint_carve(Carver &cv, AdjWs &w, int d, int K) {
     w.Ci = cv.take<double>(g * dd);
     w.T2 = cv.take<double>(g * dd);
     w.X = cv.take<double>(g * K * dd);
-    w.trp = cv.take<double>(g * K * nt * (nt + 1) / 2);
+    w.trp = cv.take<double>(g * K);
     w.Z = cv.take<double>(g * K * d);
     w.R = cv.take<double>(g * K);
     w.qpart = cv.take<double>(g * K * nJT);
@@ -499,15 +591,11 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
     SB_CUDA_TRY(cudaMemsetAsync(w.p_done, 0, sizeof(int32_t) * kMaxK, s));
     note_launch();
     k_softmax_pi<<<1, 32, 0, s>>>(n_modes, logZk, grad_logZ, w.pi);
-    const int nt = (d + TB - 1) / TB, tiles = nt * (nt + 1) / 2;
+    const int tiles = (d + SC - 1) / SC;
     const unsigned rows8 = (unsigned)((d + 7) / 8), cols32 = (unsigned)((d + 31) / 32);
     const size_t dd = (size_t)d * d, dK = (size_t)d * K, dV = (size_t)d * (K + 1);
-    // unused shared memory holds an SM to two CTAs of the GEMMs, so that their tiles, up to
-    // nt times different in length, are dealt out as SMs come free (d = 512, K = 4: 390 us per
-    // mode with every tile resident at once, 206 so)
-    constexpr int kPad = 80 * 1024;
-    SB_CUDA_TRY(cudaFuncSetAttribute(k_adj_X, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad));
-    SB_CUDA_TRY(cudaFuncSetAttribute(k_adj_dL, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad));
+    constexpr int kPad = 80 * 1024;  // two CTAs of k_adj_solve per SM
+    SB_CUDA_TRY(cudaFuncSetAttribute(k_adj_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad));
     for (int m0 = 0; m0 < n_modes; m0 += group) {
         const int nm = n_modes - m0 < group ? n_modes - m0 : group;
         const double *x = modes + (size_t)m0 * d;
@@ -542,32 +630,34 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
         launch_onehot(K, w.R, w.count, nm, w.onehot, s);
         launch_precision_needed(d, K, pv.L, w.R, w.count, w.p_done, w.p_need, w.P, s, w.onehot);
         launch_hessian_chol(d, K, nm, pv.L, w.P, w.Z, w.R, w.gbar, w.count, w.GK, w.H, w.info, w.bar, pv.status, s,
-                            w.onehot);
+                            w.onehot, true);
         launch_tri_inverse(d, nm, w.H, w.Ci, w.T2, s);
         // W [g_0 .. g_{K-1}, gbar]; X_k = C^-1 L_k and tr(W P_k)
         note_launch();
         k_pack_rhs<<<dim3((d + 255) / 256, K + 1, nm), 256, 0, s>>>(d, K, w.GK, w.gbar, w.R, w.V);
         apply_W(K + 1, w.V, dV, w.WV, dV, w.R);
         note_launch();
-        k_adj_X<<<dim3(tiles, K, nm), 256, kPad, s>>>(d, w.Ci, pv.L, w.R, w.onehot, w.X, w.trp);
+        k_adj_solve<<<dim3(K * nm, tiles), 256, kPad, s>>>(d, K, w.H, pv.L, w.R, w.onehot, w.X);
+        note_launch();
+        k_adj_trace<<<K * nm, 256, 0, s>>>(d, K, w.X, pv.L, w.R, w.onehot, w.trp);
         // P_k (W gbar - W g_k) = L_k (L_k^T (W gbar - W g_k))
         note_launch(2);
         k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.WV, dV, w.R, K, w.U, dK}, true);
         k_adj_lower<<<dim3(rows8, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.U, dK, w.R, K, w.PY, dK});
         // t = grad_x log det H, then v = W t (into V), then c, eps_k, gam_k
         note_launch();
-        k_adj_stage<<<nm, 1024, 0, s>>>(0, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, nullptr, w.T,
+        k_adj_stage<<<nm, 1024, 0, s>>>(0, d, K, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, nullptr, w.T,
                                         nullptr, nullptr);
         apply_W(1, w.T, d, w.V, d, nullptr);
         note_launch();
-        k_adj_stage<<<nm, 1024, 0, s>>>(1, d, K, tiles, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, w.V, nullptr,
+        k_adj_stage<<<nm, 1024, 0, s>>>(1, d, K, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, w.V, nullptr,
                                         w.eps, w.gam);
         // u_k = L_k^T gam_k, dmu_k += pi (-eps_k g_k + L_k u_k), dL_k
         note_launch(3);
         k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.gam, dK, w.R, K, w.U, dK}, false);
         k_adj_dmu<<<dim3(rows8, K), 256, 0, s>>>(d, nm, pv.L, w.U, w.R, pi, w.eps, w.GK, dmu);
-        k_adj_dL<<<dim3(tiles, K), 256, kPad, s>>>(d, nm, pi, w.R, w.eps, w.onehot, pv.L, x, pv.mu, w.Z, w.gam, w.U,
-                                                   w.Ci, w.X, dL);
+        k_adj_dL<<<dim3((d + 255) / 256, d, K), 256, 0, s>>>(d, nm, pi, w.R, w.eps, w.onehot, pv.L, x, pv.mu, w.Z,
+                                                             w.gam, w.U, w.X, dL);
     }
     SB_CUDA_TRY(cudaGetLastError());
     SB_CUDA_TRY(cudaStreamSynchronize(s));  // the call returns with its results written

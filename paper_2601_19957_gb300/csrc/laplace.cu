@@ -401,6 +401,17 @@ __device__ __forceinline__ double recip(double p) {
     return fma(r, fma(d, d, d), r);
 }
 
+// EXACT: with the last bit corrected
+template <bool EXACT>
+__device__ __forceinline__ double recip_as(double p) {
+    const double r = recip(p);
+    return EXACT ? fma(r, fma(-p, r, 1.0), r) : r;
+}
+
+// EXACT in the functions below (the adjoint, whose dL_k can be 1e-8 of the terms it is the
+// difference of): reciprocals as a division rounds them, and updates a_ik -= (a_ij a_kj) /
+// a_jj with the product rounded first, one instruction more per column.
+//
 // Diagonal block kb: A[kb][kb] -= A[kb][kb-1] A[kb][kb-1]^T (upd, the trailing update of the
 // step before), then its factor. Threads 0..127 hold the block in registers: lane = row i,
 // warp q the columns q, q + 4, ... Step j: the owner warp of column j publishes it unscaled
@@ -408,6 +419,7 @@ __device__ __forceinline__ double recip(double p) {
 // its later columns, a_ik -= (a_ij / a_jj) a_kj. Columns are scaled by 1 / sqrt(a_jj) at the
 // end, all square roots at once. A pivot <= 0 (not positive definite) sets the candidate's
 // info flag (read by every CTA after the next barrier).
+template <bool EXACT>
 __device__ void diag_block(int d, int kb, bool upd, double *A, int32_t *info_c) {
     __shared__ double a[NB][NB + 1];
     __shared__ double pa[NB][NB + 1];
@@ -452,14 +464,15 @@ __device__ void diag_block(int d, int kb, bool upd, double *A, int32_t *info_c) 
                         if (__double_as_longlong(p) <= 0 || p != p) s_bad = 1;
                     }
                     col[sl][i] = x[t0];
-                    mul[sl][i] = x[t0] * recip(p);
+                    mul[sl][i] = EXACT ? recip_as<true>(p) : x[t0] * recip(p);
                 }
                 asm volatile("bar.sync 1, 128;" ::: "memory");
-                const double m = mul[sl][i];
+                const double m = mul[sl][i], ci = EXACT ? col[sl][i] : 0.0;
                 // the column the next step needs comes first
 #pragma unroll
                 for (int t = 0; t < NB / 4; ++t)
-                    if (t > t0 || (t == t0 && q > qo)) x[t] = fma(-m, col[sl][4 * t + q], x[t]);
+                    if (t > t0 || (t == t0 && q > qo))
+                        x[t] = EXACT ? fma(-(ci * col[sl][4 * t + q]), m, x[t]) : fma(-m, col[sl][4 * t + q], x[t]);
             }
         }
 #pragma unroll
@@ -487,6 +500,7 @@ __device__ void diag_block(int d, int kb, bool upd, double *A, int32_t *info_c) 
 // updates its later columns, two on average (16 rows, not 32, because a warp instruction
 // takes its 64 cycles whatever the lanes: eight parts a row halve the chain).
 constexpr int TRSM_THREADS = 128, TRSM_ROWS = 16;
+template <bool EXACT>
 __device__ void trsm_block(int d, int kb, int r0, double *A) {
     __shared__ double l[NB][NB + 1];
     __shared__ double xs[TRSM_ROWS][NB + 1];
@@ -497,7 +511,7 @@ __device__ void trsm_block(int d, int kb, int r0, double *A) {
         l[i][j] = (o + i < d && o + j < d) ? __ldcg(&A[(size_t)(o + i) * d + o + j]) : (i == j ? 1.0 : 0.0);
     }
     __syncthreads();
-    if (threadIdx.x < NB) inv[threadIdx.x] = recip(l[threadIdx.x][threadIdx.x]);
+    if (threadIdx.x < NB) inv[threadIdx.x] = recip_as<EXACT>(l[threadIdx.x][threadIdx.x]);
     const int r = threadIdx.x & (TRSM_ROWS - 1), part = threadIdx.x / TRSM_ROWS;  // parts 0..7
     const int row = r0 + r;
     double x[NB / 8];
@@ -562,6 +576,7 @@ __device__ __forceinline__ bool chol_live(int c, const int32_t *onehot, const in
     return !(onehot && onehot[c] >= 0) && *reinterpret_cast<const volatile int32_t *>(&info[c]) == 0;
 }
 
+template <bool EXACT>
 __global__ void __launch_bounds__(CF_THREADS) k_chol_coop(int d, double *H, const int32_t *n_c,
                                                          const int32_t *onehot, int32_t *info, uint32_t *bar,
                                                          int32_t *err) {
@@ -575,20 +590,20 @@ __global__ void __launch_bounds__(CF_THREADS) k_chol_coop(int d, double *H, cons
     }
     const int nblk = (d + NB - 1) / NB;
     for (int c = blockIdx.x; c < nc; c += gridDim.x)
-        if (chol_live(c, onehot, info)) diag_block(d, 0, false, H + (size_t)c * d * d, info + c);
+        if (chol_live(c, onehot, info)) diag_block<EXACT>(d, 0, false, H + (size_t)c * d * d, info + c);
     if (!grid_barrier(bar, gridDim.x, err)) return;
     for (int kb = 0; kb + 1 < nblk; ++kb) {
         const int rest = nblk - kb - 1;
         for (int it = blockIdx.x; it < nc * 2 * rest; it += gridDim.x) {
             const int c = it / (2 * rest);
             if (chol_live(c, onehot, info))
-                trsm_block(d, kb, (kb + 1) * NB + (it % (2 * rest)) * TRSM_ROWS, H + (size_t)c * d * d);
+                trsm_block<EXACT>(d, kb, (kb + 1) * NB + (it % (2 * rest)) * TRSM_ROWS, H + (size_t)c * d * d);
         }
         if (!grid_barrier(bar, gridDim.x, err)) return;
         // the next diagonal block of every candidate is updated and factored at once, by
         // the first CTAs; the other trailing blocks (ii >= jj, ii > 0) go to the rest
         for (int c = blockIdx.x; c < nc; c += gridDim.x)
-            if (chol_live(c, onehot, info)) diag_block(d, kb + 1, true, H + (size_t)c * d * d, info + c);
+            if (chol_live(c, onehot, info)) diag_block<EXACT>(d, kb + 1, true, H + (size_t)c * d * d, info + c);
         const int tri = rest * (rest + 1) / 2 - 1;
         const int skip = (int)gridDim.x > 2 * nc ? nc : 0;  // CTAs that only factor in this phase
         const int b = (int)blockIdx.x - skip, nb = (int)gridDim.x - skip;
@@ -1049,7 +1064,7 @@ int laplace_sms();
 
 void launch_hessian_chol(int d, int K, int cap, const double *L, const double *P, const double *Z, const double *R,
                          const double *gbar, const int32_t *n_c, double *GK, double *H, int32_t *info,
-                         uint32_t *bar, int32_t *err, cudaStream_t s, const int32_t *onehot) {
+                         uint32_t *bar, int32_t *err, cudaStream_t s, const int32_t *onehot, bool exact) {
     note_launch();
     k_comp_grads<<<dim3(cap, K, kGradSlices), 256, sizeof(double) * d, s>>>(d, K, L, Z, R, n_c, GK);
     const int64_t dd = (int64_t)d * d;
@@ -1067,7 +1082,7 @@ void launch_hessian_chol(int d, int K, int cap, const double *L, const double *P
         cudaMemsetAsync(bar, 0, 2 * sizeof(uint32_t), fs);
         void *args[] = {&d, &H, &n_c, &onehot, &info, &bar, &err};
         note_launch();
-        cudaLaunchCooperativeKernel((const void *)k_chol_coop, dim3(G), dim3(CF_THREADS), args, 0, fs);
+        cudaLaunchCooperativeKernel((const void *)(exact ? k_chol_coop<true> : k_chol_coop<false>), dim3(G), dim3(CF_THREADS), args, 0, fs);
     };
     // (the kernel leaves at once when every live candidate is one-hot)
     factor(s);
