@@ -1230,10 +1230,30 @@ sb_status run_chisao(const Prelude &P, const sb_config *c, const sb_chisao_confi
             if (st != SB_OK) return st;
             launch_cs_ray_pick(0, n, c->n_steps, d, w.rows, w.state, w.ellp, w.lost_list, w.O, w.U, w.texit, w.X, s);
         }
-        for (int l0 = 0; !mixed && l0 < n; l0 += w.lc) {
-            const int lc = n - l0 < w.lc ? n - l0 : w.lc;
+        // Small problems form the samples of a ray in registers, so a chunk is as many rays as
+        // have room for l at their samples in V and G (written anew below), usually all of
+        // them: 4096 rays of 128 samples at d = 64 in 3 launches, not 128 x 4 (the solve
+        // 46.2 -> 43.0 ms).
+        const bool small = !mixed && small_f64_fits(d, pv.K, 0);
+        const int64_t room = 2 * (int64_t)n * d, fit = (room < (1 << 30) ? room : 1 << 30) / c->n_steps;
+        const int per = !small || fit < w.lc ? w.lc : fit < n ? (int)fit : n;
+        double *ellp = small && fit >= w.lc ? w.V : w.ellp;
+        for (int l0 = 0; !mixed && l0 < n; l0 += per) {
+            const int lc = n - l0 < per ? n - l0 : per;
             launch_cs_chunk_rows(w.cnt, w.state, l0, lc, c->n_steps, w.rows, s);
-            {
+            if (small) {
+                LikF64Args a = f64_args(pv);
+                a.c = w.O + (size_t)l0 * d;
+                a.c_ld = d;
+                a.u = w.U + (size_t)l0 * d;
+                a.texit = w.texit + l0;
+                a.n_steps = c->n_steps;
+                a.n_rows = lc * c->n_steps;
+                a.n_rows_dev = w.rows;
+                a.ell = ellp;
+                a.out_by_walker = 0;
+                launch_lik_f64_rays(a, s);
+            } else {
                 launch_cs_ray_points(l0, lc, c->n_steps, d, w.O, w.U, w.texit, w.rows, w.P, s);
                 LikF64Args a = f64_args(pv);
                 a.X = w.P;
@@ -1244,8 +1264,7 @@ sb_status run_chisao(const Prelude &P, const sb_config *c, const sb_chisao_confi
                 a.out_by_walker = 0;
                 launch_lik_f64_points(a, false, s);
             }
-            launch_cs_ray_pick(l0, lc, c->n_steps, d, w.rows, w.state, w.ellp, w.lost_list, w.O, w.U, w.texit, w.X,
-                               s);
+            launch_cs_ray_pick(l0, lc, c->n_steps, d, w.rows, w.state, ellp, w.lost_list, w.O, w.U, w.texit, w.X, s);
         }
         // anti-convergence of every sample that is not stuck (the moving list)
         if (cc->anti_steps > 0) {

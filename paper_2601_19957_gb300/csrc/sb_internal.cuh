@@ -255,7 +255,8 @@ struct LikF64Args {
     // ray source
     const double *u;          // [n_rays][d]
     const double *texit;      // [n_rays]
-    const double *c;          // [d]
+    const double *c;          // [d], or [n_rays][c_ld] when c_ld > 0 (small problems only)
+    int c_ld;
     int n_steps;
     int64_t flat0;            // first flat sample index of the chunk
     // outputs

@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) k_small_points(LikF64Args a, i
         const int out = a.out_by_walker ? w : n;
         double x[VPL], g[VPL], ell, t = 0.0;
         int r = 0;
-        if (RAYS && on) {  // x = c + t_j t_exit u_r, t_j = (j + 1) / n_steps
+        if (RAYS && on) {  // x = c + t_j t_exit u_r, t_j = (j + 1) / n_steps (c_ld: the ray's own c)
             const int64_t flat = a.flat0 + n;
             r = (int)(flat / a.n_steps);
             t = mul_rn(div_rn((double)(flat - (int64_t)r * a.n_steps + 1), (double)a.n_steps), a.texit[r]);
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) k_small_points(LikF64Args a, i
         for (int v = 0; v < VPL; ++v) {
             const int i = l + LPW * v;
             x[v] = 0.0;
-            if (on && i < a.d) x[v] = RAYS ? add_rn(a.c[i], mul_rn(t, a.u[(size_t)r * a.d + i])) : a.X[(size_t)w * a.d + i];
+            if (on && i < a.d) x[v] = RAYS ? add_rn(a.c[(size_t)r * a.c_ld + i], mul_rn(t, a.u[(size_t)r * a.d + i])) : a.X[(size_t)w * a.d + i];
         }
         evaluate<LPW, VPL>(P, x, on, lead, buf, a.Z ? a.Z + (size_t)(on ? out : 0) * a.K * a.d : nullptr,
                            a.G != nullptr, ell, g);
