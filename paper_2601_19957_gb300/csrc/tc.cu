@@ -1819,11 +1819,13 @@ __global__ void __launch_bounds__(256) k_q_sum(int n_rk, int n_ntile, const floa
 // decides which terms can matter: with the coefficients rounded to FP32 a term is off by at
 // most 2^-21 of |c0| + tau |c1| + tau^2 |c2|, and a component that stays 110 nats below the
 // largest lower bound adds an FP32 exponential of exactly 0. A CTA takes RB rays at a time
-// by JW samples and QE_PASS times that, so that (j + 1) / n_steps is divided once per thread.
+// by JW samples and up to QE_PASS times that, so that (j + 1) / n_steps is divided once per
+// thread; fewer passes where there are not four CTAs per SM with them (181 rays x 28 samples:
+// 18 us in eight passes, 8 in one).
 // Every term in FP64, twice, and a division per sample: 196 us at 16384 rays x 64 samples,
 // K = 8, 28 us now. (ns_dev given: samples past *ns_dev are skipped)
 constexpr int QE_PASS = 8;
-__global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, int JW, const double *co,
+__global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, int JW, int passes, const double *co,
                                                const float4 *cf, const double *texit, double *ell,
                                                const int32_t *ns_dev) {
     const int nj = (n_steps + JW - 1) / JW, rb = blockIdx.x / nj;
@@ -1831,8 +1833,8 @@ __global__ void __launch_bounds__(256) k_q_ell(int n_rays, int n_steps, int K, i
     if (j >= n_steps) return;
     const int64_t ns = ns_dev ? *ns_dev : (int64_t)n_rays * n_steps;
     const double tf64 = (double)(j + 1) / (double)n_steps;
-    int r = rb * RB * QE_PASS + threadIdx.x / JW;
-    for (int p = 0; p < QE_PASS; ++p, r += RB) {
+    int r = rb * RB * passes + threadIdx.x / JW;
+    for (int p = 0; p < passes; ++p, r += RB) {
         const int64_t e = (int64_t)r * n_steps + j;
         if (r >= n_rays || e >= ns) return;
         const double tau = tf64 * texit[r];
@@ -1868,10 +1870,12 @@ void launch_q_ell(int n_rays, int n_steps, int K, const TcQuadWs &q, const doubl
                   const int32_t *ns_dev, cudaStream_t s) {
     int JW = 32;
     while (JW < 256 && JW < n_steps) JW *= 2;
-    const int rays = 256 / JW * QE_PASS;
+    const int RB = 256 / JW;
+    const int64_t nj = (n_steps + JW - 1) / JW, one = (int64_t)((n_rays + RB - 1) / RB) * nj / (4 * num_sms());
+    const int passes = one < 1 ? 1 : one < QE_PASS ? (int)one : QE_PASS, rays = RB * passes;
     note_launch();
-    const int64_t grid = (int64_t)((n_rays + rays - 1) / rays) * ((n_steps + JW - 1) / JW);
-    k_q_ell<<<(unsigned)grid, 256, 0, s>>>(n_rays, n_steps, K, JW, q.co, q.cf, texit, ell, ns_dev);
+    const int64_t grid = (int64_t)((n_rays + rays - 1) / rays) * nj;
+    k_q_ell<<<(unsigned)grid, 256, 0, s>>>(n_rays, n_steps, K, JW, passes, q.co, q.cf, texit, ell, ns_dev);
 }
 
 void launch_q_split_LT(const ProbView &pv, int prec, const TcQuadWs &q, cudaStream_t s) {
