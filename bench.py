@@ -27,10 +27,10 @@ sys.path.insert(0, ROOT)
 
 # DRAM bytes per algorithmic byte of the L-BFGS step with bf16 pairs: ncu
 # dram__bytes_read.sum + dram__bytes_write.sum of step launches 40-42 of a solve at
-# d=1024, K=8, 8192 walkers (2.831 GB in all) against the step's own algorithmic-byte
+# d=1024, K=8, 8192 walkers (2.930 GB in all) against the step's own algorithmic-byte
 # count for the same three launches (4.889 GB). The second pass of the two-loop
 # recursion is served by the shared-memory ring (the newest groups) and L2.
-LBFGS_DRAM_PER_ALGORITHMIC_BYTE = 0.579
+LBFGS_DRAM_PER_ALGORITHMIC_BYTE = 0.599
 
 METRIC = "logL+grad evals/sec and evidence solves/sec at d=1024 K=8 vs plain FP64 GPU; |ΔlogZ|"
 PREC = {"fp64": 0, "tf32": 1, "bf16": 2}
