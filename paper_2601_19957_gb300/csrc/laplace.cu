@@ -418,7 +418,7 @@ __device__ __forceinline__ double recip_as(double p) {
 // and as the multipliers a_ij / a_jj, one barrier of the four warps, and every warp updates
 // its later columns, a_ik -= (a_ij / a_jj) a_kj. Columns are scaled by 1 / sqrt(a_jj) at the
 // end, all square roots at once. A pivot <= 0 (not positive definite) sets the candidate's
-// info flag (read by every CTA after the next barrier).
+// info to 1 + kb (see chol_live).
 template <bool EXACT>
 __device__ void diag_block(int d, int kb, bool upd, double *A, int32_t *info_c) {
     __shared__ double a[NB][NB + 1];
@@ -481,7 +481,7 @@ __device__ void diag_block(int d, int kb, bool upd, double *A, int32_t *info_c) 
     }
     __syncthreads();
     if (s_bad) {
-        if (tid == 0) *info_c = 1;
+        if (tid == 0) *info_c = 1 + kb;
         __syncthreads();
         return;
     }
@@ -569,11 +569,15 @@ __device__ void syrk_block(int d, int kb, int ib, int jb, double *A) {
     __syncthreads();  // the shared blocks are free for the next item
 }
 
-// Whether candidate c is factored here: live, not failed, and not one-hot (a one-hot
-// candidate's factor is L_k, copied in place by k_hessian). info[c] is read after a
-// grid barrier, so every CTA sees the same value.
-__device__ __forceinline__ bool chol_live(int c, const int32_t *onehot, const int32_t *info) {
-    return !(onehot && onehot[c] >= 0) && *reinterpret_cast<const volatile int32_t *>(&info[c]) == 0;
+// Whether candidate c still takes part in block step kb: not one-hot (a one-hot candidate's
+// factor is L_k, copied in place by k_hessian), and no diagonal block up to kb failed. info[c]
+// is 0, or 1 + the block that failed. Block kb + 1 is factored beside this step's trailing
+// updates, so a reader may see info[c] = 0 or kb + 2 there, in one warp the one and in the
+// next the other: both mean "takes part" (its update of the failed candidate is not used),
+// so that every thread of a CTA takes the same branch around the block barriers.
+__device__ __forceinline__ bool chol_live(int c, int kb, const int32_t *onehot, const int32_t *info) {
+    const int32_t failed = *reinterpret_cast<const volatile int32_t *>(&info[c]);
+    return !(onehot && onehot[c] >= 0) && (failed == 0 || failed > kb + 1);
 }
 
 template <bool EXACT>
@@ -590,26 +594,26 @@ __global__ void __launch_bounds__(CF_THREADS) k_chol_coop(int d, double *H, cons
     }
     const int nblk = (d + NB - 1) / NB;
     for (int c = blockIdx.x; c < nc; c += gridDim.x)
-        if (chol_live(c, onehot, info)) diag_block<EXACT>(d, 0, false, H + (size_t)c * d * d, info + c);
+        if (chol_live(c, 0, onehot, info)) diag_block<EXACT>(d, 0, false, H + (size_t)c * d * d, info + c);
     if (!grid_barrier(bar, gridDim.x, err)) return;
     for (int kb = 0; kb + 1 < nblk; ++kb) {
         const int rest = nblk - kb - 1;
         for (int it = blockIdx.x; it < nc * 2 * rest; it += gridDim.x) {
             const int c = it / (2 * rest);
-            if (chol_live(c, onehot, info))
+            if (chol_live(c, kb, onehot, info))
                 trsm_block<EXACT>(d, kb, (kb + 1) * NB + (it % (2 * rest)) * TRSM_ROWS, H + (size_t)c * d * d);
         }
         if (!grid_barrier(bar, gridDim.x, err)) return;
         // the next diagonal block of every candidate is updated and factored at once, by
         // the first CTAs; the other trailing blocks (ii >= jj, ii > 0) go to the rest
         for (int c = blockIdx.x; c < nc; c += gridDim.x)
-            if (chol_live(c, onehot, info)) diag_block<EXACT>(d, kb + 1, true, H + (size_t)c * d * d, info + c);
+            if (chol_live(c, kb, onehot, info)) diag_block<EXACT>(d, kb + 1, true, H + (size_t)c * d * d, info + c);
         const int tri = rest * (rest + 1) / 2 - 1;
         const int skip = (int)gridDim.x > 2 * nc ? nc : 0;  // CTAs that only factor in this phase
         const int b = (int)blockIdx.x - skip, nb = (int)gridDim.x - skip;
         for (int it = b; b >= 0 && it < nc * tri; it += nb) {
             const int c = it / tri, e = it - c * tri + 1;
-            if (!chol_live(c, onehot, info)) continue;
+            if (!chol_live(c, kb, onehot, info)) continue;
             int ii = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
             while (ii * (ii + 1) / 2 > e) --ii;
             while ((ii + 1) * (ii + 2) / 2 <= e) ++ii;
