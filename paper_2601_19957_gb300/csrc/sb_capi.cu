@@ -918,12 +918,7 @@ extern "C" sb_status sb_loglik(const sb_problem *p, int32_t prec, const double *
         double *R = cv.take<double>((size_t)n * p->K);
         int32_t *grp = ws_bytes < sb::loglik_bytes(p, prec, n, true) ? nullptr
                                                                      : cv.take<int32_t>(lik_f64_group_elems(p->K, n));
-        // setup needs c/half/logV/wmax only for box work; give it scratch inside Z (overwritten later)
-        pv.c = Z;
-        pv.half = Z + p->d;
-        pv.logV = Z + 2 * p->d;
-        pv.wmax = Z + 2 * p->d + 1;
-        launch_setup(pv, s);
+        launch_setup(pv, s);  // a_k and the checks: the box's constants (c, half, logV, wmax) are not needed
         LikF64Args la = f64_args(pv);
         la.X = x;
         la.n_rows = n;

@@ -30,7 +30,8 @@ __device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v)
 
 constexpr int kCheckRows = 8;  // rows of L per checking CTA (a warp each)
 
-// Blocks 0 .. K: the box (block 0) and component k = block - 1. Blocks beyond: finiteness
+// Blocks 0 .. K: the box (block 0; its constants are left out where pv.c, pv.half, pv.logV and
+// pv.wmax are null, its checks are not) and component k = block - 1. Blocks beyond: finiteness
 // of the lower triangles of all L_k, a warp per row, eight loads in flight per lane; it
 // reads only the triangle (33.6 MB at d = 1024, K = 8: 5 us of HBM) and addresses by row,
 // where a flat pass over the squares paid a 64-bit division per element.
@@ -65,8 +66,10 @@ __global__ void __launch_bounds__(256) k_setup(ProbView pv) {
             const double w = hi - lo;
             if (not_finite(lo) || not_finite(hi)) bad |= SB_DEV_NONFINITE;
             if (not_positive(w)) bad |= SB_DEV_INVALID;
-            pv.c[i] = 0.5 * (lo + hi);
-            pv.half[i] = 0.5 * (hi - lo);
+            if (pv.c) {
+                pv.c[i] = 0.5 * (lo + hi);
+                pv.half[i] = 0.5 * (hi - lo);
+            }
             lsum += log(w);
             const long long wb = __double_as_longlong(w);
             if (w == w && wb > wmax) wmax = wb;
@@ -81,8 +84,10 @@ __global__ void __launch_bounds__(256) k_setup(ProbView pv) {
         const int inv = __syncthreads_or(bad & SB_DEV_INVALID), nf = __syncthreads_or(bad & SB_DEV_NONFINITE);
         if (threadIdx.x == 0) {
             for (int w = 0; w < 8; ++w) wmax = shl[w] > wmax ? shl[w] : wmax;
-            pv.logV[0] = lsum;
-            pv.wmax[0] = __longlong_as_double(wmax);
+            if (pv.logV) {
+                pv.logV[0] = lsum;
+                pv.wmax[0] = __longlong_as_double(wmax);
+            }
             if (inv || nf) atomicOr(pv.status, (inv ? SB_DEV_INVALID : 0) | (nf ? SB_DEV_NONFINITE : 0));
         }
     } else {
