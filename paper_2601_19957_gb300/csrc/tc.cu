@@ -1602,8 +1602,10 @@ __device__ __forceinline__ void split_store(void *A2, size_t e, int dK, double x
 // for the ray's exit length from the box centre, min_i half_i / |u_i| as warp_exit_min (the
 // exact FP64 minimum): FP32 quotients of the truncated operands are within 2^-21, so when a
 // single one lies within 2^-18 of the smallest, its index is left in arg and one FP64
-// division per ray remains; otherwise (or with a coordinate out of FP32's range) the lanes
-// concerned go over their coordinates and divide here (arg -1). One pass over u (134 MB at
+// division per ray remains; otherwise the lanes near it go over their coordinates and
+// divide here (arg -1). A ray with a coordinate outside what the FP32 quotients hold for (a
+// half-width, a direction or their quotient near the ends of FP32's range) is left to FP64
+// altogether: every lane divides every coordinate. One pass over u (134 MB at
 // 16384 rays, d = 1024) where the split and the exit lengths were two, each bound by FP64
 // conversions: 297 us, 59 us now.
 template <int PREC>
@@ -1618,7 +1620,7 @@ __global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int 
         rows = rb < rows ? rb : rows;
     }
     const int lane = threadIdx.x & 31;
-    constexpr float kLo = 1e-30f, kHi = 1e30f;
+    constexpr float kLo = 1e-30f, kHi = 1e30f, kMinQ = 1e-36f;
     if (arg) {
         for (int i = threadIdx.x; i < d; i += blockDim.x) {
             const float h = f64_to_f32(half[i]);
@@ -1643,8 +1645,11 @@ __global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int 
                 for (int q = 0; q < 2; ++q) {
                     const float m = q ? m1 : m0;
                     if (m > 0.f) {
-                        const float h = hf[i + q], e = __fdividef(h, m);
-                        odd = odd || h < 0.f;
+                        const float e = __fdividef(hf[i + q], m);
+                        if (!(e >= kMinQ)) {  // (negative where hf is)
+                            odd = true;
+                            continue;
+                        }
                         if (e <= est * (1.0f + 0x1p-17f)) close = e * (1.0f + 0x1p-17f) < est ? 0 : close + (at >= 0);
                         if (e < est) {
                             est = e;
@@ -1655,14 +1660,15 @@ __global__ void __launch_bounds__(256) k_q_split_rows(int n_rays, int rows, int 
             }
         }
         if (arg && live) {
-            const float thr = warp_min(est) * (1.0f + 0x1p-18f);
+            // with an odd coordinate every lane counts as near, and no quotient is above thr
+            const float thr = __any_sync(0xffffffffu, odd) ? INFINITY : warp_min(est) * (1.0f + 0x1p-18f);
             const unsigned near = __ballot_sync(0xffffffffu, est <= thr);
-            const bool tie = __any_sync(0xffffffffu, odd || (est <= thr && (close || at < 0)));
+            const bool tie = __any_sync(0xffffffffu, est <= thr && (close || at < 0));
             if (__popc(near) == 1 && !tie) {
                 if (est <= thr) arg[r] = at;
             } else {
                 long long best = 0x7ff0000000000000ll;  // +inf; positive doubles order as their bits
-                if (est <= thr || odd) {
+                if (est <= thr) {
                     for (int i = 2 * lane; i < d; i += 64) {
                         for (int q = 0; q < 2 && i + q < d; ++q) {
                             const double x = ur[i + q];
