@@ -1046,8 +1046,7 @@ void launch_gather_rows(int d, int cap, const double *X, const int32_t *idx, con
 // with every tile resident at once, 274 so).
 static int precision_pad() {
     constexpr int kPad = 60 * 1024;
-    return cudaFuncSetAttribute(k_precision, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad) == cudaSuccess ? kPad
-                                                                                                               : 0;
+    return allow_smem(k_precision, kPad) == cudaSuccess ? kPad : 0;
 }
 
 void launch_onehot(int K, const double *R, const int32_t *n_c, int cap, int32_t *onehot, cudaStream_t s) {

@@ -675,9 +675,8 @@ void points_grouped(const LikF64Args &a, cudaStream_t s) {
     // different in length, are dealt out as SMs come free (all resident at once: 484 us at
     // 4096 points, d = 256, K = 4, 304 us so; 287 us of FP64 instructions)
     constexpr int kPad = 96 * 1024;
-    static const cudaError_t pad_set =
-        cudaFuncSetAttribute(k_ggemm_f64_grouped, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad);
-    k_ggemm_f64_grouped<<<dim3(n_multi + n / BM + K, nJT), NT, pad_set == cudaSuccess ? kPad : 0, s>>>(a, L, n_multi);
+    const int pad = allow_smem(k_ggemm_f64_grouped, kPad) == cudaSuccess ? kPad : 0;
+    k_ggemm_f64_grouped<<<dim3(n_multi + n / BM + K, nJT), NT, pad, s>>>(a, L, n_multi);
 }
 }  // namespace
 

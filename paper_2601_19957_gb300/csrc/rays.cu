@@ -376,9 +376,7 @@ void launch_select_starts(const double *ell_all, int n_rays, int n_steps, int n_
     cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * (size_t)nbins, s);
     cudaMemsetAsync(w.state, 0, sizeof(uint64_t) * 8, s);
     const size_t sm = sizeof(uint64_t) * RB_WARPS * n_steps + sizeof(uint32_t) * nbins;
-    static const cudaError_t attr = cudaFuncSetAttribute(k_ray_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)(sizeof(uint64_t) * RB_WARPS * 1024 + sizeof(uint32_t) * 2048));
-    (void)attr;
+    if (sm > kFreeSmem) allow_smem(k_ray_bucket, (int)sm);
     const int rb = (n_rays + RB_WARPS - 1) / RB_WARPS;
     note_launch();
     k_ray_bucket<<<rb < 608 ? rb : 608, 32 * RB_WARPS, sm, s>>>(ell_all, n_rays, n_steps, w.bucket, w.hist);

@@ -213,6 +213,15 @@ struct ProbView {
 // Bytes sb_loglik needs (lists: with its optional row lists, what the query returns).
 size_t loglik_bytes(const sb_problem *p, int32_t prec, int32_t n, bool lists);
 
+// Lets launches of kernel k use up to `bytes` of dynamic shared memory (needed above kFreeSmem).
+// The permission belongs to the current device's copy of the kernel, so it is given before
+// each launch: kept once per process, a second device would refuse the launch.
+constexpr size_t kFreeSmem = 48 * 1024;
+template <typename F>
+inline cudaError_t allow_smem(F *k, int bytes) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // Host-side count of kernel launches issued by the library (diagnostics).
 void note_launch(int64_t n = 1);
 

@@ -1334,12 +1334,9 @@ void launch_center(const TcWs &t, int d, int K, const int32_t *n_rows_dev, int n
 }
 
 size_t lse_smem(int K) {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_tc_lse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(double) * kMaxK * LSE_ROWS);
-    });
-    return sizeof(double) * (size_t)K * LSE_ROWS;
+    const size_t bytes = sizeof(double) * (size_t)K * LSE_ROWS;
+    if (bytes > kFreeSmem) allow_smem(k_tc_lse, (int)bytes);
+    return bytes;
 }
 
 TcArgs base_args(const ProbView &pv, const TcWs &t) {
