@@ -224,7 +224,9 @@ sb_status sb_evidence_host(const sb_problem *host_prob, const sb_config *cfg, do
  * stored): d log Z_m/dphi = d/dphi [l - 1/2 log det H - 1/2 v^T grad l] at the
  * mode with v = H^-1 grad_x log det H. modes: [n_modes][d]; logZk: [n_modes]
  * (device, as written by sb_evidence); dmu: [K][d]; dL: [K][d][d] (device).
- * ws: sb_evidence_backward_workspace_bytes. Synchronises `stream`.
+ * ws: sb_evidence_backward_workspace_bytes, the room for the modes it takes together (up to
+ * four). Less is accepted down to 8 (2 K + 1) d^2 bytes and a few vectors per component: fewer
+ * modes together, the same results. Synchronises `stream`.
  */
 size_t sb_evidence_backward_workspace_bytes(const sb_problem *prob);
 sb_status sb_evidence_backward(const sb_problem *prob, const double *modes, const double *logZk, int32_t n_modes,

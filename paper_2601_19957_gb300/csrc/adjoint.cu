@@ -32,7 +32,7 @@
 // diag(1 / L_ii), with no solve. Products with P_k are formed as L_k (L_k^T v); P_k itself
 // is built only for the Hessian of a mode that is not one-hot. Nothing is read back to
 // the host: every skip is decided from R and the one-hot flag on the device. Modes go
-// through the kernels in groups (adj_group), since one mode's factor, inverse and vector
+// through the kernels in groups (adjoint_group), since one mode's factor, inverse and vector
 // steps leave most of the chip idle; their shares are added to dmu and dL in mode order.
 //
 // The bound is the FP64 pipe (one warp instruction per 19 cycles and SM): per mode K d^3 /
@@ -80,8 +80,8 @@ __device__ __forceinline__ void tile_gemm(TileBuf &sm, int l0, int l1, double (&
 }
 
 // The inverses of the 32 x 32 diagonal blocks of C (identity past d): a warp per four
-// columns, lanes over rows, multiplication by the diagonal's reciprocals. Also zeroes the
-// rest of the block row, which the merges fill below the diagonal.
+// columns, lanes over rows, multiplication by the diagonal's reciprocals. (The merges fill
+// the blocks below; those above the diagonal are not read.)
 __global__ void __launch_bounds__(256) k_inv_diag(int d, const double *C, double *Ci) {
     __shared__ double Cs[TB][TB + 1];
     __shared__ double inv[TB];
@@ -473,8 +473,8 @@ __global__ void __launch_bounds__(1024) k_adj_stage(int stage, int d, int K, con
     gbar += (size_t)mo * d;
     WV += (size_t)mo * (K + 1) * d;
     trp += (size_t)mo * K;
-    PY += (size_t)mo * K * d;
     if (stage == 0) {
+        PY += (size_t)mo * K * d;
         t_out += (size_t)mo * d;
     } else {
         Wt += (size_t)mo * d;
@@ -541,18 +541,17 @@ __global__ void k_softmax_pi(int n, const double *logZk, double g, double *pi) {
 
 }  // namespace
 
-// Modes a group holds: four matrices of each kind, fewer with many components (X_k).
-static int adj_group(int K) {
+int adjoint_group(int K) {
     const int g = 32 / K;
     return g < 1 ? 1 : (g > 4 ? 4 : g);
 }
 
-void adjoint_carve(Carver &cv, AdjWs &w, int d, int K) {
-    const size_t nJT = (d + 63) / 64, nt = (d + TB - 1) / TB, dd = (size_t)d * d, g = adj_group(K);
+void adjoint_carve(Carver &cv, AdjWs &w, int d, int K, int group) {
+    const size_t nJT = (d + 63) / 64, dd = (size_t)d * d, g = group > 0 ? group : 1;
+    w.group = (int)g;
     w.P = cv.take<double>(K * dd);
     w.H = cv.take<double>(g * dd);
-    w.Ci = cv.take<double>(g * dd);
-    w.T2 = cv.take<double>(g * dd);
+    w.Ci = group > 0 ? cv.take<double>(g * dd) : w.P;
     w.X = cv.take<double>(g * K * dd);
     w.trp = cv.take<double>(g * K);
     w.Z = cv.take<double>(g * K * d);
@@ -563,12 +562,9 @@ void adjoint_carve(Carver &cv, AdjWs &w, int d, int K) {
     w.GK = cv.take<double>(g * K * d);
     w.V = cv.take<double>(g * d * (K + 1));
     w.Y = cv.take<double>(g * d * (K + 1));
-    w.WV = cv.take<double>(g * d * (K + 1));
     w.T = cv.take<double>(g * d);
     w.eps = cv.take<double>(g * K);
     w.gam = cv.take<double>(g * K * d);
-    w.U = cv.take<double>(g * K * d);
-    w.PY = cv.take<double>(g * K * d);
     w.pi = cv.take<double>(kMaxAdjModes);
     w.info = cv.take<int32_t>(g);
     w.count = cv.take<int32_t>(1);
@@ -584,7 +580,7 @@ __global__ void k_set_count(int32_t *p, int v) {
 
 sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, const double *logZk, int n_modes,
                       double grad_logZ, double *dmu, double *dL, cudaStream_t s) {
-    const int d = pv.d, K = pv.K, group = adj_group(K);
+    const int d = pv.d, K = pv.K, group = w.group;
     if (n_modes < 1 || n_modes > kMaxAdjModes) return SB_ERR_INVALID_ARG;
     SB_CUDA_TRY(cudaMemsetAsync(dmu, 0, sizeof(double) * K * d, s));
     SB_CUDA_TRY(cudaMemsetAsync(dL, 0, sizeof(double) * (size_t)K * d * d, s));
@@ -600,6 +596,7 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
         const int nm = n_modes - m0 < group ? n_modes - m0 : group;
         const double *x = modes + (size_t)m0 * d;
         const double *pi = w.pi + m0;
+        if (w.Ci == w.P) SB_CUDA_TRY(cudaMemsetAsync(w.p_done, 0, sizeof(int32_t) * kMaxK, s));
         note_launch();
         k_set_count<<<1, 32, 0, s>>>(w.count, nm);
         // W v for the nv vectors per mode of V (stride vm; those with R == 0 skipped, zero and unread)
@@ -631,33 +628,33 @@ sb_status adjoint_run(const ProbView &pv, const AdjWs &w, const double *modes, c
         launch_precision_needed(d, K, pv.L, w.R, w.count, w.p_done, w.p_need, w.P, s, w.onehot);
         launch_hessian_chol(d, K, nm, pv.L, w.P, w.Z, w.R, w.gbar, w.count, w.GK, w.H, w.info, w.bar, pv.status, s,
                             w.onehot, true);
-        launch_tri_inverse(d, nm, w.H, w.Ci, w.T2, s);
-        // W [g_0 .. g_{K-1}, gbar]; X_k = C^-1 L_k and tr(W P_k)
+        launch_tri_inverse(d, nm, w.H, w.Ci, w.X, s);
+        // W [g_0 .. g_{K-1}, gbar] in place; X_k = W L_k and tr(W P_k)
         note_launch();
         k_pack_rhs<<<dim3((d + 255) / 256, K + 1, nm), 256, 0, s>>>(d, K, w.GK, w.gbar, w.R, w.V);
-        apply_W(K + 1, w.V, dV, w.WV, dV, w.R);
+        apply_W(K + 1, w.V, dV, w.V, dV, w.R);
         note_launch();
         k_adj_solve<<<dim3(K * nm, tiles), 256, kPad, s>>>(d, K, w.H, pv.L, w.R, w.onehot, w.X);
         note_launch();
         k_adj_trace<<<K * nm, 256, 0, s>>>(d, K, w.X, pv.L, w.R, w.onehot, w.trp);
         // P_k (W gbar - W g_k) = L_k (L_k^T (W gbar - W g_k))
         note_launch(2);
-        k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.WV, dV, w.R, K, w.U, dK}, true);
-        k_adj_lower<<<dim3(rows8, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.U, dK, w.R, K, w.PY, dK});
-        // t = grad_x log det H, then v = W t (into V), then c, eps_k, gam_k
+        k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.V, dV, w.R, K, w.Y, dK}, true);
+        k_adj_lower<<<dim3(rows8, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.Y, dK, w.R, K, w.gam, dK});
+        // t = grad_x log det H, then v = W t in place, then c, eps_k, gam_k
         note_launch();
-        k_adj_stage<<<nm, 1024, 0, s>>>(0, d, K, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, nullptr, w.T,
+        k_adj_stage<<<nm, 1024, 0, s>>>(0, d, K, w.R, w.onehot, w.GK, w.gbar, w.V, w.trp, w.gam, nullptr, w.T,
                                         nullptr, nullptr);
-        apply_W(1, w.T, d, w.V, d, nullptr);
+        apply_W(1, w.T, d, w.T, d, nullptr);
         note_launch();
-        k_adj_stage<<<nm, 1024, 0, s>>>(1, d, K, w.R, w.onehot, w.GK, w.gbar, w.WV, w.trp, w.PY, w.V, nullptr,
+        k_adj_stage<<<nm, 1024, 0, s>>>(1, d, K, w.R, w.onehot, w.GK, w.gbar, w.V, w.trp, nullptr, w.T, nullptr,
                                         w.eps, w.gam);
         // u_k = L_k^T gam_k, dmu_k += pi (-eps_k g_k + L_k u_k), dL_k
         note_launch(3);
-        k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.gam, dK, w.R, K, w.U, dK}, false);
-        k_adj_dmu<<<dim3(rows8, K), 256, 0, s>>>(d, nm, pv.L, w.U, w.R, pi, w.eps, w.GK, dmu);
+        k_adj_upper<<<dim3(cols32, K, nm), 256, 0, s>>>(d, VecArgs{pv.L, 0, dd, w.gam, dK, w.R, K, w.Y, dK}, false);
+        k_adj_dmu<<<dim3(rows8, K), 256, 0, s>>>(d, nm, pv.L, w.Y, w.R, pi, w.eps, w.GK, dmu);
         k_adj_dL<<<dim3((d + 255) / 256, d, K), 256, 0, s>>>(d, nm, pi, w.R, w.eps, w.onehot, pv.L, x, pv.mu, w.Z,
-                                                             w.gam, w.U, w.X, dL);
+                                                             w.gam, w.Y, w.X, dL);
     }
     SB_CUDA_TRY(cudaGetLastError());
     SB_CUDA_TRY(cudaStreamSynchronize(s));  // the call returns with its results written

@@ -989,7 +989,7 @@ struct BwdLayout {
     AdjWs adj;
     size_t bytes;
 };
-BwdLayout bwd_layout(void *base, const sb_problem *p) {
+BwdLayout bwd_layout(void *base, const sb_problem *p, int group) {
     BwdLayout B{};
     Carver cv(base);
     B.hdr = cv.take<WsHeader>(1);
@@ -998,7 +998,7 @@ BwdLayout bwd_layout(void *base, const sb_problem *p) {
     B.half = cv.take<double>(p->d);
     B.logV = cv.take<double>(1);
     B.wmax = cv.take<double>(1);
-    adjoint_carve(cv, B.adj, p->d, p->K);
+    adjoint_carve(cv, B.adj, p->d, p->K, group);
     B.bytes = cv.bytes();
     return B;
 }
@@ -1006,7 +1006,7 @@ BwdLayout bwd_layout(void *base, const sb_problem *p) {
 
 extern "C" size_t sb_evidence_backward_workspace_bytes(const sb_problem *p) {
     if (check_problem(p) != SB_OK) return 0;
-    return bwd_layout(nullptr, p).bytes;
+    return bwd_layout(nullptr, p, adjoint_group(p->K)).bytes;
 }
 
 extern "C" sb_status sb_evidence_backward(const sb_problem *p, const double *modes, const double *logZk,
@@ -1015,7 +1015,10 @@ extern "C" sb_status sb_evidence_backward(const sb_problem *p, const double *mod
     sb_status st = check_problem(p);
     if (st != SB_OK) return st;
     if (!modes || !logZk || !dmu || !dL || !ws || n_modes < 1 || n_modes > kMaxAdjModes) return SB_ERR_INVALID_ARG;
-    const BwdLayout B = bwd_layout(ws, p);
+    // as many modes together as the workspace has room for
+    int group = adjoint_group(p->K);
+    while (group > 0 && ws_bytes < bwd_layout(nullptr, p, group).bytes) --group;
+    const BwdLayout B = bwd_layout(ws, p, group);
     if (ws_bytes < B.bytes) return SB_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     SB_CUDA_TRY(cudaMemsetAsync(B.hdr, 0, sizeof(WsHeader), s));

@@ -39,3 +39,45 @@ def test_loglik_stays_inside_its_workspace(d, n, K, prec):
     sb.lib().sb_loglik(C.byref(bad.s), C.c_int32(prec), sb._ptr(x), C.c_int32(n), sb._ptr(ell), None,
                        C.c_void_p(buf.data_ptr()), C.c_size_t(need), sb._stream())
     assert sb.lib().sb_check(C.c_void_p(buf.data_ptr()), C.c_size_t(need), sb._stream()) == sb.SB_ERR_INVALID_ARG
+
+
+def _backward(prob, modes, logzk, nbytes):
+    """sb_evidence_backward on exactly nbytes with a guard behind them."""
+    buf = torch.full((nbytes + GUARD,), 0x5A, dtype=torch.uint8, device="cuda")
+    dmu, dL = torch.empty_like(prob.mu), torch.empty_like(prob.L)
+    code = sb.lib().sb_evidence_backward(C.addressof(prob.s), sb._ptr(modes), sb._ptr(logzk), modes.shape[0], 0.7,
+                                         sb._ptr(dmu), sb._ptr(dL), C.c_void_p(buf.data_ptr()), nbytes, sb._stream())
+    assert bool((buf[nbytes:] == 0x5A).all())
+    return code, dmu, dL
+
+
+def _one_mode_bytes(d, K):
+    """Room for one mode with its own C^-1 L_k beside P_k: P_k and M_k [K][d][d], H, the
+    vectors of a mode and the constants, each on a multiple of 256 bytes."""
+    tiles, up = (d + 63) // 64, lambda n, s: (n * s + 255) // 256 * 256
+    doubles = [32, K, d, d, 1, 1, K * d * d, d * d, K * d * d, K * d, K, K * tiles, d, 1, K * d, d * (K + 1), d, d, K,
+               K * d, d, K, K * d, d, 1024]
+    return sum(up(n, 8) for n in doubles) + sum(up(n, 4) for n in (1, 1, 1, 2))
+
+
+@pytest.mark.parametrize("d,K,n_modes", [(1, 1, 1), (2, 64, 3), (5, 2, 5), (33, 8, 6), (64, 12, 5), (129, 3, 4),
+                                         (256, 2, 7)])
+def test_adjoint_results_do_not_depend_on_the_workspace(d, K, n_modes):
+    """From the queried size (up to four modes together) down to one mode's."""
+    inst = make_instance(d, K, 70 + d + K, s_range=(0.2, 0.5), mean_box=(-0.2, 0.2), sep=0.0)
+    prob = sb.Problem(inst)
+    rng = np.random.default_rng(d)
+    modes = inst.mu[rng.integers(0, K, n_modes)] + 0.05 * rng.standard_normal((n_modes, d))
+    if n_modes > 1:
+        modes[-1] += 30.0  # a one-hot mode
+    modes = torch.as_tensor(modes, device="cuda")
+    logzk = torch.as_tensor(rng.standard_normal(n_modes), device="cuda")
+    full = int(sb.lib().sb_evidence_backward_workspace_bytes(C.byref(prob.s)))
+    code, dmu, dL = _backward(prob, modes, logzk, full)
+    assert code == sb.SB_OK and bool(torch.isfinite(dmu).all()) and bool(torch.isfinite(dL).all())
+    one = min(full, _one_mode_bytes(d, K))
+    for nbytes in {one, (one + full) // 2 // 256 * 256, max(full - 256, one)}:
+        code, a, b = _backward(prob, modes, logzk, nbytes)
+        assert code == sb.SB_OK
+        assert torch.equal(a, dmu) and torch.equal(b, dL)
+    assert _backward(prob, modes, logzk, 8 * (2 * K + 1) * d * d)[0] == sb.SB_ERR_WORKSPACE
