@@ -876,8 +876,6 @@ size_t sb::loglik_bytes(const sb_problem *p, int32_t prec, int32_t n, bool lists
     } else if (prec == SB_PREC_TF32 || prec == SB_PREC_BF16) {
         TcWs t;
         carve_tc(cv, t, n, p->d, p->K, prec);
-        cv.take<float>((size_t)n);
-        cv.take<float>((size_t)n * p->d);
         cv.take<double>(2 * (size_t)p->d + 3);
     } else {
         return 0;
@@ -938,19 +936,15 @@ extern "C" sb_status sb_loglik(const sb_problem *p, int32_t prec, const double *
     } else {
         TcWs t;
         carve_tc(cv, t, n, p->d, p->K, prec);
-        float *f = cv.take<float>((size_t)n);
-        float *g = cv.take<float>((size_t)n * p->d);
         double *box = cv.take<double>(2 * (size_t)p->d + 3);
         pv.c = box;
         pv.half = box + p->d;
         pv.logV = box + 2 * p->d;
         pv.wmax = box + 2 * p->d + 1;
         launch_setup(pv, s);
-        sb_config c{};
-        c.prec = prec;
         st = tc_prepare(pv, t, s, false);  // no walker rounds here
         if (st != SB_OK) return st;
-        st = tc_loglik_points(pv, &c, t, x, n, f, grad ? g : nullptr, ell, grad, s);
+        st = tc_loglik_points(pv, t, x, n, ell, grad, s);
         if (st != SB_OK) return st;
     }
     SB_CUDA_TRY(cudaGetLastError());

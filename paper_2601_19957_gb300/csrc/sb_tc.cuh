@@ -84,7 +84,7 @@ void tc_walkers_reset(const TcWs &t, int n, cudaStream_t s);
 constexpr int kTcDistSlot = 14;
 void tc_eval_walkers(const ProbView &pv, const sb_config *c, const TcWs &t, const float *XT, const int32_t *act,
                      const int32_t *n_act, int n, float *FT, float *GT, cudaStream_t s);
-sb_status tc_loglik_points(const ProbView &pv, const sb_config *c, const TcWs &t, const double *x, int n, float *f,
-                           float *g, double *ell, double *grad, cudaStream_t s);
+sb_status tc_loglik_points(const ProbView &pv, const TcWs &t, const double *x, int n, double *ell, double *grad,
+                           cudaStream_t s);
 
 }  // namespace sb

@@ -1371,7 +1371,8 @@ void launch_scale_z(const ProbView &pv, const TcWs &t, const int32_t *n_rows_dev
 bool tc_available(int prec) { return (prec == SB_PREC_BF16 || prec == SB_PREC_TF32) && encode_fn() != nullptr; }
 
 // Layout: [0] LT, [1] LB, [2] mu32, [3] c32, [4] Z [K][rows][ldz], [5] qpart, [6] R,
-// [7] X32 (points), [8] G32 (points), [9] A1 [K][rows][ldp] (centred GEMM1 operand),
+// [7] columns of L_k for the skip bounds, [8] the autotuner's GEMM2 output (both [rows][d]),
+// [9] A1 [K][rows][ldp] (centred GEMM1 operand),
 // [10] rflag, and for the component skip of the walker rounds (k_tc_need):
 // [11] zb [rows][K], [12] jst [rows], [13] zst [rows], [14] dist [rows],
 // [15] lnorm [K], [16] zmask [row blocks][K]
@@ -2069,11 +2070,8 @@ void tc_eval_walkers(const ProbView &pv, const sb_config *c, const TcWs &t, cons
     launch_gemm_any(t.prec, MODE_G, t.bn, t.mapZ, t.mapB, a, s);
 }
 
-sb_status tc_loglik_points(const ProbView &pv, const sb_config *c, const TcWs &t, const double *x, int n, float *f,
-                           float *g, double *ell, double *grad, cudaStream_t s) {
-    (void)c;
-    (void)f;
-    (void)g;
+sb_status tc_loglik_points(const ProbView &pv, const TcWs &t, const double *x, int n, double *ell, double *grad,
+                           cudaStream_t s) {
     const int d = pv.d, K = pv.K;
     TcArgs a = base_args(pv, t);
     a.n_rows_max = n;
