@@ -86,9 +86,12 @@ __device__ __forceinline__ uint64_t dd_key(double l) {  // -0 and +0 alike
 }
 
 // |x - b| > tau, decided in FP32 on the rounded operands unless the difference lies within
-// their rounding of tau, where FP64 decides (a call: inlined it would be predicated).
+// their rounding of tau, where FP64 decides (a call: inlined it would be predicated). FP64
+// also decides where tau is so small that operands near it may be subnormal in FP32, whose
+// rounding is not relative: from 2^-100 on it is below the margin of 2^-20 tau.
 static __device__ __noinline__ bool dd_far_exact(double x, double b, double tau) { return fabs(x - b) > tau; }
 __device__ __forceinline__ bool dd_far(double x, double b, float bf, double tau, float tf) {
+    if (tf < 0x1p-100f) return dd_far_exact(x, b, tau);
     const float xf = f64_to_f32(x), df = fabsf(xf - bf), err = (fabsf(xf) + fabsf(bf)) * 0x1p-23f;
     if (df - err > tf * (1.0f + 0x1p-20f)) return true;
     if (df + err < tf * (1.0f - 0x1p-20f)) return false;
