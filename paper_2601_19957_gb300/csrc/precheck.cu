@@ -89,18 +89,19 @@ __global__ void __launch_bounds__(256) k_pre_rows(int d, const double *L, const 
     const double *zk = z0 + (size_t)k * d;
     double v[4] = {0.0, 0.0, 0.0, 0.0};  // dot and norm of row i, of row i + 1
     for (int j0 = 0; j0 <= i + 1; j0 += 128) {
-        double a[4], b[4], z[4];
+        double a[4], b[4], z[4], zi[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int j = j0 + 32 * u + lane;
             a[u] = j <= i ? row0[j] : 0.0;
             b[u] = two && j <= i + 1 ? row1[j] : 0.0;
             z[u] = j <= i + 1 && j < d ? zk[j] : 0.0;
+            zi[u] = j <= i ? z[u] : 0.0;  // z0_i+1 is no part of row i (0 times an infinity is NaN)
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (j0 + 32 * u > i + 1) break;
-            v[0] = fma(a[u], z[u], v[0]);
+            v[0] = fma(a[u], zi[u], v[0]);
             v[1] = fma(a[u], a[u], v[1]);
             v[2] = fma(b[u], z[u], v[2]);
             v[3] = fma(b[u], b[u], v[3]);

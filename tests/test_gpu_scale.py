@@ -30,3 +30,19 @@ def test_duplicates_are_merged_alike_at_every_scale(exp):
     two = sb.laplace(sb.Problem(inst), c, t(x * s), t(ell))
     assert two.n_modes == one.n_modes
     assert torch.equal(two.modes, one.modes * s)
+
+
+@pytest.mark.parametrize("j", [1, 2, 3, 32, 33, 63])
+def test_probe_of_coordinates_before_an_overflowing_one(j):
+    """A component whose z overflows at coordinate j (its term is -inf, its weight 0) leaves
+    the sensitivities of the coordinates before j as without it."""
+    d = 64
+    inst = make_instance(d, 2, 8, s_range=(0.3, 1.0), mean_box=(-2, 2), sep=0.0)
+    inst.L[1] = np.eye(d)
+    inst.L[1, j, j] = 1e160
+    inst.mu[1, j] = -1e160
+    got = sb.precheck(sb.Problem(inst)).s.cpu().numpy()
+    inst.K, inst.log_w, inst.mu, inst.L = 1, inst.log_w[:1], inst.mu[:1], inst.L[:1]
+    want = sb.precheck(sb.Problem(inst)).s.cpu().numpy()
+    assert np.isfinite(want).all()
+    np.testing.assert_allclose(got[:j], want[:j], rtol=1e-10)
