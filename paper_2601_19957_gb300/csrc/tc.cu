@@ -627,7 +627,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
 // absolute error stays below the FP32 resolution of the outputs.
 // mode 0: walkers (FT[act[n]] = -l, R); mode 2: points (ell[act[n]] = l, R). Both raise
 // rflag[block][k] when some row of the 128-row block has r_nk > 0 (GEMM2 and the scaling
-// pass skip the other (block, component) pairs, whose terms are exactly zero).
+// pass skip the other (block, component) pairs, whose terms are exactly zero). qlast: the
+// partial after the n_ntile of qpart, by point ([.][K], through act).
 // Bound by the FP64 pipe (one warp instruction per 19 cycles and SM): each e_k is formed
 // once and kept in shared memory (n_ntile + 1 FP64 instructions per row and evaluated
 // component; it was three times that, an FP64 square root and the conversions), the
@@ -638,7 +639,7 @@ __global__ void __launch_bounds__(LSE_ROWS) k_tc_lse(int mode, int K, int n_ntil
                                                      int n_rows_max, const int32_t *act, const float *qpart,
                                                      const double *a_k, float *R, float *FT, double *ell,
                                                      uint32_t *rflag, const uint32_t *zmask, float *zb, int32_t *jst,
-                                                     float *zst) {
+                                                     float *zst, const float *qlast) {
     extern __shared__ double s_e[];  // [K][LSE_ROWS]: e_k, then (as float) exp(e_k - max)
     const int n_rows = n_rows_dev ? *n_rows_dev : n_rows_max;
     if ((int)blockIdx.x * LSE_ROWS >= n_rows) return;
@@ -668,6 +669,7 @@ __global__ void __launch_bounds__(LSE_ROWS) k_tc_lse(int mode, int K, int n_ntil
             const float *qp = qpart + ((size_t)n * K + k) * n_ntile;
             double q = f32_to_f64(qp[0]);
             for (int t = 1; t < n_ntile; ++t) q += f32_to_f64(qp[t]);
+            if (qlast) q += f32_to_f64(qlast[(size_t)act[n] * K + k]);
             const double e = a_k[k] - 0.5 * q;
             slot(k) = e;
             const long long o = order(e);
@@ -919,95 +921,99 @@ __global__ void __launch_bounds__(256) k_tc_lnorm_gram(int d, int K, int k0, int
 // (rounded to FP32 on the integer units as they are read).
 // Rows from n_rows up to the next multiple of 128 and columns >= d are zeroed.
 // One thread per (row, 16-byte column group from group cg0 on): x is formed once and the
-// thread writes that column group for every component. vec: X allows 16-byte loads.
-template <int PREC, typename T>
+// thread writes that column group for every component. vec: X allows 16-byte loads. FEW: zmask
+// holds few pairs, or none: blocks without any are left out whole, and a few CTAs per SM go
+// over the elements (16384 of them that found nothing to do took 24 us).
+template <int PREC, typename T, bool FEW>
 __global__ void __launch_bounds__(256) k_tc_center(int d, int K, int rows_cap, int ldp, int cg0,
                                                    const int32_t *n_rows_dev, int n_rows_max, const int32_t *act,
                                                    const T *X, bool vec_ok, const float *mu32, void *A1,
-                                                   const uint32_t *zmask, bool mask_exact) {
+                                                   const uint32_t *zmask) {
     constexpr int VE = (PREC == SB_PREC_BF16) ? 8 : 4;  // elements per 16-byte store
     const int n_rows = n_rows_dev ? *n_rows_dev : n_rows_max;
     int rows_pad = (n_rows + BM - 1) / BM * BM;
     if (rows_pad > rows_cap) rows_pad = rows_cap;
     const int ncg = ldp / VE - cg0;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = e / ncg, cg = cg0 + e - n * ncg;
-    if (n >= rows_pad) return;
-    const uint64_t km = zmask ? block_kmask(zmask, n / BM, K, mask_exact) : ~0ull;  // pairs the |z|^2 pass visits
-    if (!km) return;
-    const int i0 = cg * VE;
-    const bool live = n < n_rows;
-    const bool vec = vec_ok && i0 + VE <= d;
-    float x[VE];
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x;; e += gridDim.x * blockDim.x) {
+        const int n = e / ncg, cg = cg0 + e - n * ncg;
+        if (n >= rows_pad) return;
+        const uint64_t km = zmask ? block_kmask(zmask, n / BM, K, FEW) : ~0ull;  // pairs the |z|^2 pass visits
+        if (FEW && !km) continue;
+        const int i0 = cg * VE;
+        const bool live = n < n_rows;
+        const bool vec = vec_ok && i0 + VE <= d;
+        float x[VE];
 #pragma unroll
-    for (int q = 0; q < VE; ++q) x[q] = 0.f;
-    if (live) {
-        const T *xr = X + (size_t)(act ? act[n] : n) * d;
-        if (vec) {
-            if constexpr (sizeof(T) == 4) {
-#pragma unroll
-                for (int q = 0; q < VE; q += 4) {
-                    const float4 t = *reinterpret_cast<const float4 *>(xr + i0 + q);
-                    x[q] = t.x;
-                    x[q + 1] = t.y;
-                    x[q + 2] = t.z;
-                    x[q + 3] = t.w;
-                }
-            } else {
-                double2 t[VE / 2];
-#pragma unroll
-                for (int q = 0; q < VE / 2; ++q) t[q] = reinterpret_cast<const double2 *>(xr + i0)[q];
-#pragma unroll
-                for (int q = 0; q < VE / 2; ++q) {
-                    x[2 * q] = f64_to_f32(t[q].x);
-                    x[2 * q + 1] = f64_to_f32(t[q].y);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < VE; ++q)
-                if (i0 + q < d) {
-                    if constexpr (sizeof(T) == 4)
-                        x[q] = xr[i0 + q];
-                    else
-                        x[q] = f64_to_f32(xr[i0 + q]);
-                }
-        }
-    }
-    const bool vmu = (d & 3) == 0 && i0 + VE <= d;
-    for (int k = 0; k < K; ++k) {
-        if (!((km >> k) & 1ull)) continue;
-        float v[VE];
-#pragma unroll
-        for (int q = 0; q < VE; ++q) v[q] = 0.f;
+        for (int q = 0; q < VE; ++q) x[q] = 0.f;
         if (live) {
-            const float *mk = mu32 + (size_t)k * d;
-            if (vmu) {
+            const T *xr = X + (size_t)(act ? act[n] : n) * d;
+            if (vec) {
+                if constexpr (sizeof(T) == 4) {
 #pragma unroll
-                for (int q = 0; q < VE; q += 4) {
-                    const float4 m4 = *reinterpret_cast<const float4 *>(mk + i0 + q);
-                    v[q] = x[q] - m4.x;
-                    v[q + 1] = x[q + 1] - m4.y;
-                    v[q + 2] = x[q + 2] - m4.z;
-                    v[q + 3] = x[q + 3] - m4.w;
+                    for (int q = 0; q < VE; q += 4) {
+                        const float4 t = *reinterpret_cast<const float4 *>(xr + i0 + q);
+                        x[q] = t.x;
+                        x[q + 1] = t.y;
+                        x[q + 2] = t.z;
+                        x[q + 3] = t.w;
+                    }
+                } else {
+                    double2 t[VE / 2];
+#pragma unroll
+                    for (int q = 0; q < VE / 2; ++q) t[q] = reinterpret_cast<const double2 *>(xr + i0)[q];
+#pragma unroll
+                    for (int q = 0; q < VE / 2; ++q) {
+                        x[2 * q] = f64_to_f32(t[q].x);
+                        x[2 * q + 1] = f64_to_f32(t[q].y);
+                    }
                 }
             } else {
 #pragma unroll
-                for (int q = 0; q < VE; ++q) v[q] = (i0 + q < d) ? x[q] - mk[i0 + q] : 0.f;
+                for (int q = 0; q < VE; ++q)
+                    if (i0 + q < d) {
+                        if constexpr (sizeof(T) == 4)
+                            x[q] = xr[i0 + q];
+                        else
+                            x[q] = f64_to_f32(xr[i0 + q]);
+                    }
             }
         }
-        const size_t o = ((size_t)k * rows_cap + n) * ldp + i0;
-        if (PREC == SB_PREC_BF16) {
-            uint4 p;
-            p.x = pack_bf16x2(v[0], v[1]);
-            p.y = pack_bf16x2(v[2], v[3]);
-            p.z = pack_bf16x2(v[4], v[5]);
-            p.w = pack_bf16x2(v[6], v[7]);
-            *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(A1) + o) = p;
-        } else {
-            *reinterpret_cast<float4 *>(reinterpret_cast<float *>(A1) + o) =
-                make_float4(to_tf32(v[0]), to_tf32(v[1]), to_tf32(v[2]), to_tf32(v[3]));
+        const bool vmu = (d & 3) == 0 && i0 + VE <= d;
+        for (int k = 0; k < K; ++k) {
+            if (!((km >> k) & 1ull)) continue;
+            float v[VE];
+#pragma unroll
+            for (int q = 0; q < VE; ++q) v[q] = 0.f;
+            if (live) {
+                const float *mk = mu32 + (size_t)k * d;
+                if (vmu) {
+#pragma unroll
+                    for (int q = 0; q < VE; q += 4) {
+                        const float4 m4 = *reinterpret_cast<const float4 *>(mk + i0 + q);
+                        v[q] = x[q] - m4.x;
+                        v[q + 1] = x[q + 1] - m4.y;
+                        v[q + 2] = x[q + 2] - m4.z;
+                        v[q + 3] = x[q + 3] - m4.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < VE; ++q) v[q] = (i0 + q < d) ? x[q] - mk[i0 + q] : 0.f;
+                }
+            }
+            const size_t o = ((size_t)k * rows_cap + n) * ldp + i0;
+            if (PREC == SB_PREC_BF16) {
+                uint4 p;
+                p.x = pack_bf16x2(v[0], v[1]);
+                p.y = pack_bf16x2(v[2], v[3]);
+                p.z = pack_bf16x2(v[4], v[5]);
+                p.w = pack_bf16x2(v[6], v[7]);
+                *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(A1) + o) = p;
+            } else {
+                *reinterpret_cast<float4 *>(reinterpret_cast<float *>(A1) + o) =
+                    make_float4(to_tf32(v[0]), to_tf32(v[1]), to_tf32(v[2]), to_tf32(v[3]));
+            }
         }
+        if (!FEW) return;
     }
 }
 
@@ -1058,7 +1064,8 @@ __global__ void __launch_bounds__(256) k_tc_lead(int n_rows, int K, float scale,
 // which are stored by point), lead[n] reduced to the component; zmask[block][k]: the blocks
 // that hold a point led by k, or one that looked to need several. cursor zeroed before.
 __global__ void __launch_bounds__(256) k_tc_place(int n_rows, int K, int32_t *lead, const int32_t *hist,
-                                                  int32_t *cursor, int32_t *act, uint32_t *zmask) {
+                                                  int32_t *cursor, int32_t *act, uint32_t *zmask, int32_t *n_more) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_more = 0;  // (k_tc_more)
     __shared__ int h[2 * kMaxK], base[2 * kMaxK], start[2 * kMaxK + 1];
     for (int k = threadIdx.x; k < 2 * K; k += blockDim.x) h[k] = 0;
     if (threadIdx.x == 0) {
@@ -1084,10 +1091,11 @@ __global__ void __launch_bounds__(256) k_tc_place(int n_rows, int K, int32_t *le
     }
 }
 // more[block][k]: the pairs the leading pass left out that some point of the block still
-// needs; zmask gains them.
+// needs; zmask gains them. *n_more: n_rows when there is such a pair, else 0 (the passes over
+// them then end at once). qlast: qpart holds all but the last tile's partials, which are qs.
 __global__ void __launch_bounds__(BM) k_tc_more(int n_rows, int K, int n_ntile, const int32_t *act, const int32_t *lead,
                                                 const float *qpart, const float *qs, const double *a_k,
-                                                uint32_t *zmask, uint32_t *more) {
+                                                uint32_t *zmask, uint32_t *more, int32_t *n_more, bool qlast) {
     const int p = blockIdx.x * BM + threadIdx.x;
     const bool valid = p < n_rows;
     const int n = valid ? act[p] : 0, j = valid ? lead[n] : 0;
@@ -1096,6 +1104,7 @@ __global__ void __launch_bounds__(BM) k_tc_more(int n_rows, int K, int n_ntile, 
         const float *qp = qpart + ((size_t)p * K + j) * n_ntile;
         double q = f32_to_f64(qp[0]);
         for (int t = 1; t < n_ntile; ++t) q += f32_to_f64(qp[t]);
+        if (qlast) q += f32_to_f64(qs[(size_t)n * K + j]);
         low = fma(-0.5, q, a_k[j]) - (double)(kSkipNats + 1.0f);
     }
     for (int k = 0; k < K; ++k) {
@@ -1105,7 +1114,10 @@ __global__ void __launch_bounds__(BM) k_tc_more(int n_rows, int K, int n_ntile, 
         const int any = __syncthreads_or(need);
         if (threadIdx.x == 0) {
             more[(size_t)blockIdx.x * K + k] = any ? 1u : 0u;
-            if (any) zmask[(size_t)blockIdx.x * K + k] = 1u;
+            if (any) {
+                zmask[(size_t)blockIdx.x * K + k] = 1u;
+                *n_more = n_rows;  // by any block: the same value
+            }
         }
     }
 }
@@ -1315,22 +1327,23 @@ void launch_gemm_any(int prec, int mode, int bn, const CUtensorMap &mapA, const 
     }
 }
 
-template <typename T>
+template <bool FEW = false, typename T>
 void launch_center(const TcWs &t, int d, int K, const int32_t *n_rows_dev, int n_rows_max, const int32_t *act,
-                   const T *X, cudaStream_t s, const uint32_t *zmask = nullptr, bool mask_exact = false, int col0 = 0) {
+                   const T *X, cudaStream_t s, const uint32_t *zmask = nullptr, int col0 = 0) {
     const int ldp = ldp_of(d, t.prec), ve = t.prec == SB_PREC_BF16 ? 8 : 4;
     const int cg0 = col0 / ve, ncg = ldp / ve - cg0;
     int rows = (n_rows_max + BM - 1) / BM * BM;
     if (rows > (int)t.rows) rows = (int)t.rows;
     const bool vec = d % (sizeof(T) == 4 ? 4 : 2) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-    const dim3 grid((unsigned)(((long long)rows * ncg + 255) / 256));
+    const long long ctas = ((long long)rows * ncg + 255) / 256;
+    const unsigned grid = (unsigned)(FEW && ctas > 8 * num_sms() ? 8 * num_sms() : ctas);
     note_launch();
     if (t.prec == SB_PREC_BF16)
-        k_tc_center<SB_PREC_BF16, T><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, cg0, n_rows_dev, n_rows_max, act, X,
-                                                          vec, (const float *)t.p[2], t.p[9], zmask, mask_exact);
+        k_tc_center<SB_PREC_BF16, T, FEW><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, cg0, n_rows_dev, n_rows_max,
+                                                               act, X, vec, (const float *)t.p[2], t.p[9], zmask);
     else
-        k_tc_center<SB_PREC_TF32, T><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, cg0, n_rows_dev, n_rows_max, act, X,
-                                                          vec, (const float *)t.p[2], t.p[9], zmask, mask_exact);
+        k_tc_center<SB_PREC_TF32, T, FEW><<<grid, 256, 0, s>>>(d, K, (int)t.rows, ldp, cg0, n_rows_dev, n_rows_max,
+                                                               act, X, vec, (const float *)t.p[2], t.p[9], zmask);
 }
 
 size_t lse_smem(int K) {
@@ -2063,7 +2076,7 @@ void tc_eval_walkers(const ProbView &pv, const sb_config *c, const TcWs &t, cons
     note_launch();
     k_tc_lse<<<(n + LSE_ROWS - 1) / LSE_ROWS, LSE_ROWS, lse_smem(pv.K), s>>>(0, pv.K, a.n_ntile, n_act, n, act, a.qpart, pv.a, (float *)t.p[6], FT,
                                              nullptr, (uint32_t *)t.p[10], zmask, (float *)t.p[11],
-                                             (int32_t *)t.p[12], (float *)t.p[13]);
+                                             (int32_t *)t.p[12], (float *)t.p[13], nullptr);
     launch_scale_z(pv, t, n_act, n, s);
     a.prof = -1;
     a.G = GT;
@@ -2082,21 +2095,30 @@ sb_status tc_loglik_points(const ProbView &pv, const TcWs &t, const double *x, i
     a.rflag = nullptr;
     // The screen's eight launches take about 60 us at 16384 points; it pays when the flops
     // it can spare, K - 1 of K components' GEMM1 less the last column tile of each, are worth
-    // about 40 us at the rate of these kernels, 1 PFLOP/s in BF16 (GEMM2 spares as many).
-    // d = 1024, K = 8, 16384 points, BF16 with the gradient: 365 us, 560 without.
+    // about 40 us at the rate of these kernels, 1 PFLOP/s in BF16. GEMM2 spares as many. With
+    // values alone the screen must also pay for its passes over every (point, component), in
+    // either precision, which takes 6e5 flops spared of each; and the last tile's partials are
+    // kept (qs), so that a mixture that spares nothing does not pay for that tile twice. 16384
+    // points, K = 8, d = 1024, components far apart / all needed / without the screen: BF16 with
+    // the gradient 302 / 677 / 627 us, values 210 / 333 / 266; at d = 768, below the second
+    // line, TF32 values with it 236 / 372, 285 without.
     const int nct = a.n_ntile, kc = t.prec == SB_PREC_BF16 ? 64 : 32;
     int chunks = 0;
     for (int nt = 0; nt < nct; ++nt) chunks += (d + kc - 1) / kc - nt * t.bn / kc;
     const double last = (double)((d + kc - 1) / kc - (nct - 1) * t.bn / kc) / chunks;
     const double spared = (double)n * d * (d + 1) * (K * (1.0 - last) - 1.0) * (t.prec == SB_PREC_BF16 ? 1.0 : 2.0);
-    if (nct >= 2 && spared >= 4.0e10) {
+    const bool keep_last = !grad;
+    const float *qlast = nullptr;
+    const double each = (double)d * (d + 1) * (1.0 - last - 1.0 / K);
+    if (nct >= 2 && spared >= 4.0e10 && (grad || each >= 6.0e5)) {
         float *qs = (float *)t.p[11];
         int32_t *lead = (int32_t *)t.p[13], *hist = (int32_t *)t.p[14];
         uint32_t *more = (uint32_t *)t.p[10];  // rflag's place, which k_tc_lse writes later
+        int32_t *n_more = (int32_t *)t.p[15];
         act = (int32_t *)t.p[12];
         zmask = (uint32_t *)t.p[16];
         SB_CUDA_TRY(cudaMemsetAsync(hist, 0, 4 * sizeof(int32_t) * kMaxK, s));
-        launch_center(t, d, K, nullptr, n, nullptr, x, s, nullptr, false, (nct - 1) * t.bn);
+        launch_center(t, d, K, nullptr, n, nullptr, x, s, nullptr, (nct - 1) * t.bn);
         TcArgs b = a;
         b.nt0 = nct - 1;
         b.nts = b.n_ntile = 1;
@@ -2105,18 +2127,25 @@ sb_status tc_loglik_points(const ProbView &pv, const TcWs &t, const double *x, i
         const unsigned gn = (unsigned)((n + 255) / 256), gb = (unsigned)((n + BM - 1) / BM);
         note_launch(2);
         k_tc_lead<<<gn, 256, 0, s>>>(n, K, (float)d / (float)(d - (nct - 1) * t.bn), qs, pv.a, lead, hist);
-        k_tc_place<<<gn, 256, 0, s>>>(n, K, lead, hist, hist + 2 * kMaxK, act, zmask);
+        k_tc_place<<<gn, 256, 0, s>>>(n, K, lead, hist, hist + 2 * kMaxK, act, zmask, n_more);
         launch_center(t, d, K, nullptr, n, act, x, s, zmask);
         a.zmask = zmask;
+        if (keep_last) {
+            a.nts = a.n_ntile = nct - 1;
+            qlast = qs;
+        }
         launch_gemm_any(t.prec, mode, t.bn, t.mapA1, t.mapT, a, s);
         note_launch();
-        k_tc_more<<<gb, BM, 0, s>>>(n, K, a.n_ntile, act, lead, a.qpart, qs, pv.a, zmask, more);
-        launch_center(t, d, K, nullptr, n, act, x, s, more, true);
+        k_tc_more<<<gb, BM, 0, s>>>(n, K, a.n_ntile, act, lead, a.qpart, qs, pv.a, zmask, more, n_more,
+                                     keep_last);
+        launch_center<true>(t, d, K, n_more, n, act, x, s, more);
         a.zmask = more;
         a.mask_exact = true;
+        a.n_rows_dev = n_more;
         launch_gemm_any(t.prec, mode, t.bn, t.mapA1, t.mapT, a, s);
         a.zmask = nullptr;
         a.mask_exact = false;
+        a.n_rows_dev = nullptr;
     } else {
         launch_center(t, d, K, nullptr, n, nullptr, x, s);
         launch_gemm_any(t.prec, mode, t.bn, t.mapA1, t.mapT, a, s);
@@ -2126,7 +2155,7 @@ sb_status tc_loglik_points(const ProbView &pv, const TcWs &t, const double *x, i
     k_tc_lse<<<(n + LSE_ROWS - 1) / LSE_ROWS, LSE_ROWS, lse_smem(K), s>>>(2, K, a.n_ntile, nullptr, n, act, a.qpart,
                                                                          pv.a, (float *)t.p[6], nullptr, ell,
                                                                          (uint32_t *)t.p[10], zmask, nullptr, nullptr,
-                                                                         nullptr);
+                                                                         nullptr, qlast);
     if (grad) {
         launch_scale_z(pv, t, nullptr, n, s);
         a.prof = -1;
