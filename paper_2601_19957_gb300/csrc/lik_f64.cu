@@ -222,12 +222,12 @@ __global__ void __launch_bounds__(NT) k_zgemm_f64_listed(LikF64Args a, const int
         __syncthreads();  // the shared tiles are free for the next one
 }
 
-// The row's place in per-component lists: one atomic per warp and component (the order
-// inside a list does not reach the results, which are stored by row).
-__device__ __forceinline__ void append(bool put, int k, int n, int K, int cap, int32_t *list, int32_t *cnt) {
+// The row's places in the lists of the components of `mask`: one atomic per warp and component
+// (the order inside a list does not reach the results, which are stored by row).
+__device__ __forceinline__ void append(uint64_t mask, int n, int K, int cap, int32_t *list, int32_t *cnt) {
     const int lane = threadIdx.x & 31;
     for (int c = 0; c < K; ++c) {
-        const unsigned m = __ballot_sync(0xffffffffu, put && k == c);
+        const unsigned m = __ballot_sync(0xffffffffu, (mask >> c) & 1ull);
         if (!m) continue;
         int base = 0;
         if (lane == __ffs(m) - 1) base = atomicAdd(&cnt[c], __popc(m));
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(128) k_grp_lead(LikF64Args a, Lists L) {
         }
         L.lead[n] = lead;
     }
-    append(n < n_rows, lead, n, K, a.n_rows, L.l1, L.c1);
+    append(n < n_rows ? 1ull << lead : 0ull, n, K, a.n_rows, L.l1, L.c1);
 }
 
 // The components a row needs besides its leading one (see the header).
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(128) k_grp_need(LikF64Args a, Lists L) {
         L.mask[n] = mask;
         mask &= ~(1ull << j);
     }
-    for (int k = 0; k < K; ++k) append((mask >> k) & 1ull, k, n, K, a.n_rows, L.l2 + 0, L.c2);
+    append(mask, n, K, a.n_rows, L.l2, L.c2);
 }
 
 // Per point: l = LSE_k (a_k - q_k/2) and the responsibilities r_k. GROUPED: over the
@@ -340,8 +340,8 @@ __global__ void __launch_bounds__(128) k_lse_f64(LikF64Args a, Lists L) {
         }
     }
     if (GROUPED && a.G) {
-        append(n < n_rows && !multi, one, n, K, a.n_rows, L.lg, L.cg);
-        append(multi, 0, n, 1, a.n_rows, L.lm, L.cm);
+        append(n < n_rows && !multi ? 1ull << one : 0ull, n, K, a.n_rows, L.lg, L.cg);
+        append(multi ? 1ull : 0ull, n, 1, a.n_rows, L.lm, L.cm);
     }
 }
 
