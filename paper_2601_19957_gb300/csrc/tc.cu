@@ -1463,7 +1463,8 @@ void tune_store_locked() {
     std::fclose(f);
 }
 
-float time_tile(const ProbView &pv, TcWs &t, int bn, cudaStream_t s) {
+// Best of `reps` launch pairs after one that warms up, in ms (-1 on failure).
+float time_tile(const ProbView &pv, TcWs &t, int bn, int reps, cudaStream_t s) {
     const int d = pv.d, K = pv.K, ldp = ldp_of(d, t.prec);
     TcWs u = t;
     u.bn = bn;
@@ -1478,10 +1479,7 @@ float time_tile(const ProbView &pv, TcWs &t, int bn, cudaStream_t s) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return -1.f;
     float best = -1.f;
-    // the best of six: one launch varies by 2 %, and a width within 3 % of another that wins by
-    // chance changes the order of the |z|^2 partial sums from one process to the next (of two
-    // launches d = 300, K = 3 in TF32 gave 128 or 256 columns)
-    for (int rep = 0; rep < 7; ++rep) {
+    for (int rep = 0; rep <= reps; ++rep) {
         cudaEventRecord(e0, s);
         launch_gemm_any(u.prec, MODE_ZW, bn, u.mapA1, u.mapT, a, s);
         launch_gemm_any(u.prec, MODE_G, bn, u.mapZ, u.mapB, a, s);
@@ -1489,7 +1487,7 @@ float time_tile(const ProbView &pv, TcWs &t, int bn, cudaStream_t s) {
         if (cudaEventSynchronize(e1) != cudaSuccess) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        if (rep > 0 && (best < 0.f || ms < best)) best = ms;  // first repetition warms up
+        if (rep > 0 && (best < 0.f || ms < best)) best = ms;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1508,16 +1506,43 @@ int pick_tile(const ProbView &pv, TcWs &t, cudaStream_t s) {
     if (cudaStreamIsCapturing(s, &cst) != cudaSuccess || cst != cudaStreamCaptureStatusNone)
         return bn;  // no timing inside a capture: the heuristic width, not remembered
     if (!(off && off[0] == '0')) {
-        // widest tile first; a narrower one must be at least 3 % faster to win,
-        // so timing noise between near-equal tiles does not flip the choice
-        float best = -1.f;
-        for (int cand : {256, 128, 64}) {
-            if (cand > 64 && (pv.d + 63) / 64 * 64 <= cand / 2) continue;  // tile mostly padding
-            const float ms = time_tile(pv, t, cand, s);
-            if (ms > 0.f && (best < 0.f || ms < 0.97f * best)) {
-                best = ms;
-                bn = cand;
+        // widest tile first; a narrower one must be at least 3 % faster to win, so timing noise
+        // between near-equal tiles does not flip the choice. Two launches each tell most widths
+        // apart; where two of them lie within twice the 2 % that a launch varies by from that
+        // line, the fast ones get four more (of two launches alone d = 300, K = 3 in TF32 gave
+        // 128 columns in one process and 256 in the next, which changes the order of the |z|^2
+        // partial sums)
+        constexpr int kCand = 3, width[kCand] = {256, 128, 64};
+        float ms[kCand], least = -1.f;
+        for (int c = 0; c < kCand; ++c) {
+            ms[c] = -1.f;
+            if (width[c] > 64 && (pv.d + 63) / 64 * 64 <= width[c] / 2) continue;  // tile mostly padding
+            ms[c] = time_tile(pv, t, width[c], 2, s);
+            if (ms[c] > 0.f && (least < 0.f || ms[c] < least)) least = ms[c];
+        }
+        auto pick = [&](bool &close) {
+            float best = -1.f;
+            int won = bn;
+            close = false;
+            for (int c = 0; c < kCand; ++c) {
+                if (!(ms[c] > 0.f)) continue;
+                if (best > 0.f) close = close || fabsf(ms[c] - 0.97f * best) < 0.04f * best;
+                if (best < 0.f || ms[c] < 0.97f * best) {
+                    best = ms[c];
+                    won = width[c];
+                }
             }
+            return won;
+        };
+        bool close = false;
+        bn = pick(close);
+        if (close) {
+            for (int c = 0; c < kCand; ++c)
+                if (ms[c] > 0.f && ms[c] < 1.1f * least) {
+                    const float again = time_tile(pv, t, width[c], 4, s);
+                    if (again > 0.f && again < ms[c]) ms[c] = again;
+                }
+            bn = pick(close);
         }
     }
     g_tune[key] = bn;
