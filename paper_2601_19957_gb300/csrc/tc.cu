@@ -1157,7 +1157,8 @@ __device__ __forceinline__ float round_op(double x) {
 }
 // x split into hi + lo of the operand precision: hi = round(x), lo = round(x - hi). x - hi =
 // (t - hi) + rest with t - hi exact; its FP32 rounding decides lo unless it falls on (bf16),
-// or next to (tf32), the midpoint of two operand values, where FP64 does.
+// or next to (tf32), the midpoint of two operand values, where FP64 does. (A remainder below
+// FP32's resolution of x, where the two cancel, is that of FP64 within 2^-48 of x.)
 template <int PREC>
 __device__ __noinline__ float split_lo_slow(double x, float hi) {
     return round_op_slow<PREC>(x - (double)hi);

@@ -150,3 +150,95 @@ def test_distance_test_at_the_ends(dev):
             with np.errstate(invalid="ignore"):
                 got, want = _far(dev, x, np.full(x.shape, b), np.full(x.shape, tau))
             assert np.array_equal(got, want), (b, tau)
+
+
+def _doubles(seed, n=200000):
+    """Random bit patterns over all exponents, with ties, ends of the ranges and specials."""
+    rng = np.random.default_rng(seed)
+    bits = rng.integers(0, 1 << 63, n, dtype=np.uint64) | (rng.integers(0, 2, n, dtype=np.uint64) << np.uint64(63))
+    near = (rng.integers(860, 1160, n, dtype=np.uint64) << np.uint64(52)) | (bits & np.uint64((1 << 52) - 1))
+    # halfway between neighbours of FP32, bf16 and tf32, and a unit beside it
+    tie = []
+    for keep in (23, 10, 7):
+        b = near & ~np.uint64((1 << (52 - keep)) - 1) | np.uint64(1 << (51 - keep))
+        tie += [b, b + np.uint64(1), b - np.uint64(1)]
+    sign = rng.integers(0, 2, n, dtype=np.uint64) << np.uint64(63)
+    special = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, -5e-324, 2.0 ** -126, 2.0 ** -149, 2.0 ** -150,
+                        2.0 ** -151, np.nextafter(2.0 ** -126, 0), 2.0 ** 128, np.nextafter(2.0 ** 128, 0),
+                        (2 - 2.0 ** -24) * 2.0 ** 127, np.finfo(np.float32).max, np.finfo(np.float64).max, 1.0, -1.0])
+    return np.concatenate([bits.view(np.float64), (near | sign).view(np.float64)] +
+                          [t.view(np.float64) for t in tie] + [special])
+
+
+def _same(a, b):
+    """Equal bits, or both NaN."""
+    u = np.uint32 if a.dtype == np.float32 else np.uint64
+    return (a.view(u) == b.view(u)) | (np.isnan(a) & np.isnan(b))
+
+
+def test_double_to_float_is_the_conversion(dev):
+    x = _doubles(1)
+    y = np.empty(x.shape, np.float32)
+    dev("t_f32", x.size, x, y)
+    with np.errstate(over="ignore", invalid="ignore", under="ignore"):
+        assert _same(y, x.astype(np.float32)).all()
+
+
+def test_float_to_double_is_the_conversion(dev):
+    rng = np.random.default_rng(2)
+    x = np.concatenate([rng.integers(0, 1 << 32, 400000, dtype=np.uint64).astype(np.uint32).view(np.float32),
+                        np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1e-45, -1e-45, 2.0 ** -126, 3.4028235e38], np.float32)])
+    y = np.empty(x.shape, np.float64)
+    dev("t_f64", x.size, x, y)
+    with np.errstate(invalid="ignore"):
+        assert _same(y, x.astype(np.float64)).all()
+
+
+def test_reciprocal_is_within_a_unit_and_the_corrected_one_rounds(dev):
+    """recip: one unit in the last place. recip_as<true>: a division's rounding, where the
+    correction step's products do not underflow (a third-order step then one of Newton)."""
+    x = _doubles(3)
+    x = x[np.isfinite(x) & (x != 0)]
+    x = np.concatenate([x, 1.0 + np.arange(2000) * 2.0 ** -52, 2.0 - np.arange(1, 2000) * 2.0 ** -52])
+    y, z = np.empty_like(x), np.empty_like(x)
+    dev("t_recip", x.size, x, y, z)
+    with np.errstate(over="ignore"):
+        want = 1.0 / x
+    ok = np.isfinite(want)
+    with np.errstate(invalid="ignore"):
+        assert np.all(np.abs(y - want)[ok] <= np.spacing(np.abs(want))[ok])
+        assert _same(y, want)[~ok].all()
+    e = (x.view(np.uint64) >> np.uint64(52)) & np.uint64(0x7ff)
+    mid = (e >= 64) & (e <= 1982)
+    assert np.array_equal(z[mid], want[mid])
+    normal = ok & (np.abs(want) >= 2.0 ** -1022)
+    assert np.all(np.abs(z - want)[normal] <= np.spacing(np.abs(want))[normal])
+
+
+def test_truncation_and_rest_add_up(dev):
+    x = _doubles(4)
+    t, r = np.empty(x.shape, np.float32), np.empty(x.shape, np.float32)
+    ok = np.empty(x.shape, np.int8)
+    dev("t_split24", x.size, x, t, r, ok)
+    a = np.abs(x)
+    inside = (a >= 2.0 ** -63) & (a < 2.0 ** 64)
+    assert np.array_equal(ok.astype(bool), inside | (x == 0))
+    x, t, r = x[inside], t[inside], r[inside]
+    rest = x - t.astype(np.float64)  # exact: x's last 29 bits
+    assert np.all(np.abs(t) <= np.abs(x)) and np.all(np.abs(rest) < np.abs(t) * 2.0 ** -22)
+    assert np.array_equal(r, rest.astype(np.float32))
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+def test_operand_split_is_the_fp64_one(dev, prec):
+    """hi always; lo wherever the remainder is above FP32's resolution of x (below it, where the
+    truncation and the rest cancel, within 2^-48 of x)."""
+    x = _doubles(5 + prec)
+    x = x[np.isfinite(x) & (np.abs(x) < 1e38)]
+    h, l, h0, l0 = (np.empty(x.shape, np.float32) for _ in range(4))
+    dev("t_split", x.size, prec, x, h, l, h0, l0)
+    assert np.array_equal(h, h0)  # (a zero may lose its sign)
+    rem = np.abs(x - h0.astype(np.float64))
+    far = rem > np.abs(x) * 2.0 ** -24
+    assert np.array_equal(l[far], l0[far]), np.count_nonzero(l[far] != l0[far])
+    assert np.all(np.abs(l.astype(np.float64) - l0) <= np.abs(x) * 2.0 ** -48)
