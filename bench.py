@@ -430,6 +430,16 @@ def fp64_roofline(sb, prof_ms, prof_n, prof_steps, lg_per_step, d, K):
             "peak_source": "of measured FP64 FMA loop (fp64_peak)"}
 
 
+def factorization_rate(d, n_modes, launches, ms, peak_tflops):
+    """FP64 rate of the factorisations of n_modes Hessians (d^3 / 3 flop each) that ran in
+    `launches` launches, a group of modes in each, taking ms together."""
+    out = {"factorizations": n_modes if launches else 0, "launches": launches}
+    if launches > 0:
+        rate = n_modes * d ** 3 / 3.0 / (ms / 1e3) / 1e12
+        out.update({"ms_per_launch": ms / launches, "fp64_TFLOPs": rate, "frac": rate / peak_tflops})
+    return out
+
+
 def run_adjoint(sb, args):
     """Forward log Z (the headline solve: discovery, ChiSao, Laplace over every final
     sample; sunburst-only with --no-chisao) and the hand-written adjoint d log Z / d mu_k,
@@ -461,8 +471,8 @@ def run_adjoint(sb, args):
     d, K, nm = inst.d, inst.K, out.n_modes
     # the blocked Cholesky runs where a mode is not one-hot: an overlapping pair of
     # components at the same d (means 2 apart, standard deviations 0.6-1, as in the
-    # adjoint's GPU test), whose backward pass factors H at both modes (d^3 / 3 flop
-    # each); CUDA events around the factorisation alone in one backward call
+    # adjoint's GPU test), whose backward pass factors H at both modes (in one launch);
+    # CUDA events around the factorisation alone in one backward call
     import numpy as np
     from paper_2601_19957_gb300.instances import SolveConfig, make_instance
 
@@ -492,12 +502,8 @@ def run_adjoint(sb, args):
     L.sb_profile_read(prof_ms, prof_n)
     peak = fp64_peak(sb)
     chol = {"workload": f"d={d}, two overlapping components (means 2 apart), {oo.n_modes} modes not one-hot",
-            "ms_backward": dt_ov * 1e3, "factorizations": int(prof_n[6]), "peak_source": peak["source"],
-            "fp64_peak_TFLOPs": peak["tflops"]}
-    if prof_n[6] > 0:
-        chol_ms = prof_ms[6] / int(prof_n[6])
-        rate = d ** 3 / 3.0 / (chol_ms / 1e3) / 1e12
-        chol.update({"ms_per_factorization": chol_ms, "fp64_TFLOPs": rate, "frac": rate / peak["tflops"]})
+            "ms_backward": dt_ov * 1e3, "peak_source": peak["source"], "fp64_peak_TFLOPs": peak["tflops"]}
+    chol.update(factorization_rate(d, oo.n_modes, int(prof_n[6]), prof_ms[6], peak["tflops"]))
     print(json.dumps({"case": "adjoint", "workload": f"d={d} K={K}, {cfg.n_starts} starts, m={cfg.m}",
                       "forward": "discovery + ChiSao + Laplace" if use_chisao else "sunburst-only discovery + Laplace",
                       "n_modes": nm, "ms_forward": dt_f * 1e3, "ms_backward": dt_b * 1e3, "overlapping_modes": chol,

@@ -13,3 +13,11 @@ def test_fp64_roofline_includes_the_step_kernels(monkeypatch):
     flop = 1.4e6 * 2 * 4 * 64 * 65
     assert r["achieved"] == pytest.approx(flop / 37e-3 / 1e9)
     assert r["frac"] == pytest.approx(r["achieved"] / 1e3)
+
+
+def test_factorizations_of_a_group_of_modes_share_a_launch():
+    """Two modes at d = 1024 factored in one launch of 1.5 ms."""
+    r = bench.factorization_rate(1024, 2, 1, 1.5, 1.0)
+    assert r["factorizations"] == 2 and r["launches"] == 1 and r["ms_per_launch"] == 1.5
+    assert r["frac"] == r["fp64_TFLOPs"] == pytest.approx(2 * 1024 ** 3 / 3 / 1.5e-3 / 1e12)
+    assert bench.factorization_rate(1024, 2, 0, 0.0, 1.0) == {"factorizations": 0, "launches": 0}
