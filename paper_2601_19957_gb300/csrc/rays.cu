@@ -170,7 +170,8 @@ __device__ __forceinline__ void sample_key(const double *ell, int64_t f, uint64_
 }
 
 // The bucket that holds the n_starts-th sample (state[0]), the rank of that sample inside it
-// (state[1], from 1), and the list of the bucket's samples (at most one per ray): every CTA
+// (state[1], from 1), and the list of the bucket's samples (one per ray at most of finite ones,
+// but every NaN sample has tier 1, rank 0, so the list has room for all samples): every CTA
 // finds the bucket from the histogram itself.
 __global__ void __launch_bounds__(256) k_cut_gather(const int32_t *bucket, int64_t total, const uint32_t *hist,
                                                     int nbins, int n_starts, uint64_t *state, int32_t *list) {

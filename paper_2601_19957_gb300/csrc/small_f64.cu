@@ -20,8 +20,8 @@
 // Every sum is formed in the order of the general path (lik_f64.cu, lbfgs.cu), whatever
 // LPW: the results are the same bits.
 // Measured against that path (GEMM tiles, five launches a round): a whole ChiSao solve at
-// d = 64, K = 4, 4096 walkers 230 -> 44.7 ms, the sunburst solve of one Gaussian at
-// d = 8, 64 walkers 3.4 -> 1.0 ms, l and grad l at one point (d = 64, K = 4) 363 -> 41 us.
+// d = 64, K = 4, 4096 walkers 231 -> 42 ms, the sunburst solve of one Gaussian at d = 8, 64
+// walkers 3.7 -> 0.88 ms, l and grad l at one point (d = 64, K = 4) 363 -> 24 us.
 #include "sb_small_f64.cuh"
 
 #include <type_traits>
